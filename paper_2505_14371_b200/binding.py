@@ -1,9 +1,10 @@
-"""Thin ctypes binding of liblq.so: argument marshalling only.
+"""Thin binding of liblq.so: argument marshalling only.
 
 Every step of the hot path runs inside the CUDA library; this module only converts torch
 tensors to raw device pointers and passes the current CUDA stream.  Function names mirror
-the C entry points declared in include/lq.h.  There is no CPU fallback: if the library is
-missing, importing it raises.
+the C entry points declared in include/lq.h.  The calls of an iteration go through `_native`
+(csrc/lq_native.cpp: the same checks, without ctypes' cost per argument), the others through
+ctypes.  There is no CPU fallback: if a library is missing, loading it raises.
 """
 from __future__ import annotations
 
@@ -15,6 +16,7 @@ import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "liblq.so")
+NATIVE_PATH = os.path.join(_HERE, "_native.so")
 
 NUM_BINS = 386
 HIST_STRIDE = 512
@@ -39,11 +41,12 @@ class LqError(RuntimeError):
 
 
 _lib = None
+_native = None
 
 
 def load_library() -> C.CDLL:
     """dlopen liblq.so and declare the C signatures.  Raises if the library was not built."""
-    global _lib
+    global _lib, _native
     if _lib is not None:
         return _lib
     if not os.path.exists(LIB_PATH):
@@ -96,7 +99,11 @@ def load_library() -> C.CDLL:
     L.lq_last_error.argtypes = []; L.lq_last_error.restype = C.c_char_p
     for name in EXPORTS:
         getattr(L, name)              # raises AttributeError if the library lacks an entry point
-    _lib = L
+    if not os.path.exists(NATIVE_PATH):
+        raise LqError(f"{NATIVE_PATH} is missing: build it with `python -m paper_2505_14371_b200.build`")
+    from . import _native as native
+    native.register_error(LqError)
+    _native, _lib = native, L
     return L
 
 
@@ -126,9 +133,8 @@ def lq_vector_norm_static(v: torch.Tensor, q: int, norm_out: torch.Tensor,
     array: no plan and no allocation below this call.  For callers whose device memory is all
     spoken for, or who cannot afford the synchronisation an allocation implies.  Calls must not
     overlap on the GPU (they share the scratch)."""
-    _check(load_library().lq_vector_norm_static(_ptr(v, torch.float32), v.numel(), int(q),
-                                                _ptr(norm_out, torch.float32), _ptr(status_out, torch.int32),
-                                                _stream()))
+    load_library()
+    _native.lq_vector_norm_static(v, int(q), norm_out, status_out)
 
 
 def lq_code_build(weights) -> List[int]:
@@ -161,7 +167,7 @@ class Plan:
         bb = (C.c_int32 * max(n, 1))(*self.bits)
         h = C.c_void_p()
         _check(L.lq_plan_create(C.byref(h), n, sizes, bb, self.q, self.num_workers, C.c_uint64(self.seed)))
-        self._h = h
+        self._h, self._addr = h, h.value
         self.num_layers = n
         self.padded_elems = int(L.lq_plan_padded_elems(h))
         self.packed_words = int(L.lq_plan_packed_words(h))
@@ -175,7 +181,7 @@ class Plan:
     def close(self) -> None:
         if getattr(self, "_h", None):
             load_library().lq_plan_destroy(self._h)
-            self._h = None
+            self._h = self._addr = None
 
     def __del__(self):
         try:
@@ -226,19 +232,14 @@ class Plan:
 
     # ---- hot path -----------------------------------------------------------------------
     def lq_layer_norms(self, grads: torch.Tensor, norms: torch.Tensor) -> None:
-        _check(load_library().lq_layer_norms(self._h, _ptr(grads, torch.float32), _ptr(norms, torch.float32),
-                                             _stream()))
+        _native.lq_layer_norms(self._addr, grads, norms)
 
     def lq_quantize_pack(self, grads, step: int, packed, norms, hist=None, prev_packed=None,
                          prev_norms=None) -> None:
-        _check(load_library().lq_quantize_pack(
-            self._h, _ptr(grads, torch.float32), C.c_uint32(step & 0xFFFFFFFF), _ptr(packed, torch.int32),
-            _ptr(norms, torch.float32), _ptr(hist, torch.int32), _ptr(prev_packed, torch.int32),
-            _ptr(prev_norms, torch.float32), _stream()))
+        _native.lq_quantize_pack(self._addr, grads, step, packed, norms, hist, prev_packed, prev_norms)
 
     def lq_fit_levels(self, hist, norms, num_samples: int) -> None:
-        _check(load_library().lq_fit_levels(self._h, _ptr(hist, torch.int32), _ptr(norms, torch.float32),
-                                            num_samples, _stream()))
+        _native.lq_fit_levels(self._addr, hist, norms, num_samples)
 
     def lq_fit_levels_shared(self, hist, norms, num_samples: int, layer_type: Sequence[int]) -> None:
         ids = (C.c_int32 * max(self.num_layers, 1))(*[int(t) for t in layer_type])
@@ -246,18 +247,14 @@ class Plan:
                                                    num_samples, ids, _stream()))
 
     def lq_decode_aggregate(self, packed, norms, gbar) -> None:
-        _check(load_library().lq_decode_aggregate(self._h, _ptr(packed, torch.int32), _ptr(norms, torch.float32),
-                                                  _ptr(gbar, torch.float32), _stream()))
+        _native.lq_decode_aggregate(self._addr, packed, norms, gbar)
 
     def qoda_init(self, X1, Y, Xhalf) -> None:
         _check(load_library().qoda_init(self._h, _ptr(X1, torch.float32), _ptr(Y, torch.float32),
                                         _ptr(Xhalf, torch.float32), _stream()))
 
     def qoda_step(self, packed, norms, X1, Y, Xhalf, X=None, gbar=None) -> None:
-        _check(load_library().qoda_step(self._h, _ptr(packed, torch.int32), _ptr(norms, torch.float32),
-                                        _ptr(X1, torch.float32), _ptr(Y, torch.float32),
-                                        _ptr(Xhalf, torch.float32), _ptr(X, torch.float32),
-                                        _ptr(gbar, torch.float32), _stream()))
+        _native.qoda_step(self._addr, packed, norms, X1, Y, Xhalf, X, gbar)
 
     def qoda_get_scalars(self):
         t, S, eta = C.c_int64(), C.c_double(), C.c_double()
@@ -265,12 +262,10 @@ class Plan:
         return t.value, S.value, eta.value
 
     def lq_level_probabilities(self, hist, norms, num_samples: int, probs, staged: bool = False) -> None:
-        _check(load_library().lq_level_probabilities(self._h, _ptr(hist, torch.int32), _ptr(norms, torch.float32),
-                                                     num_samples, 1 if staged else 0, _ptr(probs, torch.float64),
-                                                     _stream()))
+        _native.lq_level_probabilities(self._addr, hist, norms, num_samples, staged, probs)
 
     def lq_symbol_counts(self, packed, counts) -> None:
-        _check(load_library().lq_symbol_counts(self._h, _ptr(packed, torch.int32), _ptr(counts, torch.int32), _stream()))
+        _native.lq_symbol_counts(self._addr, packed, counts)
 
     # ---- entropy stage --------------------------------------------------------------------
     def lq_code_set(self, layer: int, lengths) -> None:
@@ -287,14 +282,10 @@ class Plan:
         return int(load_library().lq_plan_blocks(self._h))
 
     def lq_entropy_encode(self, packed, stream_words, block_offsets, run_offsets=None) -> None:
-        _check(load_library().lq_entropy_encode(self._h, _ptr(packed, torch.int32), _ptr(stream_words, torch.int32),
-                                                stream_words.shape[1], _ptr(block_offsets, torch.int32),
-                                                _ptr(run_offsets, torch.int16), _stream()))
+        _native.lq_entropy_encode(self._addr, packed, stream_words, block_offsets, run_offsets)
 
     def lq_entropy_decode(self, stream_words, block_offsets, packed, run_offsets=None) -> None:
-        _check(load_library().lq_entropy_decode(self._h, _ptr(stream_words, torch.int32), stream_words.shape[1],
-                                                _ptr(block_offsets, torch.int32), _ptr(run_offsets, torch.int16),
-                                                _ptr(packed, torch.int32), _stream()))
+        _native.lq_entropy_decode(self._addr, stream_words, block_offsets, run_offsets, packed)
 
     def empty_run_offsets(self, device="cuda"):
         """[K][blocks][8] int16 buffer for the run offsets of the entropy stage."""
