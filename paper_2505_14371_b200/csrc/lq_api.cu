@@ -111,7 +111,6 @@ void free_plan(lq_plan* p)
     cudaFree(p->search.lut); cudaFree(p->search.ld); cudaFree(p->search.fast);
     cudaFree(p->dev.norm_partial); cudaFree(p->dev.stat_partial); cudaFree(p->dev.sq_diff);
     cudaFree(p->dev.rnorm); cudaFree(p->dev.status); cudaFree(p->dev.scalars); cudaFree(p->d_code_enc); cudaFree(p->d_code_dec); cudaFree(p->d_code_bad); cudaFree(p->code_scratch.lane_bits); cudaFree(p->code_scratch.scan_part); cudaFree(p->d_member_off); cudaFree(p->d_member_layer); cudaFree(p->dev.alt_partial); cudaFree(p->dev.layer_total); cudaFree(p->d_row_mask[0]); cudaFree(p->d_row_mask[1]);
-    cudaFree(p->dev.block_live);
     cudaFree(p->dev.energy_partial); cudaFree(p->dev.flag_partial); cudaFree(p->dev.layer_weight);
     for (auto& r : p->prof_recs) { cudaEventDestroy(r.a); cudaEventDestroy(r.b); }
     for (auto e : p->prof_pool) cudaEventDestroy(e);
@@ -140,15 +139,15 @@ cudaError_t timed(lq_plan* p, int id, cudaStream_t s, F&& launch)
     return e;
 }
 
-// Per block the bitmask of workers that sent anything, if `packed` is the message the plan's last lq_quantize_pack
+// The zero-row masks of the message's input, if `packed` is the message the plan's last lq_quantize_pack
 // wrote for all K <= 32 workers in the layer or global scope (the decoder then leaves all-zero blocks unread);
 // otherwise nullptr.
-const uint32_t* message_masks(const lq_plan* p, const uint32_t* packed)
+const uint8_t* message_masks(const lq_plan* p, const uint32_t* packed)
 {
     const PlanDev& d = p->dev;
     if (!p->have_message || !p->masks_known || !p->message_intact || d.bucket_norm || packed != p->last_packed) return nullptr;
     if (d.worker0 != 0 || d.worker_count != d.num_workers || d.num_workers > 32) return nullptr;
-    return d.block_live;
+    return d.row_mask;
 }
 
 template <typename T>
@@ -192,13 +191,28 @@ int lq_plan_create(lq_plan** out, int32_t num_layers, const int64_t* layer_sizes
     lq_plan* p = new (std::nothrow) lq_plan;
     if (!p) return fail(LQ_ENOMEM, "host allocation failed");
     int64_t elem = 0, word = 0, ntiles = 0, blocks = 0;
-    // tile size: as large as possible while (tiles x workers) still fills the GPU several times over
-    int tile_blocks = kTileBlocks;
+    // tile size: as large as possible while (tiles x workers) still fills the GPU several times over; below 32 blocks only
+    // while the tiles do not fill it once (4 CTAs on each of the 148 SMs).  Sub-tiles likewise, without the workers (the
+    // decoder has one CTA for all of them).
+    int tile_blocks = kTileBlocks, sub_blocks = kSubBlocks, dec_blocks = kSubBlocks, most_bits = 1;
+    int64_t most_blocks = 0;
     {
         int64_t total = 0;
         for (int m = 0; m < num_layers; ++m)
-            if (layer_sizes[m] > 0) total += (layer_sizes[m] + kBlockCoords - 1) / kBlockCoords;
-        while (tile_blocks > kSubBlocks && (total / tile_blocks) * num_workers < 4096) tile_blocks /= 2;
+            if (layer_sizes[m] > 0) {
+                const int64_t n = (layer_sizes[m] + kBlockCoords - 1) / kBlockCoords;
+                total += n;
+                most_blocks = std::max(most_blocks, n);
+            }
+        constexpr int kWave = 4 * 148;
+        while (tile_blocks > 32 && (total / tile_blocks) * num_workers < 4096) tile_blocks /= 2;
+        while (tile_blocks > 8 && (total / tile_blocks) * num_workers < kWave) tile_blocks /= 2;
+        while (sub_blocks > 8 && (total / sub_blocks) * num_workers < kWave) sub_blocks /= 2;
+        sub_blocks = std::min(sub_blocks, tile_blocks);
+        // the decoder's CTAs (4 warps) serve all workers: 4 blocks while every SM has one CTA or more, else 1 block
+        dec_blocks = sub_blocks;
+        while (dec_blocks > 4 && total / dec_blocks < 2 * kWave) dec_blocks /= 2;
+        if (total < kWave) dec_blocks = 1;
     }
     try {
         p->layers.resize((size_t)num_layers);
@@ -213,6 +227,7 @@ int lq_plan_create(lq_plan** out, int32_t num_layers, const int64_t* layer_sizes
             L.first_tile = (int32_t)ntiles;
             L.ntiles = (L.nblocks + tile_blocks - 1) / tile_blocks;
             L.pad_ = 0;
+            most_bits = std::max(most_bits, b);
             L.block_off = blocks;
             blocks += L.nblocks;
             for (int t = 0; t < L.ntiles; ++t) {
@@ -236,7 +251,13 @@ int lq_plan_create(lq_plan** out, int32_t num_layers, const int64_t* layer_sizes
     PlanDev& d = p->dev;
     d.num_layers = num_layers; d.num_tiles = (int32_t)ntiles; d.num_workers = num_workers; d.q = q;
     d.worker0 = 0; d.worker_count = num_workers;
-    d.sub_tiles = tile_blocks / kSubBlocks;
+    d.sub_blocks = sub_blocks;
+    d.most_bits = most_bits;
+    d.dec_blocks = dec_blocks;
+    d.dec_shift = 0;
+    while ((dec_blocks << d.dec_shift) < tile_blocks) ++d.dec_shift;
+    d.most_blocks = (int32_t)std::min<int64_t>(most_blocks, INT32_MAX);
+    d.sub_tiles = tile_blocks / sub_blocks;
     d.sub_shift = 0;
     while ((1 << d.sub_shift) < d.sub_tiles) ++d.sub_shift;
     d.padded_elems = elem; d.packed_words = word; d.total_blocks = blocks;
@@ -293,17 +314,16 @@ int lq_plan_create(lq_plan** out, int32_t num_layers, const int64_t* layer_sizes
     if (e == cudaSuccess) e = dev_alloc_zero(&d.rnorm, KL);
     if (e == cudaSuccess) e = dev_alloc_zero(&d.status, KL);
     if (e == cudaSuccess) e = dev_alloc_zero(&d.layer_total, KL);
-    if (e == cudaSuccess) e = dev_alloc_zero(&d.block_live, (size_t)(blocks ? blocks : 1));
     if (e == cudaSuccess) e = dev_alloc_zero(&d.energy_partial, KT);
     if (e == cudaSuccess) e = dev_alloc_zero(&d.flag_partial, KT);
     if (e == cudaSuccess) e = dev_alloc_zero(&d.layer_weight, KL);
     if (e == cudaSuccess) e = dev_alloc_zero(&p->d_member_off, nl + 1);
     if (e == cudaSuccess) e = dev_alloc_zero(&p->d_member_layer, nl);
-    if (e == cudaSuccess) e = dev_alloc_zero(&d.alt_partial, 2 * (size_t)(ntiles ? ntiles : 1) * (size_t)d.sub_tiles);
+    if (e == cudaSuccess) e = dev_alloc_zero(&d.alt_partial, 2 * ((size_t)(ntiles ? ntiles : 1) << d.dec_shift));
     for (int i = 0; i < 2; ++i)
         if (e == cudaSuccess) e = dev_alloc_zero(&p->d_row_mask[i], (size_t)num_workers * (size_t)(blocks ? blocks : 1));
     d.row_mask = p->d_row_mask[0]; d.row_mask_prev = nullptr;
-    if (e == cudaSuccess) e = dev_alloc_zero(&d.scalars, 1);
+    if (e == cudaSuccess) e = dev_alloc_zero(&d.scalars, 2);
     if (e == cudaSuccess && !p->layers.empty())
         e = cudaMemcpy(p->d_layers, p->layers.data(), p->layers.size() * sizeof(LayerDesc), cudaMemcpyHostToDevice);
     if (e == cudaSuccess && !p->tiles.empty())
@@ -567,9 +587,7 @@ int qoda_step(lq_plan* plan, const uint32_t* packed, const float* norms, const f
     if (!plan->qoda_ready) return fail(LQ_ESTATE, "qoda_step before qoda_init");
     if (!plan->stat_pending) return fail(LQ_ESTATE, "qoda_step needs a new lq_quantize_pack message");
     cudaStream_t s = (cudaStream_t)stream;
-    const uint32_t* live = message_masks(plan, packed);
-    if (live)                        // folds the K workers' zero-row masks into one word per block
-        LQ_CUDA(timed(plan, LQ_KERNEL_BLOCK_LIVE, s, [&] { return launch_block_live(plan->dev, s); }));
+    const uint8_t* masks = message_masks(plan, packed);
     if (plan->xsum)                  // X_{t+1/2}, before this step overwrites it
         LQ_CUDA(timed(plan, LQ_KERNEL_AVERAGE, s, [&] { return launch_average(plan->dev, Xhalf, plan->xsum, s); }));
     if (plan->alt_qhat > 0.0) {
@@ -577,14 +595,15 @@ int qoda_step(lq_plan* plan, const uint32_t* packed, const float* norms, const f
         LQ_CUDA(timed(plan, LQ_KERNEL_QODA_SCALARS, s, [&] { return launch_alt_scalars(plan->dev, qh, s); }));
         LQ_CUDA(timed(plan, LQ_KERNEL_DECODE, s, [&] {
             return launch_decode(plan->dev, packed, norms, plan->d_levels_enc[plan->cur], X1, Y, Xhalf, X_opt,
-                                 gbar_opt, 2, live, s);
+                                 gbar_opt, 2, masks, s);
         }));
         LQ_CUDA(timed(plan, LQ_KERNEL_ALT_FINALIZE, s, [&] { return launch_alt_finalize(plan->dev, s); }));
     } else {
-        LQ_CUDA(timed(plan, LQ_KERNEL_QODA_SCALARS, s, [&] { return launch_qoda_scalars(plan->dev, s); }));
+        if (!rates_in_decoder(plan->dev))
+            LQ_CUDA(timed(plan, LQ_KERNEL_QODA_SCALARS, s, [&] { return launch_qoda_scalars(plan->dev, s); }));
         LQ_CUDA(timed(plan, LQ_KERNEL_DECODE, s, [&] {
             return launch_decode(plan->dev, packed, norms, plan->d_levels_enc[plan->cur], X1, Y, Xhalf, X_opt,
-                                 gbar_opt, 1, live, s);
+                                 gbar_opt, 1, masks, s);
         }));
     }
     plan->stat_pending = false;

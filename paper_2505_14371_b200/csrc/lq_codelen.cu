@@ -80,9 +80,9 @@ __global__ void __launch_bounds__(kThreads) symbol_counts_kernel(PlanDev p, cons
 {
     __shared__ uint32_t cnt[kMaxLevels];
     Tile tile = p.tiles[blockIdx.x >> p.sub_shift];
-    const int sub0 = (blockIdx.x & (p.sub_tiles - 1)) * kSubBlocks;
+    const int sub0 = (blockIdx.x & (p.sub_tiles - 1)) * p.sub_blocks;
     if (sub0 >= tile.nblocks) return;
-    const int sub1 = min(sub0 + kSubBlocks, tile.nblocks);
+    const int sub1 = min(sub0 + p.sub_blocks, tile.nblocks);
     const int layer = tile.layer, k = blockIdx.y;
     const LayerDesc L = p.layers[layer];
     const int C = L.bits + 1, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;

@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(kThreads, 4) entropy_encode_kernel(PlanDev p, 
     __shared__ uint32_t code[2 * kMaxLevels];
     __shared__ uint32_t buf[kModeWrite ? kWarps : 1][kModeWrite ? kCodeBufWords : 1];
     Tile tile = p.tiles[blockIdx.x >> p.sub_shift];
-    const int sub0 = (blockIdx.x & (p.sub_tiles - 1)) * kSubBlocks;
+    const int sub0 = (blockIdx.x & (p.sub_tiles - 1)) * p.sub_blocks;
     if (sub0 >= tile.nblocks) return;
     const int layer = tile.layer, k = blockIdx.y;
     const LayerDesc L = p.layers[layer];
@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(kThreads, 4) entropy_encode_kernel(PlanDev p, 
     J.runs = run_offsets ? run_offsets + ((int64_t)k * p.total_blocks + L.block_off) * LQ_CODE_RUNS : nullptr;
     J.lane_bits = lane_bits + ((int64_t)k * p.total_blocks + L.block_off) * 32;
     J.capacity = capacity; J.size = L.size;
-    J.block0 = tile.block0 + sub0; J.block1 = tile.block0 + min(sub0 + kSubBlocks, tile.nblocks);
+    J.block0 = tile.block0 + sub0; J.block1 = tile.block0 + min(sub0 + p.sub_blocks, tile.nblocks);
     uint32_t* bb = buf[kModeWrite ? (threadIdx.x >> 5) : 0];
     switch (L.bits + 1) {
 #define LQ_CASE(CC) case CC: encode_blocks<CC, kModeWrite != 0>(J, code, bb); break;
@@ -451,7 +451,7 @@ __global__ void __launch_bounds__(kThreads) entropy_decode_runs_kernel(PlanDev p
     __shared__ int ntodo;
     static_assert(kSubBlocks * LQ_CODE_RUNS == kThreads, "one thread per run of a sub-tile");
     const Tile tile = p.tiles[blockIdx.x >> p.sub_shift];
-    const int sub0 = (blockIdx.x & (p.sub_tiles - 1)) * kSubBlocks;
+    const int sub0 = (blockIdx.x & (p.sub_tiles - 1)) * p.sub_blocks;
     if (sub0 >= tile.nblocks) return;
     const int layer = tile.layer, k = blockIdx.y;
     const LayerDesc L = p.layers[layer];
@@ -483,7 +483,7 @@ __global__ void __launch_bounds__(kThreads) entropy_decode_runs_kernel(PlanDev p
     __syncthreads();
 
     bool broken = false, walk = false;
-    if (sub0 + (threadIdx.x >> 3) < tile.nblocks) {
+    if ((int)(threadIdx.x >> 3) < min(p.sub_blocks, tile.nblocks - sub0)) {
         int64_t blk;
         const RunRef r = run_ref(threadIdx.x, blk);
         uint32_t* dst = msg + blk * (int64_t)C * 32;

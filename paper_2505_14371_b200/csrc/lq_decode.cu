@@ -1,76 +1,46 @@
 // DECODE + aggregate of the K workers' messages, alone or fused with the optimistic dual averaging
 // update (Algorithm 1 lines 15-18 and line 10 of the next iteration; Eq. ODA; Eq. general_stepsize).
 //
-// One CTA per sub-tile (up to 32 blocks of 1024 coordinates of one layer, taken round-robin by 8 warps).  A lane
-// owns the same 32 coordinates it owned at encode time, so it reads (b+1) words per worker with
-// 128-byte coalesced warp loads, looks the signed decoded values up by symbol in a per-(worker, layer) table in shared
-// memory, sums them in worker order in registers, and finishes with float4 reads of Y and X_1 and
-// float4 writes of Y and X_{t+3/2}.  Every packed word and every state element is touched once.
+// One CTA of 4 warps per piece of a layer (up to 32 blocks of 1024 coordinates, one block per warp at a time; in plans
+// with fewer blocks than the GPU has warps to give them, the 4 warps share a block, 2 rows each).  A lane owns the same 32
+// coordinates it owned at encode time: it looks the signed decoded values up by symbol in a per-(worker, layer) table in
+// shared memory, sums them in worker order in registers, and finishes with float4 reads of Y and X_1 and float4 writes of
+// Y and X_{t+3/2}.  Every packed word and every state element is touched once.
+//
+// Everything a warp reads from global memory travels by 16-byte asynchronous copies into shared memory of its own: the
+// words of a few workers at a time (a unit), two units deep, and the block's rows of Y and X_1, which arrive while the
+// words are being decoded.  So 16 warps per SM keep up to 210 KB in flight, no load waits in a register, and the accumulators
+// of a whole block fit: per symbol remain shift, mask (which also adds the table's address: tables start at multiples of
+// their size), look-up and add.  The look-ups bound it for many narrow messages (one pass of the SM's shared-memory
+// pipe per 32 symbols), DRAM otherwise.
+#include <algorithm>
+#include <atomic>
+
 #include "lq_internal.cuh"
 
 namespace lq {
 
-constexpr int kWorkerChunk = 8;   // workers whose value tables sit in shared memory at once
-#ifndef LQ_DEC_PARTS
-#define LQ_DEC_PARTS 2
-#endif
-#ifndef LQ_DEC_CTAS
-#define LQ_DEC_CTAS 4
-#endif
-constexpr int kParts = LQ_DEC_PARTS;            // a block is decoded in kParts pieces of 8 / kParts rows
-constexpr int kPartSyms = 32 / kParts;          // symbols of a lane per piece
-constexpr int kPartRows = 8 / kParts;
-constexpr int kStageBytes = kWarps * 2 * kPartRows * 512;   // per CTA: each warp stages its piece's rows of Y and X_1
+constexpr int kDecWarps = 4;
+constexpr int kDecThreads = kDecWarps * 32;
+constexpr int kUnitPlanes = 20;                          // 128-byte planes of words in a unit, most
+constexpr uint32_t kUnitBytes = kUnitPlanes * 128;
+constexpr uint32_t kStateBytes = 2 * kBlockCoords * 4;   // a block's rows of Y, then of X_1
+constexpr uint32_t kTableBytes = 32 * 1024;              // most shared memory for value tables
 
-
-// Adds up to kWorkerChunk workers' decoded half blocks into acc, in worker order.  Half H of a lane's
-// string holds its symbols 16 H .. 16 H + 15 (rows 4 H .. 4 H + 3 of the block); only the words that
-// carry those symbols are read.  All workers' words are requested before the first one is used, so
-// that a warp keeps a few KB in flight.  `table[kk]` holds N * l_j at 2j and -N * l_j at 2j + 1 for
-// worker kk of the chunk.  Bucket scope: table[0] holds the plain signed levels for every worker, and `bn` points
-// at worker k0's norms of this piece's rows (one per row of 128 coordinates; the next worker's `bn_stride` further).
-template <int B, int H, bool kBucket>
-__device__ __forceinline__ void decode_accumulate(float (&acc)[kPartSyms], const uint32_t* __restrict__ words,
-                                                  int64_t worker_stride, int kc,
-                                                  const float (*table)[2 * kMaxLevels],
-                                                  const float* __restrict__ bn, int64_t bn_stride, uint32_t live)
-{
-    // `live`: bit kk clear = worker kk's block is known to be all zero words, which are then not read (their
-    // symbols are 0 and add the table's +0)
-    constexpr int C = B + 1;
-    constexpr int kFirst = (kPartSyms * H * C) >> 5;                  // first and last word of this piece
-    constexpr int kLast = ((kPartSyms * (H + 1) * C) - 1) >> 5;
-    uint32_t w[kWorkerChunk][C];
-#pragma unroll
-    for (int kk = 0; kk < kWorkerChunk; ++kk)
-#pragma unroll
-        for (int i = 0; i < C; ++i)
-            w[kk][i] = (i >= kFirst && i <= kLast && kk < kc && ((live >> kk) & 1u)) ? __ldcs(words + kk * worker_stride + i * 32) : 0u;
-    float nr[kBucket ? kWorkerChunk : 1][kPartRows];
-    if (kBucket) {
-#pragma unroll
-        for (int kk = 0; kk < kWorkerChunk; ++kk)
-#pragma unroll
-            for (int jj = 0; jj < kPartRows; ++jj) nr[kk][jj] = kk < kc ? __ldg(bn + kk * bn_stride + jj) : 0.0f;
-    }
-#pragma unroll
-    for (int kk = 0; kk < kWorkerChunk; ++kk) {
-        if (kk < kc) {
-            const char* tb = reinterpret_cast<const char*>(table[kBucket ? 0 : kk]);
-#pragma unroll
-            for (int p = 0; p < kPartSyms; ++p) {
-                const float val = *reinterpret_cast<const float*>(tb + symbol4_at<C>(w[kk], kPartSyms * H + p));
-                acc[p] += kBucket ? __fmul_rn(val, nr[kk][p >> 2]) : val;
-            }
-        }
-    }
-}
+// workers per unit, and bytes of one worker's words of a block
+template <int B>
+constexpr int kUnitWorkers = kUnitPlanes / (B + 1) < 16 ? kUnitPlanes / (B + 1) : 16;
+template <int B>
+constexpr uint32_t kBlockBytes = (B + 1) * 128;
+// workers whose value tables (2^(b+1) floats each) are in shared memory at once: whole units
+template <int B>
+constexpr int kTableWorkers = ((int)(kTableBytes >> (B + 3)) / kUnitWorkers<B>) * kUnitWorkers<B>;
 
 // The rates one QODA update uses: X_{t+1} = X_1 + eta Y_{t+1}, X_{t+3/2} = X_{t+1} - gamma gbar; eta_cur made X_t.
 struct Rates { float eta, gamma, eta_cur; };
 
 struct DecodeArgs {
-    const uint32_t* live;    // per block of 1024 coordinates: bit k set = worker k's words are not all zero; or nullptr
+    const uint8_t* masks;    // [K][total_blocks] zero-row masks of the message's input (K <= 32), or nullptr
     const uint32_t* packed;
     const float* norms;
     const float* levels;
@@ -79,76 +49,145 @@ struct DecodeArgs {
     float* Xhalf;
     float* X;
     float* gbar;
+    bool form_rates;         // mode 1: the CTAs form the step's rates (rates_in_decoder), else a kernel before has done it
+    bool vec;                // packed (and in bucket scope norms) start on a 16-byte boundary
+    uint32_t table_bytes;    // shared memory for the value tables, a multiple of their size
 };
 
-// Fills the value tables of workers k0 .. k0 + kc - 1 of one layer (CTA-wide, between two barriers); in bucket
-// scope one table of plain signed levels.
+// Fills the value tables of workers k0 .. k0 + kc - 1 of one layer (all threads); in bucket scope one table of plain
+// signed levels.  Symbol = 2 * idx + sign.
 template <bool kBucket>
 __device__ __forceinline__ void fill_tables(const PlanDev& p, const LayerDesc& L, int layer, const DecodeArgs& a,
-                                            float (*table)[2 * kMaxLevels], int k0, int kc)
+                                            float2* table, int k0, int kc)
 {
-    __syncthreads();
-    for (int i = threadIdx.x; i < (kBucket ? 1 : kc) * L.nlevels; i += blockDim.x) {
-        const int kk = i / L.nlevels, j = i - kk * L.nlevels;
-        const float lv = a.levels[(int64_t)layer * kLevelStride + j];
-        const float mag = kBucket ? lv : __fmul_rn(a.norms[(int64_t)(k0 + kk) * p.num_layers + layer], lv);
-        table[kk][2 * j] = mag;                       // symbol = 2 * idx + sign
-        table[kk][2 * j + 1] = -mag;
+    const int n = (kBucket ? 1 : kc) << L.bits;
+    for (int i = threadIdx.x; i < n; i += kDecThreads) {
+        const int kk = i >> L.bits, j = i & (L.nlevels - 1);
+        const float lv = __ldg(a.levels + (int64_t)layer * kLevelStride + j);
+        const float mag = kBucket ? lv : __fmul_rn(__ldg(a.norms + (int64_t)(k0 + kk) * p.num_layers + layer), lv);
+        table[i] = make_float2(mag, -mag);
     }
-    __syncthreads();
 }
 
-// One half block: the mean of the K decoded messages for rows 4 H .. 4 H + 3, then the update.
-// Any worker count: the accumulators live across chunks of kWorkerChunk workers; with a single chunk
-// the tables are filled once per CTA (`resident`).
-template <int B, int H, int kMode, bool kBucket>
-__device__ __forceinline__ void decode_half(const PlanDev& p, const LayerDesc& L, int layer, const DecodeArgs& a,
-                                            float (*table)[2 * kMaxLevels], const Rates& rt, float invK,
-                                            int64_t blk, bool active, bool& resident, float4* stage,
-                                            double& lam_acc, double& mu_acc, uint32_t block_live)
+// What a warp needs to walk its blocks.
+struct Walk {
+    const uint32_t* words;       // the layer's words in worker 0's message
+    const float* bnorms;         // bucket scope: the layer's bucket norms of worker 0
+    int64_t base;                // the layer's first element in a state row
+    int32_t block0, nblocks;     // the CTA's blocks of the layer
+    int32_t size;                // d_m
+    uint32_t tables, units, state;   // shared-memory addresses: value tables, this warp's two units, its state rows
+    int lane, warp;
+};
+
+// Which 16-byte pieces of a unit a lane copies: piece 32 i + lane is piece (32 i + lane) % (8 C) of the words of the
+// unit's worker (32 i + lane) / (8 C).  Worked out once per warp.
+template <int B>
+struct UnitPieces {
+    static constexpr int kPer = (B + 1) * 8, kCount = (kUnitWorkers<B> * kPer + 31) / 32;
+    int64_t off[kCount];         // bytes from the unit's first word
+    uint32_t worker[kCount];     // the worker's bit (0: no such piece)
+    __device__ __forceinline__ UnitPieces(int64_t packed_words, int lane)
+    {
+#pragma unroll
+        for (int i = 0; i < kCount; ++i) {
+            const int c = 32 * i + lane, kk = c / kPer;
+            off[i] = kk * packed_words * 4 + (c - kk * kPer) * 16;
+            worker[i] = kk < kUnitWorkers<B> ? 1u << kk : 0u;
+        }
+    }
+};
+
+// Starts the copies of the words of the workers k0 + (set bits of `live`) of block blk into a unit; in bucket scope
+// every worker's 8 norms of the block go behind the words' space.
+template <int B, bool kBucket>
+__device__ __forceinline__ void request_unit(const PlanDev& p, const DecodeArgs& a, const Walk& w, const UnitPieces<B>& up,
+                                             uint32_t unit, int64_t blk, int k0, uint32_t live)
+{
+    constexpr int C = B + 1;
+    const uint32_t* src = w.words + (int64_t)k0 * p.packed_words + blk * (C * 32);
+    const float* bn = kBucket ? w.bnorms + ((int64_t)k0 * p.total_blocks + blk) * 8 : nullptr;
+    if (a.vec) {
+        const char* from = reinterpret_cast<const char*>(src);
+#pragma unroll
+        for (int i = 0; i < UnitPieces<B>::kCount; ++i)
+            if (live & up.worker[i]) cp_async16(unit + 16 * w.lane + 512 * i, from + up.off[i], 16);
+        if (kBucket && w.lane < 2 * kUnitWorkers<B> && ((live >> (w.lane >> 1)) & 1u))
+            cp_async16(unit + kUnitBytes + 16 * w.lane, bn + (w.lane >> 1) * p.total_blocks * 8 + 4 * (w.lane & 1), 16);
+        return;
+    }
+    for (uint32_t m = live; m; m &= m - 1) {
+        const int kk = __ffs(m) - 1;
+#pragma unroll
+        for (int i = 0; i < C; ++i)
+            cp_async4(unit + kk * kBlockBytes<B> + 128 * i + 4 * w.lane, src + kk * p.packed_words + 32 * i + w.lane);
+        if (kBucket && w.lane < 8)
+            cp_async4(unit + kUnitBytes + 32 * kk + 4 * w.lane, bn + kk * p.total_blocks * 8 + w.lane);
+    }
+}
+
+// symbol p of the lane's words as (4 * symbol) | table
+template <int C>
+__device__ __forceinline__ uint32_t value_addr(const uint32_t (&w)[C], int p, uint32_t table)
+{
+    const int off = p * C, i = off >> 5, s = off & 31;
+    constexpr uint32_t mask4 = ((1u << C) - 1u) << 2;
+    uint32_t v;
+    if (s + C <= 32) v = s >= 2 ? (w[i] >> (s - 2)) : (w[i] << (2 - s));
+    else             v = __funnelshift_r(w[i], w[i + 1], s - 2);      // s >= 2 whenever a symbol straddles
+    return (v & mask4) | table;
+}
+
+// Adds a unit's workers to the sums of rows kRow0 .. kRow0 + kRows - 1, in worker order.  A clear bit of `live`: that
+// worker's block is all zero words, which would add +0 to sums that are never -0.
+template <int B, int kRow0, int kRows, bool kBucket>
+__device__ __forceinline__ void add_unit(float (&acc)[4 * kRows], uint32_t unit, int lane, uint32_t table, uint32_t live)
+{
+    constexpr int C = B + 1, kFirst = (4 * kRow0 * C) >> 5, kLast = ((4 * (kRow0 + kRows) * C) - 1) >> 5;
+    uint32_t at = unit + 4 * lane, norm_at = unit + kUnitBytes;
+#pragma unroll 1
+    for (; live; live >>= 1, at += kBlockBytes<B>, table += kBucket ? 0u : 8u << B, norm_at += 32) {
+        if (!(live & 1u)) continue;
+        uint32_t w[C];
+#pragma unroll
+        for (int i = kFirst; i <= kLast; ++i) w[i] = lds_u32(at + 128 * i);
+        float nr[kRows];
+        if (kBucket) {
+#pragma unroll
+            for (int j = 0; j < kRows; ++j) nr[j] = lds_f32(norm_at + 4 * (kRow0 + j));
+        }
+#pragma unroll
+        for (int i = 0; i < 4 * kRows; ++i) {
+            const float val = lds_f32(value_addr<C>(w, 4 * kRow0 + i, table));
+            acc[i] += kBucket ? __fmul_rn(val, nr[i >> 2]) : val;
+        }
+    }
+}
+
+template <int kRow0, int kRows>
+__device__ __forceinline__ void request_state(const DecodeArgs& a, const Walk& w, int64_t blk)
+{
+#pragma unroll
+    for (int j = kRow0; j < kRow0 + kRows; ++j) {
+        const int64_t at = blk * kBlockCoords + 128 * j + 4 * w.lane;
+        if (at < w.size) {
+            cp_async16(w.state + 512 * j + 16 * w.lane, a.Y + w.base + at, 16);
+            cp_async16(w.state + kStateBytes / 2 + 512 * j + 16 * w.lane, a.X1 + w.base + at, 16);
+        }
+    }
+}
+
+// The rows kRow0 .. of one block, from their sums: the mean, then the update.
+template <int kMode, int kRow0, int kRows>
+__device__ __forceinline__ void finish_block(const DecodeArgs& a, const Walk& w, int64_t blk, const float (&acc)[4 * kRows],
+                                             float invK, const Rates& rt, bool sent, double& lam_acc, double& mu_acc)
 {
     constexpr bool kQoda = kMode >= 1, kAlt = kMode == 2;
     const float eta = rt.eta, gamma = rt.gamma;
-    const int lane = threadIdx.x & 31;
-    const int K = p.num_workers;
-    const int64_t woff = L.word_off + blk * (int64_t)(B + 1) * 32 + lane;
-    const int64_t base = L.elem_off + blk * kBlockCoords + 4 * lane;
-    const int64_t limit = L.elem_off + L.size;
-    // the state rows of this piece travel to shared memory while the messages are read and decoded
-    // (`stage`: this lane's slots, rows of Y then rows of X_1, 32 float4 apart; only this lane reads them)
-    if (kQoda && active) {
-        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(stage);
 #pragma unroll
-        for (int jj = 0; jj < kPartRows; ++jj) {
-            const int64_t pos = base + 128 * (kPartRows * H + jj);
-            if (pos < limit) {
-                cp_async16(dst + 512u * jj, a.Y + pos, 16);
-                cp_async16(dst + 512u * (kPartRows + jj), a.X1 + pos, 16);
-            }
-        }
-        cp_async_commit();
-    }
-    float acc[kPartSyms];
-#pragma unroll
-    for (int i = 0; i < kPartSyms; ++i) acc[i] = 0.0f;
-    for (int k0 = 0; k0 < K; k0 += kWorkerChunk) {
-        const int kc = min(kWorkerChunk, K - k0);
-        // the chunk's workers in the low bits; the masks cover at most 32 workers, and beyond that (masks unknown,
-        // block_live all ones) every word is read: a shift by 32 or more is not defined
-        const uint32_t live = k0 < 32 ? block_live >> k0 : 0xffffffffu;
-        if (!resident) fill_tables<kBucket>(p, L, layer, a, table, k0, kc);
-        if (kBucket || K <= kWorkerChunk) resident = true;
-        const int64_t bn_stride = p.total_blocks * 8;
-        const float* bn = kBucket ? a.norms + (int64_t)k0 * bn_stride + (L.block_off + blk) * 8 + kPartRows * H : nullptr;
-        if (active) decode_accumulate<B, H, kBucket>(acc, a.packed + (int64_t)k0 * p.packed_words + woff, p.packed_words,
-                                                     kc, table, bn, bn_stride, live);
-    }
-    if (!active) return;
-    if (kQoda) cp_async_wait<0>();
-#pragma unroll
-    for (int jj = 0; jj < kPartRows; ++jj) {
-        const int64_t pos = base + 128 * (kPartRows * H + jj);
-        if (pos >= limit) continue;
+    for (int jj = 0; jj < kRows; ++jj) {
+        const int64_t at = blk * kBlockCoords + 128 * (kRow0 + jj) + 4 * w.lane, pos = w.base + at;
+        if (at >= w.size) continue;
         float4 g;
         g.x = __fmul_rn(acc[4 * jj + 0], invK);
         g.y = __fmul_rn(acc[4 * jj + 1], invK);
@@ -156,8 +195,8 @@ __device__ __forceinline__ void decode_half(const PlanDev& p, const LayerDesc& L
         g.w = __fmul_rn(acc[4 * jj + 3], invK);
         if (a.gbar) *reinterpret_cast<float4*>(a.gbar + pos) = g;
         if (kQoda) {
-            const float4 y0 = stage[32 * jj];
-            const float4 x1 = stage[32 * (kPartRows + jj)];
+            const float4 y0 = lds_f32x4(w.state + 512 * (kRow0 + jj) + 16 * w.lane);
+            const float4 x1 = lds_f32x4(w.state + kStateBytes / 2 + 512 * (kRow0 + jj) + 16 * w.lane);
             float4 y, x, h;
             y.x = __fsub_rn(y0.x, g.x); y.y = __fsub_rn(y0.y, g.y);
             y.z = __fsub_rn(y0.z, g.z); y.w = __fsub_rn(y0.w, g.w);
@@ -173,82 +212,213 @@ __device__ __forceinline__ void decode_half(const PlanDev& p, const LayerDesc& L
                                      __fsub_rn(fmaf(rt.eta_cur, y0.z, x1.z), x.z), __fsub_rn(fmaf(rt.eta_cur, y0.w, x1.w), x.w)};
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    if (pos + e < limit) {
+                    if (at + e < w.size) {
                         const double gd = (double)gv[e], dd = (double)dv[e];
                         lam_acc = fma(gd, gd, lam_acc);
                         mu_acc = fma(dd, dd, mu_acc);
                     }
                 }
             }
-            if (block_live) *reinterpret_cast<float4*>(a.Y + pos) = y;   // no worker sent anything here: y = y0 - 0
+            if (sent) *reinterpret_cast<float4*>(a.Y + pos) = y;         // no worker sent anything here: y = y0 - 0
             *reinterpret_cast<float4*>(a.Xhalf + pos) = h;
             if (a.X) *reinterpret_cast<float4*>(a.X + pos) = x;
         }
     }
 }
 
-template <int B, int kMode, bool kBucket>
-__device__ __forceinline__ void decode_block_chunked(const PlanDev& p, const LayerDesc& L, int layer,
-                                                     const Tile& tile, const DecodeArgs& a,
-                                                     float (*table)[2 * kMaxLevels], const Rates& rt,
-                                                     double& lam_acc, double& mu_acc)
+// A warp's blocks: warp, warp + 4, ... of the CTA's (kRows = 8), or rows kRow0, kRow0 + 1 of all of them (kRows = 2).
+// The next unit's words are always requested before the current unit is waited for; the rows of Y and X_1 as soon as
+// the block before is finished.  Per unit one copy group, per block one more for the state, so a fixed number of
+// younger groups may be under way at every wait.
+template <int B, int kMode, bool kBucket, int kRow0, int kRows>
+__device__ __forceinline__ void decode_blocks(const PlanDev& p, const LayerDesc& L, int layer, const DecodeArgs& a, const Walk& w,
+                                           float2* table, const Rates* rates, uint32_t my_live, double* sums)
 {
-    const int warp = threadIdx.x >> 5;
-    const float invK = __fdiv_rn(1.0f, (float)p.num_workers);
-    bool resident = false;
-    extern __shared__ float4 stage_mem[];                 // [warp][Y rows, X_1 rows][lane]
-    float4* stage = stage_mem + warp * (2 * kPartRows * 32) + (threadIdx.x & 31);
-    // each warp takes the tile's blocks round-robin; all warps run the same number of rounds so
-    // that the table refills (CTA-wide barriers) stay aligned
-    for (int b0 = 0; b0 < tile.nblocks; b0 += kWarps) {
-        const bool active = b0 + warp < tile.nblocks;
-        const int64_t blk = tile.block0 + b0 + warp;
-        // which workers sent anything in this block (all of them when that is not known)
-        const uint32_t block_live = (!kBucket && a.live && active) ? __ldg(a.live + L.block_off + blk) : 0xffffffffu;
-        decode_half<B, 0, kMode, kBucket>(p, L, layer, a, table, rt, invK, blk, active, resident, stage, lam_acc, mu_acc, block_live);
-        decode_half<B, 1, kMode, kBucket>(p, L, layer, a, table, rt, invK, blk, active, resident, stage, lam_acc, mu_acc, block_live);
-        if (kParts == 4) {
-            decode_half<B, 2 % kParts, kMode, kBucket>(p, L, layer, a, table, rt, invK, blk, active, resident, stage, lam_acc, mu_acc, block_live);
-            decode_half<B, 3 % kParts, kMode, kBucket>(p, L, layer, a, table, rt, invK, blk, active, resident, stage, lam_acc, mu_acc, block_live);
-        }
+    constexpr bool kQoda = kMode >= 1;
+    constexpr int kUW = kUnitWorkers<B>, kTW = kBucket ? 1 << 20 : kTableWorkers<B>;
+    constexpr int kStep = kRows == 8 ? kDecWarps : 1;
+    constexpr uint32_t kUnitStride = kUnitBytes + (kBucket ? 32 * 16 : 0);
+    const int K = p.num_workers, nu = (K + kUW - 1) / kUW;
+    const float invK = __fdiv_rn(1.0f, (float)K);
+    // the workers of unit u that sent anything in a block with `live` (kept for up to 32 workers; of more, all are read)
+    auto unit_live = [&](uint32_t live, int u) {
+        const int k0 = u * kUW;
+        const uint32_t m = K <= 32 ? live >> k0 : 0xffffffffu;
+        return K - k0 < kUW ? m & ((1u << (K - k0)) - 1u) : m & ((1u << kUW) - 1u);
+    };
+    auto block_live = [&](int i) { return __reduce_or_sync(0xffffffffu, w.lane == i ? my_live : 0u); };   // uniform
+
+    const UnitPieces<B> up(p.packed_words, w.lane);
+    int b = kRows == 8 ? w.warp : 0, i = 0;
+    uint32_t live = block_live(0);
+    if (b < w.nblocks) request_unit<B, kBucket>(p, a, w, up, w.units, w.block0 + b, 0, unit_live(live, 0));
+    cp_async_commit();
+    if (kQoda) {
+        if (b < w.nblocks) request_state<kRow0, kRows>(a, w, w.block0 + b);
+        cp_async_commit();
     }
+    fill_tables<kBucket>(p, L, layer, a, table, 0, min(K, kTW));
+    __syncthreads();
+    const Rates rt = *rates;
+    double lam_acc = 0.0, mu_acc = 0.0;
+    uint32_t stage = 0;
+    // with more workers than tables fit, all warps take the same number of turns (the refills are CTA-wide)
+    for (int b0 = 0; K > kTW ? b0 < w.nblocks : b < w.nblocks; b0 += kStep, b += kStep, ++i) {
+        const bool active = b < w.nblocks;
+        const int64_t blk = w.block0 + b;
+        const uint32_t next_live = b + kStep < w.nblocks ? block_live(i + 1) : 0u;
+        float acc[4 * kRows];
+#pragma unroll
+        for (int c = 0; c < 4 * kRows; ++c) acc[c] = 0.0f;
+        for (int u = 0; u < nu; ++u) {
+            const uint32_t other = w.units + (stage ^ 1u) * kUnitStride;
+            if (u + 1 < nu) { if (active) request_unit<B, kBucket>(p, a, w, up, other, blk, (u + 1) * kUW, unit_live(live, u + 1)); }
+            else if (b + kStep < w.nblocks) request_unit<B, kBucket>(p, a, w, up, other, blk + kStep, 0, unit_live(next_live, 0));
+            cp_async_commit();
+            const int k0 = u * kUW;
+            int k_in = k0;                                        // index of the unit's first worker in the tables
+            if (!kBucket && K > kTW) {
+                k_in = k0 % kTW;
+                if (k_in == 0 && (b0 > 0 || u > 0)) {
+                    __syncthreads();
+                    fill_tables<kBucket>(p, L, layer, a, table, k0, min(kTW, K - k0));
+                    __syncthreads();
+                }
+            }
+            if (kQoda && u == 0) cp_async_wait<2>(); else cp_async_wait<1>();
+            __syncwarp();                                         // a lane reads what other lanes have copied
+            if (active)
+                add_unit<B, kRow0, kRows, kBucket>(acc, w.units + stage * kUnitStride, w.lane,
+                                                   w.tables + (kBucket ? 0 : (uint32_t)k_in << (B + 3)), unit_live(live, u));
+            __syncwarp();                                         // ... and the unit may be overwritten
+            stage ^= 1u;
+        }
+        if (kQoda) cp_async_wait<1>();
+        if (active) finish_block<kMode, kRow0, kRows>(a, w, blk, acc, invK, rt, live != 0u, lam_acc, mu_acc);
+        if (kQoda) {
+            if (b + kStep < w.nblocks) request_state<kRow0, kRows>(a, w, blk + kStep);
+            cp_async_commit();
+        }
+        live = next_live;
+    }
+    cp_async_wait<0>();
+    if (kMode == 2) { sums[0] = lam_acc; sums[1] = mu_acc; }
 }
 
-template <int kMode, bool kBucket>
-__global__ void __launch_bounds__(kThreads, kBucket ? 2 : (kMode == 2 ? 3 : LQ_DEC_CTAS)) decode_kernel(PlanDev p, DecodeArgs a)
+// S_t = S_{t-1} + (sum over workers and layers of the squared differences) / K^2, eta_{t+1} = fp32((1 + S_t)^(-1/2)).
+__device__ __forceinline__ QodaScalars next_scalars(const QodaScalars& q0, double total, int num_workers)
 {
-    __shared__ float table[kWorkerChunk][2 * kMaxLevels];
+    QodaScalars q = q0;
+    const double K = (double)num_workers;
+    const double delta = total / (K * K);
+    q.last_delta = delta;
+    q.S = q.S + delta;
+    q.eta = (float)(1.0 / sqrt(1.0 + q.S));
+    q.gamma = q.eta;
+    q.t = q.t + 1;
+    return q;
+}
+
+// The sum of sq_diff over workers and layers in a fixed order (all threads of the CTA; valid in thread 0).
+__device__ __forceinline__ double sum_sq_diff(const PlanDev& p, double* scratch)
+{
+    const int n = p.num_workers * p.num_layers;
+    double acc = 0.0;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) acc += p.sq_diff[i];
+    return block_reduce<false>(acc, scratch);
+}
+
+// kSplit: the 4 warps share every block, 2 rows each.
+template <int kMode, bool kBucket, bool kSplit>
+__global__ void __launch_bounds__(kDecThreads, kMode == 0 ? 5 : 4) decode_kernel(PlanDev p, DecodeArgs a)
+{
+    extern __shared__ __align__(1024) unsigned char dec_smem[];
     constexpr bool kAlt = kMode == 2;
-    const int ncta = p.num_tiles * p.sub_tiles;
-    Tile tile = p.tiles[blockIdx.x >> p.sub_shift];                    // this CTA takes one sub-tile of it
-    const int sub0 = (blockIdx.x & (p.sub_tiles - 1)) * kSubBlocks;
-    if (sub0 >= tile.nblocks) {
+    constexpr uint32_t kUnitStride = kUnitBytes + (kBucket ? 32 * 16 : 0);
+    constexpr uint32_t kWarpBytes = 2 * kUnitStride + (kMode >= 1 ? kStateBytes : 0);
+    pdl_launch_next();
+    const int ncta = p.num_tiles << p.dec_shift;
+    const Tile tile = p.tiles[blockIdx.x >> p.dec_shift];              // this CTA takes a piece of it
+    const int first = (blockIdx.x & ((1 << p.dec_shift) - 1)) * p.dec_blocks;
+    if (first >= tile.nblocks) {
+        pdl_wait();
         if (kAlt && threadIdx.x == 0) { p.alt_partial[blockIdx.x] = 0.0; p.alt_partial[ncta + blockIdx.x] = 0.0; }
         return;
     }
-    tile.block0 += sub0;
-    tile.nblocks = min(kSubBlocks, tile.nblocks - sub0);
     const int layer = tile.layer;
     const LayerDesc L = p.layers[layer];
-    Rates rt{0.0f, 0.0f, 0.0f};
-    if (kMode >= 1) {
-        rt.eta = p.scalars->eta;
-        rt.gamma = kAlt ? p.scalars->gamma : rt.eta;
-        rt.eta_cur = kAlt ? p.scalars->eta_cur : 0.0f;
-    }
-    double lam_acc = 0.0, mu_acc = 0.0;
+    // tables at a multiple of their size, then a few words for the reductions, then the warps' units and state rows
+    const uint32_t base = (uint32_t)__cvta_generic_to_shared(dec_smem);
+    const uint32_t table_size = 8u << L.bits;
+    const uint32_t tables = (base + table_size - 1) & ~(table_size - 1);
+    unsigned char* after = dec_smem + a.table_bytes;
+    double* scratch = reinterpret_cast<double*>(after);
+    Rates* rates = reinterpret_cast<Rates*>(after + 64);
+    Walk w;
+    w.lane = threadIdx.x & 31; w.warp = threadIdx.x >> 5;
+    w.words = a.packed + L.word_off;
+    w.bnorms = a.norms + L.block_off * 8;
+    w.base = L.elem_off;
+    w.block0 = tile.block0 + first;
+    w.nblocks = min(p.dec_blocks, tile.nblocks - first);
+    w.size = (int32_t)L.size;
+    w.tables = tables;
+    w.units = base + a.table_bytes + 128 + w.warp * kWarpBytes;
+    w.state = w.units + 2 * kUnitStride;
+    float2* table = reinterpret_cast<float2*>(dec_smem + (tables - base));
+    pdl_wait();
 
-    switch (L.bits) {
-#define LQ_CASE(BB) case BB: decode_block_chunked<BB, kMode, kBucket>(p, L, layer, tile, a, table, rt, lam_acc, mu_acc); break;
-        LQ_CASE(1) LQ_CASE(2) LQ_CASE(3) LQ_CASE(4) LQ_CASE(5) LQ_CASE(6) LQ_CASE(7) LQ_CASE(8)
+    // lane i: which workers sent anything in this warp's i-th block (all of them when that is not known)
+    uint32_t my_live = 0xffffffffu;
+    if (!kBucket && a.masks) {
+        constexpr int kStep = kSplit ? 1 : kDecWarps;
+        const uint8_t* mk = a.masks + (int64_t)min(w.lane, p.num_workers - 1) * p.total_blocks + L.block_off + w.block0;
+        for (int i0 = 0; kStep * i0 < w.nblocks; i0 += 8) {
+            uint32_t m[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int b = (kSplit ? 0 : w.warp) + kStep * (i0 + i);
+                m[i] = b < w.nblocks && w.lane < p.num_workers ? __ldg(mk + b) : 0u;
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const uint32_t v = __ballot_sync(0xffffffffu, m[i] != 0u);
+                if (w.lane == i0 + i) my_live = v;
+            }
+        }
+    }
+    if (kMode == 1 && a.form_rates) {
+        const double total = sum_sq_diff(p, scratch);
+        if (threadIdx.x == 0) {
+            const QodaScalars q = next_scalars(p.scalars[1], total, p.num_workers);
+            *rates = Rates{q.eta, q.eta, 0.0f};
+            if (blockIdx.x == 0) p.scalars[0] = q;
+        }
+    } else if (kMode >= 1) {
+        if (threadIdx.x == 0)
+            *rates = Rates{p.scalars->eta, kAlt ? p.scalars->gamma : p.scalars->eta, kAlt ? p.scalars->eta_cur : 0.0f};
+    }
+    double sums[2] = {0.0, 0.0};
+    if constexpr (kSplit) {
+        switch (L.bits * 4 + w.warp) {
+#define LQ_ROWS(BB, R) case 4 * BB + R: decode_blocks<BB, kMode, kBucket, 2 * R, 2>(p, L, layer, a, w, table, rates, my_live, sums); break;
+#define LQ_CASE(BB) LQ_ROWS(BB, 0) LQ_ROWS(BB, 1) LQ_ROWS(BB, 2) LQ_ROWS(BB, 3)
+            LQ_CASE(1) LQ_CASE(2) LQ_CASE(3) LQ_CASE(4) LQ_CASE(5) LQ_CASE(6) LQ_CASE(7) LQ_CASE(8)
 #undef LQ_CASE
-        default: break;
+#undef LQ_ROWS
+            default: break;
+        }
+    } else {
+        switch (L.bits) {
+#define LQ_CASE(BB) case BB: decode_blocks<BB, kMode, kBucket, 0, 8>(p, L, layer, a, w, table, rates, my_live, sums); break;
+            LQ_CASE(1) LQ_CASE(2) LQ_CASE(3) LQ_CASE(4) LQ_CASE(5) LQ_CASE(6) LQ_CASE(7) LQ_CASE(8)
+#undef LQ_CASE
+            default: break;
+        }
     }
     if (kAlt) {                                  // one term per CTA, added in CTA order by the finalize kernel
-        double* scratch = reinterpret_cast<double*>(&table[0][0]);   // the tables are no longer needed (the
-                                                                     // reduction starts with a barrier)
-        const double lam = block_reduce<false>(lam_acc, scratch);
-        const double mu = block_reduce<false>(mu_acc, scratch);
+        const double lam = block_reduce<false>(sums[0], scratch);
+        const double mu = block_reduce<false>(sums[1], scratch);
         if (threadIdx.x == 0) { p.alt_partial[blockIdx.x] = lam; p.alt_partial[ncta + blockIdx.x] = mu; }
     }
 }
@@ -256,6 +426,8 @@ __global__ void __launch_bounds__(kThreads, kBucket ? 2 : (kMode == 2 ? 3 : LQ_D
 // Eq. (Alt), before the update of iteration t: eta_{t+1} and gamma_{t+1} from the sums through iteration t-1.
 __global__ void alt_scalars_kernel(PlanDev p, double qhat)
 {
+    pdl_launch_next();
+    pdl_wait();
     if (threadIdx.x == 0 && blockIdx.x == 0) {
         QodaScalars* q = p.scalars;
         q->eta_cur = q->eta;
@@ -269,7 +441,9 @@ __global__ void alt_scalars_kernel(PlanDev p, double qhat)
 __global__ void __launch_bounds__(256) alt_finalize_kernel(PlanDev p)
 {
     __shared__ double scratch[8];
-    const int n = p.num_tiles * p.sub_tiles;
+    pdl_launch_next();
+    pdl_wait();
+    const int n = p.num_tiles << p.dec_shift;
     double lam = 0.0, mu = 0.0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) { lam += p.alt_partial[i]; mu += p.alt_partial[n + i]; }
     const double lam_t = block_reduce<false>(lam, scratch);
@@ -277,25 +451,14 @@ __global__ void __launch_bounds__(256) alt_finalize_kernel(PlanDev p)
     if (threadIdx.x == 0) { p.scalars->lambda += lam_t; p.scalars->mu += mu_t; }
 }
 
-// S_t = S_{t-1} + (sum over workers and layers of the squared differences) / K^2,
-// eta_{t+1} = fp32((1 + S_t)^(-1/2)); one CTA, fixed summation order.
-__global__ void __launch_bounds__(256) qoda_scalars_kernel(PlanDev p)
+// The rates of a step in a kernel of their own (plans with many layers and workers); one CTA, fixed summation order.
+__global__ void __launch_bounds__(kThreads) qoda_scalars_kernel(PlanDev p)
 {
-    __shared__ double scratch[8];
-    const int n = p.num_workers * p.num_layers;
-    double acc = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) acc += p.sq_diff[i];
-    const double total = block_reduce<false>(acc, scratch);
-    if (threadIdx.x == 0) {
-        QodaScalars* q = p.scalars;
-        const double K = (double)p.num_workers;
-        const double delta = total / (K * K);
-        q->last_delta = delta;
-        q->S = q->S + delta;
-        q->eta = (float)(1.0 / sqrt(1.0 + q->S));
-        q->gamma = q->eta;
-        q->t = q->t + 1;
-    }
+    __shared__ double scratch[kWarps];
+    pdl_launch_next();
+    pdl_wait();
+    const double total = sum_sq_diff(p, scratch);
+    if (threadIdx.x == 0) p.scalars[0] = next_scalars(p.scalars[0], total, p.num_workers);
 }
 
 __global__ void qoda_init_kernel(PlanDev p, const float* __restrict__ X1, float* __restrict__ Y,
@@ -336,57 +499,52 @@ cudaError_t launch_average(const PlanDev& p, const float* Xhalf, double* xsum, c
 
 cudaError_t launch_decode(const PlanDev& p, const uint32_t* packed, const float* norms,
                           const float* levels, const float* X1, float* Y, float* Xhalf, float* X,
-                          float* gbar, int mode, const uint32_t* live, cudaStream_t s)
+                          float* gbar, int mode, const uint8_t* masks, cudaStream_t s)
 {
     if (p.num_tiles == 0) return cudaSuccess;
-    DecodeArgs a{live, packed, norms, levels, X1, Y, Xhalf, X, gbar};
-    const unsigned grid = (unsigned)p.num_tiles * p.sub_tiles;
-    if (p.bucket_norm) {
-        if (mode == 2)      decode_kernel<2, true><<<grid, kThreads, kStageBytes, s>>>(p, a);
-        else if (mode == 1) decode_kernel<1, true><<<grid, kThreads, kStageBytes, s>>>(p, a);
-        else                decode_kernel<0, true><<<grid, kThreads, kStageBytes, s>>>(p, a);
-    } else {
-        if (mode == 2)      decode_kernel<2, false><<<grid, kThreads, kStageBytes, s>>>(p, a);
-        else if (mode == 1) decode_kernel<1, false><<<grid, kThreads, kStageBytes, s>>>(p, a);
-        else                decode_kernel<0, false><<<grid, kThreads, kStageBytes, s>>>(p, a);
+    DecodeArgs a{masks, packed, norms, levels, X1, Y, Xhalf, X, gbar, rates_in_decoder(p), false, 0};
+    a.vec = reinterpret_cast<uintptr_t>(packed) % 16 == 0 && (!p.bucket_norm || reinterpret_cast<uintptr_t>(norms) % 16 == 0);
+    // room for the widest layer's tables (narrower layers' need less), plus what aligning 2 KB tables may skip
+    const int tables = std::min(p.bucket_norm ? 1 : p.num_workers, (int)(kTableBytes >> (p.most_bits + 3)));
+    a.table_bytes = ((uint32_t)tables << (p.most_bits + 3)) + (p.most_bits == 8 ? 1024u : 0u);
+    a.table_bytes = (a.table_bytes + 127u) & ~127u;
+    const bool split = p.dec_blocks == 1;
+    const unsigned grid = (unsigned)p.num_tiles << p.dec_shift;
+    const size_t smem = a.table_bytes + 128 + kDecWarps * (2 * (kUnitBytes + (p.bucket_norm ? 32 * 16 : 0)) + (mode ? kStateBytes : 0));
+    using Kernel = void (*)(PlanDev, DecodeArgs);
+    static const Kernel kernels[3][2][2] = {
+        {{decode_kernel<0, false, false>, decode_kernel<0, false, true>}, {decode_kernel<0, true, false>, decode_kernel<0, true, true>}},
+        {{decode_kernel<1, false, false>, decode_kernel<1, false, true>}, {decode_kernel<1, true, false>, decode_kernel<1, true, true>}},
+        {{decode_kernel<2, false, false>, decode_kernel<2, false, true>}, {decode_kernel<2, true, false>, decode_kernel<2, true, true>}}};
+    static std::atomic<uint64_t> configured{0};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev > 63 || !((configured.load(std::memory_order_relaxed) >> dev) & 1u)) {
+        for (const auto& m : kernels)
+            for (const auto& s2 : m)
+                for (Kernel k : s2) {
+                    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
+                    if (e != cudaSuccess) return e;
+                }
+        if (dev >= 0 && dev <= 63) configured.fetch_or(1ull << dev, std::memory_order_relaxed);
     }
-    return cudaGetLastError();
-}
-
-// block_live[b] = bitmask of the workers whose block b holds a nonzero value, from the K zero-row mask arrays
-__global__ void __launch_bounds__(256) block_live_kernel(PlanDev p)
-{
-    const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (b >= p.total_blocks) return;
-    uint32_t m = 0;
-    for (int k = 0; k < p.num_workers; ++k) m |= (p.row_mask[(int64_t)k * p.total_blocks + b] != 0 ? 1u : 0u) << k;
-    p.block_live[b] = m;
-}
-
-cudaError_t launch_block_live(const PlanDev& p, cudaStream_t s)
-{
-    if (p.total_blocks == 0) return cudaSuccess;
-    block_live_kernel<<<(unsigned)((p.total_blocks + 255) / 256), 256, 0, s>>>(p);
-    return cudaGetLastError();
+    return launch(kernels[mode][p.bucket_norm ? 1 : 0][split ? 1 : 0], grid, kDecThreads, smem, s, p, a);
 }
 
 cudaError_t launch_alt_scalars(const PlanDev& p, double qhat, cudaStream_t s)
 {
-    alt_scalars_kernel<<<1, 32, 0, s>>>(p, qhat);
-    return cudaGetLastError();
+    return launch(alt_scalars_kernel, 1, 32, 0, s, p, qhat);
 }
 
 cudaError_t launch_alt_finalize(const PlanDev& p, cudaStream_t s)
 {
     if (p.num_tiles == 0) return cudaSuccess;
-    alt_finalize_kernel<<<1, 256, 0, s>>>(p);
-    return cudaGetLastError();
+    return launch(alt_finalize_kernel, 1, 256, 0, s, p);
 }
 
 cudaError_t launch_qoda_scalars(const PlanDev& p, cudaStream_t s)
 {
-    qoda_scalars_kernel<<<1, 256, 0, s>>>(p);
-    return cudaGetLastError();
+    return launch(qoda_scalars_kernel, 1, kThreads, 0, s, p);
 }
 
 cudaError_t launch_qoda_init(const PlanDev& p, const float* X1, float* Y, float* Xhalf, cudaStream_t s)

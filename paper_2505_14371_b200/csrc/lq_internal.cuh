@@ -10,8 +10,10 @@ namespace lq {
 
 constexpr int kBlockCoords = 1024;    // coordinates per message block (32 lanes x 32 positions)
 constexpr int kTileBlocks = 128;      // most blocks per tile (the encoder's unit: its per-CTA tables are amortised over a
-                                      // tile); a plan uses 32, 64 or 128, the largest that still gives several waves of CTAs
-constexpr int kSubBlocks = 32;        // blocks per sub-tile (the unit of the norm and decode kernels)
+                                      // tile); a plan takes the largest power of two that still gives several waves of
+                                      // CTAs, down to 8 (one block per warp) when even a single wave is not reached
+constexpr int kSubBlocks = 32;        // most blocks per sub-tile (the unit of the norm kernel and the entropy stage), and
+                                      // of the decoder's CTAs; fewer in plans that would leave SMs idle
 constexpr int kWarps = 8;
 constexpr int kThreads = 256;
 constexpr int kLevelStride = 256;     // floats per layer in a level table
@@ -80,8 +82,13 @@ struct PlanDev {
     int32_t num_tiles;
     int32_t num_workers;
     int32_t q;            // 0 = infinity norm
-    int32_t sub_tiles;    // sub-tiles per tile: the plan's tile size / kSubBlocks (1, 2 or 4)
+    int32_t sub_tiles;    // sub-tiles per tile: the plan's tile size / sub_blocks, a power of two
     int32_t sub_shift;    // log2(sub_tiles)
+    int32_t sub_blocks;   // blocks per sub-tile
+    int32_t most_blocks;  // blocks of the plan's largest layer
+    int32_t most_bits;    // widest code of the plan
+    int32_t dec_blocks;   // blocks per decoder CTA; 1: its warps share them
+    int32_t dec_shift;    // log2(plan's tile size / dec_blocks)
     int32_t global_norm;  // 1: one norm per worker over all layers (Section 3.1), 0: one per layer
     int32_t bucket_norm;  // 1: one norm per bucket of 128 consecutive coordinates of a layer (Section 7.1)
     int32_t worker0;      // the encode-side kernels cover workers worker0 .. worker0 + worker_count - 1 (grid.y =
@@ -97,19 +104,42 @@ struct PlanDev {
     float* rnorm;         // [K][L]   1/N, or 0 for a zeroed layer
     uint32_t* status;     // [K][L]
     double* layer_total;  // [K][L]  per-layer sums (or maxima) before the root, for the global norm
-    double* alt_partial;  // [2][num_tiles * sub_tiles]  per-CTA terms of lambda and mu (Eq. Alt)
+    double* alt_partial;  // [2][num_tiles << dec_shift]  per-CTA terms of lambda and mu (Eq. Alt)
     uint8_t* row_mask;    // [K][total_blocks]  bit j of a block's byte: row j (128 values) holds a nonzero value
     const uint8_t* row_mask_prev;   // the same for the input behind the previous message, or NULL when unknown
     int64_t total_blocks; // blocks of 1024 values per worker, all layers
-    uint32_t* block_live; // [total_blocks]  bit k: worker k's block holds a nonzero value (built from row_mask; K <= 32)
     double* energy_partial;   // [K][num_tiles]  bucket scope: per-tile sums of squared bucket norms
     uint32_t* flag_partial;   // [K][num_tiles]  bucket scope: bit 0 a non-finite bucket, bit 1 a nonzero bucket
     float* layer_weight;      // [K][L]          bucket scope: sqrt of a layer's summed squared bucket norms
-    QodaScalars* scalars;
+    QodaScalars* scalars;     // [2]  the live values, and their copy as the last lq_quantize_pack found them: a decoder
+                              // whose CTAs each form the step's rates reads the copy while one of them writes the first
 };
 
 // Stores a printf-style reason for lq_last_error() (calling thread) and returns `code`.
 int lq_set_error(int code, const char* fmt, ...);
+
+// Whether the decoder's CTAs form the step's rates themselves from sq_diff (Eq. general_stepsize) instead of a kernel of
+// its own.  Up to four sums per thread: the kernel and the gap before it cost 3 to 4 us, the sums about 0.5 us per CTA.
+inline bool rates_in_decoder(const PlanDev& p) { return (int64_t)p.num_workers * p.num_layers <= 4 * kThreads && p.num_tiles > 0; }
+
+// Launches `kernel` so that it may start while the kernel before it on the stream is still finishing (programmatic
+// dependent launch).  Every kernel of the library waits for its predecessor's memory (pdl_wait) before it touches anything
+// a kernel may have written, so only the launch itself and the reading of the plan's constant tables overlap: an
+// iteration of a small plan is a chain of kernels of a few us each, and what lies between two of them shrinks from 1.7 us
+// to well below 1 us.  Grids of many waves are launched the plain way: with the attribute every CTA starts about 3 us
+// late, not just the first ones (norm pass of 37 000 CTAs 690 -> 850 us, decoder of 4 700 CTAs 451 -> 486 us).
+constexpr int64_t kDependentCtas = 148 * 8;
+template <typename... Params, typename... Args>
+cudaError_t launch(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args)
+{
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s;
+    cfg.attrs = at; cfg.numAttrs = (int64_t)grid.x * grid.y * grid.z <= kDependentCtas ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
 
 // ---- launchers (each enqueues on `s` and returns the launch status) ----
 // `write_mask`: also record the zero-row masks of `grads` in p.row_mask
@@ -135,14 +165,14 @@ cudaError_t launch_quantize_bucketed(const PlanDev& p, const float* grads, uint3
 cudaError_t launch_bucket_finalize(const PlanDev& p, cudaStream_t s);
 cudaError_t launch_stat_finalize(const PlanDev& p, cudaStream_t s);
 // mode 0: decode + aggregate only; 1: + QODA update, Eq. (general_stepsize); 2: + QODA update, Eq. (Alt)
-// live: per block the bitmask of workers whose words are not all zero, for exactly this message, or nullptr
+// masks: the zero-row masks of exactly this message's input, [K][total_blocks] with K <= 32 (a worker's all-zero
+// blocks are then not read), or nullptr
 cudaError_t launch_decode(const PlanDev& p, const uint32_t* packed, const float* norms,
                           const float* levels, const float* X1, float* Y, float* Xhalf, float* X,
-                          float* gbar, int mode, const uint32_t* live, cudaStream_t s);
+                          float* gbar, int mode, const uint8_t* masks, cudaStream_t s);
 cudaError_t launch_level_probabilities(const PlanDev& p, const uint32_t* hist, const float* norms, int num_samples,
                                        const float* levels, double* probs, cudaStream_t s);
 cudaError_t launch_symbol_counts(const PlanDev& p, const uint32_t* packed, uint32_t* counts, cudaStream_t s);
-cudaError_t launch_block_live(const PlanDev& p, cudaStream_t s);
 cudaError_t launch_alt_scalars(const PlanDev& p, double qhat, cudaStream_t s);
 cudaError_t launch_alt_finalize(const PlanDev& p, cudaStream_t s);
 cudaError_t launch_qoda_scalars(const PlanDev& p, cudaStream_t s);
@@ -157,6 +187,11 @@ cudaError_t launch_fit_shared(const PlanDev& p, const uint32_t* hist, const floa
 
 // ---- device helpers ----
 #ifdef __CUDACC__
+
+// First statements of every kernel: the next kernel of the stream may be launched from now on (its CTAs take slots as
+// this kernel's last ones leave them), and nothing written by the kernels before this one is read until they are done.
+__device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Philox4x32-10 (Salmon et al., SC'11): 10 rounds of two 32x32->64 multiplies and xors,
 // the key bumped by the Weyl constants between rounds.
@@ -179,16 +214,45 @@ __device__ __forceinline__ void philox4x32_10(uint32_t c0, uint32_t c1, uint32_t
     out[0] = c0; out[1] = c1; out[2] = c2; out[3] = c3;
 }
 
-// symbol p (pre-scaled by 4) of a lane's string of 32 symbols of C bits, held in C words
-template <int C>
-__device__ __forceinline__ uint32_t symbol4_at(const uint32_t (&w)[C], int p)
+// ---- shared-memory loads by absolute 32-bit address (volatile pins their place after the barrier or wait that
+// ---- precedes them)
+__device__ __forceinline__ uint32_t lds_u32(uint32_t a)
 {
-    const int off = p * C, i = off >> 5, s = off & 31;
-    constexpr uint32_t mask4 = ((1u << C) - 1u) << 2;
     uint32_t v;
-    if (s + C <= 32) v = s >= 2 ? (w[i] >> (s - 2)) : (w[i] << (2 - s));
-    else             v = __funnelshift_r(w[i], w[i + 1], s - 2);      // s >= 2 whenever a symbol straddles
-    return v & mask4;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ uint32_t lds_u8(uint32_t a)
+{
+    uint32_t v;
+    asm volatile("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ float lds_f32(uint32_t a)
+{
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
+    return v;
+}
+template <int kOff>
+__device__ __forceinline__ float lds_f32_at(uint32_t a)
+{
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1+%2];" : "=f"(v) : "r"(a), "n"(kOff));
+    return v;
+}
+__device__ __forceinline__ float2 lds_f32x2(uint32_t a)
+{
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a));
+    return v;
+}
+
+__device__ __forceinline__ float4 lds_f32x4(uint32_t a)
+{
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
+    return v;
 }
 
 // 16-byte asynchronous copies global -> shared (completion by commit / wait groups of the issuing thread)
@@ -196,6 +260,10 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, int by
 {
     // copies `bytes` (0..16) bytes and fills the rest of the 16 with zeros
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async4(uint32_t dst, const void* src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
@@ -256,6 +324,58 @@ __device__ __forceinline__ void accumulate(double& acc, uint32_t& maxbits, float
     }
 }
 
+// One block of 1024 values (a lane takes the float4 at 128 j + 4 lane of row j): adds its terms to the lane's
+// accumulators and returns, in every lane, the byte whose bit j says whether row j holds anything but zeros.
+template <int kMode>
+__device__ __forceinline__ uint32_t norm_block(const float* __restrict__ g, int64_t blk, int64_t size, int lane, int q,
+                                               double& acc, uint32_t& maxbits)
+{
+    const int64_t blk0 = blk * kBlockCoords, base = blk0 + 4 * lane;
+    uint32_t rows = 0;                       // bit j: this lane's part of row j holds a value that is not +-0 (NaN counts)
+    if (blk0 + kBlockCoords <= size) {
+        float4 v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            v[j] = __ldg(reinterpret_cast<const float4*>(g + base + 128 * j));
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            accumulate<kMode>(acc, maxbits, v[j].x, q);
+            accumulate<kMode>(acc, maxbits, v[j].y, q);
+            accumulate<kMode>(acc, maxbits, v[j].z, q);
+            accumulate<kMode>(acc, maxbits, v[j].w, q);
+            const float mag = (fabsf(v[j].x) + fabsf(v[j].y)) + (fabsf(v[j].z) + fabsf(v[j].w));
+            rows |= (mag != 0.0f ? 1u : 0u) << j;
+        }
+    } else {
+        for (int j = 0; j < 8; ++j) {
+            const int64_t pos = base + 128 * j;
+            float mag = 0.0f;
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (pos + e < size) {
+                    const float x = __ldg(g + pos + e);
+                    accumulate<kMode>(acc, maxbits, x, q);
+                    mag += fabsf(x);
+                }
+            rows |= (mag != 0.0f ? 1u : 0u) << j;
+        }
+    }
+    return __reduce_or_sync(0xffffffffu, rows);      // a row is live if any lane's part of it is
+}
+
+// The CTA's total of the lanes' accumulators, valid in thread 0; NaN when a value was not finite.
+template <int kMode>
+__device__ __forceinline__ double norm_cta_total(double acc, uint32_t maxbits, double* scratch)
+{
+    if (kMode == 0) {
+        // fmax drops NaNs: reduce a "bad" flag next to the maximum
+        const unsigned bad = __syncthreads_or(maxbits >= 0x7f800000u);
+        const double r = block_reduce<true>((double)__uint_as_float(maxbits), scratch);
+        return bad ? __longlong_as_double(0x7ff8000000000000LL) : r;
+    }
+    return block_reduce<false>(acc, scratch);
+}
+
 // A layer's norm from the norm pass's partials, in a fixed order: thread i < 128 takes partials i, i + 128, ...,
 // then the CTA tree; the root, the rounding to fp32, the flags and the fp32 reciprocal.  Every thread of the CTA
 // calls it (128 threads or more); the result is valid in thread 0.  `scratch`: one double per warp.
@@ -265,6 +385,25 @@ struct LayerNorm {
     uint32_t status;
     bool bad;            // a partial was NaN or Inf
 };
+__device__ __forceinline__ LayerNorm layer_norm_of_total(double total, bool bad, int q)
+{
+    LayerNorm r;
+    r.total = total;
+    r.bad = bad;
+    double n64;
+    if (q == 0 || q == 1) n64 = total;
+    else if (q == 2)      n64 = sqrt(total);
+    else                  n64 = pow(total, 1.0 / (double)q);
+    float nf = (float)n64;
+    r.status = 0;
+    if (bad || !(fabs(n64) <= 1.7976931348623157e308) || !(fabsf(nf) <= 3.402823466e38f))
+        r.status = LQ_STATUS_NONFINITE;
+    else if (nf < 1.17549435e-38f)
+        r.status = LQ_STATUS_ZERO_NORM;
+    r.norm = r.status ? 0.0f : nf;
+    r.rnorm = r.status ? 0.0f : __fdiv_rn(1.0f, nf);
+    return r;
+}
 __device__ __forceinline__ LayerNorm layer_norm_from_partials(const double* part, int n, int q, double* scratch)
 {
     double acc = 0.0;
@@ -276,22 +415,8 @@ __device__ __forceinline__ LayerNorm layer_norm_from_partials(const double* part
             if (q == 0) acc = fmax(acc, v); else acc += v;
         }
     bad = __syncthreads_or(bad);
-    LayerNorm r;
-    r.total = q == 0 ? block_reduce<true>(acc, scratch) : block_reduce<false>(acc, scratch);
-    r.bad = bad != 0;
-    double n64;
-    if (q == 0 || q == 1) n64 = r.total;
-    else if (q == 2)      n64 = sqrt(r.total);
-    else                  n64 = pow(r.total, 1.0 / (double)q);
-    float nf = (float)n64;
-    r.status = 0;
-    if (bad || !(fabs(n64) <= 1.7976931348623157e308) || !(fabsf(nf) <= 3.402823466e38f))
-        r.status = LQ_STATUS_NONFINITE;
-    else if (nf < 1.17549435e-38f)
-        r.status = LQ_STATUS_ZERO_NORM;
-    r.norm = r.status ? 0.0f : nf;
-    r.rnorm = r.status ? 0.0f : __fdiv_rn(1.0f, nf);
-    return r;
+    const double total = q == 0 ? block_reduce<true>(acc, scratch) : block_reduce<false>(acc, scratch);
+    return layer_norm_of_total(total, bad != 0, q);
 }
 
 #endif  // __CUDACC__

@@ -206,6 +206,7 @@ __global__ void __launch_bounds__(kQThreads, 4) quantize_pack_kernel(
     // one worker's whole message
     const int flat = blockIdx.y * gridDim.x + blockIdx.x;
     const int slot = flat / (int)gridDim.y, kk = flat - slot * (int)gridDim.y;
+    pdl_launch_next();
     const TileJob J = p.jobs[slot];
     const int tile_id = J.tile, layer = J.layer;
     Tile tile;
@@ -216,6 +217,7 @@ __global__ void __launch_bounds__(kQThreads, 4) quantize_pack_kernel(
     const int k = kk + p.worker0;
     const int lane = threadIdx.x & 31;
     const int64_t kl = (int64_t)k * p.num_layers + layer;
+    pdl_wait();
 
     // Everything below depends on the job record only, so all of it is requested at once: the norms, this thread's
     // two pieces of the search table, the zero-row masks of its block, the levels of its table entries.
@@ -309,12 +311,16 @@ __global__ void __launch_bounds__(kQThreads, 4) quantize_pack_kernel(
     }
 }
 
-// Adds the per-tile statistic partials of one (layer, worker) in a fixed order.
+// Adds the per-tile statistic partials of one (layer, worker) in a fixed order, and keeps the scalars as this message
+// found them.
 __global__ void __launch_bounds__(128) stat_finalize_kernel(PlanDev p)
 {
     __shared__ double scratch[4];
+    pdl_launch_next();
     const int m = blockIdx.x, k = blockIdx.y + p.worker0;
     const LayerDesc L = p.layers[m];
+    pdl_wait();
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) p.scalars[1] = p.scalars[0];
     const double* part = p.stat_partial + (int64_t)k * p.num_tiles + L.first_tile;
     double acc = 0.0;
     for (int i = threadIdx.x; i < L.ntiles; i += blockDim.x) acc += part[i];
@@ -410,22 +416,15 @@ cudaError_t launch_quantize(const PlanDev& p, const float* grads, uint32_t step,
         if (e != cudaSuccess) return e;
         configured[dev] = true;
     }
-    if (hist)
-        quantize_pack_kernel<true, true><<<grid, kQThreads, smem_hist, s>>>(p, grads, step, packed, norms, hist,
-                                                                       prev_packed, prev_norms, levels_cur, levels_prev, t);
-    else if (need_stat)
-        quantize_pack_kernel<false, true><<<grid, kQThreads, smem, s>>>(p, grads, step, packed, norms, hist,
-                                                                        prev_packed, prev_norms, levels_cur, levels_prev, t);
-    else
-        quantize_pack_kernel<false, false><<<grid, kQThreads, smem, s>>>(p, grads, step, packed, norms, hist,
-                                                                         prev_packed, prev_norms, levels_cur, levels_prev, t);
-    return cudaGetLastError();
+    const auto kernel = hist ? quantize_pack_kernel<true, true>
+                        : need_stat ? quantize_pack_kernel<false, true> : quantize_pack_kernel<false, false>;
+    return launch(kernel, grid, kQThreads, hist ? smem_hist : smem, s, p, grads, step, packed, norms, hist, prev_packed,
+                  prev_norms, levels_cur, levels_prev, t);
 }
 
 cudaError_t launch_stat_finalize(const PlanDev& p, cudaStream_t s)
 {
-    stat_finalize_kernel<<<dim3((unsigned)p.num_layers, (unsigned)p.worker_count), 128, 0, s>>>(p);
-    return cudaGetLastError();
+    return launch(stat_finalize_kernel, dim3((unsigned)p.num_layers, (unsigned)p.worker_count), 128, 0, s, p);
 }
 
 }  // namespace lq

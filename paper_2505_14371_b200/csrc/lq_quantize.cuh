@@ -43,40 +43,6 @@ constexpr uint32_t kSmSlack = kSmAlign - 16;       // which is 16-byte aligned a
 // (tables + ring + slack = 55 792 bytes: four CTAs fit in the 227 KB of an SM)
 constexpr uint32_t kHistClamp = 0x33780000u;       // bit pattern one histogram bin below 2^-24
 
-// ---- shared-memory loads by absolute 32-bit address (volatile only pins their place after the barrier that
-// ---- follows the table fill; the tables do not change afterwards)
-__device__ __forceinline__ uint32_t lds_u32(uint32_t a)
-{
-    uint32_t v;
-    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
-    return v;
-}
-__device__ __forceinline__ uint32_t lds_u8(uint32_t a)
-{
-    uint32_t v;
-    asm volatile("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(a));
-    return v;
-}
-__device__ __forceinline__ float lds_f32(uint32_t a)
-{
-    float v;
-    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
-    return v;
-}
-template <int kOff>
-__device__ __forceinline__ float lds_f32_at(uint32_t a)
-{
-    float v;
-    asm volatile("ld.shared.f32 %0, [%1+%2];" : "=f"(v) : "r"(a), "n"(kOff));
-    return v;
-}
-__device__ __forceinline__ float2 lds_f32x2(uint32_t a)
-{
-    float2 v;
-    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a));
-    return v;
-}
-
 // x + 8 when the comparison holds, else x: one compare and one predicated add
 __device__ __forceinline__ uint32_t add8_if_gt_u32(uint32_t x, uint32_t a, uint32_t b)
 {

@@ -245,12 +245,14 @@ __global__ void __launch_bounds__(kQThreads, 3) quantize_pack_bucket_kernel(
     extern __shared__ unsigned char dyn_smem[];
     uint32_t base;
     unsigned char* sm = table_base(dyn_smem, base);
+    pdl_launch_next();
     const Tile tile = p.tiles[blockIdx.x];
     const int layer = tile.layer;
     const LayerDesc L = p.layers[layer];
     const int k = blockIdx.y + p.worker0;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t kl = (int64_t)k * p.num_layers + layer;
+    pdl_wait();
     const int search = st.fast[layer];                      // 1: one lookup; 1 + R: byte table and up to R steps
 
     // the tables hold the plain levels (norm 1) and each row multiplies by its own norm
@@ -313,8 +315,11 @@ __global__ void __launch_bounds__(kQThreads, 3) quantize_pack_bucket_kernel(
 __global__ void __launch_bounds__(128) bucket_finalize_kernel(PlanDev p)
 {
     __shared__ double scratch[4];
+    pdl_launch_next();
     const int m = blockIdx.x, k = blockIdx.y + p.worker0;
     const LayerDesc L = p.layers[m];
+    pdl_wait();
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) p.scalars[1] = p.scalars[0];
     const int64_t o = (int64_t)k * p.num_tiles + L.first_tile;
     double acc = 0.0, en = 0.0;
     uint32_t fl = 0;
@@ -353,19 +358,13 @@ cudaError_t launch_quantize_bucketed(const PlanDev& p, const float* grads, uint3
         if (e != cudaSuccess) return e;
         configured[dev] = true;
     }
-    if (hist)
-        quantize_pack_bucket_kernel<true><<<grid, kQThreads, smem, s>>>(p, grads, step, packed, bucket_norms, hist,
-                                                                        prev_packed, prev_norms, levels_cur, levels_prev, t);
-    else
-        quantize_pack_bucket_kernel<false><<<grid, kQThreads, smem, s>>>(p, grads, step, packed, bucket_norms, hist,
-                                                                         prev_packed, prev_norms, levels_cur, levels_prev, t);
-    return cudaGetLastError();
+    return launch(hist ? quantize_pack_bucket_kernel<true> : quantize_pack_bucket_kernel<false>, grid, kQThreads, smem, s, p,
+                  grads, step, packed, bucket_norms, hist, prev_packed, prev_norms, levels_cur, levels_prev, t);
 }
 
 cudaError_t launch_bucket_finalize(const PlanDev& p, cudaStream_t s)
 {
-    bucket_finalize_kernel<<<dim3((unsigned)p.num_layers, (unsigned)p.worker_count), 128, 0, s>>>(p);
-    return cudaGetLastError();
+    return launch(bucket_finalize_kernel, dim3((unsigned)p.num_layers, (unsigned)p.worker_count), 128, 0, s, p);
 }
 
 }  // namespace lq
