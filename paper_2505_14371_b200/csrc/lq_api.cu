@@ -350,7 +350,7 @@ int lq_plan_create(lq_plan** out, int32_t num_layers, const int64_t* layer_sizes
         return fail(code, "plan setup: %s", cudaGetErrorString(e));
     }
     d.layers = p->d_layers; d.tiles = p->d_tiles; d.jobs = p->d_jobs;
-    e = launch_build_search(d, p->d_levels_enc[0], p->search, nullptr);
+    e = launch_build_search(d, p->d_levels_stage, p->d_levels_enc[0], p->search, nullptr);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         free_plan(p);
@@ -442,15 +442,12 @@ int lq_quantize_pack(lq_plan* plan, const float* grads, uint32_t step, uint32_t*
     LQ_ALIGNED(prev_packed, 4); LQ_ALIGNED(prev_norms, 4);
     if (plan->dev.num_layers == 0) return LQ_OK;
     cudaStream_t s = (cudaStream_t)stream;
-    const size_t lev_bytes = (size_t)plan->dev.num_layers * kLevelStride * sizeof(float);
     if (plan->stage_dirty) {
         const int next = plan->have_message ? 1 - plan->cur : plan->cur;
-        LQ_CUDA(cudaMemcpyAsync(plan->d_levels_enc[next], plan->d_levels_stage, lev_bytes,
-                                cudaMemcpyDeviceToDevice, s));
         plan->prev = plan->cur;
         plan->cur = next;
         plan->stage_dirty = false;
-        LQ_CUDA(launch_build_search(plan->dev, plan->d_levels_enc[next], plan->search, s));
+        LQ_CUDA(launch_build_search(plan->dev, plan->d_levels_stage, plan->d_levels_enc[next], plan->search, s));
     } else {
         plan->prev = plan->cur;
     }

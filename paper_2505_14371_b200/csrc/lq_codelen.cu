@@ -21,57 +21,76 @@ __device__ __forceinline__ double edge_of(int i)
     return ldexp(1.0 + (double)m * 0.0625, o - 24);
 }
 
-// One CTA per layer, one thread per level.
+// One CTA per layer, one warp per level at a time: the lanes take the bins that lie under the level's hat function (the
+// first intervals of a level set span most of the 385 bins) and the warp adds their pieces.  One thread per level walking
+// all bins took 152 us for 4-bit levels, the latency of its divisions throughout; this takes 11.
 __global__ void __launch_bounds__(kMaxLevels) level_probabilities_kernel(PlanDev p, const uint32_t* __restrict__ hist,
                                                                          const float* __restrict__ norms, int Z,
                                                                          const float* __restrict__ levels,
                                                                          double* __restrict__ probs)
 {
     __shared__ double mass[LQ_NUM_BINS];
+    __shared__ double edge[kBins + 1];
     __shared__ double lev[kMaxLevels];
+    __shared__ double weight[LQ_MAX_WORKERS];
     __shared__ double wsum_s;
-    const int m = blockIdx.x, tid = threadIdx.x;
+    const int m = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
     const LayerDesc L = p.layers[m];
     const int n = L.nlevels;
     double* out = probs + (int64_t)m * kMaxLevels;
-    if (tid == 0) {
-        double w = 0.0;
-        for (int z = 0; z < Z; ++z) { const double x = (double)norms[(int64_t)z * p.num_layers + m]; w += x * x; }
-        wsum_s = w;
+    pdl_launch_next();
+    pdl_wait();
+    for (int z = tid; z < Z; z += blockDim.x) {
+        const double x = (double)norms[(int64_t)z * p.num_layers + m];
+        weight[z] = x * x;
     }
     if (tid < n) lev[tid] = (double)levels[(int64_t)m * kLevelStride + tid];
+    for (int i = tid; i <= kBins; i += blockDim.x) edge[i] = edge_of(i);
+    __syncthreads();
+    if (tid == 0) {
+        double w = 0.0;
+        for (int z = 0; z < Z; ++z) w += weight[z];
+        wsum_s = w;
+    }
     __syncthreads();
     const double wsum = wsum_s;
-    if (!(wsum > 0.0) || L.size <= 0) { out[tid] = 0.0; return; }
+    if (tid >= n || !(wsum > 0.0) || L.size <= 0) out[tid] = 0.0;
+    if (!(wsum > 0.0) || L.size <= 0) return;
     for (int i = tid; i < LQ_NUM_BINS; i += blockDim.x) {
         double acc = 0.0;
-        for (int z = 0; z < Z; ++z) {
-            const double x = (double)norms[(int64_t)z * p.num_layers + m];
-            acc += ((x * x) / wsum) * (double)hist[((int64_t)z * p.num_layers + m) * LQ_HIST_STRIDE + i];
-        }
+        for (int z = 0; z < Z; ++z)
+            acc += (weight[z] / wsum) * (double)hist[((int64_t)z * p.num_layers + m) * LQ_HIST_STRIDE + i];
         mass[i] = acc / (double)L.size;
     }
     __syncthreads();
-    if (tid >= n) { out[tid] = 0.0; return; }
-    const int j = tid;
-    double pj = 0.0;
-    // the pieces of every bin, in ascending order of u, that lie under the two halves of hat_j
-    for (int i = 0; i < kBins; ++i) {
-        if (mass[i] == 0.0) continue;
-        const double lo = edge_of(i), hi = edge_of(i + 1), dens = mass[i] / (hi - lo);
-        if (j >= 1) {                                      // rising half on [a, c] = [l_{j-1}, l_j]
-            const double a = lev[j - 1], c = lev[j];
-            const double x0 = fmax(lo, a), x1 = fmin(hi, c);
-            if (x1 > x0) pj += dens * (x1 - x0) * (0.5 * (x0 + x1) - a) / (c - a);
+    // the bin that holds x: the largest i <= 384 with edge[i] <= x
+    auto bin_of = [&](double x) {
+        int lo = 0, hi = kBins - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (edge[mid] <= x) lo = mid; else hi = mid - 1;
         }
-        if (j <= n - 2) {                                  // falling half on [a, c] = [l_j, l_{j+1}]
-            const double a = lev[j], c = lev[j + 1];
-            const double x0 = fmax(lo, a), x1 = fmin(hi, c);
-            if (x1 > x0) pj += dens * (x1 - x0) * (c - 0.5 * (x0 + x1)) / (c - a);
+        return lo;
+    };
+    for (int j = tid >> 5; j < n; j += kMaxLevels / 32) {
+        const double prev = j > 0 ? lev[j - 1] : 0.0, at = lev[j], next = j + 1 < n ? lev[j + 1] : 1.0;
+        const int last = bin_of(next);
+        double pj = 0.0;
+        for (int i = bin_of(prev) + lane; i <= last; i += 32) {
+            if (mass[i] == 0.0) continue;
+            const double lo = edge[i], hi = edge[i + 1], dens = mass[i] / (hi - lo);
+            if (j >= 1) {                                      // rising half on [l_{j-1}, l_j]
+                const double x0 = fmax(lo, prev), x1 = fmin(hi, at);
+                if (x1 > x0) pj += dens * (x1 - x0) * (0.5 * (x0 + x1) - prev) / (at - prev);
+            }
+            if (j <= n - 2) {                                  // falling half on [l_j, l_{j+1}]
+                const double x0 = fmax(lo, at), x1 = fmin(hi, next);
+                if (x1 > x0) pj += dens * (x1 - x0) * (next - 0.5 * (x0 + x1)) / (next - at);
+            }
         }
+        pj = warp_sum(pj);
+        if (lane == 0) out[j] = j == n - 1 ? pj + mass[LQ_NUM_BINS - 1] : pj;      // the last level also has the point mass at u = 1
     }
-    if (j == n - 1) pj += mass[LQ_NUM_BINS - 1];           // the point mass at u = 1
-    out[j] = pj;
 }
 
 // One CTA per (sub-tile, worker): counts the level indices of the message's real coordinates.
@@ -115,8 +134,7 @@ cudaError_t launch_level_probabilities(const PlanDev& p, const uint32_t* hist, c
                                        const float* levels, double* probs, cudaStream_t s)
 {
     if (p.num_layers == 0) return cudaSuccess;
-    level_probabilities_kernel<<<(unsigned)p.num_layers, kMaxLevels, 0, s>>>(p, hist, norms, num_samples, levels, probs);
-    return cudaGetLastError();
+    return launch(level_probabilities_kernel, (unsigned)p.num_layers, kMaxLevels, 0, s, p, hist, norms, num_samples, levels, probs);
 }
 
 cudaError_t launch_symbol_counts(const PlanDev& p, const uint32_t* packed, uint32_t* counts, cudaStream_t s)

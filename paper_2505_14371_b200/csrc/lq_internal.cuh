@@ -152,7 +152,7 @@ struct SearchTables {
     int32_t* fast;     // [L]              1 if every bin holds at most one level; else 1 + R (byte table over the top 15
                        //                  bits in lut's place, at most R levels per bin)
 };
-cudaError_t launch_build_search(const PlanDev& p, const float* levels, SearchTables t, cudaStream_t s);
+cudaError_t launch_build_search(const PlanDev& p, const float* levels, float* kept, SearchTables t, cudaStream_t s);
 cudaError_t launch_quantize(const PlanDev& p, const float* grads, uint32_t step, uint32_t* packed,
                             const float* norms, uint32_t* hist, const uint32_t* prev_packed,
                             const float* prev_norms, const float* levels_cur,

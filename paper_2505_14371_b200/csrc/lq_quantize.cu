@@ -328,7 +328,8 @@ __global__ void __launch_bounds__(128) stat_finalize_kernel(PlanDev p)
     if (threadIdx.x == 0) p.sq_diff[(int64_t)k * p.num_layers + m] = total;
 }
 
-// One CTA per layer: derives the encode-side tables from the layer's levels.
+// One CTA per layer: derives the encode-side tables from the layer's levels, which it also copies to `kept` (the level
+// table of the messages to come).
 //   ld[tau]  = {l_tau, l_{tau+1} - l_tau}                 tau = 0..n-2 (other entries: {l_tau, 0})
 //   lut[bin] = 8 * tau0 | code << 13    bin = bits(u) >> 19, i.e. the values [lo, hi) with bits(lo) = bin << 19;
 //              tau0 = last level (<= n-2) at or below lo; code = (low 19 bits of l_{tau0+1}) - 1 if that level
@@ -338,14 +339,19 @@ __global__ void __launch_bounds__(128) stat_finalize_kernel(PlanDev p)
 //   lut8[bits(u) >> 17] = tau0 of that finer bin; tau is found by stepping up while l_{tau+1} <= u, at most R times,
 //   R = the most levels inside one bin;  fast = 1 + R.
 __global__ void __launch_bounds__(256) build_search_kernel(PlanDev p, const float* __restrict__ levels,
-                                                           SearchTables t)
+                                                           float* __restrict__ kept, SearchTables t)
 {
     __shared__ float lev[kMaxLevels];
     __shared__ int slow, most;
+    pdl_launch_next();
+    pdl_wait();
     const int m = blockIdx.x;
     const int n = p.layers[m].nlevels;
     if (threadIdx.x == 0) { slow = 0; most = 0; }
-    for (int i = threadIdx.x; i < n; i += blockDim.x) lev[i] = levels[(int64_t)m * kLevelStride + i];
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        lev[i] = levels[(int64_t)m * kLevelStride + i];
+        kept[(int64_t)m * kLevelStride + i] = lev[i];
+    }
     __syncthreads();
     for (int i = threadIdx.x; i < kMaxLevels; i += blockDim.x) {
         float2 e = make_float2(i < n ? lev[i] : 0.f, 0.f);
@@ -390,11 +396,10 @@ __global__ void __launch_bounds__(256) build_search_kernel(PlanDev p, const floa
     if (threadIdx.x == 0) t.fast[m] = slow ? 1 + most : 1;
 }
 
-cudaError_t launch_build_search(const PlanDev& p, const float* levels, SearchTables t, cudaStream_t s)
+cudaError_t launch_build_search(const PlanDev& p, const float* levels, float* kept, SearchTables t, cudaStream_t s)
 {
     if (p.num_layers == 0) return cudaSuccess;
-    build_search_kernel<<<(unsigned)p.num_layers, 256, 0, s>>>(p, levels, t);
-    return cudaGetLastError();
+    return launch(build_search_kernel, (unsigned)p.num_layers, 256, 0, s, p, levels, kept, t);
 }
 
 cudaError_t launch_quantize(const PlanDev& p, const float* grads, uint32_t step, uint32_t* packed,
