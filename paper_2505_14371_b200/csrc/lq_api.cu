@@ -473,14 +473,22 @@ int lq_quantize_pack(lq_plan* plan, const float* grads, uint32_t step, uint32_t*
         plan->stat_pending = true;
         return LQ_OK;
     }
-    LQ_CUDA(timed(plan, LQ_KERNEL_NORM_PARTIAL, s, [&] { return launch_norm_partial(d, grads, true, s); }));
-    LQ_CUDA(timed(plan, LQ_KERNEL_NORM_FINALIZE, s, [&] { return launch_norm_finalize(d, norms, s); }));
-    LQ_CUDA(timed(plan, LQ_KERNEL_QUANTIZE_PACK, s, [&] {
-        // under Eq. (Alt) nothing consumes the statistic of Eq. (general_stepsize): it is left out (and reads 0)
-        return launch_quantize(d, grads, step, packed, norms, hist, prev_packed, prev_norms, lc, lp,
-                               plan->search, plan->alt_qhat <= 0.0, s);
-    }));
-    LQ_CUDA(timed(plan, LQ_KERNEL_STAT_FINALIZE, s, [&] { return launch_stat_finalize(d, s); }));
+    // under Eq. (Alt) nothing consumes the statistic of Eq. (general_stepsize): it is left out (and reads 0)
+    const bool need_stat = plan->alt_qhat <= 0.0;
+    if (use_small(d)) {                  // one kernel
+        LQ_CUDA(timed(plan, LQ_KERNEL_QUANTIZE_PACK, s, [&] {
+            return launch_quantize_small(d, grads, step, packed, norms, hist, prev_packed, prev_norms, lc, lp, plan->search,
+                                         need_stat, s);
+        }));
+    } else {
+        LQ_CUDA(timed(plan, LQ_KERNEL_NORM_PARTIAL, s, [&] { return launch_norm_partial(d, grads, true, s); }));
+        LQ_CUDA(timed(plan, LQ_KERNEL_NORM_FINALIZE, s, [&] { return launch_norm_finalize(d, norms, s); }));
+        LQ_CUDA(timed(plan, LQ_KERNEL_QUANTIZE_PACK, s, [&] {
+            return launch_quantize(d, grads, step, packed, norms, hist, prev_packed, prev_norms, lc, lp, plan->search,
+                                   need_stat, s);
+        }));
+        LQ_CUDA(timed(plan, LQ_KERNEL_STAT_FINALIZE, s, [&] { return launch_stat_finalize(d, s); }));
+    }
     plan->have_message = true;
     plan->masks_known = true;
     plan->message_intact = true;

@@ -14,7 +14,6 @@
 // their size), look-up and add.  The look-ups bound it for many narrow messages (one pass of the SM's shared-memory
 // pipe per 32 symbols), DRAM otherwise.
 #include <algorithm>
-#include <atomic>
 
 #include "lq_internal.cuh"
 
@@ -517,17 +516,10 @@ cudaError_t launch_decode(const PlanDev& p, const uint32_t* packed, const float*
         {{decode_kernel<1, false, false>, decode_kernel<1, false, true>}, {decode_kernel<1, true, false>, decode_kernel<1, true, true>}},
         {{decode_kernel<2, false, false>, decode_kernel<2, false, true>}, {decode_kernel<2, true, false>, decode_kernel<2, true, true>}}};
     static std::atomic<uint64_t> configured{0};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev > 63 || !((configured.load(std::memory_order_relaxed) >> dev) & 1u)) {
-        for (const auto& m : kernels)
-            for (const auto& s2 : m)
-                for (Kernel k : s2) {
-                    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
-                    if (e != cudaSuccess) return e;
-                }
-        if (dev >= 0 && dev <= 63) configured.fetch_or(1ull << dev, std::memory_order_relaxed);
-    }
+    const cudaError_t e = opt_in_shared_memory(
+        configured, 100 * 1024, kernels[0][0][0], kernels[0][0][1], kernels[0][1][0], kernels[0][1][1], kernels[1][0][0], kernels[1][0][1],
+        kernels[1][1][0], kernels[1][1][1], kernels[2][0][0], kernels[2][0][1], kernels[2][1][0], kernels[2][1][1]);
+    if (e != cudaSuccess) return e;
     return launch(kernels[mode][p.bucket_norm ? 1 : 0][split ? 1 : 0], grid, kDecThreads, smem, s, p, a);
 }
 

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "lq.h"
 
 namespace lq {
@@ -129,16 +131,44 @@ inline bool rates_in_decoder(const PlanDev& p) { return (int64_t)p.num_workers *
 // to well below 1 us.  Grids of many waves are launched the plain way: with the attribute every CTA starts about 3 us
 // late, not just the first ones (norm pass of 37 000 CTAs 690 -> 850 us, decoder of 4 700 CTAs 451 -> 486 us).
 constexpr int64_t kDependentCtas = 148 * 8;
+// `cluster`: CTAs per cluster along x
+template <typename... Params, typename... Args>
+cudaError_t launch_cluster(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, unsigned cluster, cudaStream_t s,
+                           Args... args)
+{
+    cudaLaunchAttribute at[2];
+    unsigned n = 0;
+    if ((int64_t)grid.x * grid.y * grid.z <= kDependentCtas) {
+        at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 1) {
+        at[n].id = cudaLaunchAttributeClusterDimension;
+        at[n].val.clusterDim.x = cluster; at[n].val.clusterDim.y = 1; at[n++].val.clusterDim.z = 1;
+    }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s;
+    cfg.attrs = at; cfg.numAttrs = n;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
 template <typename... Params, typename... Args>
 cudaError_t launch(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args)
 {
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s;
-    cfg.attrs = at; cfg.numAttrs = (int64_t)grid.x * grid.y * grid.z <= kDependentCtas ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+    return launch_cluster(kernel, grid, block, smem, 1, s, args...);
+}
+
+// More than 48 KB of dynamic shared memory: every kernel opts in once per device (`configured`: bit d = device d is done).
+template <typename... Kernels>
+cudaError_t opt_in_shared_memory(std::atomic<uint64_t>& configured, int bytes, Kernels... kernels)
+{
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const bool known = dev >= 0 && dev < 64;
+    if (known && ((configured.load(std::memory_order_relaxed) >> dev) & 1u)) return cudaSuccess;
+    cudaError_t e = cudaSuccess;
+    ((e = e == cudaSuccess ? cudaFuncSetAttribute(kernels, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) : e), ...);
+    if (e == cudaSuccess && known) configured.fetch_or(1ull << dev, std::memory_order_relaxed);
+    return e;
 }
 
 // ---- launchers (each enqueues on `s` and returns the launch status) ----
@@ -157,6 +187,11 @@ cudaError_t launch_quantize(const PlanDev& p, const float* grads, uint32_t step,
                             const float* norms, uint32_t* hist, const uint32_t* prev_packed,
                             const float* prev_norms, const float* levels_cur,
                             const float* levels_prev, SearchTables t, bool need_stat, cudaStream_t s);
+// layer scope, plans whose layers are all small: norms, messages and statistic in one kernel
+bool use_small(const PlanDev& p);
+cudaError_t launch_quantize_small(const PlanDev& p, const float* grads, uint32_t step, uint32_t* packed, float* norms,
+                                  uint32_t* hist, const uint32_t* prev_packed, const float* prev_norms,
+                                  const float* levels_cur, const float* levels_prev, SearchTables t, bool need_stat, cudaStream_t s);
 // bucket scope: `bucket_norms` [K][8 * total_blocks] is written, `prev_norms` has the same shape
 cudaError_t launch_quantize_bucketed(const PlanDev& p, const float* grads, uint32_t step, uint32_t* packed,
                                      float* bucket_norms, uint32_t* hist, const uint32_t* prev_packed,

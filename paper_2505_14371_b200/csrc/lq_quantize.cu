@@ -24,172 +24,9 @@
 // skipped entirely.  The masks are made warp-uniform by a reduction, so the per-row tests are uniform
 // branches.  The unrolled code handles whole blocks only; a layer's last, partial block goes through a
 // plain loop (once per layer and worker).
-#include "lq_quantize.cuh"
+#include "lq_quantize_tile.cuh"
 
 namespace lq {
-
-// Everything a warp needs to walk its blocks of one (tile, worker).
-struct WarpCtx {
-    const float* g;              // first coordinate of the layer in this worker's row
-    int64_t size;                // d_m
-    int64_t nfull;               // blocks below this index lie wholly inside the layer
-    int lane;
-};
-
-// x of lane i, the same in every lane and known to be (a reduction's result is warp-uniform)
-__device__ __forceinline__ uint32_t lane_value(uint32_t x, int i, int lane)
-{
-    return __reduce_or_sync(0xffffffffu, lane == i ? x : 0u);
-}
-
-// The layer's last, partial block (one per layer and worker): a plain loop over the lane's 32 positions with a
-// binary search over the levels, the coordinates past the layer's end sending zeros.  Same arithmetic as
-// quantize_coord; speed does not matter here.
-__device__ __noinline__ double quantize_partial_block(const PlanDev& p, const QuantEnv& ev, const float* __restrict__ g,
-                                                      int64_t size, int64_t blk, int bits, uint32_t layer, uint32_t worker,
-                                                      uint32_t step, uint32_t* __restrict__ out,
-                                                      const uint32_t* __restrict__ prev, bool hist, int lane)
-{
-    const int C = bits + 1, n = 1 << bits;
-    const int64_t woff = blk * (int64_t)C * 32 + lane;
-    uint64_t acc = 0, pacc = 0;
-    int fill = 0, wi = 0, pfill = 0, pwi = 0;
-    double stat = 0.0;
-    for (int pp = 0; pp < 32; ++pp) {
-        const int64_t pos = blk * kBlockCoords + 128 * (pp >> 2) + 4 * lane + (pp & 3);
-        uint32_t sym = 0;
-        if (pos < size) {
-            const float v = __ldg(g + pos);
-            uint32_t x[4];
-            philox4x32_10((uint32_t)(pos >> 2), layer, worker, step, p.seed_lo, p.seed_hi, x);
-            const float u = __fmul_rn(fabsf(v), ev.r);
-            int tau = 0;
-            for (int s = n >> 1; s > 0; s >>= 1)
-                if (lds_f32(ev.ld + 8u * (uint32_t)(tau + s)) <= u) tau += s;
-            tau = min(tau, n - 2);
-            const float2 ld = lds_f32x2(ev.ld + 8u * (uint32_t)tau);
-            const float num = __fsub_rn(u, ld.x);
-            const float f = __uint_as_float((x[pos & 3] >> 9) | 0x3F800000u);
-            const float t = __fmaf_rn(f, ld.y, -ld.y);
-            sym = 2u * (uint32_t)(tau + (t < num ? 1 : 0)) + (v < 0.0f ? 1u : 0u);
-            if (hist) atomicAdd(ev.hist + ((max(__float_as_uint(u), kHistClamp) - kHistClamp) >> 19), 1u);
-        }
-        if (pfill < C) {
-            if (prev && pwi < C) pacc |= (uint64_t)__ldg(prev + woff + 32 * pwi) << pfill;
-            pfill += 32; ++pwi;
-        }
-        const uint32_t psym = (uint32_t)pacc & ((1u << C) - 1u);
-        pacc >>= C; pfill -= C;
-        const double dd = (double)__fsub_rn(lds_f32(ev.ld + (kSmTcur - kSmLd) + 4u * sym), lds_f32(ev.tprev + 4u * psym));
-        stat = fma(dd, dd, stat);
-        acc |= (uint64_t)sym << fill;
-        fill += C;
-        if (fill >= 32) { __stcs(out + woff + 32 * wi, (uint32_t)acc); acc >>= 32; fill -= 32; ++wi; }
-    }
-    return stat;
-}
-
-// A warp's share of a tile: the whole blocks warp, warp + 8, ...  A block whose rows are all zero in this input
-// and in the input behind the previous message is an all-zero piece of message that adds nothing to the
-// statistic: its words are stored and nothing is read.  The other blocks are taken in order.
-template <int B, int kSearch, bool kHist, bool kStat>
-__device__ __forceinline__ double quantize_tile(const PlanDev& p, const PhiloxConsts& pc, const WarpCtx& c,
-                                                const Tile& tile, uint32_t* __restrict__ out,
-                                                const uint32_t* __restrict__ prev, const QuantEnv& ev,
-                                                const uint8_t* rows_cur, const uint8_t* rows_prev, uint32_t ring_base)
-{
-    constexpr int C = B + 1;
-    const int warp = threadIdx.x >> 5, lane = c.lane;
-    double stat = 0.0;
-    const int64_t nf = c.nfull - tile.block0;                 // whole blocks of this tile
-    const int nfb = nf < tile.nblocks ? (int)nf : tile.nblocks;
-
-    // lane i < 16 keeps the masks of the warp's i-th block (this input's rows in bits 0..7, the previous input's
-    // in bits 8..15, bit 16: the block exists)
-    uint32_t mymask = 0;
-    {
-        const int b = warp + kQWarps * lane;
-        if (lane < kTileBlocks / kQWarps && b < nfb) mymask = (uint32_t)rows_cur[b] | ((uint32_t)rows_prev[b] << 8) | 0x10000u;
-    }
-    uint32_t zero = __ballot_sync(0xffffffffu, mymask == 0x10000u);
-    uint32_t todo = __ballot_sync(0xffffffffu, (mymask & 0xffffu) != 0u);
-    while (zero) {
-        const int i = __ffs(zero) - 1;
-        zero &= zero - 1;
-        const int64_t blk = tile.block0 + warp + kQWarps * i;
-        const int64_t woff = blk * (int64_t)C * 32 + lane;
-#pragma unroll
-        for (int w = 0; w < C; ++w) __stcs(out + woff + w * 32, 0u);
-        if (kHist && lane == 0) atomicAdd(ev.hist, (uint32_t)kBlockCoords);     // its coordinates all have u = 0
-    }
-    if (todo == 0u) return stat;
-
-    auto block_base = [&](int i) { return c.g + (tile.block0 + warp + kQWarps * i) * (int64_t)kBlockCoords; };
-    int i = __ffs(todo) - 1;
-    todo &= todo - 1;
-    uint32_t m = lane_value(mymask, i, lane);
-    const float* src = block_base(i) + 4 * lane;             // this lane's float4 of row 0
-    // While a lane works on row j of a block, row j of the next block with content is already on its way into
-    // the slot that row j has just left (one commit group per row slot, so waiting for all but the last 7
-    // groups means the row is there).
-    const uint32_t ring = ring_base + (uint32_t)(warp * 8 * 512 + lane * 16);
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        if ((m >> j) & 1u) cp_async16(ring + 512u * j, src + 128 * j, 16);
-        cp_async_commit();
-    }
-    for (;;) {
-        const int64_t blk = tile.block0 + warp + kQWarps * i;
-        const uint32_t rows = m & 0xffu, prows = (m >> 8) & 0xffu;
-        // the next block with content: its rows follow this block's
-        const int inext = todo ? __ffs(todo) - 1 : 0;
-        const uint32_t mnext = todo ? lane_value(mymask, inext, lane) : 0u;
-        const float* nsrc = block_base(inext) + 4 * lane;
-        uint32_t pw[C];
-#pragma unroll
-        for (int w = 0; w < C; ++w)
-            pw[w] = (kStat && prev && prows) ? __ldcs(prev + blk * (int64_t)C * 32 + lane + w * 32) : 0u;
-        uint32_t cw[C];
-        pack_begin<C>(cw, ev.ld);
-        const uint32_t ctr0 = (uint32_t)(blk * 256) + (uint32_t)lane;     // index / 4 of this lane's row 0
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            if ((rows >> j) & 1u) {
-                float4 v;
-                cp_async_wait<7>();
-                asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
-                             : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(ring + 512u * j));
-                if ((mnext >> j) & 1u) cp_async16(ring + 512u * j, nsrc + 128 * j, 16);
-                cp_async_commit();
-                uint32_t x[4];
-                philox4x32_10_folded(ctr0 + 32 * j, pc, p, x);
-                const float vv[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    quantize_coord<B, kSearch, kHist, kStat, false>(ev, vv[e], x[e], 4 * j + e, cw, pw, stat, 0.f, 0.f, true);
-            } else {
-                if ((mnext >> j) & 1u) cp_async16(ring + 512u * j, nsrc + 128 * j, 16);
-                cp_async_commit();
-                pack_zero_row<C>(cw, j, ev.ld);
-                if (kStat && ((prows >> j) & 1u)) {
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) stat_prev_only<C, false>(ev, pw, 4 * j + e, 0.f, stat);
-                }
-                if (kHist && lane == 0) atomicAdd(ev.hist, 128u);   // an all-zero row: its coordinates have u = 0
-            }
-        }
-        const int64_t woff = blk * (int64_t)C * 32 + lane;
-#pragma unroll
-        for (int w = 0; w < C; ++w) __stcs(out + woff + w * 32, cw[w]);
-        if (todo == 0u) break;
-        i = inext;
-        todo &= todo - 1;
-        m = mnext;
-        src = nsrc;
-    }
-    cp_async_wait<0>();
-    return stat;
-}
 
 template <bool kHist, bool kStat>
 __global__ void __launch_bounds__(kQThreads, 4) quantize_pack_kernel(
@@ -274,32 +111,13 @@ __global__ void __launch_bounds__(kQThreads, 4) quantize_pack_kernel(
     ev.r = rn;
     ev.refine = search - 1;
     ev.hist = reinterpret_cast<uint32_t*>(sm + kSmHist);
-    const bool zeroed = ev.r == 0.0f;
     if (step == LQ_STEP_AUTO) step = (uint32_t)p.scalars->t;      // the plan's own iteration counter (graph replays)
     const PhiloxConsts pc = philox_fold((uint32_t)layer, (uint32_t)k, step, p.seed_lo, p.seed_hi);
     uint32_t* out = packed + (int64_t)k * p.packed_words + L.word_off;
     const uint32_t* prev = prev_packed ? prev_packed + (int64_t)k * p.packed_words + L.word_off : nullptr;
 
-    double stat = 0.0;
-    switch (zeroed ? -L.bits : L.bits * 2 + (search == 1 ? 1 : 0)) {
-#define LQ_CASE(BB)                                                                              \
-    case -BB:        stat = kStat ? zeroed_tile<BB>(tile, lane, out, prev, ev.tprev)             \
-                                  : zeroed_tile<BB>(tile, lane, out, nullptr, ev.tprev); break;  \
-    case 2 * BB:     stat = quantize_tile<BB, 2, kHist, kStat>(p, pc, c, tile, out, prev, ev, rows_cur, rows_prev, base + kSmRing); break;  \
-    case 2 * BB + 1: stat = quantize_tile<BB, 1, kHist, kStat>(p, pc, c, tile, out, prev, ev, rows_cur, rows_prev, base + kSmRing); break;
-        LQ_CASE(1) LQ_CASE(2) LQ_CASE(3) LQ_CASE(4) LQ_CASE(5) LQ_CASE(6) LQ_CASE(7) LQ_CASE(8)
-#undef LQ_CASE
-        default: break;
-    }
-    // the layer's last, partial block, if this tile holds it: one warp, after its whole blocks
-    {
-        const int64_t bp = c.nfull - tile.block0;
-        if (!zeroed && (L.size % kBlockCoords) != 0 && bp >= 0 && bp < tile.nblocks && (int)(bp % kQWarps) == (threadIdx.x >> 5)) {
-            const double s2 = quantize_partial_block(p, ev, c.g, c.size, c.nfull, L.bits, (uint32_t)layer, (uint32_t)k, step, out,
-                                                     kStat ? prev : nullptr, kHist, lane);
-            if (kStat) stat += s2;
-        }
-    }
+    const double stat = quantize_blocks<kHist, kStat>(p, pc, c, tile, L.bits, search, (uint32_t)layer, (uint32_t)k, step, out, prev, ev,
+                                                      rows_cur, rows_prev, base + kSmRing);
     const double total = block_reduce<false>(stat, reinterpret_cast<double*>(sm + kSmScratch));
     if (threadIdx.x == 0) p.stat_partial[(int64_t)k * p.num_tiles + tile_id] = total;
 
@@ -411,16 +229,10 @@ cudaError_t launch_quantize(const PlanDev& p, const float* grads, uint32_t step,
     const dim3 grid((unsigned)p.num_tiles, (unsigned)p.worker_count);
     // the ring follows the tables; the histogram (histogram mode only) follows the ring
     constexpr unsigned smem = kSmTables + kRingBytes + kSmSlack, smem_hist = smem + LQ_HIST_STRIDE * 4;
-    static bool configured[64] = {};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev >= 0 && dev < 64 && !configured[dev]) {            // more than 48 KB of dynamic shared memory: opt in once
-        cudaError_t e = cudaFuncSetAttribute(quantize_pack_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_hist);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(quantize_pack_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(quantize_pack_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        configured[dev] = true;
-    }
+    static std::atomic<uint64_t> configured{0};
+    const cudaError_t e = opt_in_shared_memory(configured, (int)smem_hist, quantize_pack_kernel<true, true>,
+                                               quantize_pack_kernel<false, true>, quantize_pack_kernel<false, false>);
+    if (e != cudaSuccess) return e;
     const auto kernel = hist ? quantize_pack_kernel<true, true>
                         : need_stat ? quantize_pack_kernel<false, true> : quantize_pack_kernel<false, false>;
     return launch(kernel, grid, kQThreads, hist ? smem_hist : smem, s, p, grads, step, packed, norms, hist, prev_packed,

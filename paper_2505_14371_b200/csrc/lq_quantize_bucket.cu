@@ -348,16 +348,10 @@ cudaError_t launch_quantize_bucketed(const PlanDev& p, const float* grads, uint3
     if (p.num_tiles == 0) return cudaSuccess;
     const dim3 grid((unsigned)p.num_tiles, (unsigned)p.worker_count);
     constexpr unsigned smem = kSmTables + kRingBytes + LQ_HIST_STRIDE * 4 + kSmSlack;
-    static bool configured[64] = {};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev >= 0 && dev < 64 && !configured[dev]) {            // more than 48 KB of dynamic shared memory: opt in once
-        cudaError_t e = cudaFuncSetAttribute(quantize_pack_bucket_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(quantize_pack_bucket_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        configured[dev] = true;
-    }
+    static std::atomic<uint64_t> configured{0};
+    const cudaError_t e = opt_in_shared_memory(configured, (int)smem, quantize_pack_bucket_kernel<true>,
+                                               quantize_pack_bucket_kernel<false>);
+    if (e != cudaSuccess) return e;
     return launch(hist ? quantize_pack_bucket_kernel<true> : quantize_pack_bucket_kernel<false>, grid, kQThreads, smem, s, p,
                   grads, step, packed, bucket_norms, hist, prev_packed, prev_norms, levels_cur, levels_prev, t);
 }

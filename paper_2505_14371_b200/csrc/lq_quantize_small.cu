@@ -1,0 +1,187 @@
+// ENCODE in the layer norm scope for plans whose layers are all small: one cluster of up to 8 CTAs takes a whole (layer,
+// worker), so the norm, which every coordinate of the layer needs before its first symbol, is exchanged inside the
+// cluster (distributed shared memory, a cluster barrier) instead of through kernel boundaries: one launch where the
+// general path has four (norm partials, norms, encoder, statistic).  Such plans are a chain of launches of a few us each,
+// with nothing to fill the GPU, so latency is what bounds them.
+//
+// The rule (use_small): every layer has at most 256 blocks of 1024 coordinates (8 CTAs of 32), and the clusters of all
+// layers and workers are at most two to three waves of CTAs.  A cluster has as many CTAs as its plan's largest layer needs
+// for one block per warp; the values are read twice, the second time from L2.
+#include "lq_quantize_tile.cuh"
+
+namespace lq {
+
+namespace {
+
+// ---- cluster exchange
+__device__ __forceinline__ void st_peer(const double* mine, uint32_t rank, double v)
+{
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(mine)), "r"(rank));
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+
+template <int kMode>
+__device__ __forceinline__ double norm_of_blocks(const PlanDev& p, const float* g, int64_t size, int block0, int nblocks,
+                                                 uint8_t* rows, double* scratch)
+{
+    double acc = 0.0;
+    uint32_t maxbits = 0;
+    for (int b = threadIdx.x >> 5; b < nblocks; b += kQWarps) {
+        const uint32_t r = norm_block<kMode>(g, block0 + b, size, threadIdx.x & 31, p.q, acc, maxbits);
+        if ((threadIdx.x & 31) == 0) rows[b] = (uint8_t)r;
+    }
+    return norm_cta_total<kMode>(acc, maxbits, scratch);
+}
+
+template <bool kHist, bool kStat>
+__global__ void __launch_bounds__(kQThreads, 3) quantize_small_kernel(
+    PlanDev p, const float* __restrict__ grads, uint32_t step, uint32_t* __restrict__ packed,
+    float* __restrict__ norms, uint32_t* __restrict__ hist,
+    const uint32_t* __restrict__ prev_packed, const float* __restrict__ prev_norms,
+    const float* __restrict__ levels_cur, const float* __restrict__ levels_prev, SearchTables st)
+{
+    extern __shared__ unsigned char dyn_smem[];
+    __shared__ double norm_part[8], stat_part[8];             // per CTA of the cluster
+    uint32_t base;
+    unsigned char* sm = table_base(dyn_smem, base);
+    pdl_launch_next();
+    // grid: x = CTA of the cluster, y = layer, z = worker
+    const int ranks = gridDim.x, rank = blockIdx.x, layer = blockIdx.y, k = blockIdx.z + p.worker0;
+    cluster_arrive();                                         // (waited for before the first store into a peer)
+    const LayerDesc L = p.layers[layer];
+    const int per = (L.nblocks + ranks - 1) / ranks;
+    Tile tile;
+    tile.layer = layer; tile.block0 = rank * per; tile.nblocks = max(0, min(per, L.nblocks - tile.block0)); tile.pad_ = 0;
+    const int lane = threadIdx.x & 31;
+    const int64_t kl = (int64_t)k * p.num_layers + layer;
+    const float* g = grads + (int64_t)blockIdx.z * p.padded_elems + L.elem_off;
+    pdl_wait();
+    if (rank == 0 && layer == 0 && blockIdx.z == 0 && threadIdx.x == 0) p.scalars[1] = p.scalars[0];
+
+    // everything that does not need the norm is requested before the values
+    const float nprev = prev_norms ? prev_norms[kl] : 0.0f;
+    const int search = st.fast[layer];                      // 1: one lookup; 1 + R: byte table and up to R steps
+    const uint4* lsrc = reinterpret_cast<const uint4*>(st.lut + (int64_t)layer * kLutEntries);
+    const uint4 lut0 = __ldg(lsrc + threadIdx.x), lut1 = __ldg(lsrc + kQThreads + threadIdx.x);
+    const int64_t mask_at = (int64_t)k * p.total_blocks + L.block_off + tile.block0 + threadIdx.x;
+    uint32_t mprev = 0;
+    if (threadIdx.x < tile.nblocks)
+        mprev = (!kStat || !prev_packed) ? 0u : (p.row_mask_prev ? (uint32_t)p.row_mask_prev[mask_at] : 0xffu);
+    float lc = 0.f, lp = 0.f;
+    float2 lg = make_float2(0.f, 0.f);
+    if (threadIdx.x < L.nlevels) {
+        lc = levels_cur[(int64_t)layer * kLevelStride + threadIdx.x];
+        lp = levels_prev[(int64_t)layer * kLevelStride + threadIdx.x];
+        lg = st.ld[(int64_t)layer * kMaxLevels + threadIdx.x];
+    }
+    uint8_t* rows_cur = sm + kSmRows;
+    uint8_t* rows_prev = rows_cur + kTileBlocks;
+    double* scratch = reinterpret_cast<double*>(sm + kSmScratch);
+    const double mine = p.q == 0   ? norm_of_blocks<0>(p, g, L.size, tile.block0, tile.nblocks, rows_cur, scratch)
+                        : p.q == 1 ? norm_of_blocks<1>(p, g, L.size, tile.block0, tile.nblocks, rows_cur, scratch)
+                        : p.q == 2 ? norm_of_blocks<2>(p, g, L.size, tile.block0, tile.nblocks, rows_cur, scratch)
+                                   : norm_of_blocks<3>(p, g, L.size, tile.block0, tile.nblocks, rows_cur, scratch);
+    cluster_wait();                                          // every CTA of the cluster runs
+    if (threadIdx.x == 0)
+        for (int r = 0; r < ranks; ++r) st_peer(&norm_part[rank], r, mine);
+    cluster_arrive();
+    {
+        uint4* ldst = reinterpret_cast<uint4*>(sm + kSmLut);
+        ldst[threadIdx.x] = lut0;
+        ldst[kQThreads + threadIdx.x] = lut1;
+        if (kHist) {
+            uint32_t* h = reinterpret_cast<uint32_t*>(sm + kSmHist);
+            for (int i = threadIdx.x; i < LQ_HIST_STRIDE; i += kQThreads) h[i] = 0;
+        }
+    }
+    cluster_wait();
+    double total = 0.0;
+    bool bad = false;
+    for (int r = 0; r < ranks; ++r) {
+        const double v = norm_part[r];
+        if (!(fabs(v) <= 1.7976931348623157e308)) bad = true;
+        total = p.q == 0 ? fmax(total, v) : total + v;
+    }
+    const LayerNorm ln = layer_norm_of_total(total, bad, p.q);
+    if (threadIdx.x < L.nlevels) {
+        const float cv = __fmul_rn(ln.norm, lc), pv = __fmul_rn(nprev, lp);
+        reinterpret_cast<float2*>(sm + kSmLd)[threadIdx.x] = lg;
+        reinterpret_cast<float2*>(sm + kSmTcur)[threadIdx.x] = make_float2(cv, -cv);
+        reinterpret_cast<float2*>(sm + kSmTprev)[threadIdx.x] = make_float2(pv, -pv);
+    }
+    if (threadIdx.x < tile.nblocks) {
+        rows_prev[threadIdx.x] = (uint8_t)mprev;
+        p.row_mask[mask_at] = rows_cur[threadIdx.x];
+    }
+    if (rank == 0 && threadIdx.x == 0) { norms[kl] = ln.norm; p.rnorm[kl] = ln.rnorm; p.status[kl] = ln.status; }
+    __syncthreads();
+
+    WarpCtx c;
+    c.g = g;
+    c.size = L.size;
+    c.nfull = L.size / kBlockCoords;
+    c.lane = lane;
+    QuantEnv ev;
+    ev.lut = base + kSmLut; ev.ld = base + kSmLd; ev.tprev = base + kSmTprev;
+    ev.r = ln.rnorm;
+    ev.refine = search - 1;
+    ev.hist = reinterpret_cast<uint32_t*>(sm + kSmHist);
+    if (step == LQ_STEP_AUTO) step = (uint32_t)p.scalars->t;      // the plan's own iteration counter (graph replays)
+    const PhiloxConsts pc = philox_fold((uint32_t)layer, (uint32_t)k, step, p.seed_lo, p.seed_hi);
+    uint32_t* out = packed + (int64_t)k * p.packed_words + L.word_off;
+    const uint32_t* prev = prev_packed ? prev_packed + (int64_t)k * p.packed_words + L.word_off : nullptr;
+    const double stat = quantize_blocks<kHist, kStat>(p, pc, c, tile, L.bits, search, (uint32_t)layer, (uint32_t)k, step, out, prev, ev,
+                                                      rows_cur, rows_prev, base + kSmRing);
+    const double sum = block_reduce<false>(stat, scratch);
+    if (threadIdx.x == 0) st_peer(&stat_part[rank], 0, sum);
+    cluster_arrive();
+    if (kHist) {                                             // (block_reduce's barriers lie behind the last count)
+        uint32_t* h = hist + kl * LQ_HIST_STRIDE;
+        for (int i = threadIdx.x; i < LQ_NUM_BINS; i += blockDim.x)
+            if (ev.hist[i]) atomicAdd(h + i, ev.hist[i]);
+    }
+    cluster_wait();
+    if (rank == 0 && threadIdx.x == 0) {
+        double s = 0.0;
+        for (int r = 0; r < ranks; ++r) s += stat_part[r];
+        p.sq_diff[kl] = s;
+    }
+}
+
+int small_ranks(const PlanDev& p)
+{
+    int r = 1;
+    while (r < 8 && r * kQWarps < p.most_blocks) r *= 2;
+    return r;
+}
+
+}  // namespace
+
+bool use_small(const PlanDev& p)
+{
+    return !p.global_norm && !p.bucket_norm && p.most_blocks <= 256 && p.num_layers <= 65535 &&
+           (int64_t)p.worker_count * p.num_layers * small_ranks(p) <= 148 * 8;
+}
+
+cudaError_t launch_quantize_small(const PlanDev& p, const float* grads, uint32_t step, uint32_t* packed, float* norms,
+                                  uint32_t* hist, const uint32_t* prev_packed, const float* prev_norms,
+                                  const float* levels_cur, const float* levels_prev, SearchTables t, bool need_stat, cudaStream_t s)
+{
+    if (p.num_layers == 0) return cudaSuccess;
+    constexpr unsigned smem = kSmTables + kRingBytes + kSmSlack, smem_hist = smem + LQ_HIST_STRIDE * 4;
+    static std::atomic<uint64_t> configured{0};
+    const cudaError_t e = opt_in_shared_memory(configured, (int)smem_hist, quantize_small_kernel<true, true>,
+                                               quantize_small_kernel<false, true>, quantize_small_kernel<false, false>);
+    if (e != cudaSuccess) return e;
+    const auto kernel = hist ? quantize_small_kernel<true, true>
+                        : need_stat ? quantize_small_kernel<false, true> : quantize_small_kernel<false, false>;
+    const unsigned ranks = (unsigned)small_ranks(p);
+    return launch_cluster(kernel, dim3(ranks, (unsigned)p.num_layers, (unsigned)p.worker_count), kQThreads,
+                          hist ? smem_hist : smem, ranks, s, p, grads, step, packed, norms, hist, prev_packed, prev_norms,
+                          levels_cur, levels_prev, t);
+}
+
+}  // namespace lq
