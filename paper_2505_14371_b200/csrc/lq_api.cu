@@ -108,7 +108,7 @@ void free_plan(lq_plan* p)
     if (!p) return;
     cudaFree(p->d_layers); cudaFree(p->d_tiles); cudaFree(p->d_jobs);
     cudaFree(p->d_levels_stage); cudaFree(p->d_levels_enc[0]); cudaFree(p->d_levels_enc[1]);
-    cudaFree(p->search.lut); cudaFree(p->search.ld); cudaFree(p->search.fast);
+    cudaFree(p->search.lut); cudaFree(p->search.ld); cudaFree(p->search.how);
     cudaFree(p->dev.norm_partial); cudaFree(p->dev.stat_partial); cudaFree(p->dev.sq_diff);
     cudaFree(p->dev.rnorm); cudaFree(p->dev.status); cudaFree(p->dev.scalars); cudaFree(p->d_code_enc); cudaFree(p->d_code_dec); cudaFree(p->d_code_bad); cudaFree(p->code_scratch.lane_bits); cudaFree(p->code_scratch.scan_part); cudaFree(p->d_member_off); cudaFree(p->d_member_layer); cudaFree(p->dev.alt_partial); cudaFree(p->dev.layer_total); cudaFree(p->d_row_mask[0]); cudaFree(p->d_row_mask[1]);
     cudaFree(p->dev.energy_partial); cudaFree(p->dev.flag_partial); cudaFree(p->dev.layer_weight);
@@ -194,7 +194,7 @@ int lq_plan_create(lq_plan** out, int32_t num_layers, const int64_t* layer_sizes
     // tile size: as large as possible while (tiles x workers) still fills the GPU several times over; below 32 blocks only
     // while the tiles do not fill it once (4 CTAs on each of the 148 SMs).  Sub-tiles likewise, without the workers (the
     // decoder has one CTA for all of them).
-    int tile_blocks = kTileBlocks, sub_blocks = kSubBlocks, dec_blocks = kSubBlocks, most_bits = 1;
+    int tile_blocks = kTileBlocks, sub_blocks = kSubBlocks, dec_blocks = kSubBlocks, most_bits = 1, least_bits = num_layers ? LQ_MAX_BITS : 1;
     int64_t most_blocks = 0;
     {
         int64_t total = 0;
@@ -228,6 +228,7 @@ int lq_plan_create(lq_plan** out, int32_t num_layers, const int64_t* layer_sizes
             L.ntiles = (L.nblocks + tile_blocks - 1) / tile_blocks;
             L.pad_ = 0;
             most_bits = std::max(most_bits, b);
+            least_bits = std::min(least_bits, b);
             L.block_off = blocks;
             blocks += L.nblocks;
             for (int t = 0; t < L.ntiles; ++t) {
@@ -252,7 +253,7 @@ int lq_plan_create(lq_plan** out, int32_t num_layers, const int64_t* layer_sizes
     d.num_layers = num_layers; d.num_tiles = (int32_t)ntiles; d.num_workers = num_workers; d.q = q;
     d.worker0 = 0; d.worker_count = num_workers;
     d.sub_blocks = sub_blocks;
-    d.most_bits = most_bits;
+    d.most_bits = most_bits; d.least_bits = least_bits;
     d.dec_blocks = dec_blocks;
     d.dec_shift = 0;
     while ((dec_blocks << d.dec_shift) < tile_blocks) ++d.dec_shift;
@@ -307,7 +308,7 @@ int lq_plan_create(lq_plan** out, int32_t num_layers, const int64_t* layer_sizes
     const size_t nl = (size_t)(num_layers ? num_layers : 1);
     if (e == cudaSuccess) e = dev_alloc_zero(&p->search.lut, nl * kLutEntries);
     if (e == cudaSuccess) e = dev_alloc_zero(&p->search.ld, nl * kMaxLevels);
-    if (e == cudaSuccess) e = dev_alloc_zero(&p->search.fast, nl);
+    if (e == cudaSuccess) e = dev_alloc_zero(&p->search.how, nl);
     if (e == cudaSuccess) e = dev_alloc_zero(&d.norm_partial, KT * (size_t)d.sub_tiles);
     if (e == cudaSuccess) e = dev_alloc_zero(&d.stat_partial, KT);
     if (e == cudaSuccess) e = dev_alloc_zero(&d.sq_diff, KL);

@@ -24,10 +24,10 @@ __device__ __forceinline__ double edge_of(int i)
 // One CTA per layer, one warp per level at a time: the lanes take the bins that lie under the level's hat function (the
 // first intervals of a level set span most of the 385 bins) and the warp adds their pieces.  One thread per level walking
 // all bins took 152 us for 4-bit levels, the latency of its divisions throughout; this takes 11.
-__global__ void __launch_bounds__(kMaxLevels) level_probabilities_kernel(PlanDev p, const uint32_t* __restrict__ hist,
-                                                                         const float* __restrict__ norms, int Z,
-                                                                         const float* __restrict__ levels,
-                                                                         double* __restrict__ probs)
+__global__ void __launch_bounds__(kMaxLevels) level_probabilities_kernel(PlanDev p, const uint32_t* hist,
+                                                                         const float* norms, int Z,
+                                                                         const float* levels,
+                                                                         double* probs)
 {
     __shared__ double mass[LQ_NUM_BINS];
     __shared__ double edge[kBins + 1];

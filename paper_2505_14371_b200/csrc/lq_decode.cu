@@ -62,8 +62,8 @@ __device__ __forceinline__ void fill_tables(const PlanDev& p, const LayerDesc& L
     const int n = (kBucket ? 1 : kc) << L.bits;
     for (int i = threadIdx.x; i < n; i += kDecThreads) {
         const int kk = i >> L.bits, j = i & (L.nlevels - 1);
-        const float lv = __ldg(a.levels + (int64_t)layer * kLevelStride + j);
-        const float mag = kBucket ? lv : __fmul_rn(__ldg(a.norms + (int64_t)(k0 + kk) * p.num_layers + layer), lv);
+        const float lv = load_f32(a.levels + (int64_t)layer * kLevelStride + j);
+        const float mag = kBucket ? lv : __fmul_rn(load_f32(a.norms + (int64_t)(k0 + kk) * p.num_layers + layer), lv);
         table[i] = make_float2(mag, -mag);
     }
 }
@@ -377,7 +377,7 @@ __global__ void __launch_bounds__(kDecThreads, kMode == 0 ? 5 : 4) decode_kernel
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 const int b = (kSplit ? 0 : w.warp) + kStep * (i0 + i);
-                m[i] = b < w.nblocks && w.lane < p.num_workers ? __ldg(mk + b) : 0u;
+                m[i] = b < w.nblocks && w.lane < p.num_workers ? load_u8(mk + b) : 0u;
             }
 #pragma unroll
             for (int i = 0; i < 8; ++i) {

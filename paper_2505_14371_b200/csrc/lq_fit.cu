@@ -223,11 +223,11 @@ __device__ void objective(const FitSmem& s, const double* l, int n, int lane, do
 // whose member layers are member_layer[member_off[t] .. member_off[t+1]) (all with the same level count): the
 // histograms of all (sample, member) pairs are merged with weights N^2 (the variance to minimise is
 // sum N_s^2 sum_i sigma^2(u_i)), scaled by sum N_s^2 d_s, and the result goes to every member.
-__global__ void __launch_bounds__(kFitThreads) fit_levels_kernel(PlanDev p, const uint32_t* __restrict__ hist,
-                                                                 const float* __restrict__ norms, int Z,
-                                                                 float* __restrict__ levels_stage,
-                                                                 const int32_t* __restrict__ member_off,
-                                                                 const int32_t* __restrict__ member_layer)
+__global__ void __launch_bounds__(kFitThreads) fit_levels_kernel(PlanDev p, const uint32_t* hist,
+                                                                 const float* norms, int Z,
+                                                                 float* levels_stage,
+                                                                 const int32_t* member_off,
+                                                                 const int32_t* member_layer)
 {
     __shared__ FitSmem s;
     pdl_launch_next();

@@ -89,6 +89,7 @@ struct PlanDev {
     int32_t sub_blocks;   // blocks per sub-tile
     int32_t most_blocks;  // blocks of the plan's largest layer
     int32_t most_bits;    // widest code of the plan
+    int32_t least_bits;   // narrowest code of the plan
     int32_t dec_blocks;   // blocks per decoder CTA; 1: its warps share them
     int32_t dec_shift;    // log2(plan's tile size / dec_blocks)
     int32_t global_norm;  // 1: one norm per worker over all layers (Section 3.1), 0: one per layer
@@ -179,9 +180,17 @@ cudaError_t launch_norm_finalize(const PlanDev& p, float* norms, cudaStream_t s)
 struct SearchTables {
     uint32_t* lut;     // [L][kLutEntries] per bin: 8 * tau0 | (low 19 bits of the level inside the bin, minus 1) << 13
     float2* ld;        // [L][kMaxLevels]  {l_tau, l_{tau+1} - l_tau}
-    int32_t* fast;     // [L]              1 if every bin holds at most one level; else 1 + R (byte table over the top 15
-                       //                  bits in lut's place, at most R levels per bin)
+    int2* how;         // [L]              which search a layer takes and its parameters
 };
+// how.x & 3:
+//   kSearchOctave  bins of 1/16 octave over the whole fp32 range, at most one level in each
+//   kSearchWindow  bins of 2^s patterns, s = how.x >> 2, from the pattern how.y on (bin 0: everything below, too), at most one
+//                  level in each: level sets too dense for 16 bins per octave whose range from the first level to 1 fits
+//                  2048 bins that are fine enough (uniform 8-bit levels)
+//   kSearchStep    byte table over the top 15 bits in lut's place, and at most how.x >> 2 levels per bin: the rest
+constexpr int kSearchOctave = 1, kSearchStep = 2, kSearchWindow = 3;
+constexpr int kWindowBits = 5;      // narrowest codes with a window search: fewer levels are hardly ever that dense, and every search
+                                    // more in a kernel costs the others registers
 cudaError_t launch_build_search(const PlanDev& p, const float* levels, float* kept, SearchTables t, cudaStream_t s);
 cudaError_t launch_quantize(const PlanDev& p, const float* grads, uint32_t step, uint32_t* packed,
                             const float* norms, uint32_t* hist, const uint32_t* prev_packed,
@@ -227,6 +236,44 @@ cudaError_t launch_fit_shared(const PlanDev& p, const uint32_t* hist, const floa
 // this kernel's last ones leave them), and nothing written by the kernels before this one is read until they are done.
 __device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// What a kernel that may overlap its predecessor reads after pdl_wait, and an earlier kernel of the stream may have written,
+// must neither be read early nor through the read-only path, which takes memory as constant while the kernel runs: the
+// compiler moves such loads (__ldg, const __restrict__ parameters, and the load intrinsics, which it takes for pure functions
+// of the address) above the wait.  So: ordinary loads, the volatile ones below, or intrinsics on a pointer from fresh().
+// All go to L2.
+template <typename T>
+__device__ __forceinline__ T* fresh(T* p) { asm volatile("" : "+l"(p) :: "memory"); return p; }
+__device__ __forceinline__ float load_f32(const float* p)
+{
+    float v;
+    asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ float2 load_f32x2(const float2* p)
+{
+    float2 v;
+    asm volatile("ld.global.cg.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint32_t load_u8(const uint8_t* p)
+{
+    uint32_t v;
+    asm volatile("ld.global.cg.u8 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ int2 load_i32x2(const int2* p)
+{
+    int2 v;
+    asm volatile("ld.global.cg.v2.s32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint4 load_u32x4(const uint4* p)
+{
+    uint4 v;
+    asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+    return v;
+}
 
 // Philox4x32-10 (Salmon et al., SC'11): 10 rounds of two 32x32->64 multiplies and xors,
 // the key bumped by the Weyl constants between rounds.
@@ -359,7 +406,7 @@ __device__ __forceinline__ void accumulate(double& acc, uint32_t& maxbits, float
     }
 }
 
-// One block of 1024 values (a lane takes the float4 at 128 j + 4 lane of row j): adds its terms to the lane's
+// One block of 1024 values of a fresh() pointer (a lane takes the float4 at 128 j + 4 lane of row j): adds its terms to the lane's
 // accumulators and returns, in every lane, the byte whose bit j says whether row j holds anything but zeros.
 template <int kMode>
 __device__ __forceinline__ uint32_t norm_block(const float* __restrict__ g, int64_t blk, int64_t size, int lane, int q,
@@ -371,7 +418,7 @@ __device__ __forceinline__ uint32_t norm_block(const float* __restrict__ g, int6
         float4 v[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j)
-            v[j] = __ldg(reinterpret_cast<const float4*>(g + base + 128 * j));
+            v[j] = __ldcg(reinterpret_cast<const float4*>(g + base + 128 * j));
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             accumulate<kMode>(acc, maxbits, v[j].x, q);
@@ -388,7 +435,7 @@ __device__ __forceinline__ uint32_t norm_block(const float* __restrict__ g, int6
 #pragma unroll
             for (int e = 0; e < 4; ++e)
                 if (pos + e < size) {
-                    const float x = __ldg(g + pos + e);
+                    const float x = __ldcg(g + pos + e);
                     accumulate<kMode>(acc, maxbits, x, q);
                     mag += fabsf(x);
                 }

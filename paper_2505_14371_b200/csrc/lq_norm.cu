@@ -9,7 +9,7 @@
 namespace lq {
 
 template <int kMode>
-__global__ void __launch_bounds__(kThreads) norm_partial_kernel(PlanDev p, const float* __restrict__ grads,
+__global__ void __launch_bounds__(kThreads) norm_partial_kernel(PlanDev p, const float* grads,
                                                                 bool write_mask)
 {
     __shared__ double scratch[kThreads / 32];
@@ -20,8 +20,8 @@ __global__ void __launch_bounds__(kThreads) norm_partial_kernel(PlanDev p, const
     const LayerDesc L = p.layers[tile.layer];
     const int k = blockIdx.y + p.worker0;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const float* __restrict__ g = grads + (int64_t)blockIdx.y * p.padded_elems + L.elem_off;
     pdl_wait();
+    const float* g = fresh(grads + (int64_t)blockIdx.y * p.padded_elems + L.elem_off);
 
     double acc = 0.0;
     uint32_t maxbits = 0;
@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(128) norm_finalize_kernel(PlanDev p, float* __
     const int m = blockIdx.x, k = blockIdx.y + p.worker0;
     const LayerDesc L = p.layers[m];
     pdl_wait();
-    const double* part = p.norm_partial + ((int64_t)k * p.num_tiles + L.first_tile) * p.sub_tiles;
+    const double* part = fresh(p.norm_partial + ((int64_t)k * p.num_tiles + L.first_tile) * p.sub_tiles);
     const LayerNorm r = layer_norm_from_partials(part, L.ntiles * p.sub_tiles, p.q, scratch);
     if (threadIdx.x == 0) {
         const int64_t o = (int64_t)k * p.num_layers + m;

@@ -15,7 +15,7 @@
 // instruction issue (about 42 instructions per coordinate: 10 Philox, 7 the statistic), not by DRAM.
 //
 // The level search and the tables are described in lq_quantize.cuh.  Layers whose levels are denser than the
-// search table's bins take a byte table over finer bins and step up from its entry (build_search_kernel).
+// search table's bins take finer bins, or a byte table and steps up from its entry (build_search_kernel).
 //
 // The norm pass, which reads the same values just before, leaves one bit per row of 128 values
 // that says whether the row holds anything but zeros.  An all-zero row (untouched embedding rows)
@@ -28,12 +28,12 @@
 
 namespace lq {
 
-template <bool kHist, bool kStat>
+// kWidth: the code width of every layer of the plan, or 0 when they differ.  (A kernel of one width is compiled to what that
+// width needs: fewer spills, less code.)
+template <int kWidth, bool kHist, bool kStat>
 __global__ void __launch_bounds__(kQThreads, 4) quantize_pack_kernel(
-    PlanDev p, const float* __restrict__ grads, uint32_t step, uint32_t* __restrict__ packed,
-    const float* __restrict__ norms, uint32_t* __restrict__ hist,
-    const uint32_t* __restrict__ prev_packed, const float* __restrict__ prev_norms,
-    const float* __restrict__ levels_cur, const float* __restrict__ levels_prev, SearchTables st)
+    PlanDev p, const float* grads, uint32_t step, uint32_t* packed, const float* norms, uint32_t* hist,
+    const uint32_t* prev_packed, const float* prev_norms, const float* levels_cur, const float* levels_prev, SearchTables st)
 {
     extern __shared__ unsigned char dyn_smem[];
     uint32_t base;
@@ -58,25 +58,25 @@ __global__ void __launch_bounds__(kQThreads, 4) quantize_pack_kernel(
 
     // Everything below depends on the job record only, so all of it is requested at once: the norms, this thread's
     // two pieces of the search table, the zero-row masks of its block, the levels of its table entries.
-    const float ncur = norms[kl];
-    const float nprev = prev_norms ? prev_norms[kl] : 0.0f;
-    const float rn = p.rnorm[kl];
-    const int search = st.fast[layer];                      // 1: one lookup; 1 + R: byte table and up to R steps
+    const float ncur = load_f32(norms + kl);
+    const float nprev = prev_norms ? load_f32(prev_norms + kl) : 0.0f;
+    const float rn = load_f32(p.rnorm + kl);
+    const int2 how = load_i32x2(st.how + layer);
     const uint4* lsrc = reinterpret_cast<const uint4*>(st.lut + (int64_t)layer * kLutEntries);
-    const uint4 lut0 = __ldg(lsrc + threadIdx.x), lut1 = __ldg(lsrc + kQThreads + threadIdx.x);
+    const uint4 lut0 = load_u32x4(lsrc + threadIdx.x), lut1 = load_u32x4(lsrc + kQThreads + threadIdx.x);
     uint32_t mcur = 0, mprev = 0;
     if (threadIdx.x < tile.nblocks) {
         // a previous message whose masks are unknown is taken as nonzero everywhere
         const int64_t mb = (int64_t)k * p.total_blocks + L.block_off + tile.block0 + threadIdx.x;
-        mcur = p.row_mask[mb];
-        mprev = (!kStat || !prev_packed) ? 0u : (p.row_mask_prev ? (uint32_t)p.row_mask_prev[mb] : 0xffu);
+        mcur = load_u8(p.row_mask + mb);
+        mprev = (!kStat || !prev_packed) ? 0u : (p.row_mask_prev ? load_u8(p.row_mask_prev + mb) : 0xffu);
     }
     float lc = 0.f, lp = 0.f;
     float2 lg = make_float2(0.f, 0.f);
     if (threadIdx.x < L.nlevels) {
-        lc = levels_cur[(int64_t)layer * kLevelStride + threadIdx.x];
-        lp = levels_prev[(int64_t)layer * kLevelStride + threadIdx.x];
-        lg = st.ld[(int64_t)layer * kMaxLevels + threadIdx.x];
+        lc = load_f32(levels_cur + (int64_t)layer * kLevelStride + threadIdx.x);
+        lp = load_f32(levels_prev + (int64_t)layer * kLevelStride + threadIdx.x);
+        lg = load_f32x2(st.ld + (int64_t)layer * kMaxLevels + threadIdx.x);
     }
     {
         uint4* ldst = reinterpret_cast<uint4*>(sm + kSmLut);
@@ -93,6 +93,7 @@ __global__ void __launch_bounds__(kQThreads, 4) quantize_pack_kernel(
             for (int i = threadIdx.x; i < LQ_HIST_STRIDE; i += kQThreads) h[i] = 0;
         }
     }
+    if (threadIdx.x == 0) *reinterpret_cast<int2*>(sm + kSmHow) = how;
     uint8_t* rows_cur = sm + kSmRows;
     uint8_t* rows_prev = rows_cur + kTileBlocks;
     if (threadIdx.x < tile.nblocks) {
@@ -102,21 +103,20 @@ __global__ void __launch_bounds__(kQThreads, 4) quantize_pack_kernel(
     __syncthreads();
 
     WarpCtx c;
-    c.g = grads + (int64_t)kk * p.padded_elems + L.elem_off;
+    c.g = fresh(grads + (int64_t)kk * p.padded_elems + L.elem_off);
     c.size = L.size;
     c.nfull = L.size / kBlockCoords;
     c.lane = lane;
     QuantEnv ev;
     ev.lut = base + kSmLut; ev.ld = base + kSmLd; ev.tprev = base + kSmTprev;
     ev.r = rn;
-    ev.refine = search - 1;
     ev.hist = reinterpret_cast<uint32_t*>(sm + kSmHist);
     if (step == LQ_STEP_AUTO) step = (uint32_t)p.scalars->t;      // the plan's own iteration counter (graph replays)
     const PhiloxConsts pc = philox_fold((uint32_t)layer, (uint32_t)k, step, p.seed_lo, p.seed_hi);
     uint32_t* out = packed + (int64_t)k * p.packed_words + L.word_off;
-    const uint32_t* prev = prev_packed ? prev_packed + (int64_t)k * p.packed_words + L.word_off : nullptr;
+    const uint32_t* prev = prev_packed ? fresh(prev_packed + (int64_t)k * p.packed_words + L.word_off) : nullptr;
 
-    const double stat = quantize_blocks<kHist, kStat>(p, pc, c, tile, L.bits, search, (uint32_t)layer, (uint32_t)k, step, out, prev, ev,
+    const double stat = quantize_blocks<kWidth, kHist, kStat>(p, pc, c, tile, L.bits, how.x & 3, (uint32_t)layer, (uint32_t)k, step, out, prev, ev,
                                                       rows_cur, rows_prev, base + kSmRing);
     const double total = block_reduce<false>(stat, reinterpret_cast<double*>(sm + kSmScratch));
     if (threadIdx.x == 0) p.stat_partial[(int64_t)k * p.num_tiles + tile_id] = total;
@@ -152,20 +152,21 @@ __global__ void __launch_bounds__(128) stat_finalize_kernel(PlanDev p)
 //   lut[bin] = 8 * tau0 | code << 13    bin = bits(u) >> 19, i.e. the values [lo, hi) with bits(lo) = bin << 19;
 //              tau0 = last level (<= n-2) at or below lo; code = (low 19 bits of l_{tau0+1}) - 1 if that level
 //              (<= n-2) lies inside the bin, else all ones, so that  (bits(u) << 13) > lut[bin]  iff  u >= l_{tau0+1}
-//   fast     = 1: no bin holds two or more levels (then tau is tau0 or tau0 + 1)
-// Layers with denser levels (8-bit codes) get a byte table over the top 15 bits instead, in the same 8 KB:
+// Layers with two levels in such a bin and 5 bits or more get bins of 2^s patterns from just below the first level up to
+// 1.0, with the finest s that 2048 bins allow and the same entries (code: the low s bits, in the entry's top s bits).  If two
+// levels still share a bin, or below 5 bits, a byte table over the top 15 bits takes the same 8 KB:
 //   lut8[bits(u) >> 17] = tau0 of that finer bin; tau is found by stepping up while l_{tau+1} <= u, at most R times,
-//   R = the most levels inside one bin;  fast = 1 + R.
-__global__ void __launch_bounds__(256) build_search_kernel(PlanDev p, const float* __restrict__ levels,
-                                                           float* __restrict__ kept, SearchTables t)
+//   R = the most levels inside one bin.
+// (8-bit uniform levels took the byte table and 3 steps before: 201 M coordinates in 593 us, 419 us with one lookup.)
+__global__ void __launch_bounds__(256) build_search_kernel(PlanDev p, const float* levels, float* kept, SearchTables t)
 {
     __shared__ float lev[kMaxLevels];
-    __shared__ int slow, most;
+    __shared__ int shared_bin, most;
     pdl_launch_next();
     pdl_wait();
     const int m = blockIdx.x;
     const int n = p.layers[m].nlevels;
-    if (threadIdx.x == 0) { slow = 0; most = 0; }
+    if (threadIdx.x == 0) { shared_bin = 0; most = 0; }
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         lev[i] = levels[(int64_t)m * kLevelStride + i];
         kept[(int64_t)m * kLevelStride + i] = lev[i];
@@ -176,42 +177,64 @@ __global__ void __launch_bounds__(256) build_search_kernel(PlanDev p, const floa
         if (i <= n - 2) e.y = __fsub_rn(lev[i + 1], lev[i]);
         t.ld[(int64_t)m * kMaxLevels + i] = e;
     }
-    for (int bin = threadIdx.x; bin < kLutEntries; bin += blockDim.x) {
-        const uint32_t lob = (uint32_t)bin << 19;
-        // bins past 1.0 (and the patterns of Inf / NaN) behave like the bin of 1.0: the last interval
-        const bool top = lob >= 0x3f800000u;
-        const float lo = __uint_as_float(top ? 0x3f800000u : lob);
-        int tau0 = 0;
-        for (int j = 1; j <= n - 2; ++j) if (lev[j] <= lo) tau0 = j;
-        uint32_t code = 0x7ffffu;
-        if (!top && tau0 + 1 <= n - 2) {
-            const uint32_t nb = __float_as_uint(lev[tau0 + 1]);
-            if ((nb >> 19) == (uint32_t)bin) {                         // l_{tau0+1} > lo lies inside this bin
-                code = (nb & 0x7ffffu) - 1u;
-                if (tau0 + 2 <= n - 2 && (__float_as_uint(lev[tau0 + 2]) >> 19) == (uint32_t)bin) atomicOr(&slow, 1);
+    // the last level <= n - 2 at or below x
+    auto tau_of = [&](float x) {
+        int tau = 0;
+        for (int s = n >> 1; s > 0; s >>= 1)
+            if (lev[tau + s] <= x) tau += s;
+        return min(tau, n - 2);
+    };
+    constexpr uint32_t kOne = 0x3f800000u;               // bins past 1.0 (and Inf / NaN) behave like the bin of 1.0
+    uint32_t* lut = t.lut + (int64_t)m * kLutEntries;
+    // bins of 2^s patterns, bin i from off + i 2^s on; returns whether two levels share one
+    auto fill = [&](int s, uint32_t off) {
+        const uint32_t mask = (1u << s) - 1u;
+        for (int bin = threadIdx.x; bin < kLutEntries; bin += blockDim.x) {
+            const uint32_t lob = off + ((uint32_t)bin << s);
+            const bool top = lob >= kOne;
+            const int tau0 = tau_of(__uint_as_float(top ? kOne : lob));
+            uint32_t code = mask;
+            if (!top && tau0 + 1 <= n - 2) {
+                const uint32_t nb = __float_as_uint(lev[tau0 + 1]);
+                if ((nb >> s) == (lob >> s)) {                              // l_{tau0+1} > lo lies inside this bin
+                    code = (nb & mask) - 1u;
+                    if (tau0 + 2 <= n - 2 && (__float_as_uint(lev[tau0 + 2]) >> s) == (lob >> s)) atomicOr(&shared_bin, 1);
+                }
             }
-        }
-        const uint32_t entry = (code << 13) | (8u * (uint32_t)tau0);
-        t.lut[(int64_t)m * kLutEntries + bin] = entry;
-    }
-    __syncthreads();
-    if (slow) {
-        uint8_t* lut8 = reinterpret_cast<uint8_t*>(t.lut + (int64_t)m * kLutEntries);
-        for (int bin = threadIdx.x; bin < 4 * kLutEntries; bin += blockDim.x) {
-            const uint32_t lob = (uint32_t)bin << 17;
-            const bool top = lob >= 0x3f800000u;
-            const float lo = __uint_as_float(top ? 0x3f800000u : lob);
-            int tau0 = 0, inside = 0;
-            for (int j = 1; j <= n - 2; ++j) {
-                if (lev[j] <= lo) tau0 = j;
-                else if (!top && (__float_as_uint(lev[j]) >> 17) == (uint32_t)bin) ++inside;
-            }
-            lut8[bin] = (uint8_t)tau0;
-            atomicMax(&most, inside);
+            lut[bin] = (code << (32 - s)) | (8u * (uint32_t)tau0);
         }
         __syncthreads();
+        const int r = shared_bin;
+        __syncthreads();
+        if (threadIdx.x == 0) shared_bin = 0;
+        __syncthreads();
+        return r != 0;
+    };
+    int2 how = make_int2(kSearchOctave, 0);
+    bool dense = fill(19, 0u);
+    if (dense && n >= 1 << kWindowBits) {
+        const uint32_t first = __float_as_uint(lev[1]);
+        int s = 2;
+        while ((kOne >> s) - (first >> s) + 1u >= (uint32_t)kLutEntries) ++s;
+        const uint32_t off = ((first >> s) - 1u) << s;                     // (a level is at least 2^-100: no wrap)
+        how = make_int2(kSearchWindow | (s << 2), (int)off);
+        dense = fill(s, off);
     }
-    if (threadIdx.x == 0) t.fast[m] = slow ? 1 + most : 1;
+    if (dense) {
+        uint8_t* lut8 = reinterpret_cast<uint8_t*>(lut);
+        for (int bin = threadIdx.x; bin < 4 * kLutEntries; bin += blockDim.x) {
+            const uint32_t lob = (uint32_t)bin << 17;
+            const bool top = lob >= kOne;
+            const int tau0 = tau_of(__uint_as_float(top ? kOne : lob));
+            lut8[bin] = (uint8_t)tau0;
+            int inside = 0;
+            while (!top && tau0 + 1 + inside <= n - 2 && (__float_as_uint(lev[tau0 + 1 + inside]) >> 17) == (uint32_t)bin) ++inside;
+            if (inside) atomicMax(&most, inside);
+        }
+        __syncthreads();
+        how = make_int2(kSearchStep | (most << 2), 0);
+    }
+    if (threadIdx.x == 0) t.how[m] = how;
 }
 
 cudaError_t launch_build_search(const PlanDev& p, const float* levels, float* kept, SearchTables t, cudaStream_t s)
@@ -229,12 +252,18 @@ cudaError_t launch_quantize(const PlanDev& p, const float* grads, uint32_t step,
     const dim3 grid((unsigned)p.num_tiles, (unsigned)p.worker_count);
     // the ring follows the tables; the histogram (histogram mode only) follows the ring
     constexpr unsigned smem = kSmTables + kRingBytes + kSmSlack, smem_hist = smem + LQ_HIST_STRIDE * 4;
-    static std::atomic<uint64_t> configured{0};
-    const cudaError_t e = opt_in_shared_memory(configured, (int)smem_hist, quantize_pack_kernel<true, true>,
-                                               quantize_pack_kernel<false, true>, quantize_pack_kernel<false, false>);
+    using Kernel = void (*)(PlanDev, const float*, uint32_t, uint32_t*, const float*, uint32_t*, const uint32_t*, const float*,
+                            const float*, const float*, SearchTables);
+#define LQ_ALL(H, S) {quantize_pack_kernel<0, H, S>, quantize_pack_kernel<1, H, S>, quantize_pack_kernel<2, H, S>, \
+                      quantize_pack_kernel<3, H, S>, quantize_pack_kernel<4, H, S>, quantize_pack_kernel<5, H, S>, \
+                      quantize_pack_kernel<6, H, S>, quantize_pack_kernel<7, H, S>, quantize_pack_kernel<8, H, S>}
+    static const Kernel kernels[3][9] = {LQ_ALL(false, false), LQ_ALL(false, true), LQ_ALL(true, true)};
+#undef LQ_ALL
+    const int mode = hist ? 2 : need_stat ? 1 : 0, width = p.least_bits == p.most_bits ? p.most_bits : 0;
+    const Kernel kernel = kernels[mode][width];
+    static std::atomic<uint64_t> configured[3][9];
+    const cudaError_t e = opt_in_shared_memory(configured[mode][width], (int)smem_hist, kernel);
     if (e != cudaSuccess) return e;
-    const auto kernel = hist ? quantize_pack_kernel<true, true>
-                        : need_stat ? quantize_pack_kernel<false, true> : quantize_pack_kernel<false, false>;
     return launch(kernel, grid, kQThreads, hist ? smem_hist : smem, s, p, grads, step, packed, norms, hist, prev_packed,
                   prev_norms, levels_cur, levels_prev, t);
 }

@@ -34,6 +34,8 @@ constexpr uint32_t kSmTcur = 0x2800;
 constexpr uint32_t kSmTprev = 0x3000;
 constexpr uint32_t kSmRows = 0x3800;               // u8[kTileBlocks] rows of this input, u8[kTileBlocks] of the previous one
 constexpr uint32_t kSmScratch = 0x3900;            // double[kQWarps]
+constexpr uint32_t kSmHow = 0x3940;                // int2: SearchTables::how of the layer (here and not in registers that
+                                                   // the octave search's code would have to carry)
 constexpr uint32_t kSmTables = 0x3A00;             // end of the tables = start of the per-warp rings (a multiple of 512)
 constexpr uint32_t kSmRing = kSmTables;
 constexpr uint32_t kRingBytes = kQWarps * 8 * 512; // 8 rows of 512 bytes per warp
@@ -181,9 +183,23 @@ __device__ __forceinline__ void philox4x32_10_folded(uint32_t ctr0, const Philox
 struct QuantEnv {
     uint32_t lut, ld, tprev;
     float r;
-    int refine;          // layers whose levels are too dense for the one-lookup search: byte table over the top 15
-                         // bits, then up to `refine` steps upwards
     uint32_t* hist;      // the CTA's histogram (generic pointer), histogram mode only
+};
+
+// The parameters of a search that is not the octave search, once per warp.
+template <int kSearch>
+struct SearchPar {
+    int par;             // kSearchStep: most steps upwards from the byte table's entry; kSearchWindow: patterns per bin (log2)
+    int neg_off;         // kSearchWindow: minus the pattern at which bin 0 starts
+    __device__ __forceinline__ SearchPar(const QuantEnv& ev)
+    {
+        par = 0; neg_off = 0;
+        if (kSearch != kSearchOctave) {
+            const uint32_t at = ev.lut + (kSmHow - kSmLut);
+            par = (int)(lds_u32(at) >> 2);
+            neg_off = -(int)lds_u32(at + 4u);
+        }
+    }
 };
 
 // One coordinate: v -> symbol, added to the lane's words `cw` at position pp; its term of the step-size
@@ -192,7 +208,7 @@ struct QuantEnv {
 // norms (nrow now, pn in the previous message) scale them.  `counted`: the coordinate lies inside the layer
 // (histogram mode).
 template <int B, int kSearch, bool kHist, bool kStat, bool kBucket>
-__device__ __forceinline__ void quantize_coord(const QuantEnv& ev, float v, uint32_t x, int pp,
+__device__ __forceinline__ void quantize_coord(const QuantEnv& ev, const SearchPar<kSearch>& sp, float v, uint32_t x, int pp,
                                                uint32_t (&cw)[B + 1], const uint32_t (&pw)[B + 1], double& stat,
                                                float nrow, float pn, bool counted)
 {
@@ -202,13 +218,17 @@ __device__ __forceinline__ void quantize_coord(const QuantEnv& ev, float v, uint
     const float u = __fmul_rn(fabsf(v), ev.r);
     const uint32_t ub = __float_as_uint(u);
     uint32_t t8;                                             // address of {l_tau, gap}
-    if (kSearch == 1) {
+    if (kSearch == kSearchWindow) {
+        const uint32_t d = (uint32_t)__viaddmax_s32((int)ub, sp.neg_off, 0);
+        const uint32_t e = lds_u32(((d >> (sp.par - 2)) & 0x1FFCu) | ev.lut);
+        t8 = add8_if_gt_u32((e & 0x7F8u) | ev.ld, ub << (32 - sp.par), e);
+    } else if (kSearch == kSearchOctave) {
         const uint32_t e = lds_u32(((ub >> 17) & 0x1FFCu) | ev.lut);
         t8 = add8_if_gt_u32((e & 0x7F8u) | ev.ld, ub << 13, e);
     } else {
         // (u <= 1 + 2^-23 gives bits(u) >> 17 <= 8128; the mask keeps the pattern of a NaN inside the table too)
         t8 = ev.ld + 8u * lds_u8(((ub >> 17) & 0x1FFFu) | ev.lut);
-        for (int s = 0; s < ev.refine; ++s) t8 = add8_if_le(t8, lds_f32(t8 + 8u), u);
+        for (int s = 0; s < sp.par; ++s) t8 = add8_if_le(t8, lds_f32(t8 + 8u), u);
         t8 = min(t8, ev.ld + 8u * (uint32_t)(n - 2));
     }
     const float2 ld = lds_f32x2(t8);
@@ -254,16 +274,16 @@ __device__ __forceinline__ void fill_tables(unsigned char* sm, const SearchTable
     float* tcur = reinterpret_cast<float*>(sm + kSmTcur);
     float* tprev = reinterpret_cast<float*>(sm + kSmTprev);
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const float c = __fmul_rn(ncur, levels_cur[(int64_t)layer * kLevelStride + i]);
-        const float q = __fmul_rn(nprev, levels_prev[(int64_t)layer * kLevelStride + i]);
-        ld[i] = st.ld[(int64_t)layer * kMaxLevels + i];
+        const float c = __fmul_rn(ncur, load_f32(levels_cur + (int64_t)layer * kLevelStride + i));
+        const float q = __fmul_rn(nprev, load_f32(levels_prev + (int64_t)layer * kLevelStride + i));
+        ld[i] = load_f32x2(st.ld + (int64_t)layer * kMaxLevels + i);
         tcur[2 * i] = c;  tcur[2 * i + 1] = -c;
         tprev[2 * i] = q; tprev[2 * i + 1] = -q;
     }
     if (fast) {
         const uint4* src = reinterpret_cast<const uint4*>(st.lut + (int64_t)layer * kLutEntries);
         uint4* dst = reinterpret_cast<uint4*>(sm + kSmLut);
-        for (int i = threadIdx.x; i < kLutEntries / 4; i += blockDim.x) dst[i] = __ldg(src + i);
+        for (int i = threadIdx.x; i < kLutEntries / 4; i += blockDim.x) dst[i] = load_u32x4(src + i);
     }
     if (hist) {
         uint32_t* h = reinterpret_cast<uint32_t*>(sm + kSmHist);
@@ -284,7 +304,7 @@ __device__ __forceinline__ double zeroed_tile(const Tile& tile, int lane, uint32
         uint32_t pw[C];
 #pragma unroll
         for (int w = 0; w < C; ++w) {
-            pw[w] = prev ? __ldcs(prev + woff + w * 32) : 0u;
+            pw[w] = prev ? __ldcg(prev + woff + w * 32) : 0u;
             __stcs(out + woff + w * 32, 0u);
         }
 #pragma unroll

@@ -132,6 +132,7 @@ __device__ __forceinline__ double quantize_block(const PlanDev& p, const PhiloxC
     const int lane = c.lane;
     float my_norm, my_rnorm;                     // norm and reciprocal of row (lane >> 2)
     bool bad;
+    const SearchPar<kSearch> sp(ev);
     cp_async_wait<0>();                          // all 8 rows of the block have landed
     bucket_norms8(c.ring_ptr, c.q, lane, my_norm, my_rnorm, bad);
     if ((lane & 3) == 0) c.energy = fma((double)my_norm, (double)my_norm, c.energy);
@@ -170,7 +171,7 @@ __device__ __forceinline__ double quantize_block(const PlanDev& p, const PhiloxC
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const bool counted = !kHist || blk * kBlockCoords + 128 * j + 4 * lane + e < c.size;
-                quantize_coord<B, kSearch, kHist, true, true>(ev, vv[e], x[e], 4 * j + e, cw, pw, stat, nrow, pn, counted);
+                quantize_coord<B, kSearch, kHist, true, true>(ev, sp, vv[e], x[e], 4 * j + e, cw, pw, stat, nrow, pn, counted);
             }
         } else {
             pack_zero_row<C>(cw, j, ev.ld);
@@ -217,12 +218,12 @@ __device__ __forceinline__ double quantize_tile(const PlanDev& p, const PhiloxCo
         float prev_norm8 = 0.0f;
         uint32_t pmask = 0u;
         if (prev) {
-            if (c.lane < 8) prev_norm8 = __ldg(c.prev_bn + blk * 8 + c.lane);
+            if (c.lane < 8) prev_norm8 = __ldcg(c.prev_bn + blk * 8 + c.lane);
             pmask = __ballot_sync(0xffffffffu, prev_norm8 != 0.0f) & 0xffu;
         }
         uint32_t pw[C];
 #pragma unroll
-        for (int w = 0; w < C; ++w) pw[w] = pmask ? __ldcs(prev + blk * (int64_t)C * 32 + c.lane + w * 32) : 0u;
+        for (int w = 0; w < C; ++w) pw[w] = pmask ? __ldcg(prev + blk * (int64_t)C * 32 + c.lane + w * 32) : 0u;
         const int nb = b + kQWarps;
         const bool has_next = nb < tile.nblocks;
         const int64_t nblk = tile.block0 + nb;
@@ -237,10 +238,8 @@ __device__ __forceinline__ double quantize_tile(const PlanDev& p, const PhiloxCo
 
 template <bool kHist>
 __global__ void __launch_bounds__(kQThreads, 3) quantize_pack_bucket_kernel(
-    PlanDev p, const float* __restrict__ grads, uint32_t step, uint32_t* __restrict__ packed,
-    float* __restrict__ bucket_norms, uint32_t* __restrict__ hist,
-    const uint32_t* __restrict__ prev_packed, const float* __restrict__ prev_norms,
-    const float* __restrict__ levels_cur, const float* __restrict__ levels_prev, SearchTables st)
+    PlanDev p, const float* grads, uint32_t step, uint32_t* packed, float* bucket_norms, uint32_t* hist,
+    const uint32_t* prev_packed, const float* prev_norms, const float* levels_cur, const float* levels_prev, SearchTables st)
 {
     extern __shared__ unsigned char dyn_smem[];
     uint32_t base;
@@ -253,9 +252,10 @@ __global__ void __launch_bounds__(kQThreads, 3) quantize_pack_bucket_kernel(
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t kl = (int64_t)k * p.num_layers + layer;
     pdl_wait();
-    const int search = st.fast[layer];                      // 1: one lookup; 1 + R: byte table and up to R steps
+    const int2 how = load_i32x2(st.how + layer);
 
     // the tables hold the plain levels (norm 1) and each row multiplies by its own norm
+    if (threadIdx.x == 0) *reinterpret_cast<int2*>(sm + kSmHow) = how;
     fill_tables(sm, st, layer, L.nlevels, true, levels_cur, levels_prev, 1.0f, 1.0f, kHist);
     __syncthreads();
 
@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(kQThreads, 3) quantize_pack_bucket_kernel(
     c.ring = (uint32_t)__cvta_generic_to_shared(c.ring_ptr);
     c.lane = lane;
     const int64_t bo = (int64_t)k * p.total_blocks * 8 + L.block_off * 8;
-    c.prev_bn = prev_norms ? prev_norms + bo : nullptr;
+    c.prev_bn = prev_norms ? fresh(prev_norms + bo) : nullptr;
     c.bn_out = bucket_norms + bo;
     c.q = p.q;
     c.energy = 0.0;
@@ -274,20 +274,19 @@ __global__ void __launch_bounds__(kQThreads, 3) quantize_pack_bucket_kernel(
     QuantEnv ev;
     ev.lut = base + kSmLut; ev.ld = base + kSmLd; ev.tprev = base + kSmTprev;
     ev.r = 1.0f;
-    ev.refine = search - 1;
     ev.hist = reinterpret_cast<uint32_t*>(sm + kSmHist);
     if (step == LQ_STEP_AUTO) step = (uint32_t)p.scalars->t;      // the plan's own iteration counter (graph replays)
     const PhiloxConsts pc = philox_fold((uint32_t)layer, (uint32_t)k, step, p.seed_lo, p.seed_hi);
     uint32_t* out = packed + (int64_t)k * p.packed_words + L.word_off;
-    const uint32_t* prev = prev_packed ? prev_packed + (int64_t)k * p.packed_words + L.word_off : nullptr;
+    const uint32_t* prev = prev_packed ? fresh(prev_packed + (int64_t)k * p.packed_words + L.word_off) : nullptr;
 
     double stat = 0.0;
-    switch (L.bits * 2 + (search == 1 ? 1 : 0)) {
-#define LQ_CASE(BB)                                                                              \
-    case 2 * BB:     stat = quantize_tile<BB, 2, kHist>(p, pc, c, ev, tile, out, prev); break;  \
-    case 2 * BB + 1: stat = quantize_tile<BB, 1, kHist>(p, pc, c, ev, tile, out, prev); break;
+    switch (L.bits * 4 + (how.x & 3)) {
+#define LQ_SEARCH(BB, S) case 4 * BB + S: stat = quantize_tile<BB, S, kHist>(p, pc, c, ev, tile, out, prev); break;
+#define LQ_CASE(BB) LQ_SEARCH(BB, kSearchOctave) LQ_SEARCH(BB, kSearchStep) LQ_SEARCH(BB, kSearchWindow)
         LQ_CASE(1) LQ_CASE(2) LQ_CASE(3) LQ_CASE(4) LQ_CASE(5) LQ_CASE(6) LQ_CASE(7) LQ_CASE(8)
 #undef LQ_CASE
+#undef LQ_SEARCH
         default: break;
     }
     double* scratch = reinterpret_cast<double*>(sm + kSmScratch);

@@ -38,10 +38,8 @@ __device__ __forceinline__ double norm_of_blocks(const PlanDev& p, const float* 
 
 template <bool kHist, bool kStat>
 __global__ void __launch_bounds__(kQThreads, 3) quantize_small_kernel(
-    PlanDev p, const float* __restrict__ grads, uint32_t step, uint32_t* __restrict__ packed,
-    float* __restrict__ norms, uint32_t* __restrict__ hist,
-    const uint32_t* __restrict__ prev_packed, const float* __restrict__ prev_norms,
-    const float* __restrict__ levels_cur, const float* __restrict__ levels_prev, SearchTables st)
+    PlanDev p, const float* grads, uint32_t step, uint32_t* packed, float* norms, uint32_t* hist,
+    const uint32_t* prev_packed, const float* prev_norms, const float* levels_cur, const float* levels_prev, SearchTables st)
 {
     extern __shared__ unsigned char dyn_smem[];
     __shared__ double norm_part[8], stat_part[8];             // per CTA of the cluster
@@ -57,25 +55,25 @@ __global__ void __launch_bounds__(kQThreads, 3) quantize_small_kernel(
     tile.layer = layer; tile.block0 = rank * per; tile.nblocks = max(0, min(per, L.nblocks - tile.block0)); tile.pad_ = 0;
     const int lane = threadIdx.x & 31;
     const int64_t kl = (int64_t)k * p.num_layers + layer;
-    const float* g = grads + (int64_t)blockIdx.z * p.padded_elems + L.elem_off;
     pdl_wait();
+    const float* g = fresh(grads + (int64_t)blockIdx.z * p.padded_elems + L.elem_off);
     if (rank == 0 && layer == 0 && blockIdx.z == 0 && threadIdx.x == 0) p.scalars[1] = p.scalars[0];
 
     // everything that does not need the norm is requested before the values
-    const float nprev = prev_norms ? prev_norms[kl] : 0.0f;
-    const int search = st.fast[layer];                      // 1: one lookup; 1 + R: byte table and up to R steps
+    const float nprev = prev_norms ? load_f32(prev_norms + kl) : 0.0f;
+    const int2 how = load_i32x2(st.how + layer);
     const uint4* lsrc = reinterpret_cast<const uint4*>(st.lut + (int64_t)layer * kLutEntries);
-    const uint4 lut0 = __ldg(lsrc + threadIdx.x), lut1 = __ldg(lsrc + kQThreads + threadIdx.x);
+    const uint4 lut0 = load_u32x4(lsrc + threadIdx.x), lut1 = load_u32x4(lsrc + kQThreads + threadIdx.x);
     const int64_t mask_at = (int64_t)k * p.total_blocks + L.block_off + tile.block0 + threadIdx.x;
     uint32_t mprev = 0;
     if (threadIdx.x < tile.nblocks)
-        mprev = (!kStat || !prev_packed) ? 0u : (p.row_mask_prev ? (uint32_t)p.row_mask_prev[mask_at] : 0xffu);
+        mprev = (!kStat || !prev_packed) ? 0u : (p.row_mask_prev ? load_u8(p.row_mask_prev + mask_at) : 0xffu);
     float lc = 0.f, lp = 0.f;
     float2 lg = make_float2(0.f, 0.f);
     if (threadIdx.x < L.nlevels) {
-        lc = levels_cur[(int64_t)layer * kLevelStride + threadIdx.x];
-        lp = levels_prev[(int64_t)layer * kLevelStride + threadIdx.x];
-        lg = st.ld[(int64_t)layer * kMaxLevels + threadIdx.x];
+        lc = load_f32(levels_cur + (int64_t)layer * kLevelStride + threadIdx.x);
+        lp = load_f32(levels_prev + (int64_t)layer * kLevelStride + threadIdx.x);
+        lg = load_f32x2(st.ld + (int64_t)layer * kMaxLevels + threadIdx.x);
     }
     uint8_t* rows_cur = sm + kSmRows;
     uint8_t* rows_prev = rows_cur + kTileBlocks;
@@ -112,6 +110,7 @@ __global__ void __launch_bounds__(kQThreads, 3) quantize_small_kernel(
         reinterpret_cast<float2*>(sm + kSmTcur)[threadIdx.x] = make_float2(cv, -cv);
         reinterpret_cast<float2*>(sm + kSmTprev)[threadIdx.x] = make_float2(pv, -pv);
     }
+    if (threadIdx.x == 0) *reinterpret_cast<int2*>(sm + kSmHow) = how;
     if (threadIdx.x < tile.nblocks) {
         rows_prev[threadIdx.x] = (uint8_t)mprev;
         p.row_mask[mask_at] = rows_cur[threadIdx.x];
@@ -127,13 +126,12 @@ __global__ void __launch_bounds__(kQThreads, 3) quantize_small_kernel(
     QuantEnv ev;
     ev.lut = base + kSmLut; ev.ld = base + kSmLd; ev.tprev = base + kSmTprev;
     ev.r = ln.rnorm;
-    ev.refine = search - 1;
     ev.hist = reinterpret_cast<uint32_t*>(sm + kSmHist);
     if (step == LQ_STEP_AUTO) step = (uint32_t)p.scalars->t;      // the plan's own iteration counter (graph replays)
     const PhiloxConsts pc = philox_fold((uint32_t)layer, (uint32_t)k, step, p.seed_lo, p.seed_hi);
     uint32_t* out = packed + (int64_t)k * p.packed_words + L.word_off;
-    const uint32_t* prev = prev_packed ? prev_packed + (int64_t)k * p.packed_words + L.word_off : nullptr;
-    const double stat = quantize_blocks<kHist, kStat>(p, pc, c, tile, L.bits, search, (uint32_t)layer, (uint32_t)k, step, out, prev, ev,
+    const uint32_t* prev = prev_packed ? fresh(prev_packed + (int64_t)k * p.packed_words + L.word_off) : nullptr;
+    const double stat = quantize_blocks<0, kHist, kStat>(p, pc, c, tile, L.bits, how.x & 3, (uint32_t)layer, (uint32_t)k, step, out, prev, ev,
                                                       rows_cur, rows_prev, base + kSmRing);
     const double sum = block_reduce<false>(stat, scratch);
     if (threadIdx.x == 0) st_peer(&stat_part[rank], 0, sum);

@@ -38,7 +38,7 @@ static __device__ __noinline__ double quantize_partial_block(const PlanDev& p, c
         const int64_t pos = blk * kBlockCoords + 128 * (pp >> 2) + 4 * lane + (pp & 3);
         uint32_t sym = 0;
         if (pos < size) {
-            const float v = __ldg(g + pos);
+            const float v = __ldcg(g + pos);
             uint32_t x[4];
             philox4x32_10((uint32_t)(pos >> 2), layer, worker, step, p.seed_lo, p.seed_hi, x);
             const float u = __fmul_rn(fabsf(v), ev.r);
@@ -54,7 +54,7 @@ static __device__ __noinline__ double quantize_partial_block(const PlanDev& p, c
             if (hist) atomicAdd(ev.hist + ((max(__float_as_uint(u), kHistClamp) - kHistClamp) >> 19), 1u);
         }
         if (pfill < C) {
-            if (prev && pwi < C) pacc |= (uint64_t)__ldg(prev + woff + 32 * pwi) << pfill;
+            if (prev && pwi < C) pacc |= (uint64_t)__ldcg(prev + woff + 32 * pwi) << pfill;
             pfill += 32; ++pwi;
         }
         const uint32_t psym = (uint32_t)pacc & ((1u << C) - 1u);
@@ -102,6 +102,7 @@ __device__ __forceinline__ double quantize_tile(const PlanDev& p, const PhiloxCo
         if (kHist && lane == 0) atomicAdd(ev.hist, (uint32_t)kBlockCoords);     // its coordinates all have u = 0
     }
     if (todo == 0u) return stat;
+    const SearchPar<kSearch> sp(ev);
 
     auto block_base = [&](int i) { return c.g + (tile.block0 + warp + kQWarps * i) * (int64_t)kBlockCoords; };
     int i = __ffs(todo) - 1;
@@ -127,7 +128,7 @@ __device__ __forceinline__ double quantize_tile(const PlanDev& p, const PhiloxCo
         uint32_t pw[C];
 #pragma unroll
         for (int w = 0; w < C; ++w)
-            pw[w] = (kStat && prev && prows) ? __ldcs(prev + blk * (int64_t)C * 32 + lane + w * 32) : 0u;
+            pw[w] = (kStat && prev && prows) ? __ldcg(prev + blk * (int64_t)C * 32 + lane + w * 32) : 0u;
         uint32_t cw[C];
         pack_begin<C>(cw, ev.ld);
         const uint32_t ctr0 = (uint32_t)(blk * 256) + (uint32_t)lane;     // index / 4 of this lane's row 0
@@ -145,7 +146,7 @@ __device__ __forceinline__ double quantize_tile(const PlanDev& p, const PhiloxCo
                 const float vv[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
-                    quantize_coord<B, kSearch, kHist, kStat, false>(ev, vv[e], x[e], 4 * j + e, cw, pw, stat, 0.f, 0.f, true);
+                    quantize_coord<B, kSearch, kHist, kStat, false>(ev, sp, vv[e], x[e], 4 * j + e, cw, pw, stat, 0.f, 0.f, true);
             } else {
                 if ((mnext >> j) & 1u) cp_async16(ring + 512u * j, nsrc + 128 * j, 16);
                 cp_async_commit();
@@ -170,8 +171,24 @@ __device__ __forceinline__ double quantize_tile(const PlanDev& p, const PhiloxCo
     return stat;
 }
 
-// The CTA's blocks for the layer's code width and search; returns the thread's statistic term.
-template <bool kHist, bool kStat>
+// The whole blocks of a layer of width B.
+template <int B, bool kHist, bool kStat>
+__device__ __forceinline__ double quantize_width(const PlanDev& p, const PhiloxConsts& pc, const WarpCtx& c, const Tile& tile, int search,
+                                                 uint32_t* __restrict__ out, const uint32_t* __restrict__ prev, const QuantEnv& ev,
+                                                 const uint8_t* rows_cur, const uint8_t* rows_prev, uint32_t ring_base)
+{
+    if (ev.r == 0.0f) return zeroed_tile<B>(tile, c.lane, out, kStat ? prev : nullptr, ev.tprev);
+    if (search == kSearchOctave)
+        return quantize_tile<B, kSearchOctave, kHist, kStat>(p, pc, c, tile, out, prev, ev, rows_cur, rows_prev, ring_base);
+    if constexpr (B >= kWindowBits)
+        if (search == kSearchWindow)
+            return quantize_tile<B, kSearchWindow, kHist, kStat>(p, pc, c, tile, out, prev, ev, rows_cur, rows_prev, ring_base);
+    return quantize_tile<B, kSearchStep, kHist, kStat>(p, pc, c, tile, out, prev, ev, rows_cur, rows_prev, ring_base);
+}
+
+// The CTA's blocks for the layer's code width (kWidth, or `bits` where kWidth is 0) and search; returns the thread's
+// statistic term.
+template <int kWidth, bool kHist, bool kStat>
 __device__ __forceinline__ double quantize_blocks(const PlanDev& p, const PhiloxConsts& pc, const WarpCtx& c, const Tile& tile,
                                                   int bits, int search, uint32_t layer, uint32_t worker, uint32_t step,
                                                   uint32_t* __restrict__ out, const uint32_t* __restrict__ prev,
@@ -180,16 +197,17 @@ __device__ __forceinline__ double quantize_blocks(const PlanDev& p, const Philox
 {
     const bool zeroed = ev.r == 0.0f;
     double stat = 0.0;
-    switch (zeroed ? -bits : bits * 2 + (search == 1 ? 1 : 0)) {
-#define LQ_CASE(BB)                                                                                \
-    case -BB:        stat = kStat ? zeroed_tile<BB>(tile, c.lane, out, prev, ev.tprev)             \
-                                  : zeroed_tile<BB>(tile, c.lane, out, nullptr, ev.tprev); break;  \
-    case 2 * BB:     stat = quantize_tile<BB, 2, kHist, kStat>(p, pc, c, tile, out, prev, ev, rows_cur, rows_prev, ring_base); break;  \
-    case 2 * BB + 1: stat = quantize_tile<BB, 1, kHist, kStat>(p, pc, c, tile, out, prev, ev, rows_cur, rows_prev, ring_base); break;
-        LQ_CASE(1) LQ_CASE(2) LQ_CASE(3) LQ_CASE(4) LQ_CASE(5) LQ_CASE(6) LQ_CASE(7) LQ_CASE(8)
+    if constexpr (kWidth != 0) {
+        stat = quantize_width<kWidth, kHist, kStat>(p, pc, c, tile, search, out, prev, ev, rows_cur, rows_prev, ring_base);
+    } else {
+        switch (bits) {
+#define LQ_CASE(BB) case BB: stat = quantize_width<BB, kHist, kStat>(p, pc, c, tile, search, out, prev, ev, rows_cur, rows_prev, ring_base); break;
+            LQ_CASE(1) LQ_CASE(2) LQ_CASE(3) LQ_CASE(4) LQ_CASE(5) LQ_CASE(6) LQ_CASE(7) LQ_CASE(8)
 #undef LQ_CASE
-        default: break;
+            default: break;
+        }
     }
+    if (!kStat) stat = 0.0;
     // the layer's last, partial block, if it is among them: one warp, after its whole blocks
     const int64_t bp = c.nfull - tile.block0;
     if (!zeroed && (c.size % kBlockCoords) != 0 && bp >= 0 && bp < tile.nblocks && (int)(bp % kQWarps) == (threadIdx.x >> 5)) {
