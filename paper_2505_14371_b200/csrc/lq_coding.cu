@@ -115,51 +115,106 @@ __device__ __forceinline__ uint32_t symbol_at(const uint32_t (&w)[C + 1], int p)
     return v & ((1u << C) - 1u);
 }
 
-// Bits that a lane's 32 coordinates take in the stream.  code[symbol] = stream bits of the coordinate (word, then
-// the sign bit of a non-zero level; first bit in bit 0) | their number << 16.
+// The encoder takes two coordinates at a time.  Entry of a pair of symbols: their stream bits (word, then the sign bit of a
+// non-zero level; first bit in bit 0; at most 26 bits) in bits 0..26, the number of bits in bits 27..31.  Symbols of up to
+// kPairBits bits have a table of pairs in shared memory, wider ones join the entries of two single symbols.
+constexpr int kPairBits = 6;
+constexpr int kLenShift = 27;
+constexpr uint32_t kCodeMask = (1u << kLenShift) - 1u;
+constexpr int kEncEntries = 1 << (2 * kPairBits);
+
+__device__ __forceinline__ uint32_t join_entries(uint32_t e0, uint32_t e1)
+{
+    const uint32_t l0 = e0 >> kLenShift;
+    return ((e0 & kCodeMask) | ((e1 & kCodeMask) << l0)) | ((l0 + (e1 >> kLenShift)) << kLenShift);
+}
+
+// Entry of the coordinates pp, pp + 1 (pp even) of a lane's string.
+template <int C>
+__device__ __forceinline__ uint32_t pair_entry(const uint32_t* code, const uint32_t (&w)[C + 1], int pp)
+{
+    if constexpr (C <= kPairBits) {
+        const int off = pp * C, i = off >> 5, s = off & 31;
+        uint32_t v;                                              // 4 * (the pair's 2 C bits)
+        if (s + 2 * C <= 32) v = s >= 2 ? (w[i] >> (s - 2)) : (w[i] << (2 - s));
+        else                 v = __funnelshift_r(w[i], w[i + 1], s - 2);
+        return *reinterpret_cast<const uint32_t*>(reinterpret_cast<const char*>(code) + (v & (((1u << (2 * C)) - 1u) << 2)));
+    } else {
+        return join_entries(code[symbol_at<C>(w, pp)], code[symbol_at<C>(w, pp + 1)]);
+    }
+}
+
+// Entry of the single coordinate pp (table of pairs: its pair with symbol 0, without that one's bits).
+template <int C>
+__device__ __forceinline__ uint32_t single_entry(const uint32_t* code, const uint32_t (&w)[C + 1], int pp)
+{
+    const uint32_t e = code[symbol_at<C>(w, pp)];
+    if constexpr (C <= kPairBits) {
+        const uint32_t l = (e >> kLenShift) - (code[0] >> (kLenShift + 1));       // (code[0]: symbol 0 twice)
+        return (e & ((1u << l) - 1u)) | (l << kLenShift);
+    } else {
+        return e;
+    }
+}
+
+// Bits that a lane's 32 coordinates take in the stream.
 template <int C, bool kFull>
 __device__ __forceinline__ uint32_t lane_bits(const uint32_t* code, const uint32_t (&w)[C + 1], int64_t blk, int lane,
                                               int64_t size)
 {
     uint32_t bits = 0;
+    if (kFull) {
 #pragma unroll
-    for (int pp = 0; pp < 32; ++pp) {
-        if (!kFull && !real_coord(blk, lane, pp, size)) continue;
-        bits += code[symbol_at<C>(w, pp)] >> 16;
+        for (int pp = 0; pp < 32; pp += 2) bits += pair_entry<C>(code, w, pp) >> kLenShift;
+    } else {
+#pragma unroll
+        for (int pp = 0; pp < 32; ++pp)
+            if (real_coord(blk, lane, pp, size)) bits += single_entry<C>(code, w, pp) >> kLenShift;
     }
     return bits;
 }
 
-// Writes a lane's coordinates into the block's buffer from bit `pos` on.  The lane's bits gather in a 64-bit word and
-// leave 32 at a time: the first and the last word it touches may be shared with its neighbours (atomic OR into the
-// zeroed buffer), the words between them are its own (plain stores).  Whole blocks are taken two coordinates at a
-// time: with fewer than 32 bits waiting, two coordinates (at most 26 bits) still fit.
-template <int C, bool kFull>
-__device__ __forceinline__ void lane_emit(const uint32_t* code, const uint32_t (&w)[C + 1], int64_t blk, int lane,
-                                          int64_t size, uint32_t pos, uint32_t* buf)
+// Writes a whole block's lane into the block's buffer from bit `pos` on.  The lane's bits gather in two registers and leave
+// a word at a time.  Every lane has 32 bits or more, so it completes the word it starts in, which at most the lane before
+// it shares: completed words are stored plainly, and after all lanes have done so each ORs the bits it has left over into
+// the word that the next lane has stored (the last lane stores them).
+template <int C>
+__device__ __forceinline__ void emit_full(const uint32_t* code, const uint32_t (&w)[C + 1], int lane, uint32_t pos, uint32_t* buf)
 {
-    uint64_t acc = 0;
-    uint32_t f = pos & 31u;
+    uint32_t lo = 0, f = pos & 31u;
     uint32_t* dst = buf + (pos >> 5);
-    bool first = true;
+#pragma unroll
+    for (int pp = 0; pp < 32; pp += 2) {
+        const uint32_t e = pair_entry<C>(code, w, pp), c = e & kCodeMask;
+        lo |= c << f;
+        const uint32_t hi = __funnelshift_l(c, 0u, f);           // the bits of c that do not fit (0 when f is 0)
+        f += e >> kLenShift;
+        if (f >= 32u) { *dst++ = lo; lo = hi; f -= 32u; }
+    }
+    __syncwarp();
+    if (lane == 31) { if (f) *dst = lo; }
+    else if (f) atomicOr(dst, lo);
+}
+
+// The same for a layer's last, partial block, coordinate by coordinate into a zeroed buffer.
+template <int C>
+__device__ __forceinline__ void emit_partial(const uint32_t* code, const uint32_t (&w)[C + 1], int64_t blk, int lane,
+                                             int64_t size, uint32_t pos, uint32_t* buf)
+{
 #pragma unroll
     for (int pp = 0; pp < 32; ++pp) {
-        if (!kFull && !real_coord(blk, lane, pp, size)) continue;
-        const uint32_t e = code[symbol_at<C>(w, pp)];
-        acc |= (uint64_t)(e & 0xffffu) << f;
-        f += e >> 16;
-        if ((kFull ? (pp & 1) == 1 : true) && f >= 32u) {
-            if (first) atomicOr(dst, (uint32_t)acc); else *dst = (uint32_t)acc;
-            first = false;
-            ++dst; acc >>= 32; f -= 32u;
-        }
+        if (!real_coord(blk, lane, pp, size)) continue;
+        const uint32_t e = single_entry<C>(code, w, pp);
+        const uint64_t c = (uint64_t)(e & kCodeMask) << (pos & 31u);
+        atomicOr(buf + (pos >> 5), (uint32_t)c);
+        if (c >> 32) atomicOr(buf + (pos >> 5) + 1, (uint32_t)(c >> 32));
+        pos += e >> kLenShift;
     }
-    if (f) atomicOr(dst, (uint32_t)acc);
 }
 
 constexpr int kCodeBufWords = kBlockCoords * (kCodeMaxLen + 1) / 32;      // longest block: every coordinate 13 bits
 
-// What the warps of an encoder CTA share about their sub-tile.
+// What the warps of an encoder CTA share about their tile.
 struct EncodeJob {
     const uint32_t* msg;         // the layer's words in this worker's message
     uint32_t* off;               // this worker's block sizes / offsets, at the layer's first block
@@ -167,35 +222,49 @@ struct EncodeJob {
     uint16_t* runs;              // this worker's run offsets at the layer's first block, or NULL
     uint16_t* lane_bits;         // this worker's bits per lane and block, at the layer's first block
     int64_t capacity, size;      // words of the stream buffer; coordinates of the layer
-    int block0, block1;          // the sub-tile's blocks [block0, block1) of the layer
+    int block0, block1;          // the tile's blocks [block0, block1) of the layer
+    uint32_t zero_bits;          // bits of the word of level 0; its pattern
+    uint32_t zero_code;
 };
 
-// A warp's blocks of a sub-tile for one symbol width (its own function per width, so that each is compiled with
+// A warp's blocks of a tile for one symbol width (its own function per width, so that each is compiled with
 // its own register budget).  kWrite = false: the words each block needs -> off[block].  true: the blocks are
-// written at off[block].
+// written at off[block].  The next block's words are requested before the current one is worked on.
 template <int C, bool kWrite>
 __device__ __noinline__ void encode_blocks(const EncodeJob& J, const uint32_t* code, uint32_t* bb)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t zero_code = code[0];
+    uint32_t next[C], next_bits = 0;
+    uint32_t next_first = 0;
+    auto request = [&](int64_t blk) {
+        if (blk >= J.block1) return;
+#pragma unroll
+        for (int i = 0; i < C; ++i) next[i] = __ldcs(J.msg + blk * (int64_t)C * 32 + i * 32 + lane);
+        if (kWrite) { next_bits = J.lane_bits[blk * 32 + lane]; next_first = J.off[blk]; }       // sized by the first pass
+    };
+    request(J.block0 + warp);
     for (int64_t blk = J.block0 + warp; blk < J.block1; blk += kWarps) {
         const bool full = (blk + 1) * kBlockCoords <= J.size;
         uint32_t w[C + 1];
         uint32_t any = 0;
 #pragma unroll
         for (int i = 0; i < C; ++i) {
-            w[i] = J.msg[blk * (int64_t)C * 32 + i * 32 + lane];
+            w[i] = next[i];
             any |= w[i];
         }
         w[C] = 0u;
-        // a lane whose coordinates are all level 0 (untouched rows): 32 times the word of level 0
-        const bool plain = full && any == 0u;
-        uint32_t bits;
-        if (kWrite) bits = J.lane_bits[blk * 32 + lane];     // sized by the first pass
-        else {
-            bits = 32u * (zero_code >> 16);
+        uint32_t bits = next_bits;
+        const int64_t first = next_first;
+        request(blk + kWarps);
+        // a block whose coordinates are all level 0 (untouched rows): 1024 times the word of level 0
+        const bool plain = full && __all_sync(0xffffffffu, any == 0u);
+        if (!kWrite) {
+            bits = 32u * J.zero_bits;
             if (!plain) bits = full ? lane_bits<C, true>(code, w, blk, lane, J.size) : lane_bits<C, false>(code, w, blk, lane, J.size);
             J.lane_bits[blk * 32 + lane] = (uint16_t)bits;
+            const uint32_t total = __reduce_add_sync(0xffffffffu, bits);
+            if (lane == 0) J.off[blk] = (total + 31u) >> 5;
+            continue;
         }
         uint32_t incl = bits;                                // inclusive prefix sum over the lanes
 #pragma unroll
@@ -205,30 +274,29 @@ __device__ __noinline__ void encode_blocks(const EncodeJob& J, const uint32_t* c
         }
         const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
         const uint32_t nwords = (total + 31u) >> 5;
-        if constexpr (!kWrite) {
-            if (lane == 0) J.off[blk] = nwords;
-        } else {
-        for (uint32_t i = lane; i < nwords; i += 32) bb[i] = 0u;
-        __syncwarp();
         const uint32_t pos = incl - bits;
         // where the runs of four lanes (128 coordinates) start inside the block's stream: lets a decoder work on
         // eight runs of a block at once
         if (J.runs && (lane & 3) == 0) J.runs[blk * LQ_CODE_RUNS + (lane >> 2)] = (uint16_t)pos;
-        if (!(plain && (zero_code & 0xffffu) == 0u)) {       // (32 words "0...0" of level 0 are already there)
-            if (full) lane_emit<C, true>(code, w, blk, lane, J.size, pos, bb);
-            else      lane_emit<C, false>(code, w, blk, lane, J.size, pos, bb);
+        const bool fits = first + nwords <= J.capacity;      // a stream buffer that is too small is never overrun
+        if (plain && J.zero_code == 0u) {
+            if (fits) for (uint32_t i = lane; i < nwords; i += 32) __stcs(J.out + first + i, 0u);
+            continue;
+        }
+        if (full) {
+            emit_full<C>(code, w, lane, pos, bb);
+        } else {
+            for (uint32_t i = lane; i < nwords; i += 32) bb[i] = 0u;
+            __syncwarp();
+            emit_partial<C>(code, w, blk, lane, J.size, pos, bb);
         }
         __syncwarp();
-        const int64_t first = J.off[blk];
-        if (first + nwords <= J.capacity) {                  // a stream buffer that is too small is never overrun
-            for (uint32_t i = lane; i < nwords; i += 32) J.out[first + i] = bb[i];
-        }
+        if (fits) for (uint32_t i = lane; i < nwords; i += 32) __stcs(J.out + first + i, bb[i]);
         __syncwarp();
-        }
     }
 }
 
-// One warp per block, one CTA per sub-tile (32 blocks of one layer).
+// One warp per block, one CTA per tile (up to 128 blocks of one layer; on 32 the CTA's tables took longer than its blocks).
 // kModeWrite = 0: words needed by every block -> sizes[k][block].   1: write the blocks at their offsets.
 template <int kModeWrite>
 __global__ void __launch_bounds__(kThreads, 4) entropy_encode_kernel(PlanDev p, const uint32_t* __restrict__ packed,
@@ -238,29 +306,35 @@ __global__ void __launch_bounds__(kThreads, 4) entropy_encode_kernel(PlanDev p, 
                                                                      uint16_t* __restrict__ run_offsets,
                                                                      uint16_t* __restrict__ lane_bits)
 {
-    __shared__ uint32_t code[2 * kMaxLevels];
+    __shared__ uint32_t code[kEncEntries];
+    __shared__ uint32_t single[2 * kMaxLevels];
     __shared__ uint32_t buf[kModeWrite ? kWarps : 1][kModeWrite ? kCodeBufWords : 1];
-    Tile tile = p.tiles[blockIdx.x >> p.sub_shift];
-    const int sub0 = (blockIdx.x & (p.sub_tiles - 1)) * p.sub_blocks;
-    if (sub0 >= tile.nblocks) return;
-    const int layer = tile.layer, k = blockIdx.y;
-    const LayerDesc L = p.layers[layer];
+    const TileJob T = p.jobs[blockIdx.x];
+    const int layer = T.layer, k = blockIdx.y;
     // per symbol (2 * level + sign): the level's word, the sign bit behind it unless the level is 0, and their length
-    for (int sym = threadIdx.x; sym < 2 * L.nlevels; sym += blockDim.x) {
+    const int C = T.bits + 1, nsym = 1 << C;
+    uint32_t* one = C <= kPairBits ? single : code;
+    for (int sym = threadIdx.x; sym < nsym; sym += blockDim.x) {
         const uint32_t e = enc_tables[(int64_t)layer * kMaxLevels + (sym >> 1)], l = e >> 16;
-        code[sym] = (sym >> 1) ? ((e & 0xffffu) | ((uint32_t)(sym & 1) << l) | ((l + 1u) << 16)) : e;
+        one[sym] = (sym >> 1) ? ((e & 0xffffu) | ((uint32_t)(sym & 1) << l) | ((l + 1u) << kLenShift)) : ((e & 0xffffu) | (l << kLenShift));
     }
     __syncthreads();
+    const uint32_t zero = one[0];
+    if (C <= kPairBits) {
+        for (int i = threadIdx.x; i < 1 << (2 * C); i += blockDim.x) code[i] = join_entries(single[i & (nsym - 1)], single[i >> C]);
+        __syncthreads();
+    }
     EncodeJob J;
-    J.msg = packed + (int64_t)k * p.packed_words + L.word_off;
-    J.off = offsets + (int64_t)k * (p.total_blocks + 1) + L.block_off;
+    J.msg = packed + (int64_t)k * p.packed_words + T.word_off;
+    J.off = offsets + (int64_t)k * (p.total_blocks + 1) + T.block_off;
     J.out = out + (int64_t)k * capacity;
-    J.runs = run_offsets ? run_offsets + ((int64_t)k * p.total_blocks + L.block_off) * LQ_CODE_RUNS : nullptr;
-    J.lane_bits = lane_bits + ((int64_t)k * p.total_blocks + L.block_off) * 32;
-    J.capacity = capacity; J.size = L.size;
-    J.block0 = tile.block0 + sub0; J.block1 = tile.block0 + min(sub0 + p.sub_blocks, tile.nblocks);
+    J.runs = run_offsets ? run_offsets + ((int64_t)k * p.total_blocks + T.block_off) * LQ_CODE_RUNS : nullptr;
+    J.lane_bits = lane_bits + ((int64_t)k * p.total_blocks + T.block_off) * 32;
+    J.capacity = capacity; J.size = T.size;
+    J.block0 = T.block0; J.block1 = T.block0 + T.nblocks;
+    J.zero_bits = zero >> kLenShift; J.zero_code = zero & kCodeMask;
     uint32_t* bb = buf[kModeWrite ? (threadIdx.x >> 5) : 0];
-    switch (L.bits + 1) {
+    switch (C) {
 #define LQ_CASE(CC) case CC: encode_blocks<CC, kModeWrite != 0>(J, code, bb); break;
         LQ_CASE(2) LQ_CASE(3) LQ_CASE(4) LQ_CASE(5) LQ_CASE(6) LQ_CASE(7) LQ_CASE(8) LQ_CASE(9)
 #undef LQ_CASE
@@ -545,7 +619,7 @@ cudaError_t launch_entropy_encode(const PlanDev& p, const uint32_t* packed, cons
                                   EncodeScratch scratch, cudaStream_t s)
 {
     if (p.num_tiles == 0) return cudaSuccess;
-    const dim3 grid((unsigned)p.num_tiles * p.sub_tiles, (unsigned)p.num_workers);
+    const dim3 grid((unsigned)p.num_tiles, (unsigned)p.num_workers);
     const dim3 chunks((unsigned)((p.total_blocks + 1023) / 1024), (unsigned)p.num_workers);
     entropy_encode_kernel<0><<<grid, kThreads, 0, s>>>(p, packed, enc_tables, offsets, out, capacity, nullptr, scratch.lane_bits);
     entropy_scan_sums_kernel<<<chunks, 1024, 0, s>>>(p, offsets, scratch.scan_part);
