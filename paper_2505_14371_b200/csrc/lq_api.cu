@@ -914,7 +914,7 @@ int lq_entropy_decode(lq_plan* plan, const uint32_t* stream_words, int64_t capac
     LQ_ALIGNED(packed, 4); LQ_ALIGNED(stream_words, 4); LQ_ALIGNED(block_offsets, 4);
     const int rc = ensure_codes(plan);
     if (rc != LQ_OK) return rc;
-    LQ_CUDA(launch_entropy_decode(plan->dev, stream_words, capacity_words, block_offsets, run_offsets, plan->d_code_dec,
+    LQ_CUDA(launch_entropy_decode(plan->dev, stream_words, capacity_words, block_offsets, run_offsets, plan->d_code_enc, plan->d_code_dec,
                                   packed, plan->d_code_bad, (cudaStream_t)stream));
     return LQ_OK;
 }

@@ -94,6 +94,24 @@ void build_code_tables_host(const uint8_t* len, const uint32_t* code, int n, uin
             dec[rev | (hi << l)] = (uint16_t)((2u * (uint32_t)s + sign) | ((uint32_t)(l + (s != 0 ? 1 : 0)) << kDecLenShift));
         }
     }
+    int C = 1;
+    while ((1 << C) < 2 * n) ++C;
+    if (C > kDecPairBits) return;
+    // what follows a window's first coordinate is the window shifted right: a smaller value (or 0 again), so going down
+    // every entry looked at is still a single one
+    for (uint32_t w = kDecEntries; w-- > 0;) {
+        const uint32_t e = dec[w], l = e >> kDecLenShift;
+        uint32_t out;
+        if (e & kDecInvalid) {
+            out = kDecPairInvalid | kDecSingle | (1u << kDecLenShift);
+        } else {
+            const uint32_t e1 = dec[w >> l], l1 = e1 >> kDecLenShift;
+            const bool second = !(e1 & kDecInvalid) && l + l1 <= (uint32_t)kDecBits;
+            out = (e & 0x1ffu) | (l << kDecLenShift) | kDecSingle;
+            if (second) out = (e & 0x1ffu) | ((e1 & 0x1ffu) << C) | ((l + l1) << kDecLenShift);
+        }
+        dec[w] = (uint16_t)out;
+    }
 }
 
 // ---- device ------------------------------------------------------------------------------------
@@ -416,9 +434,20 @@ __global__ void __launch_bounds__(1024) entropy_scan_apply_kernel(PlanDev p, uin
     if (i < p.total_blocks) a[i] = base_s + red[warp] + incl - v;
 }
 
+// One coordinate from the next 13 stream bits: its symbol, the bits it takes and whether no word matched.
+struct OneCoord { uint32_t sym, bits; bool invalid; };
+__device__ __forceinline__ OneCoord decode_one(uint32_t e, int C, const uint32_t* enc)
+{
+    if (C > kDecPairBits) return OneCoord{e & 0x1ffu, e >> kDecLenShift, (e & kDecInvalid) != 0u};
+    OneCoord r{e & ((1u << C) - 1u), e >> kDecLenShift, (e & kDecPairInvalid) != 0u};
+    if (!(e & kDecSingle)) r.bits = (enc[r.sym >> 1] >> 16) + (r.sym > 1u ? 1u : 0u);      // the first one's share of the pair's
+    return r;
+}
+
 // One thread per (block, worker): walks the block's stream and rebuilds the fixed-width words.
 __global__ void __launch_bounds__(128) entropy_decode_kernel(PlanDev p, const uint32_t* __restrict__ in, int64_t capacity,
                                                              const uint32_t* __restrict__ offsets,
+                                                             const uint32_t* __restrict__ enc_tables,
                                                              const uint16_t* __restrict__ dec_tables,
                                                              uint32_t* __restrict__ packed, uint32_t* __restrict__ bad)
 {
@@ -433,6 +462,7 @@ __global__ void __launch_bounds__(128) entropy_decode_kernel(PlanDev p, const ui
     const int64_t blk = g - L.block_off;
     const int C = L.bits + 1;
     const uint16_t* dec = dec_tables + (int64_t)layer * kDecEntries;
+    const uint32_t* enc = enc_tables + (int64_t)layer * kMaxLevels;
     const uint32_t* off_k = offsets + (int64_t)k * (p.total_blocks + 1);
     const int64_t first = off_k[g], last = min((int64_t)off_k[g + 1], capacity);
     const uint32_t* src = in + (int64_t)k * capacity;
@@ -446,28 +476,32 @@ __global__ void __launch_bounds__(128) entropy_decode_kernel(PlanDev p, const ui
         for (int pp = 0; pp < 32; ++pp) {
             if (!real_coord(blk, lane, pp, L.size)) continue;
             while (have <= 32) { const uint32_t x = wi < last ? src[wi] : 0u; ++wi; window |= (uint64_t)x << have; have += 32; }
-            const uint32_t e = dec[window & (uint32_t)(kDecEntries - 1)];
-            if (e & kDecInvalid) { broken = true; continue; }
-            const uint32_t sym = e & 0x1ffu, l = e >> kDecLenShift;
-            window >>= l; have -= (int)l;
+            const OneCoord c = decode_one(dec[window & (uint32_t)(kDecEntries - 1)], C, enc);
+            window >>= c.bits; have -= (int)c.bits;
+            if (c.invalid) { broken = true; continue; }
             const int off = pp * C, i = off >> 5, s = off & 31;
-            cw[i] |= sym << s;
-            if (s + C > 32) cw[i + 1] |= sym >> (32 - s);
+            cw[i] |= c.sym << s;
+            if (s + C > 32) cw[i + 1] |= c.sym >> (32 - s);
         }
         for (int i = 0; i < C; ++i) dst[i * 32 + lane] = cw[i];
     }
     if (broken || wi - 2 > last) atomicOr(bad, 1u);           // no valid word, or the block ran past its end
 }
 
-// Decoder on the run offsets.  A run is four lanes (128 coordinates) of a block; one CTA takes a sub-tile (32 blocks
-// of one layer = 256 runs) with the layer's decode table in shared memory.  First every thread looks at one run: a
+// Decoder on the run offsets.  A run is four lanes (128 coordinates) of a block; one CTA takes a tile (up to 128 blocks of
+// one layer = 1024 runs) with the layer's decode table in shared memory.  First every thread looks at some runs: a
 // run of 128 zero bits where "0" is the word of level 0 (what untouched rows turn into) is written as zeros at once;
 // the other runs are collected in a list, so that the walk below is done by full warps and not by the few lanes of
-// every warp whose run happens to hold values.  Then thread i walks the i-th run of the list from its recorded bit
-// offset: the next 13 stream bits come from a funnel shift over two of three words kept in registers, one table
-// lookup gives the symbol and the bits taken (the words are refilled every second coordinate).  A run that meets no
-// valid word, that would read past the block's end, or that does not end where the next run starts reports a broken
-// stream; nothing is read or written out of bounds.
+// every warp whose run happens to hold values.  Then the warps take 32 runs of the list at a time and a thread walks one
+// run from its recorded bit offset: the next 13 stream bits come from a funnel shift over two of three words kept in
+// registers, one table lookup gives two coordinates (one, where symbols are wider than 5 bits or two do not fit 13 bits),
+// A run that meets no valid word, that would read past the block's end, or
+// that does not end where the next run starts reports a broken stream; nothing is read or written out of bounds.
+//
+// What bounds the walk is its instructions (per two coordinates about 16, and 10 more when one lane's pair does not fit) and,
+// before, its loads: a thread that read its run word by word from global memory touched 16 lines a load and waited for
+// every second one, so a run's words are brought to shared memory at once.  Mostly zero tiles were walked by one or two warps
+// of a CTA while it took a CTA per 32 blocks, and each had its table to fetch first.
 struct RunRef {
     const uint32_t* src;     // first word of the block's stream
     int nwords;              // words of the block that may be read
@@ -477,75 +511,133 @@ struct RunRef {
 
 __device__ __forceinline__ uint32_t stream_word(const RunRef& r, int i) { return i < r.nwords ? __ldg(r.src + i) : 0u; }
 
-template <int C, bool kFull>
-__device__ __forceinline__ bool decode_run(const RunRef& r, const uint16_t* dec, int64_t blk, int run, int64_t size,
-                                           uint32_t* __restrict__ dst)
+// Shared memory of a CTA: decode table, list of runs, word lengths, then room for the stream words of every thread's run, an
+// odd number of 16-byte pieces; a broken run can read up to 13 * 128 bits on from its first word.
+constexpr int kRunsPerTile = kTileBlocks * LQ_CODE_RUNS;
+__host__ __device__ constexpr int run_pieces(int C) { return (C + 2) | 1; }
+constexpr int kRunList = kDecEntries * 2, kRunLen = kRunList + kRunsPerTile * 2, kRunTaken = kRunLen + 64;
+constexpr int kRunSmem(int bits) { return kRunTaken + kThreads * 16 * run_pieces(bits + 1) + 256; }
+extern __shared__ __align__(16) unsigned char run_smem[];
+
+__device__ __forceinline__ uint32_t run_entry(uint32_t bits)
 {
-    int wi = (int)(r.start_bit >> 5);
-    uint32_t lo = stream_word(r, wi), hi = stream_word(r, wi + 1), nx = stream_word(r, wi + 2);
-    wi += 3;                                                  // next word to load; `lo` is word wi - 3
-    uint32_t sh = r.start_bit & 31u, flags = 0, win = 0;
-    // Coordinates are taken in pairs: with sh < 32 the 32 bits from the current position lie inside {lo, hi}, and
-    // after the first coordinate (at most 13 bits) they still hold the second one whole.
+    return *reinterpret_cast<const uint16_t*>(run_smem + ((bits << 1) & (2u * kDecEntries - 2u)));
+}
+
+// Whole block, words in shared memory: `at` is the address of the run's first word.  `len`: bits of every symbol's word and
+// sign (pair tables).  Word i of lane l4 of the run goes to dst[32 i + l4].
+template <int C>
+__device__ __forceinline__ bool walk_run(const RunRef& r, uint32_t at, const uint8_t* len, uint32_t* dst)
+{
+    constexpr bool kPair = C <= kDecPairBits;
+    const uint32_t at0 = at;
+    uint32_t lo = lds_u32(at), hi = lds_u32(at + 4u), nx = lds_u32(at + 8u);       // `lo` is the word at `at`
+    uint32_t sh = r.start_bit & 31u, flags = 0;
 #pragma unroll 1
     for (int l4 = 0; l4 < 4; ++l4) {
-        const int lane = 4 * run + l4;
         uint32_t cw[C + 1];
 #pragma unroll
         for (int i = 0; i <= C; ++i) cw[i] = 0u;
 #pragma unroll
-        for (int pp = 0; pp < 32; ++pp) {
-            if (!kFull && !(blk * kBlockCoords + 128 * (pp >> 2) + 4 * lane + (pp & 3) < size)) continue;
-            if (kFull ? (pp & 1) == 0 : true) {
-                if (sh >= 32u) { sh -= 32u; lo = hi; hi = nx; nx = stream_word(r, wi); ++wi; }
-                win = __funnelshift_r(lo, hi, sh);           // 32 stream bits from the current position
+        for (int pp = 0; pp < 32; pp += 2) {
+            // with sh < 32 the 32 bits from the current position lie inside {lo, hi}; two coordinates take at most 26
+            asm volatile("{\n\t.reg .pred p;\n\tsetp.ge.u32 p, %3, 32;\n\t@p mov.u32 %0, %1;\n\t@p mov.u32 %1, %2;\n\t"
+                         "@p ld.shared.u32 %2, [%4+12];\n\t@p add.u32 %4, %4, 4;\n\tand.b32 %3, %3, 31;\n\t}"
+                         : "+r"(lo), "+r"(hi), "+r"(nx), "+r"(sh), "+r"(at));
+            const uint32_t win = __funnelshift_r(lo, hi, sh);
+            const uint32_t e = run_entry(win);
+            uint32_t sy, bits = e >> kDecLenShift;
+            if (kPair) {
+                sy = e & ((1u << (2 * C)) - 1u);
+                if (e & kDecSingle) {
+                    const uint32_t e1 = run_entry(win >> bits), s1 = e1 & ((1u << C) - 1u);
+                    flags |= e | e1;
+                    sy |= s1 << C;
+                    bits += (e1 & kDecSingle) ? e1 >> kDecLenShift : (uint32_t)len[s1];
+                }
+            } else {
+                const uint32_t e1 = run_entry(win >> bits);
+                flags |= e | e1;
+                sy = (e & 0x1ffu) | ((e1 & 0x1ffu) << C);
+                bits += e1 >> kDecLenShift;
             }
-            const uint32_t e = dec[win & (uint32_t)(kDecEntries - 1)];
-            flags |= e;
-            win >>= e >> kDecLenShift;                       // at least 19 bits are left for the pair's second coordinate
-            sh += e >> kDecLenShift;
-            const uint32_t sym = e & 0x1ffu;
+            sh += bits;
             const int off = pp * C, i = off >> 5, s = off & 31;
-            cw[i] += sym << s;                               // the fields do not overlap: a multiply-add
-            if (s + C > 32) cw[i + 1] |= sym >> (32 - s);
+            cw[i] += sy << s;                                // the fields do not overlap: a multiply-add
+            if (s + 2 * C > 32) cw[i + 1] |= sy >> (32 - s);
         }
 #pragma unroll
-        for (int i = 0; i < C; ++i) dst[i * 32 + lane] = cw[i];
+        for (int i = 0; i < C; ++i) __stcs(dst + 32 * i + l4, cw[i]);
     }
-    if (sh >= 32u) { sh -= 32u; ++wi; }                      // (what the next pair's refill would have done)
-    const uint32_t used = 32u * (uint32_t)(wi - 3) + sh;
-    return (flags & kDecInvalid) != 0u || (r.check_end ? used != r.end_bit : used > 32u * (uint32_t)r.nwords);
+    const uint32_t used = (r.start_bit & ~31u) + 8u * (at - at0) + sh;
+    return (flags & (kPair ? kDecPairInvalid : kDecInvalid)) != 0u || (r.check_end ? used != r.end_bit : used > 32u * (uint32_t)r.nwords);
 }
 
-__global__ void __launch_bounds__(kThreads) entropy_decode_runs_kernel(PlanDev p, const uint32_t* __restrict__ in, int64_t capacity,
+// The other runs (a layer's last, partial block; more words than there is room for): coordinate by coordinate, from global
+// memory.
+static __device__ __noinline__ bool walk_run_plain(const RunRef r, int C, const uint32_t* enc, int64_t blk, int run, int64_t size,
+                                                   uint32_t* dst)
+{
+    uint32_t pos = r.start_bit;
+    bool invalid = false;
+    for (int l4 = 0; l4 < 4; ++l4) {
+        uint64_t acc = 0;
+        int fill = 0, word = 0;
+        for (int pp = 0; pp < 32; ++pp) {
+            uint32_t sym = 0;
+            if (real_coord(blk, 4 * run + l4, pp, size)) {
+                const int i = (int)(pos >> 5);
+                const uint32_t win = __funnelshift_r(stream_word(r, i), stream_word(r, i + 1), pos & 31u);
+                const OneCoord c = decode_one(run_entry(win), C, enc);
+                invalid |= c.invalid;
+                sym = c.invalid ? 0u : c.sym;
+                pos += c.bits;
+            }
+            acc |= (uint64_t)sym << fill;
+            fill += C;
+            if (fill >= 32) { dst[32 * word++ + l4] = (uint32_t)acc; acc >>= 32; fill -= 32; }
+        }
+    }
+    return invalid || (r.check_end ? pos != r.end_bit : pos > 32u * (uint32_t)r.nwords);
+}
+
+// The C words of each of a run's four lanes, which are neighbours: 16 bytes per plane where the message allows it.
+__device__ __forceinline__ void store_zero_lanes(uint32_t* dst, bool vec)
+{
+    if (vec) { __stcs(reinterpret_cast<uint4*>(dst), make_uint4(0u, 0u, 0u, 0u)); return; }
+    dst[0] = 0u; dst[1] = 0u; dst[2] = 0u; dst[3] = 0u;
+}
+
+__global__ void __launch_bounds__(kThreads, 4) entropy_decode_runs_kernel(PlanDev p, const uint32_t* __restrict__ in, int64_t capacity,
                                                                        const uint32_t* __restrict__ offsets,
                                                                        const uint16_t* __restrict__ run_offsets,
+                                                                       const uint32_t* __restrict__ enc_tables,
                                                                        const uint16_t* __restrict__ dec_tables,
-                                                                       uint32_t* __restrict__ packed, uint32_t* __restrict__ bad)
+                                                                       uint32_t* __restrict__ packed, uint32_t* __restrict__ bad, bool vec)
 {
-    __shared__ __align__(16) uint16_t dec[kDecEntries];
-    __shared__ uint8_t todo[kSubBlocks * LQ_CODE_RUNS];
     __shared__ int ntodo;
-    static_assert(kSubBlocks * LQ_CODE_RUNS == kThreads, "one thread per run of a sub-tile");
-    const Tile tile = p.tiles[blockIdx.x >> p.sub_shift];
-    const int sub0 = (blockIdx.x & (p.sub_tiles - 1)) * p.sub_blocks;
-    if (sub0 >= tile.nblocks) return;
-    const int layer = tile.layer, k = blockIdx.y;
-    const LayerDesc L = p.layers[layer];
+    uint16_t* dec = reinterpret_cast<uint16_t*>(run_smem);
+    uint16_t* todo = reinterpret_cast<uint16_t*>(run_smem + kRunList);
+    uint8_t* len = run_smem + kRunLen;
+    const TileJob T = p.jobs[blockIdx.x];
+    const int layer = T.layer, k = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int C = T.bits + 1;
     {
         const uint4* src = reinterpret_cast<const uint4*>(dec_tables + (int64_t)layer * kDecEntries);
         uint4* dst = reinterpret_cast<uint4*>(dec);
-        for (int i = threadIdx.x; i < kDecEntries / 8; i += blockDim.x) dst[i] = __ldg(src + i);
+#pragma unroll
+        for (int i = 0; i < kDecEntries / 8 / kThreads; ++i) dst[i * kThreads + threadIdx.x] = __ldg(src + i * kThreads + threadIdx.x);
+        if (C <= kDecPairBits && threadIdx.x < 1 << C)
+            len[threadIdx.x] = (uint8_t)((enc_tables[(int64_t)layer * kMaxLevels + (threadIdx.x >> 1)] >> 16) + (threadIdx.x > 1 ? 1 : 0));
     }
     if (threadIdx.x == 0) ntodo = 0;
-    const int C = L.bits + 1;
     const uint32_t* off_k = offsets + (int64_t)k * (p.total_blocks + 1);
     const uint32_t* stream = in + (int64_t)k * capacity;
-    uint32_t* msg = packed + (int64_t)k * p.packed_words + L.word_off;
-    // the run with index t of this sub-tile: block sub0 + t / 8, run t % 8
+    uint32_t* msg = packed + (int64_t)k * p.packed_words + T.word_off;
+    // the run with index t of this tile: block t / 8, run t % 8
     auto run_ref = [&](int t, int64_t& blk) {
-        blk = tile.block0 + sub0 + (t >> 3);
-        const int64_t g = L.block_off + blk;
+        blk = T.block0 + (t >> 3);
+        const int64_t g = T.block_off + blk;
         const int64_t first = off_k[g], last = min((int64_t)off_k[g + 1], capacity);
         const uint16_t* ro = run_offsets + ((int64_t)k * p.total_blocks + g) * LQ_CODE_RUNS;
         const int run = t & 7;
@@ -558,55 +650,74 @@ __global__ void __launch_bounds__(kThreads) entropy_decode_runs_kernel(PlanDev p
         return r;
     };
     __syncthreads();
+    const bool zero_bit = dec[0] == (uint16_t)zero_bit_entry(C);
 
-    bool broken = false, walk = false;
-    if ((int)(threadIdx.x >> 3) < min(p.sub_blocks, tile.nblocks - sub0)) {
-        int64_t blk;
-        const RunRef r = run_ref(threadIdx.x, blk);
-        uint32_t* dst = msg + blk * (int64_t)C * 32;
-        const int run = threadIdx.x & 7;
-        walk = true;
-        if ((int64_t)(r.start_bit >> 5) > (int64_t)r.nwords) {            // an offset that points past the block's end:
-            broken = true; walk = false;                                 // the run's words are still written (zeros)
-            for (int i = 0; i < C; ++i) *reinterpret_cast<uint4*>(dst + i * 32 + 4 * run) = make_uint4(0u, 0u, 0u, 0u);
-        } else if ((blk + 1) * kBlockCoords <= L.size && dec[0] == (uint16_t)kDecZeroBit) {
-            // 128 coordinates of level 0 are 128 zero bits; the last run of a block is followed by zero padding
-            // up to the block's last word
-            const uint32_t nbits = r.check_end ? r.end_bit - r.start_bit : 32u * (uint32_t)r.nwords - r.start_bit;
-            if (r.check_end ? nbits == 128u : (nbits >= 128u && nbits < 160u)) {
-                const uint32_t end = r.start_bit + nbits;
-                const int w0 = (int)(r.start_bit >> 5), w1 = (int)(end >> 5);
-                uint32_t any = stream_word(r, w0) >> (r.start_bit & 31u);
+    bool broken = false;
+    for (int t0 = 0; t0 < T.nblocks * LQ_CODE_RUNS; t0 += kThreads) {
+        const int t = t0 + threadIdx.x;
+        bool walk = false;
+        if (t < T.nblocks * LQ_CODE_RUNS) {
+            int64_t blk;
+            const RunRef r = run_ref(t, blk);
+            uint32_t* dst = msg + blk * (int64_t)C * 32 + 4 * (t & 7);
+            walk = true;
+            if ((int64_t)(r.start_bit >> 5) > (int64_t)r.nwords) {            // an offset that points past the block's end:
+                broken = true; walk = false;                                 // the run's words are still written (zeros)
+            } else if (zero_bit && (blk + 1) * kBlockCoords <= T.size) {
+                // 128 coordinates of level 0 are 128 zero bits; the last run of a block is followed by zero padding
+                // up to the block's last word
+                const uint32_t nbits = r.check_end ? r.end_bit - r.start_bit : 32u * (uint32_t)r.nwords - r.start_bit;
+                if (r.check_end ? nbits == 128u : (nbits >= 128u && nbits < 160u)) {
+                    const uint32_t end = r.start_bit + nbits;
+                    const int w0 = (int)(r.start_bit >> 5), w1 = (int)(end >> 5);
+                    uint32_t any = stream_word(r, w0) >> (r.start_bit & 31u);
 #pragma unroll
-                for (int i = 1; i < 6; ++i) {
-                    const uint32_t x = stream_word(r, w0 + i);
-                    if (w0 + i < w1) any |= x;
-                    else if (w0 + i == w1 && (end & 31u)) any |= x << (32u - (end & 31u));
-                }
-                if (any == 0u) {
-                    walk = false;
-                    for (int i = 0; i < C; ++i) *reinterpret_cast<uint4*>(dst + i * 32 + 4 * run) = make_uint4(0u, 0u, 0u, 0u);
+                    for (int i = 1; i < 6; ++i) {
+                        const uint32_t x = stream_word(r, w0 + i);
+                        if (w0 + i < w1) any |= x;
+                        else if (w0 + i == w1 && (end & 31u)) any |= x << (32u - (end & 31u));
+                    }
+                    walk = any != 0u;
                 }
             }
+            if (!walk)
+                for (int i = 0; i < C; ++i) store_zero_lanes(dst + i * 32, vec);
         }
-    }
-    {
         const uint32_t m = __ballot_sync(0xffffffffu, walk);
         int at = 0;
-        if ((threadIdx.x & 31) == 0 && m) at = atomicAdd(&ntodo, __popc(m));
+        if (lane == 0 && m) at = atomicAdd(&ntodo, __popc(m));
         at = __shfl_sync(0xffffffffu, at, 0);
-        if (walk) todo[at + __popc(m & ((1u << (threadIdx.x & 31)) - 1u))] = (uint8_t)threadIdx.x;
+        if (walk) todo[at + __popc(m & ((1u << lane) - 1u))] = (uint16_t)t;
     }
     __syncthreads();
-    if ((int)threadIdx.x < ntodo) {
-        const int t = todo[threadIdx.x];
+    const int n = ntodo;
+    const int pieces = run_pieces(C);
+    const uint32_t taken = (uint32_t)__cvta_generic_to_shared(run_smem + kRunTaken) + threadIdx.x * pieces * 16;
+    const bool in_vec = reinterpret_cast<uintptr_t>(in) % 16 == 0;
+    for (int i0 = warp * 32; i0 < n; i0 += kThreads) {
+        if (i0 + lane >= n) continue;
+        const int t = todo[i0 + lane];
         int64_t blk;
         const RunRef r = run_ref(t, blk);
-        uint32_t* dst = msg + blk * (int64_t)C * 32;
-        const bool full = (blk + 1) * kBlockCoords <= L.size;
-        switch (full ? C : -C) {
-#define LQ_CASE(CC) case CC:  broken |= decode_run<CC, true>(r, dec, blk, t & 7, L.size, dst); break;  \
-                    case -CC: broken |= decode_run<CC, false>(r, dec, blk, t & 7, L.size, dst); break;
+        uint32_t* dst = msg + blk * (int64_t)C * 32 + 4 * (t & 7);
+        const int w0 = (int)(r.start_bit >> 5), w1 = r.check_end ? min((int)((r.end_bit + 31u) >> 5), r.nwords) : r.nwords;
+        const uintptr_t at = reinterpret_cast<uintptr_t>(r.src + w0), to = reinterpret_cast<uintptr_t>(r.src + w1);
+        const uintptr_t from = at & ~(uintptr_t)15;
+        if (w1 <= w0 || to - from > (uintptr_t)(16 * pieces) || (blk + 1) * kBlockCoords > T.size) {
+            broken |= walk_run_plain(r, C, enc_tables + (int64_t)layer * kMaxLevels, blk, t & 7, T.size, dst);
+            continue;
+        }
+        if (in_vec) {
+            for (uintptr_t f = from; f < to; f += 16)
+                cp_async16(taken + (uint32_t)(f - from), reinterpret_cast<const void*>(f), (int)min((uintptr_t)16, to - f));
+        } else {
+            for (uintptr_t f = at; f < to; f += 4) cp_async4(taken + (uint32_t)(f - from), reinterpret_cast<const void*>(f));
+        }
+        cp_async_commit();
+        cp_async_wait<0>();
+        const uint32_t first = taken + (uint32_t)(at - from);
+        switch (C) {
+#define LQ_CASE(CC) case CC: broken |= walk_run<CC>(r, first, len, dst); break;
             LQ_CASE(2) LQ_CASE(3) LQ_CASE(4) LQ_CASE(5) LQ_CASE(6) LQ_CASE(7) LQ_CASE(8) LQ_CASE(9)
 #undef LQ_CASE
             default: break;
@@ -632,17 +743,21 @@ cudaError_t launch_entropy_encode(const PlanDev& p, const uint32_t* packed, cons
 }
 
 cudaError_t launch_entropy_decode(const PlanDev& p, const uint32_t* in, int64_t capacity, const uint32_t* offsets,
-                                  const uint16_t* run_offsets, const uint16_t* dec_tables, uint32_t* packed, uint32_t* bad,
-                                  cudaStream_t s)
+                                  const uint16_t* run_offsets, const uint32_t* enc_tables, const uint16_t* dec_tables,
+                                  uint32_t* packed, uint32_t* bad, cudaStream_t s)
 {
     if (p.total_blocks == 0) return cudaSuccess;
     if (run_offsets) {
-        const dim3 grid_r((unsigned)p.num_tiles * p.sub_tiles, (unsigned)p.num_workers);
-        entropy_decode_runs_kernel<<<grid_r, kThreads, 0, s>>>(p, in, capacity, offsets, run_offsets, dec_tables, packed, bad);
+        static std::atomic<uint64_t> configured{0};
+        const cudaError_t e = opt_in_shared_memory(configured, kRunSmem(LQ_MAX_BITS), entropy_decode_runs_kernel);
+        if (e != cudaSuccess) return e;
+        const dim3 grid_r((unsigned)p.num_tiles, (unsigned)p.num_workers);
+        entropy_decode_runs_kernel<<<grid_r, kThreads, kRunSmem(p.most_bits), s>>>(
+            p, in, capacity, offsets, run_offsets, enc_tables, dec_tables, packed, bad, reinterpret_cast<uintptr_t>(packed) % 16 == 0);
         return cudaGetLastError();
     }
     const dim3 grid((unsigned)((p.total_blocks + 127) / 128), (unsigned)p.num_workers);
-    entropy_decode_kernel<<<grid, 128, 0, s>>>(p, in, capacity, offsets, dec_tables, packed, bad);
+    entropy_decode_kernel<<<grid, 128, 0, s>>>(p, in, capacity, offsets, enc_tables, dec_tables, packed, bad);
     return cudaGetLastError();
 }
 

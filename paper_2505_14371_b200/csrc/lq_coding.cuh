@@ -1,9 +1,12 @@
 // Decode table of the entropy stage (shared by the code that builds it and the kernels that read it).
 // One entry per value of the next kDecBits = 13 stream bits (first bit in bit 0): a code word is at most
 // kCodeMaxLen = 12 bits and a non-zero level is followed by its sign bit, so 13 bits always hold one whole
-// coordinate.  entry = symbol (2 * level index + sign, bits 0..8) | bits taken (word + sign, 1..13) << 12;
-// where no word matches (incomplete codes) the entry is kDecInvalid | 1 << 12: the flag (bit 9, which no valid entry
-// sets) is sticky when entries are OR-ed together, and a walker still advances.
+// coordinate.  Symbol = 2 * level index + sign, of C = b + 1 bits.
+//   C <= kDecPairBits: the symbols of two coordinates (bits 0..4 and C up) and the bits that both take << kDecLenShift; where
+//     13 bits do not hold the second one, the first symbol, its bits and kDecSingle; no word matches (incomplete codes):
+//     kDecSingle, kDecPairInvalid and 1 bit.
+//   wider: symbol (bits 0..8) | bits taken (word + sign, 1..13) << kDecLenShift; no match: kDecInvalid | 1 bit.
+// The invalid flags are sticky when entries are OR-ed together, and a walker still advances.
 #pragma once
 #include "lq_internal.cuh"
 
@@ -13,8 +16,11 @@ constexpr int kDecBits = kCodeMaxLen + 1;
 constexpr int kDecEntries = 1 << kDecBits;
 constexpr uint32_t kDecInvalid = 1u << 9;
 constexpr int kDecLenShift = 12;
-constexpr uint32_t kDecZeroBit = 1u << kDecLenShift;         // the entry of "level 0 in one bit": symbol 0, one bit taken
-
+constexpr int kDecPairBits = 5;
+constexpr uint32_t kDecSingle = 1u << 10;
+constexpr uint32_t kDecPairInvalid = 1u << 11;
+// entry 0 when level 0 is the word "0": symbol 0 in one bit, or two of them in two
+__host__ __device__ constexpr uint32_t zero_bit_entry(int C) { return (C <= kDecPairBits ? 2u : 1u) << kDecLenShift; }
 
 // ---- host side of the stage (lq_coding.cu) ----
 bool huffman_lengths_host(const double* w, int n, int max_len, uint8_t* len);
@@ -31,7 +37,7 @@ cudaError_t launch_entropy_encode(const PlanDev& p, const uint32_t* packed, cons
                                   uint32_t* offsets, uint32_t* out, int64_t capacity, uint16_t* run_offsets,
                                   EncodeScratch scratch, cudaStream_t s);
 cudaError_t launch_entropy_decode(const PlanDev& p, const uint32_t* in, int64_t capacity, const uint32_t* offsets,
-                                  const uint16_t* run_offsets, const uint16_t* dec_tables, uint32_t* packed, uint32_t* bad,
+                                  const uint16_t* run_offsets, const uint32_t* enc_tables, const uint16_t* dec_tables, uint32_t* packed, uint32_t* bad,
                                   cudaStream_t s);
 
 }  // namespace lq
