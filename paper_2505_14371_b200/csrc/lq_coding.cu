@@ -574,11 +574,14 @@ __device__ __forceinline__ bool walk_run(const RunRef& r, uint32_t at, const uin
 }
 
 // The other runs (a layer's last, partial block; more words than there is room for): coordinate by coordinate, from global
-// memory.
+// memory, a word ahead of the 64 bits being read.
 static __device__ __noinline__ bool walk_run_plain(const RunRef r, int C, const uint32_t* enc, int64_t blk, int run, int64_t size,
                                                    uint32_t* dst)
 {
-    uint32_t pos = r.start_bit;
+    int i = (int)(r.start_bit >> 5);
+    uint64_t window = stream_word(r, i) >> (r.start_bit & 31u);
+    int have = 32 - (int)(r.start_bit & 31u);
+    uint32_t next = stream_word(r, ++i), pos = r.start_bit;
     bool invalid = false;
     for (int l4 = 0; l4 < 4; ++l4) {
         uint64_t acc = 0;
@@ -586,12 +589,15 @@ static __device__ __noinline__ bool walk_run_plain(const RunRef r, int C, const 
         for (int pp = 0; pp < 32; ++pp) {
             uint32_t sym = 0;
             if (real_coord(blk, 4 * run + l4, pp, size)) {
-                const int i = (int)(pos >> 5);
-                const uint32_t win = __funnelshift_r(stream_word(r, i), stream_word(r, i + 1), pos & 31u);
-                const OneCoord c = decode_one(run_entry(win), C, enc);
+                if (have < kDecBits) {
+                    window |= (uint64_t)next << have;
+                    have += 32;
+                    next = stream_word(r, ++i);
+                }
+                const OneCoord c = decode_one(run_entry((uint32_t)window), C, enc);
                 invalid |= c.invalid;
                 sym = c.invalid ? 0u : c.sym;
-                pos += c.bits;
+                pos += c.bits; window >>= c.bits; have -= (int)c.bits;
             }
             acc |= (uint64_t)sym << fill;
             fill += C;

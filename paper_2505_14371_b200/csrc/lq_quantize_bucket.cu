@@ -236,7 +236,20 @@ __device__ __forceinline__ double quantize_tile(const PlanDev& p, const PhiloxCo
     return stat;
 }
 
-template <bool kHist>
+// The blocks of a tile of width B.
+template <int B, bool kHist>
+__device__ __forceinline__ double quantize_width(const PlanDev& p, const PhiloxConsts& pc, BucketCtx& c, const QuantEnv& ev,
+                                                 const Tile& tile, int search, uint32_t* __restrict__ out,
+                                                 const uint32_t* __restrict__ prev)
+{
+    if (search == kSearchOctave) return quantize_tile<B, kSearchOctave, kHist>(p, pc, c, ev, tile, out, prev);
+    if constexpr (B >= kWindowBits)
+        if (search == kSearchWindow) return quantize_tile<B, kSearchWindow, kHist>(p, pc, c, ev, tile, out, prev);
+    return quantize_tile<B, kSearchStep, kHist>(p, pc, c, ev, tile, out, prev);
+}
+
+// kWidth: the code width of every layer of the plan, or 0 when they differ (see quantize_pack_kernel).
+template <int kWidth, bool kHist>
 __global__ void __launch_bounds__(kQThreads, 3) quantize_pack_bucket_kernel(
     PlanDev p, const float* grads, uint32_t step, uint32_t* packed, float* bucket_norms, uint32_t* hist,
     const uint32_t* prev_packed, const float* prev_norms, const float* levels_cur, const float* levels_prev, SearchTables st)
@@ -281,13 +294,16 @@ __global__ void __launch_bounds__(kQThreads, 3) quantize_pack_bucket_kernel(
     const uint32_t* prev = prev_packed ? fresh(prev_packed + (int64_t)k * p.packed_words + L.word_off) : nullptr;
 
     double stat = 0.0;
-    switch (L.bits * 4 + (how.x & 3)) {
-#define LQ_SEARCH(BB, S) case 4 * BB + S: stat = quantize_tile<BB, S, kHist>(p, pc, c, ev, tile, out, prev); break;
-#define LQ_CASE(BB) LQ_SEARCH(BB, kSearchOctave) LQ_SEARCH(BB, kSearchStep) LQ_SEARCH(BB, kSearchWindow)
-        LQ_CASE(1) LQ_CASE(2) LQ_CASE(3) LQ_CASE(4) LQ_CASE(5) LQ_CASE(6) LQ_CASE(7) LQ_CASE(8)
+    const int search = how.x & 3;
+    if constexpr (kWidth != 0) {
+        stat = quantize_width<kWidth, kHist>(p, pc, c, ev, tile, search, out, prev);
+    } else {
+        switch (L.bits) {
+#define LQ_CASE(BB) case BB: stat = quantize_width<BB, kHist>(p, pc, c, ev, tile, search, out, prev); break;
+            LQ_CASE(1) LQ_CASE(2) LQ_CASE(3) LQ_CASE(4) LQ_CASE(5) LQ_CASE(6) LQ_CASE(7) LQ_CASE(8)
 #undef LQ_CASE
-#undef LQ_SEARCH
-        default: break;
+            default: break;
+        }
     }
     double* scratch = reinterpret_cast<double*>(sm + kSmScratch);
     const double total = block_reduce<false>(stat, scratch);
@@ -347,12 +363,19 @@ cudaError_t launch_quantize_bucketed(const PlanDev& p, const float* grads, uint3
     if (p.num_tiles == 0) return cudaSuccess;
     const dim3 grid((unsigned)p.num_tiles, (unsigned)p.worker_count);
     constexpr unsigned smem = kSmTables + kRingBytes + LQ_HIST_STRIDE * 4 + kSmSlack;
-    static std::atomic<uint64_t> configured{0};
-    const cudaError_t e = opt_in_shared_memory(configured, (int)smem, quantize_pack_bucket_kernel<true>,
-                                               quantize_pack_bucket_kernel<false>);
+    using Kernel = void (*)(PlanDev, const float*, uint32_t, uint32_t*, float*, uint32_t*, const uint32_t*, const float*,
+                            const float*, const float*, SearchTables);
+#define LQ_ALL(H) {quantize_pack_bucket_kernel<0, H>, quantize_pack_bucket_kernel<1, H>, quantize_pack_bucket_kernel<2, H>, \
+                   quantize_pack_bucket_kernel<3, H>, quantize_pack_bucket_kernel<4, H>, quantize_pack_bucket_kernel<5, H>, \
+                   quantize_pack_bucket_kernel<6, H>, quantize_pack_bucket_kernel<7, H>, quantize_pack_bucket_kernel<8, H>}
+    static const Kernel kernels[2][9] = {LQ_ALL(false), LQ_ALL(true)};
+#undef LQ_ALL
+    const int mode = hist ? 1 : 0, width = p.least_bits == p.most_bits ? p.most_bits : 0;
+    static std::atomic<uint64_t> configured[2][9];
+    const cudaError_t e = opt_in_shared_memory(configured[mode][width], (int)smem, kernels[mode][width]);
     if (e != cudaSuccess) return e;
-    return launch(hist ? quantize_pack_bucket_kernel<true> : quantize_pack_bucket_kernel<false>, grid, kQThreads, smem, s, p,
-                  grads, step, packed, bucket_norms, hist, prev_packed, prev_norms, levels_cur, levels_prev, t);
+    return launch(kernels[mode][width], grid, kQThreads, smem, s, p, grads, step, packed, bucket_norms, hist, prev_packed, prev_norms,
+                  levels_cur, levels_prev, t);
 }
 
 cudaError_t launch_bucket_finalize(const PlanDev& p, cudaStream_t s)
