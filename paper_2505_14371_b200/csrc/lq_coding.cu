@@ -524,11 +524,13 @@ __device__ __forceinline__ uint32_t run_entry(uint32_t bits)
     return *reinterpret_cast<const uint16_t*>(run_smem + ((bits << 1) & (2u * kDecEntries - 2u)));
 }
 
-// Whole block, words in shared memory: `at` is the address of the run's first word.  `len`: bits of every symbol's word and
+// A run of a whole (kFull) or partial block, words in shared memory: `at` is the address of the run's first word.  `len`: bits of every symbol's word and
 // sign (pair tables).  Word i of lane l4 of the run goes to dst[32 i + l4].
-template <int C>
-__device__ __forceinline__ bool walk_run(const RunRef& r, uint32_t at, const uint8_t* len, uint32_t* dst)
+// A lane of a partial block holds the first `real` of its 32 positions: rows before the layer's end, and its share of the last.
+template <int C, bool kFull>
+__device__ __forceinline__ bool walk_run(const RunRef& r, uint32_t at, const uint8_t* len, int64_t blk, int run, int64_t size, uint32_t* dst)
 {
+    const int rest = kFull ? 0 : (int)(size - blk * kBlockCoords);
     constexpr bool kPair = C <= kDecPairBits;
     const uint32_t at0 = at;
     uint32_t lo = lds_u32(at), hi = lds_u32(at + 4u), nx = lds_u32(at + 8u);       // `lo` is the word at `at`
@@ -538,8 +540,10 @@ __device__ __forceinline__ bool walk_run(const RunRef& r, uint32_t at, const uin
         uint32_t cw[C + 1];
 #pragma unroll
         for (int i = 0; i <= C; ++i) cw[i] = 0u;
+        const int real = kFull ? 32 : 4 * (rest >> 7) + max(0, min(4, (rest & 127) - 4 * (4 * run + l4)));
 #pragma unroll
         for (int pp = 0; pp < 32; pp += 2) {
+            if (!kFull && pp >= real) break;
             // with sh < 32 the 32 bits from the current position lie inside {lo, hi}; two coordinates take at most 26
             asm volatile("{\n\t.reg .pred p;\n\tsetp.ge.u32 p, %3, 32;\n\t@p mov.u32 %0, %1;\n\t@p mov.u32 %1, %2;\n\t"
                          "@p ld.shared.u32 %2, [%4+12];\n\t@p add.u32 %4, %4, 4;\n\tand.b32 %3, %3, 31;\n\t}"
@@ -549,17 +553,25 @@ __device__ __forceinline__ bool walk_run(const RunRef& r, uint32_t at, const uin
             uint32_t sy, bits = e >> kDecLenShift;
             if (kPair) {
                 sy = e & ((1u << (2 * C)) - 1u);
-                if (e & kDecSingle) {
+                if (!kFull && pp + 1 == real) {
+                    sy = e & ((1u << C) - 1u);
+                    flags |= (e & kDecSingle) ? e : 0u;
+                    if (!(e & kDecSingle)) bits = len[sy];             // the first one's share of the pair's
+                } else if (e & kDecSingle) {
                     const uint32_t e1 = run_entry(win >> bits), s1 = e1 & ((1u << C) - 1u);
                     flags |= e | e1;
                     sy |= s1 << C;
                     bits += (e1 & kDecSingle) ? e1 >> kDecLenShift : (uint32_t)len[s1];
                 }
             } else {
-                const uint32_t e1 = run_entry(win >> bits);
-                flags |= e | e1;
-                sy = (e & 0x1ffu) | ((e1 & 0x1ffu) << C);
-                bits += e1 >> kDecLenShift;
+                flags |= e;
+                sy = e & 0x1ffu;
+                if (kFull || pp + 1 < real) {
+                    const uint32_t e1 = run_entry(win >> bits);
+                    flags |= e1;
+                    sy |= (e1 & 0x1ffu) << C;
+                    bits += e1 >> kDecLenShift;
+                }
             }
             sh += bits;
             const int off = pp * C, i = off >> 5, s = off & 31;
@@ -573,9 +585,9 @@ __device__ __forceinline__ bool walk_run(const RunRef& r, uint32_t at, const uin
     return (flags & (kPair ? kDecPairInvalid : kDecInvalid)) != 0u || (r.check_end ? used != r.end_bit : used > 32u * (uint32_t)r.nwords);
 }
 
-// The other runs (a layer's last, partial block; more words than there is room for): coordinate by coordinate, from global
+// Runs of more words than there is room for: coordinate by coordinate, from global
 // memory, a word ahead of the 64 bits being read.
-static __device__ __noinline__ bool walk_run_plain(const RunRef r, int C, const uint32_t* enc, int64_t blk, int run, int64_t size,
+static __device__ __noinline__ bool walk_run_plain(const RunRef r, int C, const uint8_t* len, int64_t blk, int run, int64_t size,
                                                    uint32_t* dst)
 {
     int i = (int)(r.start_bit >> 5);
@@ -583,9 +595,12 @@ static __device__ __noinline__ bool walk_run_plain(const RunRef r, int C, const 
     int have = 32 - (int)(r.start_bit & 31u);
     uint32_t next = stream_word(r, ++i), pos = r.start_bit;
     bool invalid = false;
+    const bool pairs = C <= kDecPairBits;
+#pragma unroll 1
     for (int l4 = 0; l4 < 4; ++l4) {
         uint64_t acc = 0;
         int fill = 0, word = 0;
+#pragma unroll 4
         for (int pp = 0; pp < 32; ++pp) {
             uint32_t sym = 0;
             if (real_coord(blk, 4 * run + l4, pp, size)) {
@@ -594,10 +609,17 @@ static __device__ __noinline__ bool walk_run_plain(const RunRef r, int C, const 
                     have += 32;
                     next = stream_word(r, ++i);
                 }
-                const OneCoord c = decode_one(run_entry((uint32_t)window), C, enc);
-                invalid |= c.invalid;
-                sym = c.invalid ? 0u : c.sym;
-                pos += c.bits; window >>= c.bits; have -= (int)c.bits;
+                const uint32_t e = run_entry((uint32_t)window);
+                uint32_t bits = e >> kDecLenShift;
+                if (pairs) {
+                    sym = e & ((1u << C) - 1u);
+                    invalid |= (e & kDecPairInvalid) != 0u;
+                    if (!(e & kDecSingle)) bits = len[sym];            // the first one's share of the pair's
+                } else {
+                    sym = e & 0x1ffu;
+                    invalid |= (e & kDecInvalid) != 0u;
+                }
+                pos += bits; window >>= bits; have -= (int)bits;
             }
             acc |= (uint64_t)sym << fill;
             fill += C;
@@ -709,8 +731,8 @@ __global__ void __launch_bounds__(kThreads, 4) entropy_decode_runs_kernel(PlanDe
         const int w0 = (int)(r.start_bit >> 5), w1 = r.check_end ? min((int)((r.end_bit + 31u) >> 5), r.nwords) : r.nwords;
         const uintptr_t at = reinterpret_cast<uintptr_t>(r.src + w0), to = reinterpret_cast<uintptr_t>(r.src + w1);
         const uintptr_t from = at & ~(uintptr_t)15;
-        if (w1 <= w0 || to - from > (uintptr_t)(16 * pieces) || (blk + 1) * kBlockCoords > T.size) {
-            broken |= walk_run_plain(r, C, enc_tables + (int64_t)layer * kMaxLevels, blk, t & 7, T.size, dst);
+        if (w1 <= w0 || to - from > (uintptr_t)(16 * pieces)) {
+            broken |= walk_run_plain(r, C, len, blk, t & 7, T.size, dst);
             continue;
         }
         if (in_vec) {
@@ -722,8 +744,9 @@ __global__ void __launch_bounds__(kThreads, 4) entropy_decode_runs_kernel(PlanDe
         cp_async_commit();
         cp_async_wait<0>();
         const uint32_t first = taken + (uint32_t)(at - from);
-        switch (C) {
-#define LQ_CASE(CC) case CC: broken |= walk_run<CC>(r, first, len, dst); break;
+        switch ((blk + 1) * kBlockCoords <= T.size ? C : -C) {
+#define LQ_CASE(CC) case CC:  broken |= walk_run<CC, true>(r, first, len, blk, t & 7, T.size, dst); break;  \
+                    case -CC: broken |= walk_run<CC, false>(r, first, len, blk, t & 7, T.size, dst); break;
             LQ_CASE(2) LQ_CASE(3) LQ_CASE(4) LQ_CASE(5) LQ_CASE(6) LQ_CASE(7) LQ_CASE(8) LQ_CASE(9)
 #undef LQ_CASE
             default: break;
