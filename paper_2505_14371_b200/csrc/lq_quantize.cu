@@ -249,7 +249,6 @@ cudaError_t launch_quantize(const PlanDev& p, const float* grads, uint32_t step,
                             const float* levels_prev, SearchTables t, bool need_stat, cudaStream_t s)
 {
     if (p.num_tiles == 0) return cudaSuccess;
-    const dim3 grid((unsigned)p.num_tiles, (unsigned)p.worker_count);
     // the ring follows the tables; the histogram (histogram mode only) follows the ring
     constexpr unsigned smem = kSmTables + kRingBytes + kSmSlack, smem_hist = smem + LQ_HIST_STRIDE * 4;
     using Kernel = void (*)(PlanDev, const float*, uint32_t, uint32_t*, const float*, uint32_t*, const uint32_t*, const float*,
@@ -259,13 +258,25 @@ cudaError_t launch_quantize(const PlanDev& p, const float* grads, uint32_t step,
                       quantize_pack_kernel<6, H, S>, quantize_pack_kernel<7, H, S>, quantize_pack_kernel<8, H, S>}
     static const Kernel kernels[3][9] = {LQ_ALL(false, false), LQ_ALL(false, true), LQ_ALL(true, true)};
 #undef LQ_ALL
-    const int mode = hist ? 2 : need_stat ? 1 : 0, width = p.least_bits == p.most_bits ? p.most_bits : 0;
-    const Kernel kernel = kernels[mode][width];
     static std::atomic<uint64_t> configured[3][9];
-    const cudaError_t e = opt_in_shared_memory(configured[mode][width], (int)smem_hist, kernel);
-    if (e != cudaSuccess) return e;
-    return launch(kernel, grid, kQThreads, hist ? smem_hist : smem, s, p, grads, step, packed, norms, hist, prev_packed,
-                  prev_norms, levels_cur, levels_prev, t);
+    const int mode = hist ? 2 : need_stat ? 1 : 0;
+    auto run = [&](const PlanDev& pw, int width, int jobs) {
+        const Kernel kernel = kernels[mode][width];
+        const cudaError_t e = opt_in_shared_memory(configured[mode][width], (int)smem_hist, kernel);
+        if (e != cudaSuccess) return e;
+        return launch(kernel, dim3((unsigned)jobs, (unsigned)p.worker_count), kQThreads, hist ? smem_hist : smem, s, pw, grads, step, packed,
+                      norms, hist, prev_packed, prev_norms, levels_cur, levels_prev, t);
+    };
+    if (p.width_job[1] < 0) return run(p, p.least_bits == p.most_bits ? p.most_bits : 0, p.num_tiles);
+    for (int b = 1; b <= LQ_MAX_BITS; ++b) {
+        const int jobs = p.width_job[b + 1] - p.width_job[b];
+        if (jobs == 0) continue;
+        PlanDev pw = p;
+        pw.jobs += p.width_job[b];
+        const cudaError_t e = run(pw, b, jobs);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t launch_stat_finalize(const PlanDev& p, cudaStream_t s)
