@@ -132,8 +132,9 @@ inline bool rates_in_decoder(const PlanDev& p) { return (int64_t)p.num_workers *
 // a kernel may have written, so only the launch itself and the reading of the plan's constant tables overlap: an
 // iteration of a small plan is a chain of kernels of a few us each, and what lies between two of them shrinks from 1.7 us
 // to well below 1 us.  Grids of many waves are launched the plain way: with the attribute every CTA starts about 3 us
-// late, not just the first ones (norm pass of 37 000 CTAs 690 -> 850 us, decoder of 4 700 CTAs 451 -> 486 us).
-constexpr int64_t kDependentCtas = 148 * 8;
+// late, not just the first ones (norm pass of 37 000 CTAs 690 -> 850 us, decoder of 4 700 CTAs 451 -> 486 us).  The line: up to 24 CTAs per
+// SM no case got slower (with 8: WGAN step 174 -> 170 us, in bucket scope 175 -> 167, low-rank factors 336 -> 328).
+constexpr int64_t kDependentCtas = 148 * 24;
 // `cluster`: CTAs per cluster along x
 template <typename... Params, typename... Args>
 cudaError_t launch_cluster(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, unsigned cluster, cudaStream_t s,
