@@ -1,10 +1,11 @@
 // Python entry of the calls that a program makes every iteration: torch tensors -> raw device pointers -> the C
-// functions of lq.h on torch's current stream.  The checks and messages are those of binding.py's ctypes route, which
-// still serves the calls made once.  What bounds a small iteration is the host: per call the ctypes route took about
+// functions of lq.h on torch's current stream.  The checks are those of binding.py's ctypes route, which still serves the
+// calls made once.  What bounds a small iteration is the host: per call the ctypes route took about
 // 8 us (eight attribute look-ups and conversions per tensor), this one takes well under 1 us beside the launches.
 #include <Python.h>
 
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include "lq.h"
@@ -54,11 +55,8 @@ bool plan_of(PyObject* o, lq_plan** out)
 
 bool int_of(PyObject* o, int32_t* out)
 {
-    const long v = PyLong_AsLong(o);
-    if (v == -1 && PyErr_Occurred()) return false;
-    if (v < INT32_MIN || v > INT32_MAX) { PyErr_SetString(PyExc_OverflowError, "does not fit in 32 bits"); return false; }
-    *out = static_cast<int32_t>(v);
-    return true;
+    *out = static_cast<int32_t>(PyLong_AsUnsignedLongMask(o));       // (ctypes takes the low 32 bits as well)
+    return !PyErr_Occurred();
 }
 
 PyObject* done(int code)
@@ -72,16 +70,10 @@ PyObject* done(int code)
 template <typename F>
 PyObject* call(F&& f)
 {
-    void* s = nullptr;
-    try {
-        s = static_cast<void*>(c10::cuda::getCurrentCUDAStream().stream());
-    } catch (const std::exception& e) {                       // no device
-        PyErr_SetString(PyExc_RuntimeError, e.what());
-        return nullptr;
-    }
+    void* s = static_cast<void*>(c10::cuda::getCurrentCUDAStream().stream());
     int code;
     Py_BEGIN_ALLOW_THREADS
-    code = f(s);
+    try { code = f(s); } catch (...) { code = LQ_ENOMEM; }    // (nothing but an allocation can throw there)
     Py_END_ALLOW_THREADS
     return done(code);
 }
@@ -175,9 +167,9 @@ PyObject* entropy_decode(PyObject*, PyObject* const* a, Py_ssize_t n)
 PyObject* vector_norm_static(PyObject*, PyObject* const* a, Py_ssize_t n)
 {
     float *v, *out; uint32_t* st; int32_t q;
-    if (!arity(n, 4) || !pointer(a[0], kF32, &v) || !int_of(a[1], &q) || !pointer(a[2], kF32, &out) || !pointer(a[3], kI32, &st))
+    if (!arity(n, 4) || (a[0] == Py_None && !fail("expected a contiguous CUDA tensor")) || !pointer(a[0], kF32, &v) || !int_of(a[1], &q) || !pointer(a[2], kF32, &out) || !pointer(a[3], kI32, &st))
         return nullptr;
-    const int64_t len = a[0] == Py_None ? 0 : THPVariable_Unpack(a[0]).numel();
+    const int64_t len = THPVariable_Unpack(a[0]).numel();
     return call([&](void* s) { return lq_vector_norm_static(v, len, q, out, st, s); });
 }
 
@@ -189,7 +181,17 @@ PyObject* register_error(PyObject*, PyObject* cls)
     Py_RETURN_NONE;
 }
 
-#define LQ_FAST(name, fn) {name, (PyCFunction)(void (*)(void))fn, METH_FASTCALL, nullptr}
+// Every entry runs inside this: torch's accessors throw for tensors without plain memory (sparse ones, subclasses that answer
+// for their layout themselves), and no C++ exception may leave through the interpreter's C frames.
+template <PyObject* (*kEntry)(PyObject*, PyObject* const*, Py_ssize_t)>
+PyObject* guarded(PyObject* self, PyObject* const* a, Py_ssize_t n)
+{
+    HANDLE_TH_ERRORS
+    return kEntry(self, a, n);
+    END_HANDLE_TH_ERRORS
+}
+
+#define LQ_FAST(name, fn) {name, (PyCFunction)(void (*)(void))guarded<fn>, METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {LQ_FAST("lq_quantize_pack", quantize_pack), LQ_FAST("qoda_step", step_qoda),
                          LQ_FAST("lq_layer_norms", layer_norms), LQ_FAST("lq_decode_aggregate", decode_aggregate),
                          LQ_FAST("lq_fit_levels", fit_levels), LQ_FAST("lq_level_probabilities", level_probabilities),

@@ -240,3 +240,37 @@ def test_universal_code_lengths_match_the_recursive_code(orc):
         assert lqm.lq_code_universal(n) == [len(orc.elias_omega(j + 1)) for j in range(n)]
     with pytest.raises(lqm.LqError):
         lqm.lq_code_universal(64)                                      # its last word would have 13 bits
+
+
+_FOREIGN_TENSORS = """
+import torch
+import paper_2505_14371_b200.binding as b
+b.load_library()
+
+class Refuses(torch.Tensor):                       # a CUDA tensor to look at, whose layout is asked of Python
+    @staticmethod
+    def __new__(cls):
+        return torch.Tensor._make_wrapper_subclass(cls, (64,), dtype=torch.float32, device="cuda",
+                                                   dispatch_sizes_strides_policy="strides")
+    @classmethod
+    def __torch_dispatch__(cls, func, types, args=(), kwargs=None):
+        raise KeyError("no layout")
+
+def refused(call):
+    try:
+        call()
+    except Exception as e:
+        return type(e).__name__
+    return "accepted"
+
+print(refused(lambda: b._native.lq_layer_norms(None, Refuses(), None)),
+      refused(lambda: b.lq_vector_norm_static(None, 2, None)))
+"""
+
+
+def test_native_entries_turn_torch_exceptions_into_python_ones():
+    """A tensor whose accessors throw: an exception, not the end of the process (in a child for that reason); and a vector
+    that is None stays refused."""
+    r = subprocess.run([sys.executable, "-c", _FOREIGN_TENSORS], capture_output=True, text=True, cwd=ROOT)
+    assert r.returncode == 0, r.stderr[-500:]
+    assert r.stdout.split() == ["KeyError", "LqError"]
