@@ -44,14 +44,20 @@ def _native_link(obj: str, out: str) -> list:
             "-lc10_cuda"]
 
 
+def _outdated(src: str, obj: str, common: float) -> bool:
+    """(an object as old as its source counts as outdated: the clock of a file system may be coarse)"""
+    return not os.path.exists(obj) or os.path.getmtime(obj) <= max(common, os.path.getmtime(src))
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     if not force and not _stale():
         return OUT
     nvcc = os.environ.get("NVCC", "nvcc")
     bdir = os.path.join(HERE, "_build")
     os.makedirs(bdir, exist_ok=True)
-    headers = max(os.path.getmtime(os.path.join(d, f)) for d in (CSRC, os.path.join(ROOT, "include"))
-                  for f in os.listdir(d) if f.endswith((".cuh", ".h")))
+    # what every object hangs on: the headers, and this file's flags
+    common = max([os.path.getmtime(__file__)] + [os.path.getmtime(os.path.join(d, f)) for d in (CSRC, os.path.join(ROOT, "include"))
+                                                 for f in os.listdir(d) if f.endswith((".cuh", ".h"))])
     objs, procs = [], []
     native_obj = os.path.join(bdir, "lq_native.o")
     jobs = [(os.path.join(CSRC, "lq_native.cpp"), native_obj, lambda: _native_compile(native_obj))]
@@ -61,7 +67,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         jobs.append((os.path.join(CSRC, src), obj, lambda cmd=cmd: cmd))
         objs.append(obj)
     for src, obj, command in jobs:
-        if force or not os.path.exists(obj) or os.path.getmtime(obj) < max(headers, os.path.getmtime(src)):
+        if force or _outdated(src, obj, common):
             cmd = command()
             procs.append((cmd, obj, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
     failed = []

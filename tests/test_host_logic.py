@@ -274,3 +274,38 @@ def test_native_entries_turn_torch_exceptions_into_python_ones():
     r = subprocess.run([sys.executable, "-c", _FOREIGN_TENSORS], capture_output=True, text=True, cwd=ROOT)
     assert r.returncode == 0, r.stderr[-500:]
     assert r.stdout.split() == ["KeyError", "LqError"]
+
+
+def test_objects_are_compiled_again_when_the_build_flags_change(tmp_path, monkeypatch):
+    """A newer build.py (its flags) makes every object outdated, like a newer header."""
+    from paper_2505_14371_b200 import build as b
+    for d in ("csrc", "include", "_build"):
+        (tmp_path / d).mkdir()
+    names = ["lq_native.cpp"] + [src for src, _ in b.SOURCES]
+    for n in names:
+        (tmp_path / "csrc" / n).write_text("")
+        (tmp_path / "_build" / (n.rsplit(".", 1)[0] + ".o")).write_text("")
+    (tmp_path / "build.py").write_text("")
+    for a, v in dict(HERE=str(tmp_path), ROOT=str(tmp_path), CSRC=str(tmp_path / "csrc"), OUT=str(tmp_path / "liblq.so"),
+                     NATIVE=str(tmp_path / "_native.so"), __file__=str(tmp_path / "build.py")).items():
+        monkeypatch.setattr(b, a, v)
+    (tmp_path / "include" / "lq.h").write_text("")
+    def at(path, t):
+        os.utime(path, (t, t))
+    for root, _, files in os.walk(tmp_path):
+        for f in files:
+            at(os.path.join(root, f), 2000 if f.endswith(".o") else 1000)
+    ran = []
+    class Done:
+        returncode = 0
+        def communicate(self):
+            return "", None
+    monkeypatch.setattr(b.subprocess, "Popen", lambda cmd, **k: ran.append(cmd[cmd.index("-c") + 1]) or Done())
+    monkeypatch.setattr(b.subprocess, "check_call", lambda cmd: open(cmd[cmd.index("-o") + 1], "w").close())
+    b.build()
+    assert ran == []
+    for f in (b.OUT, b.NATIVE):
+        at(f, 2000)
+    at(tmp_path / "build.py", 3000)
+    b.build()
+    assert sorted(os.path.basename(c) for c in ran) == sorted(names)
