@@ -434,6 +434,10 @@ int lq_layer_norms(lq_plan* plan, const float* grads, float* norms, void* stream
     if (plan->dev.num_layers == 0) return LQ_OK;
     cudaStream_t s = (cudaStream_t)stream;
     const PlanDev& d = plan->dev;
+    if (use_small(d)) {                  // the order of lq_quantize_pack's sums on such a plan
+        LQ_CUDA(timed(plan, LQ_KERNEL_NORM_PARTIAL, s, [&] { return launch_layer_norms_small(d, grads, norms, s); }));
+        return LQ_OK;
+    }
     LQ_CUDA(timed(plan, LQ_KERNEL_NORM_PARTIAL, s, [&] { return launch_norm_partial(d, grads, false, s); }));
     LQ_CUDA(timed(plan, LQ_KERNEL_NORM_FINALIZE, s, [&] { return launch_norm_finalize(d, norms, s); }));
     return LQ_OK;

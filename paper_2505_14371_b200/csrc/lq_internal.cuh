@@ -201,6 +201,7 @@ cudaError_t launch_quantize(const PlanDev& p, const float* grads, uint32_t step,
                             const float* levels_prev, SearchTables t, bool need_stat, cudaStream_t s);
 // layer scope, plans whose layers are all small: norms, messages and statistic in one kernel
 bool use_small(const PlanDev& p);
+cudaError_t launch_layer_norms_small(const PlanDev& p, const float* grads, float* norms, cudaStream_t s);
 cudaError_t launch_quantize_small(const PlanDev& p, const float* grads, uint32_t step, uint32_t* packed, float* norms,
                                   uint32_t* hist, const uint32_t* prev_packed, const float* prev_norms,
                                   const float* levels_cur, const float* levels_prev, SearchTables t, bool need_stat, cudaStream_t s);

@@ -5,8 +5,13 @@
 // with nothing to fill the GPU, so latency is what bounds them.
 //
 // The rule (use_small): every layer has at most 256 blocks of 1024 coordinates (8 CTAs of 32), and the clusters of all
-// layers and workers are at most two to three waves of CTAs.  A cluster has as many CTAs as its plan's largest layer needs
+// layers and all of the plan's workers run at once: 3 CTAs per SM, or for whole clusters, which have to fit an SM group
+// each, 352 CTAs.  It asks for nothing but the plan's constants: a worker range does not change which kernel encodes a
+// layer, nor the order in which the layer's sums are formed.  A cluster has as many CTAs as its plan's largest layer needs
 // for one block per warp; the values are read twice, the second time from L2.
+// lq_quantize_pack at 3 bits and 4 workers, this kernel and the general path: layers of one block 18.9 and 25.0 us at 444
+// CTAs, 34.8 and 26.9 at 592; of 64 blocks 27.5 and 38.9 at 352 CTAs, 46.7 and 40.1 at 416; of 256 blocks 52.0 and 60.6 at
+// 352, 75.7 and 65.7 at 416 (there the second wave waits for whole clusters).
 #include "lq_quantize_tile.cuh"
 
 namespace lq {
@@ -36,6 +41,62 @@ __device__ __forceinline__ double norm_of_blocks(const PlanDev& p, const float* 
     return norm_cta_total<kMode>(acc, maxbits, scratch);
 }
 
+// What a CTA of a cluster takes of its layer: an equal share of consecutive blocks.
+__device__ __forceinline__ Tile cluster_share(const LayerDesc& L, int layer, int rank, int ranks)
+{
+    const int per = (L.nblocks + ranks - 1) / ranks;
+    Tile t;
+    t.layer = layer; t.block0 = rank * per; t.nblocks = max(0, min(per, L.nblocks - t.block0)); t.pad_ = 0;
+    return t;
+}
+
+// The layer's norm from all CTAs of the cluster: each sends its sum to every other, and all add them in rank order.  What
+// is done between the two calls overlaps the exchange.  (The caller has arrived at the cluster's barrier once before.)
+__device__ __forceinline__ void cluster_norm_send(const PlanDev& p, const float* g, const LayerDesc& L, const Tile& t, int rank,
+                                                  int ranks, uint8_t* rows, double* scratch, double* part)
+{
+    const double mine = p.q == 0   ? norm_of_blocks<0>(p, g, L.size, t.block0, t.nblocks, rows, scratch)
+                        : p.q == 1 ? norm_of_blocks<1>(p, g, L.size, t.block0, t.nblocks, rows, scratch)
+                        : p.q == 2 ? norm_of_blocks<2>(p, g, L.size, t.block0, t.nblocks, rows, scratch)
+                                   : norm_of_blocks<3>(p, g, L.size, t.block0, t.nblocks, rows, scratch);
+    cluster_wait();                                          // every CTA of the cluster runs
+    if (threadIdx.x == 0)
+        for (int r = 0; r < ranks; ++r) st_peer(&part[rank], r, mine);
+    cluster_arrive();
+}
+__device__ __forceinline__ LayerNorm cluster_norm_receive(const PlanDev& p, int ranks, const double* part)
+{
+    cluster_wait();
+    double total = 0.0;
+    bool bad = false;
+    for (int r = 0; r < ranks; ++r) {
+        const double v = part[r];
+        if (!(fabs(v) <= 1.7976931348623157e308)) bad = true;
+        total = p.q == 0 ? fmax(total, v) : total + v;
+    }
+    return layer_norm_of_total(total, bad, p.q);
+}
+__device__ __forceinline__ void store_norm(const PlanDev& p, const LayerNorm& n, float* norms, int64_t kl)
+{
+    norms[kl] = n.norm; p.rnorm[kl] = n.rnorm; p.status[kl] = n.status;
+}
+
+// The norms alone, in the encoder's order (lq_layer_norms gives the very norms that lq_quantize_pack sends).
+__global__ void __launch_bounds__(kQThreads) layer_norms_small_kernel(PlanDev p, const float* grads, float* norms)
+{
+    __shared__ double part[8], scratch[kQWarps];
+    __shared__ uint8_t rows[32];                             // (8 CTAs for up to 256 blocks)
+    pdl_launch_next();
+    const int ranks = gridDim.x, rank = blockIdx.x, layer = blockIdx.y, k = blockIdx.z + p.worker0;
+    cluster_arrive();
+    const LayerDesc L = p.layers[layer];
+    const Tile t = cluster_share(L, layer, rank, ranks);
+    pdl_wait();
+    cluster_norm_send(p, fresh(grads + (int64_t)blockIdx.z * p.padded_elems + L.elem_off), L, t, rank, ranks, rows, scratch, part);
+    const LayerNorm n = cluster_norm_receive(p, ranks, part);
+    if (rank == 0 && threadIdx.x == 0) store_norm(p, n, norms, (int64_t)k * p.num_layers + layer);
+}
+
 template <bool kHist, bool kStat>
 __global__ void __launch_bounds__(kQThreads, 3) quantize_small_kernel(
     PlanDev p, const float* grads, uint32_t step, uint32_t* packed, float* norms, uint32_t* hist,
@@ -50,9 +111,7 @@ __global__ void __launch_bounds__(kQThreads, 3) quantize_small_kernel(
     const int ranks = gridDim.x, rank = blockIdx.x, layer = blockIdx.y, k = blockIdx.z + p.worker0;
     cluster_arrive();                                         // (waited for before the first store into a peer)
     const LayerDesc L = p.layers[layer];
-    const int per = (L.nblocks + ranks - 1) / ranks;
-    Tile tile;
-    tile.layer = layer; tile.block0 = rank * per; tile.nblocks = max(0, min(per, L.nblocks - tile.block0)); tile.pad_ = 0;
+    const Tile tile = cluster_share(L, layer, rank, ranks);
     const int lane = threadIdx.x & 31;
     const int64_t kl = (int64_t)k * p.num_layers + layer;
     pdl_wait();
@@ -78,14 +137,7 @@ __global__ void __launch_bounds__(kQThreads, 3) quantize_small_kernel(
     uint8_t* rows_cur = sm + kSmRows;
     uint8_t* rows_prev = rows_cur + kTileBlocks;
     double* scratch = reinterpret_cast<double*>(sm + kSmScratch);
-    const double mine = p.q == 0   ? norm_of_blocks<0>(p, g, L.size, tile.block0, tile.nblocks, rows_cur, scratch)
-                        : p.q == 1 ? norm_of_blocks<1>(p, g, L.size, tile.block0, tile.nblocks, rows_cur, scratch)
-                        : p.q == 2 ? norm_of_blocks<2>(p, g, L.size, tile.block0, tile.nblocks, rows_cur, scratch)
-                                   : norm_of_blocks<3>(p, g, L.size, tile.block0, tile.nblocks, rows_cur, scratch);
-    cluster_wait();                                          // every CTA of the cluster runs
-    if (threadIdx.x == 0)
-        for (int r = 0; r < ranks; ++r) st_peer(&norm_part[rank], r, mine);
-    cluster_arrive();
+    cluster_norm_send(p, g, L, tile, rank, ranks, rows_cur, scratch, norm_part);
     {
         uint4* ldst = reinterpret_cast<uint4*>(sm + kSmLut);
         ldst[threadIdx.x] = lut0;
@@ -95,15 +147,7 @@ __global__ void __launch_bounds__(kQThreads, 3) quantize_small_kernel(
             for (int i = threadIdx.x; i < LQ_HIST_STRIDE; i += kQThreads) h[i] = 0;
         }
     }
-    cluster_wait();
-    double total = 0.0;
-    bool bad = false;
-    for (int r = 0; r < ranks; ++r) {
-        const double v = norm_part[r];
-        if (!(fabs(v) <= 1.7976931348623157e308)) bad = true;
-        total = p.q == 0 ? fmax(total, v) : total + v;
-    }
-    const LayerNorm ln = layer_norm_of_total(total, bad, p.q);
+    const LayerNorm ln = cluster_norm_receive(p, ranks, norm_part);
     if (threadIdx.x < L.nlevels) {
         const float cv = __fmul_rn(ln.norm, lc), pv = __fmul_rn(nprev, lp);
         reinterpret_cast<float2*>(sm + kSmLd)[threadIdx.x] = lg;
@@ -115,7 +159,7 @@ __global__ void __launch_bounds__(kQThreads, 3) quantize_small_kernel(
         rows_prev[threadIdx.x] = (uint8_t)mprev;
         p.row_mask[mask_at] = rows_cur[threadIdx.x];
     }
-    if (rank == 0 && threadIdx.x == 0) { norms[kl] = ln.norm; p.rnorm[kl] = ln.rnorm; p.status[kl] = ln.status; }
+    if (rank == 0 && threadIdx.x == 0) store_norm(p, ln, norms, kl);
     __syncthreads();
 
     WarpCtx c;
@@ -160,8 +204,16 @@ int small_ranks(const PlanDev& p)
 
 bool use_small(const PlanDev& p)
 {
-    return !p.global_norm && !p.bucket_norm && p.most_blocks <= 256 && p.num_layers <= 65535 &&
-           (int64_t)p.worker_count * p.num_layers * small_ranks(p) <= 148 * 8;
+    const int ranks = small_ranks(p);
+    return !p.global_norm && !p.bucket_norm && p.most_blocks <= 256 &&
+           (int64_t)p.num_workers * p.num_layers * ranks <= (ranks == 1 ? 3 * 148 : 352);
+}
+
+cudaError_t launch_layer_norms_small(const PlanDev& p, const float* grads, float* norms, cudaStream_t s)
+{
+    const unsigned ranks = (unsigned)small_ranks(p);
+    return launch_cluster(layer_norms_small_kernel, dim3(ranks, (unsigned)p.num_layers, (unsigned)p.worker_count), kQThreads, 0, ranks,
+                          s, p, grads, norms);
 }
 
 cudaError_t launch_quantize_small(const PlanDev& p, const float* grads, uint32_t step, uint32_t* packed, float* norms,

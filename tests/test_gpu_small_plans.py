@@ -46,3 +46,41 @@ def test_small_plan(orc, sizes, bits, K, q, hist):
             assert np.array_equal(h.cpu().numpy().view(np.uint32), ref["hist"])
         plan.qoda_step(pk[c], nm[c], X1, Y, Xh); model.qoda_step()
         assert np.max(np.abs(to_unpadded(plan, Y) - model.Y)) <= 1e-6 * np.max(np.abs(model.Y))
+
+
+def test_worker_range_keeps_the_order_of_the_sums():
+    """A plan whose clusters for all 8 workers are more than the small path takes, while those of one worker alone would not
+    be: a process of one worker emits the messages, norms and statistic of the process of all, to the last bit."""
+    import paper_2505_14371_b200 as lqm
+    lqm.load_library()
+    sizes, K = [33 * 1024 + 5] * 20, 8
+    whole, part = lqm.Plan(sizes, 3, 2, K, 7), lqm.Plan(sizes, 3, 2, K, 7)
+    part.lq_set_worker_range(5, 1)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    pk = [[p.empty_packed(), p.empty_packed()] for p in (whole, part)]
+    nm = [[p.empty_norms(), p.empty_norms()] for p in (whole, part)]
+    for t in (1, 2, 3):
+        grads = torch.randn((K, whole.padded_elems), generator=g, device="cuda")
+        c, p = t % 2, (t + 1) % 2
+        for i, (plan, rows) in enumerate(((whole, grads), (part, grads[5:6].contiguous()))):
+            plan.lq_quantize_pack(rows, t, pk[i][c], nm[i][c], prev_packed=pk[i][p] if t > 1 else None,
+                                  prev_norms=nm[i][p] if t > 1 else None)
+        assert torch.equal(pk[0][c][5], pk[1][c][5]) and torch.equal(nm[0][c][5], nm[1][c][5])
+        a, b = (plan.lq_get_statistics()[0][5] for plan in (whole, part))
+        assert torch.equal(a, b)
+
+
+def test_layer_norms_are_the_norms_of_the_message():
+    """A sum that lies half way between two floats up to terms that a large partial sum swallows and a small one keeps: the
+    order of the additions decides the norm, so both calls have to use the same."""
+    import paper_2505_14371_b200 as lqm
+    lqm.load_library()
+    plan = lqm.Plan([196 * 1024, 5], 3, 1, 2, 7)
+    grads = torch.zeros((2, plan.padded_elems), device="cuda")
+    grads[:, 0], grads[:, 1] = 2.0 ** 24, 1.0                   # 2^24 + 1: between 2^24 and 2^24 + 2
+    for blk, worker in ((8, 0), (16, 0), (24, 1), (100, 1)):
+        grads[worker, blk * 1024: blk * 1024 + 4] = 2.0 ** -30  # lost one by one beside 2^24, not 4 of them together
+    alone, sent = plan.empty_norms(), plan.empty_norms()
+    plan.lq_layer_norms(grads, alone)
+    plan.lq_quantize_pack(grads, 1, plan.empty_packed(), sent)
+    assert torch.equal(alone, sent)
