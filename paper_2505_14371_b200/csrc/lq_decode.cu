@@ -225,6 +225,11 @@ __device__ __forceinline__ void finish_block(const DecodeArgs& a, const Walk& w,
     }
 }
 
+// All warps of the CTA.  Not __syncthreads(): where the warps share a block (kSplit) each is in a decode_blocks of its own rows,
+// and that is defined only for a barrier that all threads meet at one place of the program.  A numbered barrier counts
+// arrivals, wherever they come from.
+__device__ __forceinline__ void warps_meet() { asm volatile("barrier.sync 1, %0;" ::"n"(kDecThreads) : "memory"); }
+
 // A warp's blocks: warp, warp + 4, ... of the CTA's (kRows = 8), or rows kRow0, kRow0 + 1 of all of them (kRows = 2).
 // The next unit's words are always requested before the current unit is waited for; the rows of Y and X_1 as soon as
 // the block before is finished.  Per unit one copy group, per block one more for the state, so a fixed number of
@@ -257,7 +262,7 @@ __device__ __forceinline__ void decode_blocks(const PlanDev& p, const LayerDesc&
         cp_async_commit();
     }
     fill_tables<kBucket>(p, L, layer, a, table, 0, min(K, kTW));
-    __syncthreads();
+    warps_meet();
     const Rates rt = *rates;
     double lam_acc = 0.0, mu_acc = 0.0;
     uint32_t stage = 0;
@@ -279,9 +284,9 @@ __device__ __forceinline__ void decode_blocks(const PlanDev& p, const LayerDesc&
             if (!kBucket && K > kTW) {
                 k_in = k0 % kTW;
                 if (k_in == 0 && (b0 > 0 || u > 0)) {
-                    __syncthreads();
+                    warps_meet();
                     fill_tables<kBucket>(p, L, layer, a, table, k0, min(kTW, K - k0));
-                    __syncthreads();
+                    warps_meet();
                 }
             }
             if (kQoda && u == 0) cp_async_wait<2>(); else cp_async_wait<1>();
