@@ -135,14 +135,14 @@ inline bool rates_in_decoder(const PlanDev& p) { return (int64_t)p.num_workers *
 // late, not just the first ones (norm pass of 37 000 CTAs 690 -> 850 us, decoder of 4 700 CTAs 451 -> 486 us).  The line: up to 24 CTAs per
 // SM no case got slower (with 8: WGAN step 174 -> 170 us, in bucket scope 175 -> 167, low-rank factors 336 -> 328).
 constexpr int64_t kDependentCtas = 148 * 24;
-// `cluster`: CTAs per cluster along x
+// `cluster`: CTAs per cluster along x.  A launch that fails leaves no error behind for the next call to find.
 template <typename... Params, typename... Args>
-cudaError_t launch_cluster(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, unsigned cluster, cudaStream_t s,
-                           Args... args)
+cudaError_t launch_as(bool dependent, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, unsigned cluster, cudaStream_t s,
+                      Args... args)
 {
     cudaLaunchAttribute at[2];
     unsigned n = 0;
-    if ((int64_t)grid.x * grid.y * grid.z <= kDependentCtas) {
+    if (dependent) {
         at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         at[n++].val.programmaticStreamSerializationAllowed = 1;
     }
@@ -153,7 +153,15 @@ cudaError_t launch_cluster(void (*kernel)(Params...), dim3 grid, dim3 block, siz
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s;
     cfg.attrs = at; cfg.numAttrs = n;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
+}
+template <typename... Params, typename... Args>
+cudaError_t launch_cluster(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, unsigned cluster, cudaStream_t s,
+                           Args... args)
+{
+    return launch_as((int64_t)grid.x * grid.y * grid.z <= kDependentCtas, kernel, grid, block, smem, cluster, s, args...);
 }
 template <typename... Params, typename... Args>
 cudaError_t launch(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args)
