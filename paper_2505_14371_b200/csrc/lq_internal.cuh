@@ -90,8 +90,6 @@ struct PlanDev {
     int32_t most_blocks;  // blocks of the plan's largest layer
     int32_t most_bits;    // widest code of the plan
     int32_t least_bits;   // narrowest code of the plan
-    int32_t width_job[LQ_MAX_BITS + 2];   // plans of several widths and many waves of encoder CTAs: jobs are in order of
-                          // their width, width b's are [width_job[b], width_job[b + 1]); other plans: width_job[1] = -1
     int32_t dec_blocks;   // blocks per decoder CTA; 1: its warps share them
     int32_t dec_shift;    // log2(plan's tile size / dec_blocks)
     int32_t global_norm;  // 1: one norm per worker over all layers (Section 3.1), 0: one per layer

@@ -260,23 +260,12 @@ cudaError_t launch_quantize(const PlanDev& p, const float* grads, uint32_t step,
 #undef LQ_ALL
     static std::atomic<uint64_t> configured[3][9];
     const int mode = hist ? 2 : need_stat ? 1 : 0;
-    auto run = [&](const PlanDev& pw, int width, int jobs) {
-        const Kernel kernel = kernels[mode][width];
-        const cudaError_t e = opt_in_shared_memory(configured[mode][width], (int)smem_hist, kernel);
-        if (e != cudaSuccess) return e;
-        return launch(kernel, dim3((unsigned)jobs, (unsigned)p.worker_count), kQThreads, hist ? smem_hist : smem, s, pw, grads, step, packed,
-                      norms, hist, prev_packed, prev_norms, levels_cur, levels_prev, t);
-    };
-    if (p.width_job[1] < 0) return run(p, p.least_bits == p.most_bits ? p.most_bits : 0, p.num_tiles);
-    for (int b = 1; b <= LQ_MAX_BITS; ++b) {
-        const int jobs = p.width_job[b + 1] - p.width_job[b];
-        if (jobs == 0) continue;
-        PlanDev pw = p;
-        pw.jobs += p.width_job[b];
-        const cudaError_t e = run(pw, b, jobs);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    const int width = p.least_bits == p.most_bits ? p.most_bits : 0;
+    const Kernel kernel = kernels[mode][width];
+    const cudaError_t e = opt_in_shared_memory(configured[mode][width], (int)smem_hist, kernel);
+    if (e != cudaSuccess) return e;
+    return launch(kernel, dim3((unsigned)p.num_tiles, (unsigned)p.worker_count), kQThreads, hist ? smem_hist : smem, s, p, grads, step,
+                  packed, norms, hist, prev_packed, prev_norms, levels_cur, levels_prev, t);
 }
 
 cudaError_t launch_stat_finalize(const PlanDev& p, cudaStream_t s)

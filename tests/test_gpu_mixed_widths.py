@@ -1,4 +1,4 @@
-"""ENCODE of a plan with layers of several code widths and many waves of CTAs: one launch per width over its share of the jobs.
+"""ENCODE of a plan with layers of several code widths and many waves of CTAs, which take the tiles width by width.
 Messages, norms and flags against the oracle bit by bit, the statistic within the tolerance of its summation order."""
 import numpy as np
 import pytest
