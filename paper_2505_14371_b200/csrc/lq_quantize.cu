@@ -264,8 +264,9 @@ cudaError_t launch_quantize(const PlanDev& p, const float* grads, uint32_t step,
     const Kernel kernel = kernels[mode][width];
     const cudaError_t e = opt_in_shared_memory(configured[mode][width], (int)smem_hist, kernel);
     if (e != cudaSuccess) return e;
-    return launch(kernel, dim3((unsigned)p.num_tiles, (unsigned)p.worker_count), kQThreads, hist ? smem_hist : smem, s, p, grads, step,
-                  packed, norms, hist, prev_packed, prev_norms, levels_cur, levels_prev, t);
+    return launch_as(encoder_dependent(p), kernel, dim3((unsigned)p.num_tiles, (unsigned)p.worker_count), kQThreads,
+                     hist ? smem_hist : smem, 1, s, p, grads, step, packed, norms, hist, prev_packed, prev_norms, levels_cur,
+                     levels_prev, t);
 }
 
 cudaError_t launch_stat_finalize(const PlanDev& p, cudaStream_t s)

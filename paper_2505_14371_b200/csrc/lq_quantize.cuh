@@ -45,6 +45,17 @@ constexpr uint32_t kSmSlack = kSmAlign - 16;       // which is 16-byte aligned a
 // (tables + ring + slack = 55 792 bytes: four CTAs fit in the 227 KB of an SM)
 constexpr uint32_t kHistClamp = 0x33780000u;       // bit pattern one histogram bin below 2^-24
 
+// Whether an encoder launch is a dependent one.  CTAs of more than a block per warp that all fit at once (4 per SM) are not:
+// started while the pass before still holds most SMs, several of them share the few that are free, and no later CTA evens
+// that out (one of 8 workers, 3 950 blocks in 124 tiles: 54 us so launched, 37 plainly; 12 000 blocks in 420 tiles 56.9 and
+// 48.3; with a block per warp, 880 blocks in 110 tiles, 30.5 and 35.9 the other way round).  Of several code widths up to two
+// waves, as their CTAs differ in cost (624 of them 315 and 271; of one width 79.5 and 82.3 at 620, the other way round).
+inline bool encoder_dependent(const PlanDev& p)
+{
+    const int64_t ctas = (int64_t)p.num_tiles * p.worker_count;
+    return ctas <= kDependentCtas && (p.sub_blocks * p.sub_tiles <= kQWarps || ctas > (p.least_bits == p.most_bits ? 4 : 8) * 148);
+}
+
 // x + 8 when the comparison holds, else x: one compare and one predicated add
 __device__ __forceinline__ uint32_t add8_if_gt_u32(uint32_t x, uint32_t a, uint32_t b)
 {

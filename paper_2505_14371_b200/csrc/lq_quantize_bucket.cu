@@ -374,7 +374,7 @@ cudaError_t launch_quantize_bucketed(const PlanDev& p, const float* grads, uint3
     static std::atomic<uint64_t> configured[2][9];
     const cudaError_t e = opt_in_shared_memory(configured[mode][width], (int)smem, kernels[mode][width]);
     if (e != cudaSuccess) return e;
-    return launch(kernels[mode][width], grid, kQThreads, smem, s, p, grads, step, packed, bucket_norms, hist, prev_packed, prev_norms,
+    return launch_as(encoder_dependent(p), kernels[mode][width], grid, kQThreads, smem, 1, s, p, grads, step, packed, bucket_norms, hist, prev_packed, prev_norms,
                   levels_cur, levels_prev, t);
 }
 
