@@ -585,8 +585,9 @@ __device__ __forceinline__ bool walk_run(const RunRef& r, uint32_t at, const uin
     return (flags & (kPair ? kDecPairInvalid : kDecInvalid)) != 0u || (r.check_end ? used != r.end_bit : used > 32u * (uint32_t)r.nwords);
 }
 
-// Runs of more words than there is room for: coordinate by coordinate, from global
-// memory, a word ahead of the 64 bits being read.
+// Runs of more words than there is room for, and broken ones: coordinate by coordinate, from global memory, a word ahead of
+// the 64 bits being read.  What a broken run decodes to is thereby the stream's doing alone: the walk goes on over the
+// block's other words, and zeros past its end.
 static __device__ __noinline__ bool walk_run_plain(const RunRef r, int C, const uint8_t* len, int64_t blk, int run, int64_t size,
                                                    uint32_t* dst)
 {
@@ -731,26 +732,27 @@ __global__ void __launch_bounds__(kThreads, 4) entropy_decode_runs_kernel(PlanDe
         const int w0 = (int)(r.start_bit >> 5), w1 = r.check_end ? min((int)((r.end_bit + 31u) >> 5), r.nwords) : r.nwords;
         const uintptr_t at = reinterpret_cast<uintptr_t>(r.src + w0), to = reinterpret_cast<uintptr_t>(r.src + w1);
         const uintptr_t from = at & ~(uintptr_t)15;
-        if (w1 <= w0 || to - from > (uintptr_t)(16 * pieces)) {
-            broken |= walk_run_plain(r, C, len, blk, t & 7, T.size, dst);
-            continue;
-        }
-        if (in_vec) {
-            for (uintptr_t f = from; f < to; f += 16)
-                cp_async16(taken + (uint32_t)(f - from), reinterpret_cast<const void*>(f), (int)min((uintptr_t)16, to - f));
-        } else {
-            for (uintptr_t f = at; f < to; f += 4) cp_async4(taken + (uint32_t)(f - from), reinterpret_cast<const void*>(f));
-        }
-        cp_async_commit();
-        cp_async_wait<0>();
-        const uint32_t first = taken + (uint32_t)(at - from);
-        switch ((blk + 1) * kBlockCoords <= T.size ? C : -C) {
-#define LQ_CASE(CC) case CC:  broken |= walk_run<CC, true>(r, first, len, blk, t & 7, T.size, dst); break;  \
-                    case -CC: broken |= walk_run<CC, false>(r, first, len, blk, t & 7, T.size, dst); break;
-            LQ_CASE(2) LQ_CASE(3) LQ_CASE(4) LQ_CASE(5) LQ_CASE(6) LQ_CASE(7) LQ_CASE(8) LQ_CASE(9)
+        bool again = w1 <= w0 || to - from > (uintptr_t)(16 * pieces);
+        if (!again) {
+            if (in_vec) {
+                for (uintptr_t f = from; f < to; f += 16)
+                    cp_async16(taken + (uint32_t)(f - from), reinterpret_cast<const void*>(f), (int)min((uintptr_t)16, to - f));
+            } else {
+                for (uintptr_t f = at; f < to; f += 4) cp_async4(taken + (uint32_t)(f - from), reinterpret_cast<const void*>(f));
+            }
+            cp_async_commit();
+            cp_async_wait<0>();
+            const uint32_t first = taken + (uint32_t)(at - from);
+            switch ((blk + 1) * kBlockCoords <= T.size ? C : -C) {
+#define LQ_CASE(CC) case CC:  again = walk_run<CC, true>(r, first, len, blk, t & 7, T.size, dst); break;  \
+                    case -CC: again = walk_run<CC, false>(r, first, len, blk, t & 7, T.size, dst); break;
+                LQ_CASE(2) LQ_CASE(3) LQ_CASE(4) LQ_CASE(5) LQ_CASE(6) LQ_CASE(7) LQ_CASE(8) LQ_CASE(9)
 #undef LQ_CASE
-            default: break;
+                default: break;
+            }
         }
+        // a broken run has read on past its own words into other threads': its words are formed again, from the block's
+        if (again) broken |= walk_run_plain(r, C, len, blk, t & 7, T.size, dst);
     }
     if (broken) atomicOr(bad, 1u);
 }
