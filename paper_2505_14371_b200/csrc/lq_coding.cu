@@ -444,7 +444,13 @@ __device__ __forceinline__ OneCoord decode_one(uint32_t e, int C, const uint32_t
     return r;
 }
 
-// One thread per (block, worker): walks the block's stream and rebuilds the fixed-width words.
+// Coordinates of lane `lane` inside a layer's last block, which holds `rest` of them: the first of its 32 positions (whole
+// rows, then its share of the row that the layer ends in).
+__device__ __forceinline__ int real_positions(int rest, int lane) { return 4 * (rest >> 7) + max(0, min(4, (rest & 127) - 4 * lane)); }
+
+// One thread per (block, worker): walks the block's stream and rebuilds the fixed-width words, two coordinates per look-up
+// where the table holds pairs.  Its chain of dependent look-ups bounds it: 300 000 coordinates at 4 bits, 4 workers, 344 us
+// one by one, 416 with a second look-up (the first one's share of a pair's bits) for each, 203 by pairs.
 __global__ void __launch_bounds__(128) entropy_decode_kernel(PlanDev p, const uint32_t* __restrict__ in, int64_t capacity,
                                                              const uint32_t* __restrict__ offsets,
                                                              const uint32_t* __restrict__ enc_tables,
@@ -467,25 +473,45 @@ __global__ void __launch_bounds__(128) entropy_decode_kernel(PlanDev p, const ui
     const int64_t first = off_k[g], last = min((int64_t)off_k[g + 1], capacity);
     const uint32_t* src = in + (int64_t)k * capacity;
     uint32_t* dst = packed + (int64_t)k * p.packed_words + L.word_off + blk * (int64_t)C * 32;
+    const int rest = (int)min((int64_t)kBlockCoords, L.size - blk * kBlockCoords);
     int64_t wi = first;                                       // next word to load
     uint64_t window = 0; int have = 0;                        // `have` valid bits in the low end of `window`
     bool broken = false;
+    uint32_t pos = 0, last_at = 0, last_pair = 0;             // bits taken; where the last look-up was made; its entry if a pair's
     for (int lane = 0; lane < 32; ++lane) {
         uint32_t cw[LQ_MAX_BITS + 2];
         for (int i = 0; i <= C; ++i) cw[i] = 0u;
-        for (int pp = 0; pp < 32; ++pp) {
-            if (!real_coord(blk, lane, pp, L.size)) continue;
+        const int real = real_positions(rest, lane);
+        for (int pp = 0; pp < real; pp += 2) {
             while (have <= 32) { const uint32_t x = wi < last ? src[wi] : 0u; ++wi; window |= (uint64_t)x << have; have += 32; }
-            const OneCoord c = decode_one(dec[window & (uint32_t)(kDecEntries - 1)], C, enc);
-            window >>= c.bits; have -= (int)c.bits;
-            if (c.invalid) { broken = true; continue; }
+            const uint32_t e = dec[window & (uint32_t)(kDecEntries - 1)];
+            uint32_t two, bits;                               // the symbols of coordinates pp and pp + 1 (a pattern without a word: 0)
+            last_at = pos; last_pair = 0;
+            if (C <= kDecPairBits && pp + 1 < real && !(e & kDecSingle)) {
+                two = e & ((1u << (2 * C)) - 1u);
+                bits = e >> kDecLenShift;
+                last_pair = e;
+            } else {
+                const OneCoord c = decode_one(e, C, enc);
+                two = c.sym; bits = c.bits;
+                broken |= c.invalid;
+                if (pp + 1 < real) {
+                    const OneCoord c1 = decode_one(dec[(window >> bits) & (uint32_t)(kDecEntries - 1)], C, enc);
+                    last_at = pos + bits;
+                    two |= c1.sym << C; bits += c1.bits;
+                    broken |= c1.invalid;
+                }
+            }
+            window >>= bits; have -= (int)bits; pos += bits;
             const int off = pp * C, i = off >> 5, s = off & 31;
-            cw[i] |= c.sym << s;
-            if (s + C > 32) cw[i + 1] |= c.sym >> (32 - s);
+            cw[i] |= two << s;
+            if (s + 2 * C > 32) cw[i + 1] |= two >> (32 - s);
         }
         for (int i = 0; i < C; ++i) dst[i * 32 + lane] = cw[i];
     }
-    if (broken || wi - 2 > last) atomicOr(bad, 1u);           // no valid word, or the block ran past its end
+    if (last_pair) last_at += decode_one(last_pair, C, enc).bits;
+    // no valid word, or a last coordinate that starts past the word behind the block's end
+    if (broken || first + (int64_t)(last_at >> 5) > last) atomicOr(bad, 1u);
 }
 
 // Decoder on the run offsets.  A run is four lanes (128 coordinates) of a block; one CTA takes a tile (up to 128 blocks of
@@ -540,7 +566,7 @@ __device__ __forceinline__ bool walk_run(const RunRef& r, uint32_t at, const uin
         uint32_t cw[C + 1];
 #pragma unroll
         for (int i = 0; i <= C; ++i) cw[i] = 0u;
-        const int real = kFull ? 32 : 4 * (rest >> 7) + max(0, min(4, (rest & 127) - 4 * (4 * run + l4)));
+        const int real = kFull ? 32 : real_positions(rest, 4 * run + l4);
 #pragma unroll
         for (int pp = 0; pp < 32; pp += 2) {
             if (!kFull && pp >= real) break;
