@@ -84,6 +84,7 @@ struct lq_plan {
     std::vector<int32_t> h_members;        // host staging of both lists (kept alive for the asynchronous copy)
     uint32_t* d_code_enc = nullptr;        // [L][256]   entropy stage, allocated at its first use
     uint16_t* d_code_dec = nullptr;        // [L][kDecEntries]
+    bool codes_ready = false;              // ... and all of the following allocated, the tables made
     uint32_t* d_code_bad = nullptr;        // [1] set by a decode that met an invalid stream
     EncodeScratch code_scratch{nullptr, nullptr};   // allocated with the tables
     std::vector<uint8_t> code_len;         // [L][256] host copy of the word lengths
@@ -798,44 +799,54 @@ int lq_profile_read(lq_plan* plan, double* total_ms, int64_t* launches)
 
 namespace {
 
-// Uploads the tables of one layer's code.
-int upload_code(lq_plan* plan, int layer, const uint8_t* len, int n)
+// The encode entries of one layer's code.
+int code_entries(int layer, const uint8_t* len, int n, uint32_t* enc)
 {
-    std::vector<uint32_t> code(kMaxLevels, 0), enc(kMaxLevels, 0);
-    std::vector<uint16_t> dec((size_t)kDecEntries);
-    if (!canonical_codes_host(len, n, kCodeMaxLen, code.data()))
+    uint32_t code[kMaxLevels] = {};
+    if (!canonical_codes_host(len, n, kCodeMaxLen, code))
         return fail(LQ_EINVAL, "layer %d: lengths must lie in [1, %d] and satisfy Kraft's inequality", layer, kCodeMaxLen);
-    build_code_tables_host(len, code.data(), n, enc.data(), dec.data());
-    LQ_CUDA(cudaMemcpy(plan->d_code_enc + (size_t)layer * kMaxLevels, enc.data(), kMaxLevels * sizeof(uint32_t),
+    build_code_table_host(len, code, n, enc);
+    return LQ_OK;
+}
+
+// Uploads the encode entries of `layers` layers from `layer` on and has the decode tables made from them; waits for both.
+int upload_codes(lq_plan* plan, int layer, int layers, const uint32_t* enc)
+{
+    LQ_CUDA(cudaMemcpy(plan->d_code_enc + (size_t)layer * kMaxLevels, enc, (size_t)layers * kMaxLevels * sizeof(uint32_t),
                        cudaMemcpyHostToDevice));
-    LQ_CUDA(cudaMemcpy(plan->d_code_dec + (size_t)layer * kDecEntries, dec.data(), dec.size() * sizeof(uint16_t),
-                       cudaMemcpyHostToDevice));
-    std::copy(len, len + n, plan->code_len.begin() + (size_t)layer * kMaxLevels);
+    LQ_CUDA(launch_build_decode_tables(plan->dev, layer, layers, plan->d_code_enc, plan->d_code_dec, nullptr));
+    LQ_CUDA(cudaStreamSynchronize(nullptr));
     return LQ_OK;
 }
 
 // First use of the entropy stage: tables for every layer, initialised to the flat code (b bits per index).
 int ensure_codes(lq_plan* plan)
 {
-    if (plan->d_code_enc) return LQ_OK;
+    if (plan->codes_ready) return LQ_OK;
     const size_t L = (size_t)(plan->dev.num_layers ? plan->dev.num_layers : 1);
+    const size_t K = (size_t)plan->dev.num_workers, nb = (size_t)(plan->dev.total_blocks ? plan->dev.total_blocks : 1);
     LQ_CUDA(cudaDeviceSynchronize());
-    LQ_CUDA(dev_alloc_zero(&plan->d_code_enc, L * kMaxLevels));
-    LQ_CUDA(dev_alloc_zero(&plan->d_code_dec, L * (size_t)kDecEntries));
-    LQ_CUDA(dev_alloc_zero(&plan->d_code_bad, 1));
-    {
-        const size_t K = (size_t)plan->dev.num_workers, nb = (size_t)(plan->dev.total_blocks ? plan->dev.total_blocks : 1);
-        LQ_CUDA(dev_alloc_zero(&plan->code_scratch.lane_bits, K * nb * 32));
-        LQ_CUDA(dev_alloc_zero(&plan->code_scratch.scan_part, K * ((nb + 1023) / 1024)));
-    }
-    try { plan->code_len.assign(L * kMaxLevels, 0); } catch (const std::bad_alloc&) { return fail(LQ_ENOMEM, "host allocation failed"); }
-    for (int m = 0; m < plan->dev.num_layers; ++m) {
-        const LayerDesc& Ld = plan->layers[(size_t)m];
-        uint8_t flat[kMaxLevels];
-        for (int j = 0; j < Ld.nlevels; ++j) flat[j] = (uint8_t)Ld.bits;
-        const int rc = upload_code(plan, m, flat, Ld.nlevels);
+    if (!plan->d_code_enc) LQ_CUDA(dev_alloc_zero(&plan->d_code_enc, L * kMaxLevels));
+    if (!plan->d_code_dec) LQ_CUDA(dev_alloc_zero(&plan->d_code_dec, L * (size_t)kDecEntries));
+    if (!plan->d_code_bad) LQ_CUDA(dev_alloc_zero(&plan->d_code_bad, 1));
+    if (!plan->code_scratch.lane_bits) LQ_CUDA(dev_alloc_zero(&plan->code_scratch.lane_bits, K * nb * 32));
+    if (!plan->code_scratch.scan_part) LQ_CUDA(dev_alloc_zero(&plan->code_scratch.scan_part, K * ((nb + 1023) / 1024)));
+    try {
+        plan->code_len.assign(L * kMaxLevels, 0);
+        std::vector<uint32_t> enc(L * kMaxLevels, 0);
+        for (int m = 0; m < plan->dev.num_layers; ++m) {
+            const LayerDesc& Ld = plan->layers[(size_t)m];
+            uint8_t* flat = plan->code_len.data() + (size_t)m * kMaxLevels;
+            std::fill(flat, flat + Ld.nlevels, (uint8_t)Ld.bits);
+            const int rc = code_entries(m, flat, Ld.nlevels, enc.data() + (size_t)m * kMaxLevels);
+            if (rc != LQ_OK) return rc;
+        }
+        const int rc = upload_codes(plan, 0, plan->dev.num_layers, enc.data());
         if (rc != LQ_OK) return rc;
+    } catch (const std::bad_alloc&) {
+        return fail(LQ_ENOMEM, "host allocation failed");
     }
+    plan->codes_ready = true;
     return LQ_OK;
 }
 
@@ -880,10 +891,16 @@ int lq_code_set(lq_plan* plan, int32_t layer, const uint8_t* lengths, int32_t n)
     if (!plan || !lengths) return fail(LQ_EINVAL, "NULL argument");
     if (layer < 0 || layer >= plan->dev.num_layers) return fail(LQ_EINVAL, "layer %d out of range", layer);
     if (n != plan->layers[(size_t)layer].nlevels) return fail(LQ_EINVAL, "layer %d has %d levels, got %d", layer, plan->layers[(size_t)layer].nlevels, n);
-    const int rc = ensure_codes(plan);
+    int rc = ensure_codes(plan);
+    if (rc != LQ_OK) return rc;
+    uint32_t enc[kMaxLevels];
+    rc = code_entries(layer, lengths, n, enc);
     if (rc != LQ_OK) return rc;
     LQ_CUDA(cudaDeviceSynchronize());
-    return upload_code(plan, layer, lengths, n);
+    rc = upload_codes(plan, layer, 1, enc);
+    if (rc != LQ_OK) return rc;
+    std::copy(lengths, lengths + n, plan->code_len.begin() + (size_t)layer * kMaxLevels);
+    return LQ_OK;
 }
 
 int lq_code_get(lq_plan* plan, int32_t layer, uint8_t* lengths, int32_t n)

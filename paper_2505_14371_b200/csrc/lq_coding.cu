@@ -80,42 +80,45 @@ static uint32_t reverse_bits(uint32_t v, int l)
     return r;
 }
 
-// enc[level] = word with its first bit in bit 0 | length << 16.  dec: the table of lq_coding.cuh.
-void build_code_tables_host(const uint8_t* len, const uint32_t* code, int n, uint32_t* enc, uint16_t* dec)
+// enc[level] = word with its first bit in bit 0 | length << 16 (the decode table is made from these on the device).
+void build_code_table_host(const uint8_t* len, const uint32_t* code, int n, uint32_t* enc)
 {
-    for (int i = 0; i < kMaxLevels; ++i) enc[i] = 0;
-    for (int i = 0; i < kDecEntries; ++i) dec[i] = (uint16_t)(kDecInvalid | (1u << kDecLenShift));
-    for (int s = 0; s < n; ++s) {
-        const int l = len[s];
-        const uint32_t rev = reverse_bits(code[s], l);
-        enc[s] = rev | ((uint32_t)l << 16);
-        for (uint32_t hi = 0; hi < ((uint32_t)1 << (kDecBits - l)); ++hi) {
-            const uint32_t sign = s != 0 ? (hi & 1u) : 0u;             // the bit right after the word
-            dec[rev | (hi << l)] = (uint16_t)((2u * (uint32_t)s + sign) | ((uint32_t)(l + (s != 0 ? 1 : 0)) << kDecLenShift));
-        }
-    }
-    int C = 1;
-    while ((1 << C) < 2 * n) ++C;
-    if (C > kDecPairBits) return;
-    // what follows a window's first coordinate is the window shifted right: a smaller value (or 0 again), so going down
-    // every entry looked at is still a single one
-    for (uint32_t w = kDecEntries; w-- > 0;) {
-        const uint32_t e = dec[w], l = e >> kDecLenShift;
-        uint32_t out;
-        if (e & kDecInvalid) {
-            out = kDecPairInvalid | kDecSingle | (1u << kDecLenShift);
-        } else {
-            const uint32_t e1 = dec[w >> l], l1 = e1 >> kDecLenShift;
-            const bool second = !(e1 & kDecInvalid) && l + l1 <= (uint32_t)kDecBits;
-            out = (e & 0x1ffu) | (l << kDecLenShift) | kDecSingle;
-            if (second) out = (e & 0x1ffu) | ((e1 & 0x1ffu) << C) | ((l + l1) << kDecLenShift);
-        }
-        dec[w] = (uint16_t)out;
-    }
+    for (int i = 0; i < kMaxLevels; ++i) enc[i] = i < n ? reverse_bits(code[i], len[i]) | ((uint32_t)len[i] << 16) : 0u;
 }
 
 // ---- device ------------------------------------------------------------------------------------
 namespace {
+
+// The decode tables (lq_coding.cuh) of layers layer0, layer0 + 1, ... from their encode entries, a CTA per layer.  A code may
+// be renewed as often as the levels: on the host the 8192 entries and their pairs took 21 us a layer.
+__global__ void __launch_bounds__(1024) build_decode_tables_kernel(PlanDev p, int layer0, const uint32_t* enc_tables, uint16_t* dec_tables)
+{
+    __shared__ uint16_t one[kDecEntries];                       // a single coordinate per entry
+    const int layer = layer0 + blockIdx.x, n = p.layers[layer].nlevels, C = p.layers[layer].bits + 1;
+    const uint32_t* enc = enc_tables + (int64_t)layer * kMaxLevels;
+    uint16_t* dec = dec_tables + (int64_t)layer * kDecEntries;
+    for (int i = threadIdx.x; i < kDecEntries; i += blockDim.x) one[i] = (uint16_t)(kDecInvalid | (1u << kDecLenShift));
+    __syncthreads();
+    for (int s = threadIdx.x >> 5; s < n; s += (int)(blockDim.x >> 5)) {
+        const uint32_t e = enc[s], rev = e & 0xffffu, l = e >> 16;
+        for (uint32_t hi = threadIdx.x & 31; hi < 1u << (kDecBits - l); hi += 32) {
+            const uint32_t sign = s != 0 ? (hi & 1u) : 0u;             // the bit right after the word
+            one[rev | (hi << l)] = (uint16_t)((2u * (uint32_t)s + sign) | ((l + (s != 0 ? 1u : 0u)) << kDecLenShift));
+        }
+    }
+    __syncthreads();
+    for (uint32_t w = threadIdx.x; w < (uint32_t)kDecEntries; w += blockDim.x) {
+        const uint32_t e = one[w], l = e >> kDecLenShift;
+        uint32_t out = e;
+        if (C <= kDecPairBits) {
+            const uint32_t e1 = one[w >> l], l1 = e1 >> kDecLenShift;  // what follows a window's first coordinate
+            if (e & kDecInvalid) out = kDecPairInvalid | kDecSingle | (1u << kDecLenShift);
+            else if (!(e1 & kDecInvalid) && l + l1 <= (uint32_t)kDecBits) out = (e & 0x1ffu) | ((e1 & 0x1ffu) << C) | ((l + l1) << kDecLenShift);
+            else out = (e & 0x1ffu) | (l << kDecLenShift) | kDecSingle;
+        }
+        dec[w] = (uint16_t)out;
+    }
+}
 
 // Number of real coordinates among the 32 of this lane in block `blk`: coordinate of position p is
 // blk * 1024 + 128 * (p / 4) + 4 * lane + p % 4.
@@ -787,6 +790,13 @@ __global__ void __launch_bounds__(kThreads, 4) entropy_decode_runs_kernel(PlanDe
 }
 
 }  // namespace
+
+cudaError_t launch_build_decode_tables(const PlanDev& p, int layer0, int layers, const uint32_t* enc_tables, uint16_t* dec_tables,
+                                       cudaStream_t s)
+{
+    if (layers == 0) return cudaSuccess;
+    return launch_as(false, build_decode_tables_kernel, (unsigned)layers, 1024, 0, 1, s, p, layer0, enc_tables, dec_tables);
+}
 
 cudaError_t launch_entropy_encode(const PlanDev& p, const uint32_t* packed, const uint32_t* enc_tables,
                                   uint32_t* offsets, uint32_t* out, int64_t capacity, uint16_t* run_offsets,

@@ -1,4 +1,4 @@
-// Decode table of the entropy stage (shared by the code that builds it and the kernels that read it).
+// Decode table of the entropy stage (shared by the kernel that builds it and the ones that read it).
 // One entry per value of the next kDecBits = 13 stream bits (first bit in bit 0): a code word is at most
 // kCodeMaxLen = 12 bits and a non-zero level is followed by its sign bit, so 13 bits always hold one whole
 // coordinate.  Symbol = 2 * level index + sign, of C = b + 1 bits.
@@ -25,7 +25,7 @@ __host__ __device__ constexpr uint32_t zero_bit_entry(int C) { return (C <= kDec
 // ---- host side of the stage (lq_coding.cu) ----
 bool huffman_lengths_host(const double* w, int n, int max_len, uint8_t* len);
 bool canonical_codes_host(const uint8_t* len, int n, int max_len, uint32_t* code);
-void build_code_tables_host(const uint8_t* len, const uint32_t* code, int n, uint32_t* enc, uint16_t* dec);
+void build_code_table_host(const uint8_t* len, const uint32_t* code, int n, uint32_t* enc);
 
 // Scratch of the encoder, owned by the plan: the bits every lane of every block takes (filled by the sizing pass and
 // read by the writing pass, so that a lane's coordinates are sized once) and the per-1024-blocks sums of the scan.
@@ -33,6 +33,8 @@ struct EncodeScratch {
     uint16_t* lane_bits;     // [K][total_blocks][32]
     uint32_t* scan_part;     // [K][ceil(total_blocks / 1024)]
 };
+cudaError_t launch_build_decode_tables(const PlanDev& p, int layer0, int layers, const uint32_t* enc_tables, uint16_t* dec_tables,
+                                       cudaStream_t s);
 cudaError_t launch_entropy_encode(const PlanDev& p, const uint32_t* packed, const uint32_t* enc_tables,
                                   uint32_t* offsets, uint32_t* out, int64_t capacity, uint16_t* run_offsets,
                                   EncodeScratch scratch, cudaStream_t s);
