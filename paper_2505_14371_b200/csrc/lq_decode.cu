@@ -19,8 +19,6 @@
 
 namespace lq {
 
-constexpr int kDecWarps = 4;
-constexpr int kDecThreads = kDecWarps * 32;
 constexpr int kUnitPlanes = 20;                          // 128-byte planes of words in a unit, most
 constexpr uint32_t kUnitBytes = kUnitPlanes * 128;
 constexpr uint32_t kStateBytes = 2 * kBlockCoords * 4;   // a block's rows of Y, then of X_1

@@ -10,6 +10,7 @@
 
 namespace lq {
 
+constexpr int kSms = 148;             // of a B200: what grids and waves are counted in
 constexpr int kBlockCoords = 1024;    // coordinates per message block (32 lanes x 32 positions)
 constexpr int kTileBlocks = 128;      // most blocks per tile (the encoder's unit: its per-CTA tables are amortised over a
                                       // tile); a plan takes the largest power of two that still gives several waves of
@@ -18,6 +19,8 @@ constexpr int kSubBlocks = 32;        // most blocks per sub-tile (the unit of t
                                       // of the decoder's CTAs; fewer in plans that would leave SMs idle
 constexpr int kWarps = 8;
 constexpr int kThreads = 256;
+constexpr int kDecWarps = 4;          // of the decoder's CTAs
+constexpr int kDecThreads = kDecWarps * 32;
 constexpr int kLevelStride = 256;     // floats per layer in a level table
 constexpr int kMaxLevels = 256;
 constexpr int kCodeMaxLen = 12;       // longest code word of the entropy stage (LQ_CODE_MAX_LEN)
@@ -122,8 +125,14 @@ struct PlanDev {
 int lq_set_error(int code, const char* fmt, ...);
 
 // Whether the decoder's CTAs form the step's rates themselves from sq_diff (Eq. general_stepsize) instead of a kernel of
-// its own.  Up to four sums per thread: the kernel and the gap before it cost 3 to 4 us, the sums about 0.5 us per CTA.
-inline bool rates_in_decoder(const PlanDev& p) { return (int64_t)p.num_workers * p.num_layers <= 4 * kThreads && p.num_tiles > 0; }
+// its own, which with the gap before it takes 2 to 4 us: two sums per thread, four where the CTAs fit at once (4 per SM).
+// The step with 8 workers, by the decoder and by the kernel: 32 small layers 48.9 and 50.4 us, 64 of them 67.6 and 68.8; but 64
+// layers of 245 blocks 373 and 370, 128 small ones 119.6 and 117.7.
+inline bool rates_in_decoder(const PlanDev& p)
+{
+    const int64_t sums = (int64_t)p.num_workers * p.num_layers, ctas = (int64_t)p.num_tiles << p.dec_shift;
+    return p.num_tiles > 0 && (sums <= 2 * kDecThreads || (sums <= 4 * kDecThreads && ctas <= 4 * kSms));
+}
 
 // Launches `kernel` so that it may start while the kernel before it on the stream is still finishing (programmatic
 // dependent launch).  Every kernel of the library waits for its predecessor's memory (pdl_wait) before it touches anything

@@ -50,3 +50,24 @@ def test_mean_of_messages(orc, scope, sizes, bits, K):
     plan.qoda_step(packed, norms, X1, Y, Xh, None, gbar3)          # the message's own buffer: all-zero blocks are not read
     assert np.array_equal(to_unpadded(plan, gbar3), want)
     assert np.array_equal(to_unpadded(plan, Y), -want)
+
+
+@pytest.mark.parametrize("layers, size", [(32, 2000), (33, 2000), (64, 2000), (65, 2000), (64, 300000)])
+def test_rates_on_both_sides_of_their_rule(layers, size):
+    """The step size from 8 x `layers` statistics, formed by the decoder's CTAs or by a kernel before: the sum of what
+    lq_get_statistics returns, in another order."""
+    import paper_2505_14371_b200 as lqm
+    lqm.load_library()
+    plan = lqm.Plan([size] * layers, 4, 2, 8, 5)
+    g = torch.Generator(device="cuda").manual_seed(layers)
+    X1 = torch.randn(plan.padded_elems, generator=g, device="cuda")
+    Y, Xh = torch.empty_like(X1), torch.empty_like(X1)
+    plan.qoda_init(X1, Y, Xh)
+    total = 0.0
+    for t in (1, 2):
+        packed, norms = plan.empty_packed(), plan.empty_norms()
+        plan.lq_quantize_pack(torch.randn((8, plan.padded_elems), generator=g, device="cuda"), t, packed, norms)
+        total += float(plan.lq_get_statistics()[0].numpy().sum()) / 64.0
+        plan.qoda_step(packed, norms, X1, Y, Xh)
+    now, S, eta = plan.qoda_get_scalars()
+    assert now == 3 and abs(S - total) <= 8 * layers * 2.0 ** -52 * total and eta == float(np.float32((1.0 + S) ** -0.5))
