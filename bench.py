@@ -38,7 +38,7 @@ METRIC = "quantize+pack and decode+aggregate+QODA GB/s (fp32 in)"
 # of a launch is a * E + b * N for E worker-coordinates in the embedding (90 % zero rows) and N in the other layers,
 # and (a, b) solve the two captures.  `inst` is the same for executed warp instructions (smsp__inst_executed.sum).
 KERNEL_SOURCES = {"norm_partial": ["lq_norm.cu", "lq_internal.cuh"],
-                  "quantize_pack": ["lq_quantize.cu", "lq_quantize.cuh", "lq_internal.cuh"],
+                  "quantize_pack": ["lq_quantize.cu", "lq_quantize_tile.cuh", "lq_quantize.cuh", "lq_internal.cuh"],
                   "decode": ["lq_decode.cu", "lq_internal.cuh"]}
 NCU_SCALED = {"transformer_xl": {          # kernel: bytes per embedding / other worker-coordinate, warp instr likewise
     "norm_partial": {"bytes": (4.0063, 4.0085), "inst": (0.15710, 0.16787), "sources": "16beee4053b150a1"},
@@ -514,7 +514,7 @@ def run_gpu(args) -> None:
         roofline["achieved"], roofline["frac"] = kd["gbs_algorithmic"], kd["frac_algorithmic"]
         roofline["note"] = "no ncu counters for this configuration: achieved = algorithmic bytes / time"
     call_kernels = {"lq_quantize_pack": ("norm_partial", "norm_finalize", "quantize_pack", "stat_finalize"),
-                    "qoda_step": ("qoda_scalars", "block_live", "decode")}
+                    "qoda_step": ("qoda_scalars", "decode")}
     qp_alg = ((4.0 + 2 * (c + 4.0 / 128.0)) if bucket else (8.0 + 2 * c)) * K * D * share
     call_alg = {"lq_quantize_pack": qp_alg, "qoda_step": alg["decode"]}
     calls = {}

@@ -366,7 +366,7 @@ int lq_vector_norm_static(const float* v, int64_t n, int32_t q, float* norm_out,
 #define LQ_KERNEL_FIT            6
 #define LQ_KERNEL_ALT_FINALIZE   7
 #define LQ_KERNEL_AVERAGE        8
-#define LQ_KERNEL_BLOCK_LIVE     9
+#define LQ_KERNEL_BLOCK_LIVE     9    /* not launched any more (the decoder reads the masks itself): stays 0 */
 #define LQ_NUM_KERNELS           10
 int lq_profile_enable(lq_plan* plan, int32_t enable);
 int lq_profile_read(lq_plan* plan, double* total_ms, int64_t* launches);

@@ -193,8 +193,8 @@ int lq_plan_create(lq_plan** out, int32_t num_layers, const int64_t* layer_sizes
     if (!p) return fail(LQ_ENOMEM, "host allocation failed");
     int64_t elem = 0, word = 0, ntiles = 0, blocks = 0;
     // tile size: as large as possible while (tiles x workers) still fills the GPU several times over; below 32 blocks only
-    // while the tiles do not fill it once (4 CTAs on each of the 148 SMs).  Sub-tiles likewise, without the workers (the
-    // decoder has one CTA for all of them).
+    // while the tiles do not fill it once (4 CTAs on each SM).  Sub-tiles likewise; the decoder has one CTA for all workers and
+    // a size of its own.
     int tile_blocks = kTileBlocks, sub_blocks = kSubBlocks, dec_blocks = kSubBlocks, most_bits = 1, least_bits = num_layers ? LQ_MAX_BITS : 1;
     int64_t most_blocks = 0;
     {
@@ -205,7 +205,7 @@ int lq_plan_create(lq_plan** out, int32_t num_layers, const int64_t* layer_sizes
                 total += n;
                 most_blocks = std::max(most_blocks, n);
             }
-        constexpr int kWave = 4 * 148;
+        constexpr int kWave = 4 * kSms;
         while (tile_blocks > 32 && (total / tile_blocks) * num_workers < 4096) tile_blocks /= 2;
         while (tile_blocks > 8 && (total / tile_blocks) * num_workers < kWave) tile_blocks /= 2;
         while (sub_blocks > 8 && (total / sub_blocks) * num_workers < kWave) sub_blocks /= 2;

@@ -826,7 +826,7 @@ cudaError_t launch_entropy_decode(const PlanDev& p, const uint32_t* in, int64_t 
         // others' runs makes room for a CTA more (of more than fit at once): 306 layers, 2 800 blocks, 12 workers at 8 bits, 88.0 us with
         // 256 walkers and 73.9 with 128
         const int walkers = LQ_CODE_RUNS * p.total_blocks <= (kThreads / 2) * (int64_t)p.num_tiles &&
-                                    (int64_t)p.num_tiles * p.num_workers > 3 * 148 ? kThreads / 2 : kThreads;
+                                    (int64_t)p.num_tiles * p.num_workers > 3 * kSms ? kThreads / 2 : kThreads;
         entropy_decode_runs_kernel<<<grid_r, kThreads, kRunSmem(p.most_bits, walkers), s>>>(
             p, in, capacity, offsets, run_offsets, enc_tables, dec_tables, packed, bad, reinterpret_cast<uintptr_t>(packed) % 16 == 0,
             walkers);

@@ -494,7 +494,7 @@ __global__ void __launch_bounds__(256) average_kernel(const float* __restrict__ 
 cudaError_t launch_average(const PlanDev& p, const float* Xhalf, double* xsum, cudaStream_t s)
 {
     const int64_t n4 = p.padded_elems / 4;
-    const unsigned blocks = (unsigned)((n4 + 255) / 256 < 148 * 16 ? (n4 + 255) / 256 + 1 : 148 * 16);
+    const unsigned blocks = (unsigned)((n4 + 255) / 256 < kSms * 16 ? (n4 + 255) / 256 + 1 : kSms * 16);
     average_kernel<<<blocks, 256, 0, s>>>(Xhalf, xsum, n4);
     return cudaGetLastError();
 }
@@ -545,7 +545,7 @@ cudaError_t launch_qoda_scalars(const PlanDev& p, cudaStream_t s)
 cudaError_t launch_qoda_init(const PlanDev& p, const float* X1, float* Y, float* Xhalf, cudaStream_t s)
 {
     const int64_t n4 = p.padded_elems / 4;
-    const unsigned blocks = (unsigned)((n4 + 255) / 256 < 148 * 8 ? (n4 + 255) / 256 + 1 : 148 * 8);
+    const unsigned blocks = (unsigned)((n4 + 255) / 256 < kSms * 8 ? (n4 + 255) / 256 + 1 : kSms * 8);
     qoda_init_kernel<<<blocks, 256, 0, s>>>(p, X1, Y, Xhalf);
     return cudaGetLastError();
 }

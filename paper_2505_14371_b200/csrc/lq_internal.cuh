@@ -15,7 +15,7 @@ constexpr int kBlockCoords = 1024;    // coordinates per message block (32 lanes
 constexpr int kTileBlocks = 128;      // most blocks per tile (the encoder's unit: its per-CTA tables are amortised over a
                                       // tile); a plan takes the largest power of two that still gives several waves of
                                       // CTAs, down to 8 (one block per warp) when even a single wave is not reached
-constexpr int kSubBlocks = 32;        // most blocks per sub-tile (the unit of the norm kernel and the entropy stage), and
+constexpr int kSubBlocks = 32;        // most blocks per sub-tile (the unit of the norm kernel and the symbol counts), and
                                       // of the decoder's CTAs; fewer in plans that would leave SMs idle
 constexpr int kWarps = 8;
 constexpr int kThreads = 256;
@@ -141,7 +141,7 @@ inline bool rates_in_decoder(const PlanDev& p)
 // to well below 1 us.  Grids of many waves are launched the plain way: with the attribute every CTA starts about 3 us
 // late, not just the first ones (norm pass of 37 000 CTAs 690 -> 850 us, decoder of 4 700 CTAs 451 -> 486 us).  The line: up to 24 CTAs per
 // SM no case got slower (with 8: WGAN step 174 -> 170 us, in bucket scope 175 -> 167, low-rank factors 336 -> 328).
-constexpr int64_t kDependentCtas = 148 * 24;
+constexpr int64_t kDependentCtas = kSms * 24;
 // `cluster`: CTAs per cluster along x.  A launch that fails leaves no error behind for the next call to find.
 template <typename... Params, typename... Args>
 cudaError_t launch_as(bool dependent, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, unsigned cluster, cudaStream_t s,
@@ -511,7 +511,7 @@ __device__ __forceinline__ LayerNorm layer_norm_from_partials(const double* part
     int bad = 0;
     if (threadIdx.x < 128)
         for (int i = threadIdx.x; i < n; i += 128) {
-            const double v = __ldcg(part + i);                   // (from L2: another CTA of this launch may have written it)
+            const double v = __ldcg(part + i);
             if (!(fabs(v) <= 1.7976931348623157e308)) bad = 1;
             if (q == 0) acc = fmax(acc, v); else acc += v;
         }

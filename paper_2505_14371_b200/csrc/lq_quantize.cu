@@ -11,8 +11,8 @@
 // while they wait; every lane reads back only the bytes it copied itself, so the ring needs no
 // barrier.  Per row the lane draws one Philox4x32-10 block (4 uniforms); after 8 rows it holds
 // exactly b+1 words of symbols, which it stores plane by plane (128 contiguous bytes per warp and
-// plane).  No shuffles, ballots or atomics on the per-coordinate path.  The kernel is bound by
-// instruction issue (about 42 instructions per coordinate: 10 Philox, 7 the statistic), not by DRAM.
+// plane).  No shuffles, ballots or atomics on the per-coordinate path.  The kernel is bound by its
+// arithmetic pipes and the issue of some 40 instructions per coordinate (10 Philox, 7 the statistic), not by DRAM.
 //
 // The level search and the tables are described in lq_quantize.cuh.  Layers whose levels are denser than the
 // search table's bins take finer bins, or a byte table and steps up from its entry (build_search_kernel).
@@ -28,8 +28,9 @@
 
 namespace lq {
 
-// kWidth: the code width of every layer of the plan, or 0 when they differ.  (A kernel of one width is compiled to what that
-// width needs: fewer spills, less code.)
+// kWidth: the code width of every layer of the plan, or 0 when they differ.  (A kernel of one width has less code to fetch and,
+// at widths 1 to 4 without histogram, no spills: 0 bytes of stores and loads against 8 and 32; widths 5 to 8 spill 8 to 28
+// bytes of stores, with histogram widths 1, 2, 4, 5 and 6 44 to 52, all widths in one 20.)
 template <int kWidth, bool kHist, bool kStat>
 __global__ void __launch_bounds__(kQThreads, 4) quantize_pack_kernel(
     PlanDev p, const float* grads, uint32_t step, uint32_t* packed, const float* norms, uint32_t* hist,

@@ -53,7 +53,7 @@ constexpr uint32_t kHistClamp = 0x33780000u;       // bit pattern one histogram 
 inline bool encoder_dependent(const PlanDev& p)
 {
     const int64_t ctas = (int64_t)p.num_tiles * p.worker_count;
-    return ctas <= kDependentCtas && (p.sub_blocks * p.sub_tiles <= kQWarps || ctas > (p.least_bits == p.most_bits ? 4 : 8) * 148);
+    return ctas <= kDependentCtas && (p.sub_blocks * p.sub_tiles <= kQWarps || ctas > (p.least_bits == p.most_bits ? 4 : 8) * kSms);
 }
 
 // x + 8 when the comparison holds, else x: one compare and one predicated add
@@ -277,7 +277,7 @@ __device__ __forceinline__ void stat_prev_only(const QuantEnv& ev, const uint32_
 
 // Fills the CTA's tables (all threads; the caller synchronises afterwards).  `sm` is the generic pointer to the
 // aligned base.  ncur / nprev: the norms that scale the value tables (1 in bucket scope).
-__device__ __forceinline__ void fill_tables(unsigned char* sm, const SearchTables& st, int layer, int n, bool fast,
+__device__ __forceinline__ void fill_tables(unsigned char* sm, const SearchTables& st, int layer, int n,
                                             const float* __restrict__ levels_cur, const float* __restrict__ levels_prev,
                                             float ncur, float nprev, bool hist)
 {
@@ -291,11 +291,9 @@ __device__ __forceinline__ void fill_tables(unsigned char* sm, const SearchTable
         tcur[2 * i] = c;  tcur[2 * i + 1] = -c;
         tprev[2 * i] = q; tprev[2 * i + 1] = -q;
     }
-    if (fast) {
-        const uint4* src = reinterpret_cast<const uint4*>(st.lut + (int64_t)layer * kLutEntries);
-        uint4* dst = reinterpret_cast<uint4*>(sm + kSmLut);
-        for (int i = threadIdx.x; i < kLutEntries / 4; i += blockDim.x) dst[i] = load_u32x4(src + i);
-    }
+    const uint4* src = reinterpret_cast<const uint4*>(st.lut + (int64_t)layer * kLutEntries);
+    uint4* dst = reinterpret_cast<uint4*>(sm + kSmLut);
+    for (int i = threadIdx.x; i < kLutEntries / 4; i += blockDim.x) dst[i] = load_u32x4(src + i);
     if (hist) {
         uint32_t* h = reinterpret_cast<uint32_t*>(sm + kSmHist);
         for (int i = threadIdx.x; i < LQ_HIST_STRIDE; i += blockDim.x) h[i] = 0;

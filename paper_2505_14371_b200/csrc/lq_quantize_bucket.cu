@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(kQThreads, 3) quantize_pack_bucket_kernel(
 
     // the tables hold the plain levels (norm 1) and each row multiplies by its own norm
     if (threadIdx.x == 0) *reinterpret_cast<int2*>(sm + kSmHow) = how;
-    fill_tables(sm, st, layer, L.nlevels, true, levels_cur, levels_prev, 1.0f, 1.0f, kHist);
+    fill_tables(sm, st, layer, L.nlevels, levels_cur, levels_prev, 1.0f, 1.0f, kHist);
     __syncthreads();
 
     BucketCtx c;

@@ -206,7 +206,7 @@ bool use_small(const PlanDev& p)
 {
     const int ranks = small_ranks(p);
     return !p.global_norm && !p.bucket_norm && p.most_blocks <= 256 &&
-           (int64_t)p.num_workers * p.num_layers * ranks <= (ranks == 1 ? 3 * 148 : 352);
+           (int64_t)p.num_workers * p.num_layers * ranks <= (ranks == 1 ? 3 * kSms : 352);
 }
 
 cudaError_t launch_layer_norms_small(const PlanDev& p, const float* grads, float* norms, cudaStream_t s)

@@ -165,7 +165,6 @@ __device__ __forceinline__ double quantize_tile(const PlanDev& p, const PhiloxCo
         i = inext;
         todo &= todo - 1;
         m = mnext;
-        src = nsrc;
     }
     cp_async_wait<0>();
     return stat;

@@ -1,6 +1,7 @@
 """ENCODE of plans whose layers are all small (one cluster per layer and worker): sizes around a cluster's capacity, CTAs of
-a cluster that have no block, empty layers, worker ranges; messages, norms, flags and masks against the oracle bit by bit, the
-statistic within the tolerance of its summation order."""
+a cluster that have no block, empty layers, worker ranges; messages, norms and flags against the oracle bit by bit (the zero-row
+masks through the updates and statistics that leave rows out by them), the statistic within the tolerance of its summation
+order."""
 import numpy as np
 import pytest
 import torch
