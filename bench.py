@@ -43,7 +43,7 @@ KERNEL_SOURCES = {"norm_partial": ["lq_norm.cu", "lq_internal.cuh"],
 NCU_SCALED = {"transformer_xl": {          # kernel: bytes per embedding / other worker-coordinate, warp instr likewise
     "norm_partial": {"bytes": (4.0067, 4.0092), "inst": (0.15637, 0.16913), "sources": "618bfbec8b934517"},
     "quantize_pack": {"bytes": (1.3163, 5.3143), "inst": (0.22824, 1.28637), "sources": "8b9eb003e975ea00"},
-    "decode": {"bytes": (2.0863, 2.5274), "inst": (0.13197, 0.22909), "sources": "cb264e803c848c59"}}}
+    "decode": {"bytes": (2.0863, 2.5274), "inst": (0.13197, 0.22909), "sources": "79467e8b33f1c270"}}}
 NCU_DIRECT = {"flat:26:4:8:2": {           # kernel: bytes and warp instructions of one launch
     "quantize_pack": {"bytes": 2484224768.0 + 347961088.0, "inst": 676171776.0, "sources": "8b9eb003e975ea00"}}}
 DENSE_POINT = "flat:26:4:8:2"             # dense companion of the headline workload: no zero rows to skip

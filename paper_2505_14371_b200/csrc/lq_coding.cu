@@ -208,7 +208,7 @@ __device__ __forceinline__ uint32_t lane_bits(const uint32_t* code, const uint32
         const int real = real_positions((int)(size - blk * kBlockCoords), lane);
 #pragma unroll
         for (int pp = 0; pp < 32; pp += kPartialStep<C>)
-            if (pp < real) bits += partial_entry<C>(code, w, pp, real) >> kLenShift;
+            if (C <= kPairBits ? pp < real : real_coord(blk, lane, pp, size)) bits += partial_entry<C>(code, w, pp, real) >> kLenShift;
     }
     return bits;
 }
@@ -244,7 +244,7 @@ __device__ __forceinline__ void emit_partial(const uint32_t* code, const uint32_
     const int real = real_positions((int)(size - blk * kBlockCoords), lane);
 #pragma unroll
     for (int pp = 0; pp < 32; pp += kPartialStep<C>) {
-        if (pp >= real) continue;
+        if (C <= kPairBits ? pp >= real : !real_coord(blk, lane, pp, size)) continue;
         const uint32_t e = partial_entry<C>(code, w, pp, real);
         const uint64_t c = (uint64_t)(e & kCodeMask) << (pos & 31u);
         atomicOr(buf + (pos >> 5), (uint32_t)c);

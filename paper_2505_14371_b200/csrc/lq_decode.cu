@@ -223,10 +223,15 @@ __device__ __forceinline__ void finish_block(const DecodeArgs& a, const Walk& w,
     }
 }
 
-// All warps of the CTA.  Not __syncthreads(): where the warps share a block (kSplit) each is in a decode_blocks of its own rows,
-// and that is defined only for a barrier that all threads meet at one place of the program.  A numbered barrier counts
-// arrivals, wherever they come from.
-__device__ __forceinline__ void warps_meet() { asm volatile("barrier.sync 1, %0;" ::"n"(kDecThreads) : "memory"); }
+// All warps of the CTA.  Where the warps share a block (kSplit, 2 rows each) every warp is in a decode_blocks of its own rows, and
+// __syncthreads() is defined only where all threads meet at one place of the program; a numbered barrier counts arrivals,
+// wherever they come from.
+template <int kRows>
+__device__ __forceinline__ void warps_meet()
+{
+    if constexpr (kRows == 8) __syncthreads();
+    else asm volatile("bar.sync 1, %0;" ::"n"(kDecThreads) : "memory");
+}
 
 // A warp's blocks: warp, warp + 4, ... of the CTA's (kRows = 8), or rows kRow0, kRow0 + 1 of all of them (kRows = 2).
 // The next unit's words are always requested before the current unit is waited for; the rows of Y and X_1 as soon as
@@ -260,7 +265,7 @@ __device__ __forceinline__ void decode_blocks(const PlanDev& p, const LayerDesc&
         cp_async_commit();
     }
     fill_tables<kBucket>(p, L, layer, a, table, 0, min(K, kTW));
-    warps_meet();
+    warps_meet<kRows>();
     const Rates rt = *rates;
     double lam_acc = 0.0, mu_acc = 0.0;
     uint32_t stage = 0;
@@ -282,9 +287,9 @@ __device__ __forceinline__ void decode_blocks(const PlanDev& p, const LayerDesc&
             if (!kBucket && K > kTW) {
                 k_in = k0 % kTW;
                 if (k_in == 0 && (b0 > 0 || u > 0)) {
-                    warps_meet();
+                    warps_meet<kRows>();
                     fill_tables<kBucket>(p, L, layer, a, table, k0, min(kTW, K - k0));
-                    warps_meet();
+                    warps_meet<kRows>();
                 }
             }
             if (kQoda && u == 0) cp_async_wait<2>(); else cp_async_wait<1>();
