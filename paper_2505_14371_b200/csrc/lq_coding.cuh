@@ -27,17 +27,17 @@ bool huffman_lengths_host(const double* w, int n, int max_len, uint8_t* len);
 bool canonical_codes_host(const uint8_t* len, int n, int max_len, uint32_t* code);
 void build_code_table_host(const uint8_t* len, const uint32_t* code, int n, uint32_t* enc);
 
-// Scratch of the encoder, owned by the plan: the bits every lane of every block takes (filled by the sizing pass and
-// read by the writing pass, so that a lane's coordinates are sized once) and the per-1024-blocks sums of the scan.
+// Scratch of the encoder, owned by the plan: a counter from which its CTAs take their tiles, then what every (worker, tile)
+// tells the tiles behind it; cleared before each encode.
 struct EncodeScratch {
-    uint16_t* lane_bits;     // [K][total_blocks][32]
-    uint32_t* scan_part;     // [K][ceil(total_blocks / 1024)]
+    uint64_t* states;        // [1 + K * num_tiles]
+    size_t bytes;
 };
 cudaError_t launch_build_decode_tables(const PlanDev& p, int layer0, int layers, const uint32_t* enc_tables, uint16_t* dec_tables,
                                        cudaStream_t s);
 cudaError_t launch_entropy_encode(const PlanDev& p, const uint32_t* packed, const uint32_t* enc_tables,
                                   uint32_t* offsets, uint32_t* out, int64_t capacity, uint16_t* run_offsets,
-                                  EncodeScratch scratch, cudaStream_t s);
+                                  EncodeScratch scratch, uint32_t* bad, cudaStream_t s);
 cudaError_t launch_entropy_decode(const PlanDev& p, const uint32_t* in, int64_t capacity, const uint32_t* offsets,
                                   const uint16_t* run_offsets, const uint32_t* enc_tables, const uint16_t* dec_tables, uint32_t* packed, uint32_t* bad,
                                   cudaStream_t s);

@@ -1,0 +1,57 @@
+"""The entropy encoder where its tiles meet: plans of fewer and of more tiles than a tile looks back over at a time, so that a
+tile's place in the stream comes from one or several looks; blocks with rows of zeros under codes whose word for level 0 is
+one zero bit, several, or not zeros at all.  Every block of every worker against the oracle's encoder, and the way back."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+def _code(lqm, kind, n):
+    if kind == "zero_long":                                  # level 0 has the longest word, all ones
+        return lqm.lq_code_build([0.001] + [0.5 ** min(j, 9) for j in range(1, n)])
+    return [n.bit_length() - 1] * n if kind == "flat" else lqm.lq_code_build([0.9] + [0.1 / n] * (n - 1))
+
+
+@pytest.mark.parametrize("bits, kind", [(1, "fitted"), (2, "zero_long"), (3, "flat"), (4, "fitted"), (5, "zero_long"), (8, "flat")])
+@pytest.mark.parametrize("layers", [1, 32, 33, 70])
+def test_streams_of_many_tiles(orc, layers, bits, kind):
+    import paper_2505_14371_b200 as lqm
+    lqm.load_library()
+    K, rng = 3, np.random.default_rng(layers + bits)
+    sizes = [int(x) for x in rng.choice([1, 1023, 1024, 1025, 2500, 9 * 1024 + 7], layers)]
+    plan = lqm.Plan(sizes, bits, 2, K, 5 + bits)
+    gen = torch.Generator(device="cuda").manual_seed(bits)
+    grads = torch.randn((K, plan.padded_elems), generator=gen, device="cuda")
+    grads.view(K, -1, 32)[:, ::3] = 0.0                      # a third of the rows' quarters
+    grads[:, 2048:4096] = 0.0
+    packed, norms = plan.empty_packed(), plan.empty_norms()
+    plan.lq_quantize_pack(grads, 1, packed, norms)
+    lengths = _code(lqm, kind, 1 << bits)
+    for m in range(layers):
+        plan.lq_code_set(m, lengths)
+    stream = torch.full((K, plan.lq_plan_blocks() * 416), -1, dtype=torch.int32, device="cuda")
+    offs = torch.zeros((K, plan.lq_plan_blocks() + 1), dtype=torch.int32, device="cuda")
+    runs = plan.empty_run_offsets()
+    for _ in range(2):                                       # the second encode finds the first one's scratch
+        plan.lq_entropy_encode(packed, stream, offs, runs)
+    pk, S, O = packed.cpu().numpy().view(np.uint32), stream.cpu().numpy().view(np.uint32), offs.cpu().numpy().astype(np.int64)
+    l = np.uint8(lengths)
+    c = orc.canonical_codes(l)
+    for k in range(K):
+        pos = g = 0
+        for m, d in enumerate(sizes):
+            at = plan.word_offsets[m]
+            idx, sg = orc.unpack_layer(pk[k, at: at + orc.packed_words(d, bits)], d, bits)
+            for lo in range(0, d, 1024):
+                words, _ = orc.entropy_encode_block(idx[lo: lo + 1024], sg[lo: lo + 1024], l, c)
+                assert O[k, g] == pos and np.array_equal(S[k, pos: pos + words.size], words), (k, m, lo)
+                pos += words.size
+                g += 1
+        assert O[k, g] == pos and np.all(S[k, pos:] == 0xffffffff)
+    back, again = torch.full_like(packed, -1), torch.full_like(stream, -1)
+    plan.lq_entropy_decode(stream, offs, back, runs)
+    assert plan.lq_entropy_status() == 0
+    plan.lq_entropy_encode(back, again, offs, runs)
+    assert torch.equal(again, stream)
