@@ -356,6 +356,13 @@ __device__ __forceinline__ float4 lds_f32x4(uint32_t a)
     return v;
 }
 
+// a0 += b0 and a1 += b1, each rounded as a plain addition, in one instruction
+__device__ __forceinline__ void add_f32x2(float& a0, float& a1, float b0, float b1)
+{
+    asm("{\n\t.reg .b64 a, b;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 b, {%2, %3};\n\tadd.rn.f32x2 a, a, b;\n\tmov.b64 {%0, %1}, a;\n\t}"
+        : "+f"(a0), "+f"(a1) : "f"(b0), "f"(b1));
+}
+
 // 16-byte asynchronous copies global -> shared (completion by commit / wait groups of the issuing thread)
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, int bytes)
 {
