@@ -196,7 +196,7 @@ cudaError_t launch_norm_partial(const PlanDev& p, const float* grads, bool write
 cudaError_t launch_norm_finalize(const PlanDev& p, float* norms, cudaStream_t s);
 // Encode-side tables derived from one level table (rebuilt whenever the levels change).
 struct SearchTables {
-    uint32_t* lut;     // [L][kLutEntries] per bin: 8 * tau0 | (low 19 bits of the level inside the bin, minus 1) << 13
+    uint32_t* lut;     // [L][kLutEntries] per bin: what added to a value's pattern gives tau << 19 (build_search_kernel)
     float2* ld;        // [L][kMaxLevels]  {l_tau, l_{tau+1} - l_tau}
     int2* how;         // [L]              which search a layer takes and its parameters
 };

@@ -150,11 +150,11 @@ __global__ void __launch_bounds__(128) stat_finalize_kernel(PlanDev p)
 // One CTA per layer: derives the encode-side tables from the layer's levels, which it also copies to `kept` (the level
 // table of the messages to come).
 //   ld[tau]  = {l_tau, l_{tau+1} - l_tau}                 tau = 0..n-2 (other entries: {l_tau, 0})
-//   lut[bin] = 8 * tau0 | code << 13    bin = bits(u) >> 19, i.e. the values [lo, hi) with bits(lo) = bin << 19;
-//              tau0 = last level (<= n-2) at or below lo; code = (low 19 bits of l_{tau0+1}) - 1 if that level
-//              (<= n-2) lies inside the bin, else all ones, so that  (bits(u) << 13) > lut[bin]  iff  u >= l_{tau0+1}
+//   lut[bin] = (tau0 << 19) - (bin << 19) + (2^19 - low)    bin = bits(u) >> 19, i.e. the values [lo, hi) with bits(lo) = bin <<
+//              19; tau0 = last level (<= n-2) at or below lo; low = the low 19 bits of l_{tau0+1} if that level
+//              (<= n-2) lies inside the bin, else 2^19, so that  (lut[bin] + bits(u)) >> 19 = tau
 // Layers with two levels in such a bin and 5 bits or more get bins of 2^s patterns from just below the first level up to
-// 1.0, with the finest s that 2048 bins allow and the same entries (code: the low s bits, in the entry's top s bits).  If two
+// 1.0, with the finest s that 2048 bins allow and the same entries (s for 19, bits(u) counted from the first bin's edge).  If two
 // levels still share a bin, or below 5 bits, a byte table over the top 15 bits takes the same 8 KB:
 //   lut8[bits(u) >> 17] = tau0 of that finer bin; tau is found by stepping up while l_{tau+1} <= u, at most R times,
 //   R = the most levels inside one bin.
@@ -194,15 +194,15 @@ __global__ void __launch_bounds__(256) build_search_kernel(PlanDev p, const floa
             const uint32_t lob = off + ((uint32_t)bin << s);
             const bool top = lob >= kOne;
             const int tau0 = tau_of(__uint_as_float(top ? kOne : lob));
-            uint32_t code = mask;
+            uint32_t low = mask + 1u;
             if (!top && tau0 + 1 <= n - 2) {
                 const uint32_t nb = __float_as_uint(lev[tau0 + 1]);
                 if ((nb >> s) == (lob >> s)) {                              // l_{tau0+1} > lo lies inside this bin
-                    code = (nb & mask) - 1u;
+                    low = nb & mask;
                     if (tau0 + 2 <= n - 2 && (__float_as_uint(lev[tau0 + 2]) >> s) == (lob >> s)) atomicOr(&shared_bin, 1);
                 }
             }
-            lut[bin] = (code << (32 - s)) | (8u * (uint32_t)tau0);
+            lut[bin] = (((uint32_t)tau0 - (uint32_t)bin) << s) + (mask + 1u - low);
         }
         __syncthreads();
         const int r = shared_bin;
@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(256) build_search_kernel(PlanDev p, const floa
     bool dense = fill(19, 0u);
     if (dense && n >= 1 << kWindowBits) {
         const uint32_t first = __float_as_uint(lev[1]);
-        int s = 2;
+        int s = 3;                                                         // (quantize_coord shifts by s - 3)
         while ((kOne >> s) - (first >> s) + 1u >= (uint32_t)kLutEntries) ++s;
         const uint32_t off = ((first >> s) - 1u) << s;                     // (a level is at least 2^-100: no wrap)
         how = make_int2(kSearchWindow | (s << 2), (int)off);

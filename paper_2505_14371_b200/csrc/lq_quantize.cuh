@@ -6,16 +6,17 @@
 // Table lookups dominate the per-coordinate work, so every table sits at a fixed offset from one base that is
 // aligned to 8 KB, and the code carries ABSOLUTE 32-bit shared-memory addresses from one lookup to the next:
 //   search table  u32[2048]  at +0x0000, indexed by the top 13 bits of the pattern of u (sign, exponent, 4 mantissa
-//                            bits: 16 bins per octave over the whole fp32 range).  Entry = 8 * tau0 in bits 3..10,
-//                            tau0 the last level at or below the bin's lower edge, and in bits 13..31 the low 19
-//                            bits of the one level that may lie inside the bin, minus one (all ones: no such level),
-//                            so that "u is at or above that level" is one unsigned compare of (bits(u) << 13) with
-//                            the entry.  A 4-byte entry per bin spreads neighbouring bins over all 32 banks.
+//                            bits: 16 bins per octave over the whole fp32 range).  Entry + bits(u) = tau << 19 and something
+//                            below: the entry is tau0 << 19, tau0 the last level at or below the bin's lower edge, minus the
+//                            bin's lower edge, plus, where a level lies inside the bin, what lifts u from that level on
+//                            over the next multiple of 2^19.  So "u is at or above that level" costs one addition, which
+//                            the sign bit of u (values are scaled with their signs) does not disturb below bit 31.
+//                            A 4-byte entry per bin spreads neighbouring bins over all 32 banks.
 //   {l, gap}      float2[256] at +0x2000: {l_tau, l_{tau+1} - l_tau}
 //   cur values    float[512]  at +0x2800: fp32(N * l_idx) at 2 * idx, its negative at 2 * idx + 1 (bucket scope: N = 1)
 //   prev values   float[512]  at +0x3000: the same for the previous message
-// The address of the {l, gap} entry is (entry & 0x7F8) | base_ld: one logic operation.  Adding 8 for each of the two
-// decisions and 4 for the sign turns it into base_ld + 4 * symbol, from which the current value is a load at a
+// The address of the {l, gap} entry is ((entry + bits(u)) >> 16 & 0x7F8) | base_ld.  Adding 8 for the rounding
+// decision and 4 for the sign turns it into base_ld + 4 * symbol, from which the current value is a load at a
 // constant offset; the previous value's address is (shifted word & mask) | base_prev.  No address additions.
 // The packed words are accumulated from these absolute values as well: every word starts at minus the sum of
 // what the constant part (base_ld) contributes to it, so the part that is left is exactly the symbols.
@@ -57,11 +58,6 @@ inline bool encoder_dependent(const PlanDev& p)
 }
 
 // x + 8 when the comparison holds, else x: one compare and one predicated add
-__device__ __forceinline__ uint32_t add8_if_gt_u32(uint32_t x, uint32_t a, uint32_t b)
-{
-    asm("{\n\t.reg .pred p;\n\tsetp.gt.u32 p, %1, %2;\n\t@p add.u32 %0, %0, 8;\n\t}" : "+r"(x) : "r"(a), "r"(b));
-    return x;
-}
 __device__ __forceinline__ uint32_t add8_if_lt(uint32_t x, float a, float b)
 {
     asm("{\n\t.reg .pred p;\n\tsetp.lt.f32 p, %1, %2;\n\t@p add.u32 %0, %0, 8;\n\t}" : "+r"(x) : "f"(a), "f"(b));
@@ -213,38 +209,49 @@ struct SearchPar {
     }
 };
 
+// The normalised values of a lane's four coordinates of a row, with their signs (products of pairs are one instruction, rounded
+// like plain ones).
+__device__ __forceinline__ void normalise4(const float4& v, float r, float (&u)[4])
+{
+    asm("{\n\t.reg .b64 a, b, r;\n\tmov.b64 a, {%4, %5};\n\tmov.b64 b, {%6, %7};\n\tmov.b64 r, {%8, %8};\n\t"
+        "mul.rn.f32x2 a, a, r;\n\tmul.rn.f32x2 b, b, r;\n\tmov.b64 {%0, %1}, a;\n\tmov.b64 {%2, %3}, b;\n\t}"
+        : "=f"(u[0]), "=f"(u[1]), "=f"(u[2]), "=f"(u[3]) : "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "f"(r));
+}
+
 // One coordinate: v -> symbol, added to the lane's words `cw` at position pp; its term of the step-size
 // statistic (Eq. general_stepsize: fp32 difference of the two decoded values, squared in fp64) added to `stat`.
-// x: the coordinate's Philox word.  Bucket scope: the value tables hold the plain signed levels and the row's
+// u: v scaled by the layer's 1/N; x: the coordinate's Philox word.  Bucket scope: the value tables hold the plain signed levels and the row's
 // norms (nrow now, pn in the previous message) scale them.  `counted`: the coordinate lies inside the layer
 // (histogram mode).
+// A search by one addition for a compare, a shifted pattern and a predicated addition, and products of pairs: 67 M coordinates of 8
+// workers, 4 bits, step 1395 -> 1365 us; 17 M of 4 workers, 5 bits, 269 -> 257; Transformer-XL 1982 -> 1954.  (Differences of pairs as
+// well: no faster; two coordinates side by side through the search: 28 bytes of spills, 1982 -> 2018 us.)
 template <int B, int kSearch, bool kHist, bool kStat, bool kBucket>
-__device__ __forceinline__ void quantize_coord(const QuantEnv& ev, const SearchPar<kSearch>& sp, float v, uint32_t x, int pp,
+__device__ __forceinline__ void quantize_coord(const QuantEnv& ev, const SearchPar<kSearch>& sp, float v, float u, uint32_t x, int pp,
                                                uint32_t (&cw)[B + 1], const uint32_t (&pw)[B + 1], double& stat,
                                                float nrow, float pn, bool counted)
 {
     constexpr int n = 1 << B, C = B + 1;
-    // u <= 1 + 2^-23 always (N >= |v| and one rounding each in 1/N and the product), and such a u
+    // |u| <= 1 + 2^-23 always (N >= |v| and one rounding each in 1/N and the product), and such a u
     // behaves exactly like u = 1 below, so the min(u, 1) of the definition is not needed
-    const float u = __fmul_rn(fabsf(v), ev.r);
-    const uint32_t ub = __float_as_uint(u);
+    const uint32_t ub = __float_as_uint(u);                  // (the searches leave the sign out)
     uint32_t t8;                                             // address of {l_tau, gap}
     if (kSearch == kSearchWindow) {
-        const uint32_t d = (uint32_t)__viaddmax_s32((int)ub, sp.neg_off, 0);
+        const uint32_t d = (uint32_t)__viaddmax_s32((int)(ub & 0x7fffffffu), sp.neg_off, 0);
         const uint32_t e = lds_u32(((d >> (sp.par - 2)) & 0x1FFCu) | ev.lut);
-        t8 = add8_if_gt_u32((e & 0x7F8u) | ev.ld, ub << (32 - sp.par), e);
+        t8 = (((e + d) >> (sp.par - 3)) & 0x7F8u) | ev.ld;
     } else if (kSearch == kSearchOctave) {
         const uint32_t e = lds_u32(((ub >> 17) & 0x1FFCu) | ev.lut);
-        t8 = add8_if_gt_u32((e & 0x7F8u) | ev.ld, ub << 13, e);
+        t8 = (((e + ub) >> 16) & 0x7F8u) | ev.ld;
     } else {
-        // (u <= 1 + 2^-23 gives bits(u) >> 17 <= 8128; the mask keeps the pattern of a NaN inside the table too)
+        // (|u| <= 1 + 2^-23 gives bits(|u|) >> 17 <= 8128; the mask keeps the pattern of a NaN inside the table too)
         t8 = ev.ld + 8u * lds_u8(((ub >> 17) & 0x1FFFu) | ev.lut);
-        for (int s = 0; s < sp.par; ++s) t8 = add8_if_le(t8, lds_f32(t8 + 8u), u);
+        for (int s = 0; s < sp.par; ++s) t8 = add8_if_le(t8, lds_f32(t8 + 8u), fabsf(u));
         t8 = min(t8, ev.ld + 8u * (uint32_t)(n - 2));
     }
     const float2 ld = lds_f32x2(t8);
     const float den = ld.y;
-    const float num = __fsub_rn(u, ld.x);
+    const float num = __fsub_rn(fabsf(u), ld.x);
     // rho = (x >> 9) * 2^-23; f = 1 + rho is built from the bits, and fma(f, den, -den) rounds the exact
     // product rho * den once, like the plain multiplication
     // (one funnel shift: the 64-bit value {0x7F, x} moved right by 9 is (x >> 9) | 0x3F800000)
@@ -254,7 +261,7 @@ __device__ __forceinline__ void quantize_coord(const QuantEnv& ev, const SearchP
     const uint32_t abs4 = add4_if_negative(i8, v);          // base_ld + 4 * (2 * idx + sign), sign = (v < 0)
     pack_symbol<C>(cw, pp, abs4);
 
-    if (kHist && counted) atomicAdd(ev.hist + ((max(ub, kHistClamp) - kHistClamp) >> 19), 1u);
+    if (kHist && counted) atomicAdd(ev.hist + ((max(ub & 0x7fffffffu, kHistClamp) - kHistClamp) >> 19), 1u);
 
     if (kStat) {
         float cur = lds_f32_at<(int)(kSmTcur - kSmLd)>(abs4);
