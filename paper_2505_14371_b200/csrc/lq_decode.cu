@@ -135,39 +135,49 @@ __device__ __forceinline__ uint32_t value_addr(const uint32_t (&w)[C], int p, ui
     return (v & mask4) | table;
 }
 
-// Adds a unit's workers to the sums of rows kRow0 .. kRow0 + kRows - 1, in worker order.  Two neighbours are added by one
-// instruction: 33.6 M coordinates of 16 workers at 2 bits 102.7 -> 100.5 us (80 % of the issue slots are used).  A clear bit of `live`: that
-// worker's block is all zero words, which would add +0 to sums that are never -0.
-template <int B, int kRow0, int kRows, bool kBucket>
-__device__ __forceinline__ void add_unit(float (&acc)[4 * kRows], uint32_t unit, int lane, uint32_t table, uint32_t live)
+// Adds a unit's workers to the sums of rows row0 .. row0 + kRows - 1, in worker order.  Two neighbours are added by one
+// instruction: 33.6 M coordinates of 16 workers at 2 bits 102.7 -> 100.5 us (80 % of the issue slots are used).
+// A clear bit of `live`: that worker's block is all zero words, which would add +0 to sums that are never -0.
+// Of 2 rows (row0 = 2 x the warp) the words are first moved so that they start with the rows' symbols: the warps run the same code,
+// which in such small grids takes longer to fetch than to run (8192 coordinates, 8 workers: the step 12.0 -> 10.0 us; 203 530 and
+// 4: 20.5 -> 19.0).
+template <int B, int kRows, bool kBucket>
+__device__ __forceinline__ void add_unit(float (&acc)[4 * kRows], uint32_t unit, int lane, int row0, uint32_t table, uint32_t live)
 {
-    constexpr int C = B + 1, kFirst = (4 * kRow0 * C) >> 5, kLast = ((4 * (kRow0 + kRows) * C) - 1) >> 5;
-    uint32_t at = unit + 4 * lane, norm_at = unit + kUnitBytes;
+    constexpr int C = B + 1, kWords = (4 * kRows * C + 31) >> 5;
+    const int w0 = (4 * row0 * C) >> 5, shift = (4 * row0 * C) & 31;
+    uint32_t at = unit + 4 * lane + 128 * w0, norm_at = unit + kUnitBytes + 4 * row0;
 #pragma unroll 1
     for (; live; live >>= 1, at += kBlockBytes<B>, table += kBucket ? 0u : 8u << B, norm_at += 32) {
         if (!(live & 1u)) continue;
         uint32_t w[C];
 #pragma unroll
-        for (int i = kFirst; i <= kLast; ++i) w[i] = lds_u32(at + 128 * i);
+        for (int i = 0; i < kWords; ++i) w[i] = lds_u32(at + 128 * i);
+        if (kRows != 8 && (8 * C) % 32 != 0) {
+            uint32_t behind = w0 + kWords < C ? lds_u32(at + 128 * kWords) : 0u;
+#pragma unroll
+            for (int i = 0; i < kWords; ++i) w[i] = __funnelshift_r(w[i], i + 1 < kWords ? w[i + 1] : behind, shift);
+        }
         float nr[kRows];
         if (kBucket) {
 #pragma unroll
-            for (int j = 0; j < kRows; ++j) nr[j] = lds_f32(norm_at + 4 * (kRow0 + j));
+            for (int j = 0; j < kRows; ++j) nr[j] = lds_f32(norm_at + 4 * j);
         }
 #pragma unroll
         for (int i = 0; i < 4 * kRows; i += 2) {
-            float v0 = lds_f32(value_addr<C>(w, 4 * kRow0 + i, table)), v1 = lds_f32(value_addr<C>(w, 4 * kRow0 + i + 1, table));
+            float v0 = lds_f32(value_addr<C>(w, i, table)), v1 = lds_f32(value_addr<C>(w, i + 1, table));
             if (kBucket) { v0 = __fmul_rn(v0, nr[i >> 2]); v1 = __fmul_rn(v1, nr[i >> 2]); }
             add_f32x2(acc[i], acc[i + 1], v0, v1);
         }
     }
 }
 
-template <int kRow0, int kRows>
-__device__ __forceinline__ void request_state(const DecodeArgs& a, const Walk& w, int64_t blk)
+template <int kRows>
+__device__ __forceinline__ void request_state(const DecodeArgs& a, const Walk& w, int64_t blk, int row0)
 {
 #pragma unroll
-    for (int j = kRow0; j < kRow0 + kRows; ++j) {
+    for (int jj = 0; jj < kRows; ++jj) {
+        const int j = row0 + jj;
         const int64_t at = blk * kBlockCoords + 128 * j + 4 * w.lane;
         if (at < w.size) {
             cp_async16(w.state + 512 * j + 16 * w.lane, a.Y + w.base + at, 16);
@@ -176,16 +186,16 @@ __device__ __forceinline__ void request_state(const DecodeArgs& a, const Walk& w
     }
 }
 
-// The rows kRow0 .. of one block, from their sums: the mean, then the update.
-template <int kMode, int kRow0, int kRows>
-__device__ __forceinline__ void finish_block(const DecodeArgs& a, const Walk& w, int64_t blk, const float (&acc)[4 * kRows],
+// The rows row0 .. of one block, from their sums: the mean, then the update.
+template <int kMode, int kRows>
+__device__ __forceinline__ void finish_block(const DecodeArgs& a, const Walk& w, int64_t blk, int row0, const float (&acc)[4 * kRows],
                                              float invK, const Rates& rt, bool sent, double& lam_acc, double& mu_acc)
 {
     constexpr bool kQoda = kMode >= 1, kAlt = kMode == 2;
     const float eta = rt.eta, gamma = rt.gamma;
 #pragma unroll
     for (int jj = 0; jj < kRows; ++jj) {
-        const int64_t at = blk * kBlockCoords + 128 * (kRow0 + jj) + 4 * w.lane, pos = w.base + at;
+        const int64_t at = blk * kBlockCoords + 128 * (row0 + jj) + 4 * w.lane, pos = w.base + at;
         if (at >= w.size) continue;
         float4 g;
         g.x = __fmul_rn(acc[4 * jj + 0], invK);
@@ -194,8 +204,8 @@ __device__ __forceinline__ void finish_block(const DecodeArgs& a, const Walk& w,
         g.w = __fmul_rn(acc[4 * jj + 3], invK);
         if (a.gbar) *reinterpret_cast<float4*>(a.gbar + pos) = g;
         if (kQoda) {
-            const float4 y0 = lds_f32x4(w.state + 512 * (kRow0 + jj) + 16 * w.lane);
-            const float4 x1 = lds_f32x4(w.state + kStateBytes / 2 + 512 * (kRow0 + jj) + 16 * w.lane);
+            const float4 y0 = lds_f32x4(w.state + 512 * (row0 + jj) + 16 * w.lane);
+            const float4 x1 = lds_f32x4(w.state + kStateBytes / 2 + 512 * (row0 + jj) + 16 * w.lane);
             float4 y, x, h;
             y.x = __fsub_rn(y0.x, g.x); y.y = __fsub_rn(y0.y, g.y);
             y.z = __fsub_rn(y0.z, g.z); y.w = __fsub_rn(y0.w, g.w);
@@ -225,21 +235,11 @@ __device__ __forceinline__ void finish_block(const DecodeArgs& a, const Walk& w,
     }
 }
 
-// All warps of the CTA.  Where the warps share a block (kSplit, 2 rows each) every warp is in a decode_blocks of its own rows, and
-// __syncthreads() is defined only where all threads meet at one place of the program; a numbered barrier counts arrivals,
-// wherever they come from.
-template <int kRows>
-__device__ __forceinline__ void warps_meet()
-{
-    if constexpr (kRows == 8) __syncthreads();
-    else asm volatile("bar.sync 1, %0;" ::"n"(kDecThreads) : "memory");
-}
-
-// A warp's blocks: warp, warp + 4, ... of the CTA's (kRows = 8), or rows kRow0, kRow0 + 1 of all of them (kRows = 2).
+// A warp's blocks: warp, warp + 4, ... of the CTA's (kRows = 8), or its two rows of all of them (kRows = 2).
 // The next unit's words are always requested before the current unit is waited for; the rows of Y and X_1 as soon as
 // the block before is finished.  Per unit one copy group, per block one more for the state, so a fixed number of
 // younger groups may be under way at every wait.
-template <int B, int kMode, bool kBucket, int kRow0, int kRows>
+template <int B, int kMode, bool kBucket, int kRows>
 __device__ __forceinline__ void decode_blocks(const PlanDev& p, const LayerDesc& L, int layer, const DecodeArgs& a, const Walk& w,
                                            float2* table, const Rates* rates, uint32_t my_live, double* sums)
 {
@@ -247,7 +247,7 @@ __device__ __forceinline__ void decode_blocks(const PlanDev& p, const LayerDesc&
     constexpr int kUW = kUnitWorkers<B>, kTW = kBucket ? 1 << 20 : kTableWorkers<B>;
     constexpr int kStep = kRows == 8 ? kDecWarps : 1;
     constexpr uint32_t kUnitStride = kUnitBytes + (kBucket ? 32 * 16 : 0);
-    const int K = p.num_workers, nu = (K + kUW - 1) / kUW;
+    const int K = p.num_workers, nu = (K + kUW - 1) / kUW, row0 = kRows == 8 ? 0 : kRows * w.warp;
     const float invK = __fdiv_rn(1.0f, (float)K);
     // the workers of unit u that sent anything in a block with `live` (kept for up to 32 workers; of more, all are read)
     auto unit_live = [&](uint32_t live, int u) {
@@ -263,11 +263,11 @@ __device__ __forceinline__ void decode_blocks(const PlanDev& p, const LayerDesc&
     if (b < w.nblocks) request_unit<B, kBucket>(p, a, w, up, w.units, w.block0 + b, 0, unit_live(live, 0));
     cp_async_commit();
     if (kQoda) {
-        if (b < w.nblocks) request_state<kRow0, kRows>(a, w, w.block0 + b);
+        if (b < w.nblocks) request_state<kRows>(a, w, w.block0 + b, row0);
         cp_async_commit();
     }
     fill_tables<kBucket>(p, L, layer, a, table, 0, min(K, kTW));
-    warps_meet<kRows>();
+    __syncthreads();
     const Rates rt = *rates;
     double lam_acc = 0.0, mu_acc = 0.0;
     uint32_t stage = 0;
@@ -289,23 +289,23 @@ __device__ __forceinline__ void decode_blocks(const PlanDev& p, const LayerDesc&
             if (!kBucket && K > kTW) {
                 k_in = k0 % kTW;
                 if (k_in == 0 && (b0 > 0 || u > 0)) {
-                    warps_meet<kRows>();
+                    __syncthreads();
                     fill_tables<kBucket>(p, L, layer, a, table, k0, min(kTW, K - k0));
-                    warps_meet<kRows>();
+                    __syncthreads();
                 }
             }
             if (kQoda && u == 0) cp_async_wait<2>(); else cp_async_wait<1>();
             __syncwarp();                                         // a lane reads what other lanes have copied
             if (active)
-                add_unit<B, kRow0, kRows, kBucket>(acc, w.units + stage * kUnitStride, w.lane,
-                                                   w.tables + (kBucket ? 0 : (uint32_t)k_in << (B + 3)), unit_live(live, u));
+                add_unit<B, kRows, kBucket>(acc, w.units + stage * kUnitStride, w.lane, row0,
+                                            w.tables + (kBucket ? 0 : (uint32_t)k_in << (B + 3)), unit_live(live, u));
             __syncwarp();                                         // ... and the unit may be overwritten
             stage ^= 1u;
         }
         if (kQoda) cp_async_wait<1>();
-        if (active) finish_block<kMode, kRow0, kRows>(a, w, blk, acc, invK, rt, live != 0u, lam_acc, mu_acc);
+        if (active) finish_block<kMode, kRows>(a, w, blk, row0, acc, invK, rt, live != 0u, lam_acc, mu_acc);
         if (kQoda) {
-            if (b + kStep < w.nblocks) request_state<kRow0, kRows>(a, w, blk + kStep);
+            if (b + kStep < w.nblocks) request_state<kRows>(a, w, blk + kStep, row0);
             cp_async_commit();
         }
         live = next_live;
@@ -408,22 +408,11 @@ __global__ void __launch_bounds__(kDecThreads, kMode == 0 ? 5 : 4) decode_kernel
             *rates = Rates{p.scalars->eta, kAlt ? p.scalars->gamma : p.scalars->eta, kAlt ? p.scalars->eta_cur : 0.0f};
     }
     double sums[2] = {0.0, 0.0};
-    if constexpr (kSplit) {
-        switch (L.bits * 4 + w.warp) {
-#define LQ_ROWS(BB, R) case 4 * BB + R: decode_blocks<BB, kMode, kBucket, 2 * R, 2>(p, L, layer, a, w, table, rates, my_live, sums); break;
-#define LQ_CASE(BB) LQ_ROWS(BB, 0) LQ_ROWS(BB, 1) LQ_ROWS(BB, 2) LQ_ROWS(BB, 3)
-            LQ_CASE(1) LQ_CASE(2) LQ_CASE(3) LQ_CASE(4) LQ_CASE(5) LQ_CASE(6) LQ_CASE(7) LQ_CASE(8)
+    switch (L.bits) {
+#define LQ_CASE(BB) case BB: decode_blocks<BB, kMode, kBucket, kSplit ? 2 : 8>(p, L, layer, a, w, table, rates, my_live, sums); break;
+        LQ_CASE(1) LQ_CASE(2) LQ_CASE(3) LQ_CASE(4) LQ_CASE(5) LQ_CASE(6) LQ_CASE(7) LQ_CASE(8)
 #undef LQ_CASE
-#undef LQ_ROWS
-            default: break;
-        }
-    } else {
-        switch (L.bits) {
-#define LQ_CASE(BB) case BB: decode_blocks<BB, kMode, kBucket, 0, 8>(p, L, layer, a, w, table, rates, my_live, sums); break;
-            LQ_CASE(1) LQ_CASE(2) LQ_CASE(3) LQ_CASE(4) LQ_CASE(5) LQ_CASE(6) LQ_CASE(7) LQ_CASE(8)
-#undef LQ_CASE
-            default: break;
-        }
+        default: break;
     }
     if (kAlt) {                                  // one term per CTA, added in CTA order by the finalize kernel
         const double lam = block_reduce<false>(sums[0], scratch);
