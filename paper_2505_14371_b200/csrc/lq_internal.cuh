@@ -190,6 +190,20 @@ cudaError_t opt_in_shared_memory(std::atomic<uint64_t>& configured, int bytes, K
     return e;
 }
 
+// Clusters of up to 16 CTAs: likewise.
+template <typename... Kernels>
+cudaError_t allow_clusters(std::atomic<uint64_t>& configured, Kernels... kernels)
+{
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const bool known = dev >= 0 && dev < 64;
+    if (known && ((configured.load(std::memory_order_relaxed) >> dev) & 1u)) return cudaSuccess;
+    cudaError_t e = cudaSuccess;
+    ((e = e == cudaSuccess ? cudaFuncSetAttribute(kernels, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : e), ...);
+    if (e == cudaSuccess && known) configured.fetch_or(1ull << dev, std::memory_order_relaxed);
+    return e;
+}
+
 // ---- launchers (each enqueues on `s` and returns the launch status) ----
 // `write_mask`: also record the zero-row masks of `grads` in p.row_mask
 cudaError_t launch_norm_partial(const PlanDev& p, const float* grads, bool write_mask, cudaStream_t s);

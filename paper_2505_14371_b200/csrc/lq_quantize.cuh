@@ -109,6 +109,18 @@ __device__ __forceinline__ void pack_begin(uint32_t (&w)[C], uint32_t base_ld)
         w[i] = 0u - (a2 * m + (cs ? (a2 >> cs) : 0u));
     }
 }
+// The same for a string's first four symbols alone.
+template <int C>
+__device__ __forceinline__ void pack_first_row(uint32_t (&w)[C], uint32_t base_ld)
+{
+    const uint32_t a2 = base_ld >> 2;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const int off = e * C, i = off >> 5, s = off & 31;
+        w[i] -= a2 << s;
+        if (s + C > 32) w[i + 1] -= a2 >> (32 - s);
+    }
+}
 // Adds symbol p given as base_ld + 4 * symbol.
 template <int C>
 __device__ __forceinline__ void pack_symbol(uint32_t (&w)[C], int p, uint32_t abs4)

@@ -1,22 +1,28 @@
-// ENCODE in the layer norm scope for plans whose layers are all small: one cluster of up to 8 CTAs takes a whole (layer,
+// ENCODE in the layer norm scope for plans whose layers are all small: one cluster of up to 16 CTAs takes a whole (layer,
 // worker), so the norm, which every coordinate of the layer needs before its first symbol, is exchanged inside the
 // cluster (distributed shared memory, a cluster barrier) instead of through kernel boundaries: one launch where the
 // general path has four (norm partials, norms, encoder, statistic).  Such plans are a chain of launches of a few us each,
-// with nothing to fill the GPU, so latency is what bounds them.
+// with nothing to fill the GPU, so latency is what bounds them, and more than that of sums and look-ups the latency of fetching
+// code: warp j of a CTA takes row j of each of its blocks, and all warps run the same code.
 //
-// The rule (use_small): every layer has at most 256 blocks of 1024 coordinates (8 CTAs of 32), and the clusters of all
-// layers and all of the plan's workers run at once: 3 CTAs per SM, or for whole clusters, which have to fit an SM group
-// each, 352 CTAs.  It asks for nothing but the plan's constants: a worker range does not change which kernel encodes a
-// layer, nor the order in which the layer's sums are formed.  A cluster has as many CTAs as its plan's largest layer needs
-// for one block per warp; the values are read twice, the second time from L2.
-// lq_quantize_pack at 3 bits and 4 workers, this kernel and the general path: layers of one block 18.9 and 25.0 us at 444
-// CTAs, 34.8 and 26.9 at 592; of 64 blocks 27.5 and 38.9 at 352 CTAs, 46.7 and 40.1 at 416; of 256 blocks 52.0 and 60.6 at
-// 352, 75.7 and 65.7 at 416 (there the second wave waits for whole clusters).
-#include "lq_quantize_tile.cuh"
+// The rule (use_small): layers of up to 8 blocks of 1024 coordinates, a CTA each, always; larger ones, of up to 256 blocks, while
+// the clusters are not too many: 1280 CTAs of up to 8 blocks each, 352 of more, and of more than 24 where there are 2600 blocks
+// of all workers or more (those chains of rows are longer than the general path's launches otherwise).  It asks for nothing but the plan's constants: a
+// worker range does not change which kernel encodes a layer, nor the order in which the layer's sums are formed.
+// The step in us, this kernel and the general path.  One CTA a layer: layers of one block, 320 (layer, worker) pairs 11 and 36, 2400 of them
+// 38 and 104, 9600 128 and 387; of 1 to 8 blocks, 2400 pairs 58 and 108, 4896 111 and 224.  Clusters of up to 8 blocks a CTA: 640 CTAs
+// 28 and 42, 1280 of them 52 and 55 or, most with one block or none, 31 and 38, 1920 57 and 58, 2560 95 and 83.  Of more: 256
+// CTAs of 29 blocks 46 and 52, 288 of 24 27 and 31, 576 34 and 33, 512 of 29 85 and 77; 288 of 32 in 2300 blocks 34 and 30, 192
+// of 32 in 4000 35 and 44.
+#include "lq_quantize.cuh"
 
 namespace lq {
 
 namespace {
+
+constexpr int kMostRanks = 16, kMostShare = 32;              // CTAs of a cluster (more than 8 have to be asked for); blocks of a CTA
+// room for the words of a CTA's blocks
+__host__ __device__ constexpr int kSmallWords(int blocks, int C) { return blocks * C * 32; }
 
 // ---- cluster exchange
 __device__ __forceinline__ void st_peer(const double* mine, uint32_t rank, double v)
@@ -28,15 +34,43 @@ __device__ __forceinline__ void st_peer(const double* mine, uint32_t rank, doubl
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 
-template <int kMode>
-__device__ __forceinline__ double norm_of_blocks(const PlanDev& p, const float* g, int64_t size, int block0, int nblocks,
-                                                 uint8_t* rows, double* scratch)
+// This lane's four values of row j of block blk (fresh() pointer), zeros behind the layer's end.
+__device__ __forceinline__ float4 row_values(const float* g, int64_t blk, int j, int64_t size, int lane)
 {
+    const int64_t pos = blk * kBlockCoords + 128 * j + 4 * lane;
+    if (pos + 4 <= size) return __ldcg(reinterpret_cast<const float4*>(g + pos));
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (pos < size) v.x = __ldcg(g + pos);
+    if (pos + 1 < size) v.y = __ldcg(g + pos + 1);
+    if (pos + 2 < size) v.z = __ldcg(g + pos + 2);
+    return v;
+}
+
+// Warp j takes row j of all of the CTA's blocks.  `rows` (zeroed): bit j of a block's word says whether its row j holds anything
+// but zeros.  `first`: the lane's values of the first block's row.
+template <int kMode>
+__device__ __forceinline__ double norm_of_rows(const PlanDev& p, const float* g, int64_t size, int block0, int nblocks,
+                                               uint32_t* rows, double* scratch, float4& first)
+{
+    const int lane = threadIdx.x & 31, j = threadIdx.x >> 5;
     double acc = 0.0;
     uint32_t maxbits = 0;
-    for (int b = threadIdx.x >> 5; b < nblocks; b += kQWarps) {
-        const uint32_t r = norm_block<kMode>(g, block0 + b, size, threadIdx.x & 31, p.q, acc, maxbits);
-        if ((threadIdx.x & 31) == 0) rows[b] = (uint8_t)r;
+    constexpr int kAhead = 4;
+    for (int b0 = 0; b0 < nblocks; b0 += kAhead) {
+        float4 v[kAhead];
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i)
+            v[i] = b0 + i < nblocks ? row_values(g, block0 + b0 + i, j, size, lane) : make_float4(0.f, 0.f, 0.f, 0.f);
+        if (b0 == 0) first = v[0];
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) {
+            accumulate<kMode>(acc, maxbits, v[i].x, p.q);
+            accumulate<kMode>(acc, maxbits, v[i].y, p.q);
+            accumulate<kMode>(acc, maxbits, v[i].z, p.q);
+            accumulate<kMode>(acc, maxbits, v[i].w, p.q);
+            const float mag = (fabsf(v[i].x) + fabsf(v[i].y)) + (fabsf(v[i].z) + fabsf(v[i].w));
+            if (__any_sync(0xffffffffu, mag != 0.0f) && lane == 0) atomicOr(rows + b0 + i, 1u << j);
+        }
     }
     return norm_cta_total<kMode>(acc, maxbits, scratch);
 }
@@ -53,12 +87,12 @@ __device__ __forceinline__ Tile cluster_share(const LayerDesc& L, int layer, int
 // The layer's norm from all CTAs of the cluster: each sends its sum to every other, and all add them in rank order.  What
 // is done between the two calls overlaps the exchange.  (The caller has arrived at the cluster's barrier once before.)
 __device__ __forceinline__ void cluster_norm_send(const PlanDev& p, const float* g, const LayerDesc& L, const Tile& t, int rank,
-                                                  int ranks, uint8_t* rows, double* scratch, double* part)
+                                                  int ranks, uint32_t* rows, double* scratch, double* part, float4& first)
 {
-    const double mine = p.q == 0   ? norm_of_blocks<0>(p, g, L.size, t.block0, t.nblocks, rows, scratch)
-                        : p.q == 1 ? norm_of_blocks<1>(p, g, L.size, t.block0, t.nblocks, rows, scratch)
-                        : p.q == 2 ? norm_of_blocks<2>(p, g, L.size, t.block0, t.nblocks, rows, scratch)
-                                   : norm_of_blocks<3>(p, g, L.size, t.block0, t.nblocks, rows, scratch);
+    const double mine = p.q == 0   ? norm_of_rows<0>(p, g, L.size, t.block0, t.nblocks, rows, scratch, first)
+                        : p.q == 1 ? norm_of_rows<1>(p, g, L.size, t.block0, t.nblocks, rows, scratch, first)
+                        : p.q == 2 ? norm_of_rows<2>(p, g, L.size, t.block0, t.nblocks, rows, scratch, first)
+                                   : norm_of_rows<3>(p, g, L.size, t.block0, t.nblocks, rows, scratch, first);
     cluster_wait();                                          // every CTA of the cluster runs
     if (threadIdx.x == 0)
         for (int r = 0; r < ranks; ++r) st_peer(&part[rank], r, mine);
@@ -84,17 +118,101 @@ __device__ __forceinline__ void store_norm(const PlanDev& p, const LayerNorm& n,
 // The norms alone, in the encoder's order (lq_layer_norms gives the very norms that lq_quantize_pack sends).
 __global__ void __launch_bounds__(kQThreads) layer_norms_small_kernel(PlanDev p, const float* grads, float* norms)
 {
-    __shared__ double part[8], scratch[kQWarps];
-    __shared__ uint8_t rows[32];                             // (8 CTAs for up to 256 blocks)
+    __shared__ double part[kMostRanks], scratch[kQWarps];
+    __shared__ uint32_t rows[kMostShare];                    // (not used)
+    float4 first;
     pdl_launch_next();
     const int ranks = gridDim.x, rank = blockIdx.x, layer = blockIdx.y, k = blockIdx.z + p.worker0;
     cluster_arrive();
     const LayerDesc L = p.layers[layer];
     const Tile t = cluster_share(L, layer, rank, ranks);
     pdl_wait();
-    cluster_norm_send(p, fresh(grads + (int64_t)blockIdx.z * p.padded_elems + L.elem_off), L, t, rank, ranks, rows, scratch, part);
+    cluster_norm_send(p, fresh(grads + (int64_t)blockIdx.z * p.padded_elems + L.elem_off), L, t, rank, ranks, rows, scratch, part, first);
     const LayerNorm n = cluster_norm_receive(p, ranks, part);
     if (rank == 0 && threadIdx.x == 0) store_norm(p, n, norms, (int64_t)k * p.num_layers + layer);
+}
+
+// What the warps of a CTA share about their blocks.
+struct SmallJob {
+    const float* g;              // first coordinate of the layer in this worker's row
+    const uint32_t* prev;        // the layer's words in the previous message, or NULL
+    int64_t size;                // d_m
+    int block0, nblocks;         // the CTA's blocks of the layer
+    const uint32_t* rows;        // per block: bits 0..7 its rows that hold anything, bits 8..15 those of the previous input
+    uint32_t words;              // shared-memory address of the blocks' words, zeroed
+    bool counts;                 // histogram mode, and the layer is not sent as zeros
+};
+
+// Row j of all of the CTA's blocks (of a layer's partial block, too: coordinates behind the layer's end are zeros and turn into
+// symbols 0), by warp j.  A row's four symbols a lane are 4 C bits of the lane's string: they are formed as the first four of a string,
+// moved into place and ORed into the block's words, and so with the previous message's, so that all rows run the same code:
+// fetching code that no warp has run yet is what takes longest here.  Steps of 8192 coordinates and 8 workers, and of a perceptron's
+// 203 530 and 4: a warp a block, 8 rows of it unrolled, 16.7 and 26.8 us; a row a warp, code of its own for each, 13.5 and 24.8; the
+// same code for all 12.0 and 20.5.  (Two blocks side by side: 0.6 us slower.)
+template <int B, int kSearch, bool kHist, bool kStat>
+__device__ __forceinline__ double quantize_rows(const PlanDev& p, const PhiloxConsts& pc, const SmallJob& job, const QuantEnv& ev, float4 first,
+                                                int lane, int j)
+{
+    constexpr int C = B + 1;
+    const SearchPar<kSearch> sp(ev);
+    const int w0 = (4 * C * j) >> 5, shift = (4 * C * j) & 31;
+    const bool two = shift + 4 * C > 32;                         // the row's bits reach into a second word
+    double stat = 0.0;
+    float4 next = first;
+    uint32_t pnext0, pnext1;
+    auto request_prev = [&](int b) {
+        const uint32_t* from = job.prev + (int64_t)(job.block0 + b) * (C * 32) + lane + 32 * w0;
+        pnext0 = kStat && job.prev ? __ldcg(from) : 0u;
+        pnext1 = kStat && job.prev && two ? __ldcg(from + 32) : 0u;
+    };
+    request_prev(0);
+#pragma unroll 1
+    for (int b = 0; b < job.nblocks; ++b) {
+        const float4 v = next;
+        uint32_t pw[C], cw[C];
+#pragma unroll
+        for (int i = 0; i < C; ++i) { pw[i] = 0u; cw[i] = 0u; }
+        pw[0] = __funnelshift_r(pnext0, pnext1, shift);
+        pw[1] = pnext1 >> shift;
+        if (b + 1 < job.nblocks) {
+            next = row_values(job.g, job.block0 + b + 1, j, job.size, lane);
+            request_prev(b + 1);
+        }
+        const uint32_t m = job.rows[b] >> j;
+        const int64_t pos = (int64_t)(job.block0 + b) * kBlockCoords + 128 * j;          // of the row
+        if (m & 1u) {
+            uint32_t x[4];
+            philox4x32_10_folded((uint32_t)((job.block0 + b) * 256 + 32 * j + lane), pc, p, x);
+            const float vv[4] = {v.x, v.y, v.z, v.w};
+            float u[4];
+            normalise4(v, ev.r, u);
+            pack_first_row<C>(cw, ev.ld);
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                quantize_coord<B, kSearch, kHist, kStat, false>(ev, sp, vv[e], u[e], x[e], e, cw, pw, stat, 0.f, 0.f, pos + 4 * lane + e < job.size);
+            const uint32_t at = job.words + 4u * (uint32_t)(b * (C * 32) + lane + 32 * w0);
+            asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(at), "r"(cw[0] << shift) : "memory");
+            if (two) asm volatile("red.shared.or.b32 [%0+128], %1;" ::"r"(at), "r"(__funnelshift_l(cw[0], cw[1], shift)) : "memory");
+        } else {
+            if (kStat && ((m >> 8) & 1u)) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) stat_prev_only<C, false>(ev, pw, e, 0.f, stat);
+            }
+            if (kHist && job.counts && lane == 0 && pos < job.size)       // its coordinates have u = 0
+                atomicAdd(ev.hist, (uint32_t)min((int64_t)128, job.size - pos));
+        }
+    }
+    return stat;
+}
+
+template <int B, bool kHist, bool kStat>
+__device__ __forceinline__ double quantize_rows_by(const PlanDev& p, const PhiloxConsts& pc, const SmallJob& job, const QuantEnv& ev, int search,
+                                                   float4 first, int lane, int j)
+{
+    if (search == kSearchOctave) return quantize_rows<B, kSearchOctave, kHist, kStat>(p, pc, job, ev, first, lane, j);
+    if constexpr (B >= kWindowBits)
+        if (search == kSearchWindow) return quantize_rows<B, kSearchWindow, kHist, kStat>(p, pc, job, ev, first, lane, j);
+    return quantize_rows<B, kSearchStep, kHist, kStat>(p, pc, job, ev, first, lane, j);
 }
 
 template <bool kHist, bool kStat>
@@ -103,7 +221,8 @@ __global__ void __launch_bounds__(kQThreads, 3) quantize_small_kernel(
     const uint32_t* prev_packed, const float* prev_norms, const float* levels_cur, const float* levels_prev, SearchTables st)
 {
     extern __shared__ unsigned char dyn_smem[];
-    __shared__ double norm_part[8], stat_part[8];             // per CTA of the cluster
+    __shared__ double norm_part[kMostRanks], stat_part[kMostRanks];             // per CTA of the cluster
+    __shared__ uint32_t rows[kMostShare];
     uint32_t base;
     unsigned char* sm = table_base(dyn_smem, base);
     pdl_launch_next();
@@ -112,8 +231,15 @@ __global__ void __launch_bounds__(kQThreads, 3) quantize_small_kernel(
     cluster_arrive();                                         // (waited for before the first store into a peer)
     const LayerDesc L = p.layers[layer];
     const Tile tile = cluster_share(L, layer, rank, ranks);
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, C = L.bits + 1;
     const int64_t kl = (int64_t)k * p.num_layers + layer;
+    uint32_t* words = reinterpret_cast<uint32_t*>(sm + kSmRing);                // the blocks' words, behind them the histogram
+    uint32_t* counts = words + kSmallWords(tile.nblocks, C);
+    if (threadIdx.x < tile.nblocks) rows[threadIdx.x] = 0u;
+    for (int i = threadIdx.x; i < tile.nblocks * C * 32; i += kQThreads) words[i] = 0u;
+    if (kHist)
+        for (int i = threadIdx.x; i < LQ_HIST_STRIDE; i += kQThreads) counts[i] = 0u;
+    __syncthreads();
     pdl_wait();
     const float* g = fresh(grads + (int64_t)blockIdx.z * p.padded_elems + L.elem_off);
     if (rank == 0 && layer == 0 && blockIdx.z == 0 && threadIdx.x == 0) p.scalars[1] = p.scalars[0];
@@ -134,18 +260,13 @@ __global__ void __launch_bounds__(kQThreads, 3) quantize_small_kernel(
         lp = load_f32(levels_prev + (int64_t)layer * kLevelStride + threadIdx.x);
         lg = load_f32x2(st.ld + (int64_t)layer * kMaxLevels + threadIdx.x);
     }
-    uint8_t* rows_cur = sm + kSmRows;
-    uint8_t* rows_prev = rows_cur + kTileBlocks;
     double* scratch = reinterpret_cast<double*>(sm + kSmScratch);
-    cluster_norm_send(p, g, L, tile, rank, ranks, rows_cur, scratch, norm_part);
+    float4 first;
+    cluster_norm_send(p, g, L, tile, rank, ranks, rows, scratch, norm_part, first);
     {
         uint4* ldst = reinterpret_cast<uint4*>(sm + kSmLut);
         ldst[threadIdx.x] = lut0;
         ldst[kQThreads + threadIdx.x] = lut1;
-        if (kHist) {
-            uint32_t* h = reinterpret_cast<uint32_t*>(sm + kSmHist);
-            for (int i = threadIdx.x; i < LQ_HIST_STRIDE; i += kQThreads) h[i] = 0;
-        }
     }
     const LayerNorm ln = cluster_norm_receive(p, ranks, norm_part);
     if (threadIdx.x < L.nlevels) {
@@ -155,35 +276,47 @@ __global__ void __launch_bounds__(kQThreads, 3) quantize_small_kernel(
         reinterpret_cast<float2*>(sm + kSmTprev)[threadIdx.x] = make_float2(pv, -pv);
     }
     if (threadIdx.x == 0) *reinterpret_cast<int2*>(sm + kSmHow) = how;
-    if (threadIdx.x < tile.nblocks) {
-        rows_prev[threadIdx.x] = (uint8_t)mprev;
-        p.row_mask[mask_at] = rows_cur[threadIdx.x];
+    if (threadIdx.x < tile.nblocks) {                        // (the rows' bits lie behind norm_cta_total's barriers)
+        const uint32_t live = rows[threadIdx.x];
+        p.row_mask[mask_at] = (uint8_t)live;
+        rows[threadIdx.x] = (ln.rnorm != 0.0f ? live : 0u) | (mprev << 8);        // a layer without a norm sends zeros
     }
     if (rank == 0 && threadIdx.x == 0) store_norm(p, ln, norms, kl);
     __syncthreads();
 
-    WarpCtx c;
-    c.g = g;
-    c.size = L.size;
-    c.nfull = L.size / kBlockCoords;
-    c.lane = lane;
+    SmallJob job;
+    job.g = g;
+    job.prev = prev_packed ? fresh(prev_packed + (int64_t)k * p.packed_words + L.word_off) : nullptr;
+    job.size = L.size;
+    job.block0 = tile.block0; job.nblocks = tile.nblocks;
+    job.rows = rows;
+    job.words = base + kSmRing;
+    job.counts = ln.rnorm != 0.0f;
     QuantEnv ev;
     ev.lut = base + kSmLut; ev.ld = base + kSmLd; ev.tprev = base + kSmTprev;
     ev.r = ln.rnorm;
-    ev.hist = reinterpret_cast<uint32_t*>(sm + kSmHist);
+    ev.hist = counts;
     if (step == LQ_STEP_AUTO) step = (uint32_t)p.scalars->t;      // the plan's own iteration counter (graph replays)
     const PhiloxConsts pc = philox_fold((uint32_t)layer, (uint32_t)k, step, p.seed_lo, p.seed_hi);
-    uint32_t* out = packed + (int64_t)k * p.packed_words + L.word_off;
-    const uint32_t* prev = prev_packed ? fresh(prev_packed + (int64_t)k * p.packed_words + L.word_off) : nullptr;
-    const double stat = quantize_blocks<0, kHist, kStat>(p, pc, c, tile, L.bits, how.x & 3, (uint32_t)layer, (uint32_t)k, step, out, prev, ev,
-                                                      rows_cur, rows_prev, base + kSmRing);
-    const double sum = block_reduce<false>(stat, scratch);
+    double stat = 0.0;
+    if (tile.nblocks > 0) {
+        switch (L.bits) {
+#define LQ_CASE(BB) case BB: stat = quantize_rows_by<BB, kHist, kStat>(p, pc, job, ev, how.x & 3, first, lane, (int)(threadIdx.x >> 5)); break;
+            LQ_CASE(1) LQ_CASE(2) LQ_CASE(3) LQ_CASE(4) LQ_CASE(5) LQ_CASE(6) LQ_CASE(7) LQ_CASE(8)
+#undef LQ_CASE
+            default: break;
+        }
+    }
+    const double sum = block_reduce<false>(kStat ? stat : 0.0, scratch);
     if (threadIdx.x == 0) st_peer(&stat_part[rank], 0, sum);
     cluster_arrive();
-    if (kHist) {                                             // (block_reduce's barriers lie behind the last count)
+    // (block_reduce's barriers lie behind the last word and the last count)
+    uint32_t* out = packed + (int64_t)k * p.packed_words + L.word_off + (int64_t)tile.block0 * (C * 32);
+    for (int i = threadIdx.x; i < tile.nblocks * C * 32; i += kQThreads) __stcs(out + i, words[i]);
+    if (kHist) {
         uint32_t* h = hist + kl * LQ_HIST_STRIDE;
         for (int i = threadIdx.x; i < LQ_NUM_BINS; i += blockDim.x)
-            if (ev.hist[i]) atomicAdd(h + i, ev.hist[i]);
+            if (counts[i]) atomicAdd(h + i, counts[i]);
     }
     cluster_wait();
     if (rank == 0 && threadIdx.x == 0) {
@@ -193,10 +326,14 @@ __global__ void __launch_bounds__(kQThreads, 3) quantize_small_kernel(
     }
 }
 
+// CTAs of a plan's clusters: as many as its largest layer needs for 8 blocks each, up to 8, and more, while there are blocks for
+// them and SMs (2 CTAs on each): 784 blocks of 203 530 coordinates and 4 workers on 8 CTAs each 27.7, on 16 20.5 us.
 int small_ranks(const PlanDev& p)
 {
+    const int64_t pairs = (int64_t)p.num_workers * p.num_layers;
     int r = 1;
     while (r < 8 && r * kQWarps < p.most_blocks) r *= 2;
+    while (r < kMostRanks && r < p.most_blocks && pairs * 2 * r <= 2 * kSms) r *= 2;
     return r;
 }
 
@@ -204,14 +341,19 @@ int small_ranks(const PlanDev& p)
 
 bool use_small(const PlanDev& p)
 {
+    if (p.global_norm || p.bucket_norm || p.most_blocks > 8 * kMostShare || p.num_layers > 65535) return false;      // (grid.y)
     const int ranks = small_ranks(p);
-    return !p.global_norm && !p.bucket_norm && p.most_blocks <= 256 &&
-           (int64_t)p.num_workers * p.num_layers * ranks <= (ranks == 1 ? 3 * kSms : 352);
+    const int64_t ctas = (int64_t)p.num_workers * p.num_layers * ranks;
+    if (p.most_blocks > 24 * ranks && p.num_workers * p.total_blocks < 2600) return false;
+    return ranks == 1 || ctas <= (p.most_blocks <= ranks * kQWarps ? 1280 : 352);
 }
 
 cudaError_t launch_layer_norms_small(const PlanDev& p, const float* grads, float* norms, cudaStream_t s)
 {
     const unsigned ranks = (unsigned)small_ranks(p);
+    static std::atomic<uint64_t> configured{0};
+    const cudaError_t e = allow_clusters(configured, layer_norms_small_kernel);
+    if (e != cudaSuccess) return e;
     return launch_cluster(layer_norms_small_kernel, dim3(ranks, (unsigned)p.num_layers, (unsigned)p.worker_count), kQThreads, 0, ranks,
                           s, p, grads, norms);
 }
@@ -221,17 +363,20 @@ cudaError_t launch_quantize_small(const PlanDev& p, const float* grads, uint32_t
                                   const float* levels_cur, const float* levels_prev, SearchTables t, bool need_stat, cudaStream_t s)
 {
     if (p.num_layers == 0) return cudaSuccess;
-    constexpr unsigned smem = kSmTables + kRingBytes + kSmSlack, smem_hist = smem + LQ_HIST_STRIDE * 4;
-    static std::atomic<uint64_t> configured{0};
-    const cudaError_t e = opt_in_shared_memory(configured, (int)smem_hist, quantize_small_kernel<true, true>,
-                                               quantize_small_kernel<false, true>, quantize_small_kernel<false, false>);
+    constexpr unsigned tables = kSmRing + kSmSlack, most = tables + kSmallWords(kMostShare, LQ_MAX_BITS + 1) * 4 + LQ_HIST_STRIDE * 4;
+    static std::atomic<uint64_t> configured{0}, clusters{0};
+    cudaError_t e = opt_in_shared_memory(configured, (int)most, quantize_small_kernel<true, true>,
+                                         quantize_small_kernel<false, true>, quantize_small_kernel<false, false>);
+    if (e == cudaSuccess)
+        e = allow_clusters(clusters, quantize_small_kernel<true, true>, quantize_small_kernel<false, true>, quantize_small_kernel<false, false>);
     if (e != cudaSuccess) return e;
     const auto kernel = hist ? quantize_small_kernel<true, true>
                         : need_stat ? quantize_small_kernel<false, true> : quantize_small_kernel<false, false>;
     const unsigned ranks = (unsigned)small_ranks(p);
-    return launch_cluster(kernel, dim3(ranks, (unsigned)p.num_layers, (unsigned)p.worker_count), kQThreads,
-                          hist ? smem_hist : smem, ranks, s, p, grads, step, packed, norms, hist, prev_packed, prev_norms,
-                          levels_cur, levels_prev, t);
+    const int share = (p.most_blocks + (int)ranks - 1) / (int)ranks;
+    const unsigned smem = tables + kSmallWords(share, p.most_bits + 1) * 4 + (hist ? LQ_HIST_STRIDE * 4 : 0);
+    return launch_cluster(kernel, dim3(ranks, (unsigned)p.num_layers, (unsigned)p.worker_count), kQThreads, smem, ranks, s, p, grads, step,
+                          packed, norms, hist, prev_packed, prev_norms, levels_cur, levels_prev, t);
 }
 
 }  // namespace lq

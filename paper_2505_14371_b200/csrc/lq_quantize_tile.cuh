@@ -1,6 +1,5 @@
 // A CTA's share of one (layer, worker) in the layer and global norm scopes, with the CTA's tables in place: the blocks of
-// a run of consecutive blocks of the layer, taken round-robin by the warps.  Shared by the kernel that takes a tile per CTA
-// (lq_quantize.cu) and the one whose clusters take whole layers, norm included (lq_quantize_small.cu).
+// a run of consecutive blocks of the layer, taken round-robin by the warps (lq_quantize.cu).
 #pragma once
 
 #include "lq_quantize.cuh"
