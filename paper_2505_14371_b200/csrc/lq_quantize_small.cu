@@ -34,18 +34,6 @@ __device__ __forceinline__ void st_peer(const double* mine, uint32_t rank, doubl
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 
-// This lane's four values of row j of block blk (fresh() pointer), zeros behind the layer's end.
-__device__ __forceinline__ float4 row_values(const float* g, int64_t blk, int j, int64_t size, int lane)
-{
-    const int64_t pos = blk * kBlockCoords + 128 * j + 4 * lane;
-    if (pos + 4 <= size) return __ldcg(reinterpret_cast<const float4*>(g + pos));
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (pos < size) v.x = __ldcg(g + pos);
-    if (pos + 1 < size) v.y = __ldcg(g + pos + 1);
-    if (pos + 2 < size) v.z = __ldcg(g + pos + 2);
-    return v;
-}
-
 // Warp j takes row j of all of the CTA's blocks.  `rows` (zeroed): bit j of a block's word says whether its row j holds anything
 // but zeros.  `first`: the lane's values of the first block's row.
 template <int kMode>
