@@ -22,18 +22,63 @@
 // is never fetched, draws no random numbers and needs no search: its symbols are 0.  If the
 // previous message is all zero there as well, the row adds nothing to the statistic and is
 // skipped entirely.  The masks are made warp-uniform by a reduction, so the per-row tests are uniform
-// branches.  The unrolled code handles whole blocks only; a layer's last, partial block goes through a
-// plain loop (once per layer and worker).
+// branches.  The unrolled code handles whole blocks only; a layer's last, partial block is taken by all warps, a row
+// each (once per layer and worker).
 #include "lq_quantize_tile.cuh"
 
 namespace lq {
 
-// kWidth: the code width of every layer of the plan, or 0 when they differ.  (A kernel of one width has less code to fetch and,
-// at widths 1 to 4 without histogram, no spills: 0 bytes of stores and loads against 8 and 32; widths 5 to 8 spill 8 to 28
-// bytes of stores, with histogram widths 1, 2, 4, 5 and 6 44 to 52, all widths in one 20.)
+// The layer's last, partial block, by all warps of the CTA that has it, a row each, once they are done with their whole blocks; its
+// words are gathered where the rings were.  It looks everything up again, so that the whole blocks' code carries nothing for it
+// (as arguments it took that code 844 -> 950 us on the Transformer-XL shapes).  Returns the thread's statistic term.
+// One warp that went through the 32 positions of its lanes one by one, each with a load and a binary search to wait for, took some 20
+// us, behind the last whole block of its layer: steps of 1 365 blocks in 40 layers and 2 workers 53.9 -> 39.6, of 504 blocks in
+// 30 layers 53.7 -> 32.1 us.
+template <int B, bool kHist, bool kStat>
+__device__ __noinline__ double quantize_last_block(const PlanDev& p, const float* grads, uint32_t step, uint32_t* packed,
+                                                   const uint32_t* prev_packed)
+{
+    extern __shared__ unsigned char dyn_smem[];
+    constexpr int C = B + 1;
+    uint32_t base;
+    unsigned char* sm = table_base(dyn_smem, base);
+    const int flat = blockIdx.y * gridDim.x + blockIdx.x, slot = flat / (int)gridDim.y, kk = flat - slot * (int)gridDim.y;
+    const TileJob J = p.jobs[slot];
+    const int k = kk + p.worker0, b = J.nblocks - 1, lane = threadIdx.x & 31, j = threadIdx.x >> 5;
+    uint32_t* words = reinterpret_cast<uint32_t*>(sm + kSmRing);
+    RowsJob job;
+    job.g = fresh(grads + (int64_t)kk * p.padded_elems + J.elem_off);
+    job.prev = kStat && prev_packed ? fresh(prev_packed + (int64_t)k * p.packed_words + J.word_off) : nullptr;
+    job.size = J.size;
+    job.block0 = J.block0 + b; job.nblocks = 1;
+    job.rows = words + C * 32;
+    job.words = base + kSmRing;
+    job.counts = true;
+    const float4 first = row_values(job.g, job.block0, j, job.size, lane);
+    __syncthreads();
+    for (int i = threadIdx.x; i < C * 32; i += kQThreads) words[i] = 0u;
+    if (threadIdx.x == 0) words[C * 32] = (uint32_t)sm[kSmRows + b] | ((uint32_t)sm[kSmRows + kTileBlocks + b] << 8);
+    __syncthreads();
+    QuantEnv ev;
+    ev.lut = base + kSmLut; ev.ld = base + kSmLd; ev.tprev = base + kSmTprev;
+    ev.r = p.rnorm[(int64_t)k * p.num_layers + J.layer];
+    ev.hist = reinterpret_cast<uint32_t*>(sm + kSmHist);
+    if (step == LQ_STEP_AUTO) step = (uint32_t)p.scalars->t;
+    const PhiloxConsts pc = philox_fold((uint32_t)J.layer, (uint32_t)k, step, p.seed_lo, p.seed_hi);
+    const double stat = quantize_rows_by<B, kHist, kStat>(p, pc, job, ev, reinterpret_cast<const int2*>(sm + kSmHow)->x & 3, first, lane, j);
+    __syncthreads();
+    uint32_t* out = packed + (int64_t)k * p.packed_words + J.word_off + (int64_t)job.block0 * (C * 32);
+    for (int i = threadIdx.x; i < C * 32; i += kQThreads) __stcs(out + i, words[i]);
+    return stat;
+}
+
+// kWidth: the code width of every layer of the plan, or 0 when they differ (a kernel of one width has less code to fetch).
+// The plan is a grid constant: a function that is handed it by reference otherwise makes every thread copy it to its stack (288
+// bytes: WGAN step 166 -> 180 us).  With it and the partial block out of the way the widths but 8 have no spills (0 to 52 bytes
+// before): Transformer-XL step 1938 -> 1911 us, low-rank factors 322 -> 267, widths 2, 3, 4 and 8 side by side 2396 -> 2280.
 template <int kWidth, bool kHist, bool kStat>
 __global__ void __launch_bounds__(kQThreads, 4) quantize_pack_kernel(
-    PlanDev p, const float* grads, uint32_t step, uint32_t* packed, const float* norms, uint32_t* hist,
+    const __grid_constant__ PlanDev p, const float* grads, uint32_t step, uint32_t* packed, const float* norms, uint32_t* hist,
     const uint32_t* prev_packed, const float* prev_norms, const float* levels_cur, const float* levels_prev, SearchTables st)
 {
     extern __shared__ unsigned char dyn_smem[];
@@ -94,7 +139,11 @@ __global__ void __launch_bounds__(kQThreads, 4) quantize_pack_kernel(
             for (int i = threadIdx.x; i < LQ_HIST_STRIDE; i += kQThreads) h[i] = 0;
         }
     }
-    if (threadIdx.x == 0) *reinterpret_cast<int2*>(sm + kSmHow) = how;
+    if (threadIdx.x == 0) {
+        *reinterpret_cast<int2*>(sm + kSmHow) = how;
+        // whether the tile ends in the layer's partial block, which is not part of a message of zeros
+        *reinterpret_cast<int*>(sm + kSmLast) = rn != 0.0f && (J.block0 + J.nblocks) * (int64_t)kBlockCoords > J.size;
+    }
     uint8_t* rows_cur = sm + kSmRows;
     uint8_t* rows_prev = rows_cur + kTileBlocks;
     if (threadIdx.x < tile.nblocks) {
@@ -117,8 +166,19 @@ __global__ void __launch_bounds__(kQThreads, 4) quantize_pack_kernel(
     uint32_t* out = packed + (int64_t)k * p.packed_words + L.word_off;
     const uint32_t* prev = prev_packed ? fresh(prev_packed + (int64_t)k * p.packed_words + L.word_off) : nullptr;
 
-    const double stat = quantize_blocks<kWidth, kHist, kStat>(p, pc, c, tile, L.bits, how.x & 3, (uint32_t)layer, (uint32_t)k, step, out, prev, ev,
-                                                      rows_cur, rows_prev, base + kSmRing);
+    double stat = quantize_blocks<kWidth, kHist, kStat>(p, pc, c, tile, L.bits, how.x & 3, out, prev, ev, rows_cur, rows_prev, base + kSmRing);
+    if (*reinterpret_cast<volatile int*>(sm + kSmLast)) {
+        if constexpr (kWidth != 0) {
+            stat += quantize_last_block<kWidth, kHist, kStat>(p, grads, step, packed, prev_packed);
+        } else {
+            switch (L.bits) {
+#define LQ_CASE(BB) case BB: stat += quantize_last_block<BB, kHist, kStat>(p, grads, step, packed, prev_packed); break;
+                LQ_CASE(1) LQ_CASE(2) LQ_CASE(3) LQ_CASE(4) LQ_CASE(5) LQ_CASE(6) LQ_CASE(7) LQ_CASE(8)
+#undef LQ_CASE
+                default: break;
+            }
+        }
+    }
     const double total = block_reduce<false>(stat, reinterpret_cast<double*>(sm + kSmScratch));
     if (threadIdx.x == 0) p.stat_partial[(int64_t)k * p.num_tiles + tile_id] = total;
 

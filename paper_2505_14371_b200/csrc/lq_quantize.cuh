@@ -37,6 +37,7 @@ constexpr uint32_t kSmRows = 0x3800;               // u8[kTileBlocks] rows of th
 constexpr uint32_t kSmScratch = 0x3900;            // double[kQWarps]
 constexpr uint32_t kSmHow = 0x3940;                // int2: SearchTables::how of the layer (here and not in registers that
                                                    // the octave search's code would have to carry)
+constexpr uint32_t kSmLast = kSmHow + 8;           // int: the tile ends in the layer's partial block (lq_quantize.cu)
 constexpr uint32_t kSmTables = 0x3A00;             // end of the tables = start of the per-warp rings (a multiple of 512)
 constexpr uint32_t kSmRing = kSmTables;
 constexpr uint32_t kRingBytes = kQWarps * 8 * 512; // 8 rows of 512 bytes per warp

@@ -2,7 +2,7 @@
 // a run of consecutive blocks of the layer, taken round-robin by the warps (lq_quantize.cu).
 #pragma once
 
-#include "lq_quantize.cuh"
+#include "lq_quantize_rows.cuh"
 
 namespace lq {
 
@@ -18,53 +18,6 @@ struct WarpCtx {
 __device__ __forceinline__ uint32_t lane_value(uint32_t x, int i, int lane)
 {
     return __reduce_or_sync(0xffffffffu, lane == i ? x : 0u);
-}
-
-// The layer's last, partial block (one per layer and worker): a plain loop over the lane's 32 positions with a
-// binary search over the levels, the coordinates past the layer's end sending zeros.  Same arithmetic as
-// quantize_coord; speed does not matter here.
-static __device__ __noinline__ double quantize_partial_block(const PlanDev& p, const QuantEnv& ev, const float* __restrict__ g,
-                                                      int64_t size, int64_t blk, int bits, uint32_t layer, uint32_t worker,
-                                                      uint32_t step, uint32_t* __restrict__ out,
-                                                      const uint32_t* __restrict__ prev, bool hist, int lane)
-{
-    const int C = bits + 1, n = 1 << bits;
-    const int64_t woff = blk * (int64_t)C * 32 + lane;
-    uint64_t acc = 0, pacc = 0;
-    int fill = 0, wi = 0, pfill = 0, pwi = 0;
-    double stat = 0.0;
-    for (int pp = 0; pp < 32; ++pp) {
-        const int64_t pos = blk * kBlockCoords + 128 * (pp >> 2) + 4 * lane + (pp & 3);
-        uint32_t sym = 0;
-        if (pos < size) {
-            const float v = __ldcg(g + pos);
-            uint32_t x[4];
-            philox4x32_10((uint32_t)(pos >> 2), layer, worker, step, p.seed_lo, p.seed_hi, x);
-            const float u = __fmul_rn(fabsf(v), ev.r);
-            int tau = 0;
-            for (int s = n >> 1; s > 0; s >>= 1)
-                if (lds_f32(ev.ld + 8u * (uint32_t)(tau + s)) <= u) tau += s;
-            tau = min(tau, n - 2);
-            const float2 ld = lds_f32x2(ev.ld + 8u * (uint32_t)tau);
-            const float num = __fsub_rn(u, ld.x);
-            const float f = __uint_as_float((x[pos & 3] >> 9) | 0x3F800000u);
-            const float t = __fmaf_rn(f, ld.y, -ld.y);
-            sym = 2u * (uint32_t)(tau + (t < num ? 1 : 0)) + (v < 0.0f ? 1u : 0u);
-            if (hist) atomicAdd(ev.hist + ((max(__float_as_uint(u), kHistClamp) - kHistClamp) >> 19), 1u);
-        }
-        if (pfill < C) {
-            if (prev && pwi < C) pacc |= (uint64_t)__ldcg(prev + woff + 32 * pwi) << pfill;
-            pfill += 32; ++pwi;
-        }
-        const uint32_t psym = (uint32_t)pacc & ((1u << C) - 1u);
-        pacc >>= C; pfill -= C;
-        const double dd = (double)__fsub_rn(lds_f32(ev.ld + (kSmTcur - kSmLd) + 4u * sym), lds_f32(ev.tprev + 4u * psym));
-        stat = fma(dd, dd, stat);
-        acc |= (uint64_t)sym << fill;
-        fill += C;
-        if (fill >= 32) { __stcs(out + woff + 32 * wi, (uint32_t)acc); acc >>= 32; fill -= 32; ++wi; }
-    }
-    return stat;
 }
 
 // A warp's share of a tile: the whole blocks warp, warp + 8, ...  A block whose rows are all zero in this input
@@ -186,16 +139,14 @@ __device__ __forceinline__ double quantize_width(const PlanDev& p, const PhiloxC
     return quantize_tile<B, kSearchStep, kHist, kStat>(p, pc, c, tile, out, prev, ev, rows_cur, rows_prev, ring_base);
 }
 
-// The CTA's blocks for the layer's code width (kWidth, or `bits` where kWidth is 0) and search; returns the thread's
+// The CTA's whole blocks for the layer's code width (kWidth, or `bits` where kWidth is 0) and search; returns the thread's
 // statistic term.
 template <int kWidth, bool kHist, bool kStat>
 __device__ __forceinline__ double quantize_blocks(const PlanDev& p, const PhiloxConsts& pc, const WarpCtx& c, const Tile& tile,
-                                                  int bits, int search, uint32_t layer, uint32_t worker, uint32_t step,
-                                                  uint32_t* __restrict__ out, const uint32_t* __restrict__ prev,
+                                                  int bits, int search, uint32_t* __restrict__ out, const uint32_t* __restrict__ prev,
                                                   const QuantEnv& ev, const uint8_t* rows_cur, const uint8_t* rows_prev,
                                                   uint32_t ring_base)
 {
-    const bool zeroed = ev.r == 0.0f;
     double stat = 0.0;
     if constexpr (kWidth != 0) {
         stat = quantize_width<kWidth, kHist, kStat>(p, pc, c, tile, search, out, prev, ev, rows_cur, rows_prev, ring_base);
@@ -207,15 +158,7 @@ __device__ __forceinline__ double quantize_blocks(const PlanDev& p, const Philox
             default: break;
         }
     }
-    if (!kStat) stat = 0.0;
-    // the layer's last, partial block, if it is among them: one warp, after its whole blocks
-    const int64_t bp = c.nfull - tile.block0;
-    if (!zeroed && (c.size % kBlockCoords) != 0 && bp >= 0 && bp < tile.nblocks && (int)(bp % kQWarps) == (threadIdx.x >> 5)) {
-        const double s2 = quantize_partial_block(p, ev, c.g, c.size, c.nfull, bits, layer, worker, step, out,
-                                                 kStat ? prev : nullptr, kHist, c.lane);
-        if (kStat) stat += s2;
-    }
-    return stat;
+    return kStat ? stat : 0.0;
 }
 
 }  // namespace lq

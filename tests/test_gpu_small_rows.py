@@ -1,6 +1,7 @@
 """ENCODE of small plans, a row of 128 coordinates a warp: layers that end inside a row, inside a lane's four coordinates and on
 the edges of rows and blocks, rows without values now or before, many (layer, worker) pairs of one CTA each, clusters of every
-size up to 16, every code width, and layers sent as zeros; against the oracle.  The same plan encoded for one worker of a range."""
+size up to 16, every code width, and layers sent as zeros; against the oracle.  The same plan encoded for one worker of a range.
+The last, partial blocks of large layers are encoded by the same rows, behind the whole blocks of the general encoder."""
 import numpy as np
 import pytest
 import torch
@@ -14,7 +15,9 @@ ENDS = [1, 3, 4, 127, 128, 129, 255, 511, 513, 900, 1023, 1024, 1025, 1151, 2047
 @pytest.mark.parametrize("sizes, bits, K, q", [
     (ENDS, 3, 5, 2), (ENDS * 4, 5, 7, 2), ([8 * 1024 - 1] + ENDS, 8, 2, 0), ([9 * 1024, 5, 129], 1, 2, 1),
     ([5 * 1024 + 385], 6, 1, 2), ([17 * 1024 + 2], 7, 2, 3), ([16 * 1024 - 130, 77], 2, 3, 2), ([40 * 1024 + 1, 600], 4, 16, 2),
-    (ENDS[:8] + [30 * 1024], [1, 2, 3, 4, 5, 6, 7, 8, 8], 4, 2)])
+    (ENDS[:8] + [30 * 1024], [1, 2, 3, 4, 5, 6, 7, 8, 8], 4, 2),
+    ([257 * 1024 + 3, 129], 3, 2, 2), ([258 * 1024 + 900, 1023, 2048], 8, 2, 0), ([257 * 1024 + 385, 511], 5, 1, 1),
+    ([257 * 1024 + 129] + ENDS[:8], [7, 1, 2, 3, 4, 5, 6, 7, 8], 2, 2)])
 @pytest.mark.parametrize("hist", [False, True])
 def test_rows_of_small_plans(orc, sizes, bits, K, q, hist):
     import paper_2505_14371_b200 as lqm
