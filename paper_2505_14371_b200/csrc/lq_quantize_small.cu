@@ -5,22 +5,19 @@
 // with nothing to fill the GPU, so latency is what bounds them, and more than that of sums and look-ups the latency of fetching
 // code: warp j of a CTA takes row j of each of its blocks, and all warps run the same code.
 //
-// The rule (use_small): layers of up to 8 blocks of 1024 coordinates, a CTA each, always; larger ones, of up to 256 blocks, while
-// the clusters are not too many: 1280 CTAs of up to 8 blocks each, 352 of more, and of more than 24 where there are 2600 blocks
-// of all workers or more (those chains of rows are longer than the general path's launches otherwise).  It asks for nothing but the plan's constants: a
+// The rule (use_small): layers of up to 8 blocks of 1024 coordinates, a CTA each, always; larger ones while a CTA has at most 13
+// blocks and the clusters at most 444 CTAs (3 on each SM).  It asks for nothing but the plan's constants: a
 // worker range does not change which kernel encodes a layer, nor the order in which the layer's sums are formed.
-// The step in us, this kernel and the general path.  One CTA a layer: layers of one block, 320 (layer, worker) pairs 11 and 36, 2400 of them
-// 38 and 104, 9600 128 and 387; of 1 to 8 blocks, 2400 pairs 58 and 108, 4896 111 and 224.  Clusters of up to 8 blocks a CTA: 640 CTAs
-// 28 and 42, 1280 of them 52 and 55 or, most with one block or none, 31 and 38, 1920 57 and 58, 2560 95 and 83.  Of more: 256
-// CTAs of 29 blocks 46 and 52, 288 of 24 27 and 31, 576 34 and 33, 512 of 29 85 and 77; 288 of 32 in 2300 blocks 34 and 30, 192
-// of 32 in 4000 35 and 44.
+// The step in us, this kernel and the general path.  One CTA a layer: layers of one block, 80 (layer, worker) pairs 13 and 20, 2400 of them
+// 38 and 46, 9600 128 and 153; of 1 to 8 blocks, 2400 pairs 58 and 64, 4896 111 and 129.  Clusters of up to 8 blocks a CTA: 160 CTAs
+// 12 and 18, 320 15 and 20, 640 20.4 and 19.6, 1280 31 and 24.  256 CTAs of 13 blocks 19 and 22, 128 of 16 26 and 23, 288 of 24 27 and 24.
 #include "lq_quantize_rows.cuh"
 
 namespace lq {
 
 namespace {
 
-constexpr int kMostRanks = 16, kMostShare = 32;              // CTAs of a cluster (more than 8 have to be asked for); blocks of a CTA
+constexpr int kMostRanks = 16, kMostShare = 13;              // CTAs of a cluster (more than 8 have to be asked for); blocks of a CTA
 // room for the words of a CTA's blocks
 __host__ __device__ constexpr int kSmallWords(int blocks, int C) { return blocks * C * 32; }
 
@@ -246,11 +243,9 @@ int small_ranks(const PlanDev& p)
 
 bool use_small(const PlanDev& p)
 {
-    if (p.global_norm || p.bucket_norm || p.most_blocks > 8 * kMostShare || p.num_layers > 65535) return false;      // (grid.y)
+    if (p.global_norm || p.bucket_norm || p.num_layers > 65535) return false;      // (grid.y)
     const int ranks = small_ranks(p);
-    const int64_t ctas = (int64_t)p.num_workers * p.num_layers * ranks;
-    if (p.most_blocks > 24 * ranks && p.num_workers * p.total_blocks < 2600) return false;
-    return ranks == 1 || ctas <= (p.most_blocks <= ranks * kQWarps ? 1280 : 352);
+    return ranks == 1 || (p.most_blocks <= ranks * kMostShare && (int64_t)p.num_workers * p.num_layers * ranks <= 3 * kSms);
 }
 
 cudaError_t launch_layer_norms_small(const PlanDev& p, const float* grads, float* norms, cudaStream_t s)
