@@ -38,14 +38,14 @@ METRIC = "quantize+pack and decode+aggregate+QODA GB/s (fp32 in)"
 # of a launch is a * E + b * N for E worker-coordinates in the embedding (90 % zero rows) and N in the other layers,
 # and (a, b) solve the two captures.  `inst` is the same for executed warp instructions (smsp__inst_executed.sum).
 KERNEL_SOURCES = {"norm_partial": ["lq_norm.cu", "lq_internal.cuh"],
-                  "quantize_pack": ["lq_quantize.cu", "lq_quantize_tile.cuh", "lq_quantize.cuh", "lq_internal.cuh"],
+                  "quantize_pack": ["lq_quantize.cu", "lq_quantize_tile.cuh", "lq_quantize_rows.cuh", "lq_quantize.cuh", "lq_internal.cuh"],
                   "decode": ["lq_decode.cu", "lq_internal.cuh"]}
 NCU_SCALED = {"transformer_xl": {          # kernel: bytes per embedding / other worker-coordinate, warp instr likewise
-    "norm_partial": {"bytes": (4.0067, 4.0092), "inst": (0.15637, 0.16913), "sources": "618bfbec8b934517"},
-    "quantize_pack": {"bytes": (1.3163, 5.3143), "inst": (0.22824, 1.28637), "sources": "8b9eb003e975ea00"},
-    "decode": {"bytes": (2.0863, 2.5274), "inst": (0.13197, 0.22909), "sources": "79467e8b33f1c270"}}}
+    "norm_partial": {"bytes": (4.0063, 4.0087), "inst": (0.15735, 0.17059), "sources": "ef7e30f7939bb94e"},
+    "quantize_pack": {"bytes": (1.2880, 5.2472), "inst": (0.21352, 1.19445), "sources": "c6377c45b8a58006"},
+    "decode": {"bytes": (2.0844, 2.5285), "inst": (0.12434, 0.21056), "sources": "c5c4255238a4cc86"}}}
 NCU_DIRECT = {"flat:26:4:8:2": {           # kernel: bytes and warp instructions of one launch
-    "quantize_pack": {"bytes": 2484224768.0 + 347961088.0, "inst": 676171776.0, "sources": "8b9eb003e975ea00"}}}
+    "quantize_pack": {"bytes": 2484451584.0 + 322569472.0, "inst": 630599680.0, "sources": "c6377c45b8a58006"}}}
 DENSE_POINT = "flat:26:4:8:2"             # dense companion of the headline workload: no zero rows to skip
 ISSUE_PEAK = 148 * 4 * 1.965e9            # warp instructions per second: 148 SMs x 4 schedulers x 1 per clock at 1965 MHz
 
