@@ -502,6 +502,9 @@ __global__ void __launch_bounds__(kThreads, 5) entropy_encode_kernel(PlanDev p, 
     __shared__ uint32_t slot_s, before_s, total_s;
     if (threadIdx.x == 0) slot_s = atomicAdd(ticket, 1u);
     __syncthreads();
+    // Overlapping encodes of one plan, which the caller has to order, clear the counter under each other: more numbers are drawn
+    // then than there are tiles.  What they write is wrong, but lies in the call's buffers.
+    if (slot_s >= gridDim.x) return;
     const int t = (int)(slot_s / (uint32_t)p.num_workers), k = (int)(slot_s - (uint32_t)t * (uint32_t)p.num_workers);
     const Tile T = p.tiles[t];
     const int layer = T.layer, lane = threadIdx.x & 31;

@@ -55,3 +55,38 @@ def test_streams_of_many_tiles(orc, layers, bits, kind):
     assert plan.lq_entropy_status() == 0
     plan.lq_entropy_encode(back, again, offs, runs)
     assert torch.equal(again, stream)
+
+
+def test_overlapping_encodes_stay_in_their_buffers():
+    """Two encodes of one plan on two streams, which the caller should have ordered: each clears the counter from which the
+    other's CTAs take their tiles, so that more numbers are drawn than there are tiles.  What comes out is undefined; nothing
+    outside the buffers is written, and an encode after them is right again."""
+    import paper_2505_14371_b200 as lqm
+    lqm.load_library()
+    K = 8
+    plan = lqm.Plan([8 * 1024 - 5] * 30, 4, 2, K, 3)         # 240 CTAs: those of both calls run at once
+    grads = torch.randn((K, plan.padded_elems), generator=torch.Generator(device="cuda").manual_seed(1), device="cuda")
+    packed, norms = plan.empty_packed(), plan.empty_norms()
+    plan.lq_quantize_pack(grads, 1, packed, norms)
+    cap, blocks = plan.packed_words, plan.lq_plan_blocks()
+
+    def buffers():                                           # a row more than the call is given, as a guard
+        return torch.full((K + 1, cap), -1, dtype=torch.int32, device="cuda"), torch.full((K + 1, blocks + 1), -1, dtype=torch.int32, device="cuda")
+    want, mine, theirs = buffers(), buffers(), buffers()
+    plan.lq_entropy_encode(packed, want[0][:K], want[1][:K])
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    for _ in range(50):
+        for s, (words, offs) in zip(streams, (mine, theirs)):
+            with torch.cuda.stream(s):
+                plan.lq_entropy_encode(packed, words[:K], offs[:K])
+    torch.cuda.synchronize()
+    for words, offs in (mine, theirs):
+        assert bool((words[K] == -1).all()) and bool((offs[K] == -1).all())
+    plan.lq_entropy_status()
+    plan.lq_entropy_encode(packed, mine[0][:K], mine[1][:K])
+    assert plan.lq_entropy_status() == 0
+    assert torch.equal(mine[1], want[1])
+    for k in range(K):
+        n = int(want[1][k, blocks])
+        assert torch.equal(mine[0][k, :n], want[0][k, :n])
