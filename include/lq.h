@@ -275,17 +275,27 @@ int lq_symbol_counts(const lq_plan* plan, const uint32_t* packed, uint32_t* coun
  *                   the bit offsets inside the block's stream at which its LQ_CODE_RUNS = 8 runs of 128 coordinates
  *                   (four lanes) start: side data of 16 bytes per block (1/8 bit per coordinate) that is not part of
  *                   the stream and lets the decoder work on the eight runs of a block in parallel.
- *                   The call uses scratch that the plan allocates at the first use of the stage (64 bytes per block
- *                   and worker): two encodes of one plan must not overlap on the GPU.
+ *                   The call uses scratch that the plan allocates at the first use of the stage (8 bytes per worker and
+ *                   tile of 8 to 128 blocks): two encodes of one plan must not overlap on the GPU.  The tiles are
+ *                   encoded side by side, and each waits for the words that the ones before it take.  If these do not
+ *                   come (the GPU stopped for seconds, or encodes that overlap), the tile gives up: the offsets of its
+ *                   blocks, and the worker's length if it is the last tile, become 0xffffffff, which a decode reports
+ *                   as broken; its run offsets and words are not written, and lq_entropy_status returns LQ_CODE_GAVE_UP.
+ *   lq_entropy_wait: how often a tile looks for the words before it until it gives up: `looks` >= 0, 0 = not once, at
+ *                   most and by default 2^22 (some seconds).  For tests, and callers that would rather encode again.
  *   lq_entropy_decode: the inverse, packed fully overwritten; it equals the encoded message except that the sign
  *                   bit of a coordinate with level index 0 comes back as 0 (the stream carries no sign there; the
  *                   decoded value is zero either way).  With run_offsets (as written by lq_entropy_encode for this
  *                   stream) one thread decodes each run of 128 coordinates, and runs of untouched rows are not
- *                   walked; with NULL one thread walks a whole block (an order of magnitude slower).  A stream with no valid word, a block that runs past its end,
- *                   or a run that does not end where the next one starts, sets a flag that lq_entropy_status
- *                   returns (and clears); nothing faults. */
+ *                   walked; with NULL one thread walks a whole block (an order of magnitude slower).  A stream with no
+ *                   valid word, a block that runs past its end, or a run that does not end where the next one starts,
+ *                   sets LQ_CODE_BROKEN; nothing faults.
+ *   lq_entropy_status: what the plan's encodes and decodes have reported since the last call, which clears it: 0, or
+ *                   LQ_CODE_BROKEN and LQ_CODE_GAVE_UP added up.  Synchronises. */
 #define LQ_CODE_MAX_LEN 12
 #define LQ_CODE_RUNS    8
+#define LQ_CODE_BROKEN  1u   /* a decode met an invalid stream */
+#define LQ_CODE_GAVE_UP 2u   /* an encode waited in vain: encode again */
 int lq_code_build(const double* weights, int32_t n, uint8_t* lengths);
 int lq_code_universal(int32_t n, uint8_t* lengths);
 int lq_code_set(lq_plan* plan, int32_t layer, const uint8_t* lengths, int32_t n);
@@ -295,6 +305,7 @@ int lq_entropy_encode(lq_plan* plan, const uint32_t* packed, uint32_t* stream_wo
                       uint32_t* block_offsets, uint16_t* run_offsets, void* stream);
 int lq_entropy_decode(lq_plan* plan, const uint32_t* stream_words, int64_t capacity_words,
                       const uint32_t* block_offsets, const uint16_t* run_offsets, uint32_t* packed, void* stream);
+int lq_entropy_wait(lq_plan* plan, int32_t looks);
 int lq_entropy_status(lq_plan* plan, uint32_t* host_flag);
 
 /* Ergodic average (the guarantees of Section 5 are stated for X-bar_{T+1/2} = sum_{t=1..T} X_{t+1/2} / T).

@@ -22,6 +22,8 @@ NUM_BINS = 386
 HIST_STRIDE = 512
 STATUS_ZERO_NORM = 1
 STATUS_NONFINITE = 2
+CODE_BROKEN = 1                 # a decode met an invalid stream
+CODE_GAVE_UP = 2                # an encode waited in vain
 STEP_AUTO = 0xFFFFFFFF          # lq_quantize_pack: take the step index from the plan's device-side iteration counter
 
 EXPORTS = ["lq_plan_create", "lq_plan_destroy", "lq_plan_padded_elems", "lq_plan_packed_words",
@@ -29,7 +31,7 @@ EXPORTS = ["lq_plan_create", "lq_plan_destroy", "lq_plan_padded_elems", "lq_plan
            "lq_side_data_import", "lq_set_levels", "lq_get_levels", "lq_layer_norms",
            "lq_quantize_pack", "lq_fit_levels", "lq_fit_levels_shared", "lq_decode_aggregate", "qoda_init", "qoda_step",
            "qoda_get_scalars", "lq_code_build", "lq_code_universal", "lq_code_set", "lq_code_get", "lq_plan_blocks", "lq_entropy_encode",
-           "lq_entropy_decode", "lq_entropy_status", "lq_level_probabilities", "lq_symbol_counts", "qoda_set_alt_rates", "qoda_set_average", "qoda_get_alt_scalars", "lq_get_statistics", "lq_vector_norm_static", "lq_profile_enable",
+           "lq_entropy_decode", "lq_entropy_wait", "lq_entropy_status", "lq_level_probabilities", "lq_symbol_counts", "qoda_set_alt_rates", "qoda_set_average", "qoda_get_alt_scalars", "lq_get_statistics", "lq_vector_norm_static", "lq_profile_enable",
            "lq_profile_read",
            "lq_error_string", "lq_last_error"]
 KERNEL_NAMES = ["norm_partial", "norm_finalize", "quantize_pack", "stat_finalize", "qoda_scalars",
@@ -85,6 +87,7 @@ def load_library() -> C.CDLL:
     L.lq_plan_blocks.argtypes = [vp]; L.lq_plan_blocks.restype = i64
     L.lq_entropy_encode.argtypes = [vp, vp, vp, i64, vp, vp, vp]
     L.lq_entropy_decode.argtypes = [vp, vp, i64, vp, vp, vp, vp]
+    L.lq_entropy_wait.argtypes = [vp, i32]
     L.lq_entropy_status.argtypes = [vp, C.POINTER(u32)]
     L.lq_level_probabilities.argtypes = [vp, vp, vp, i32, i32, vp, vp]
     L.lq_symbol_counts.argtypes = [vp, vp, vp, vp]
@@ -291,7 +294,12 @@ class Plan:
         """[K][blocks][8] int16 buffer for the run offsets of the entropy stage."""
         return torch.zeros((self.num_workers, self.lq_plan_blocks(), 8), dtype=torch.int16, device=device)
 
+    def lq_entropy_wait(self, looks: int = 1 << 22) -> None:
+        """How often a tile of an encode looks for the words before it until it gives up."""
+        _check(load_library().lq_entropy_wait(self._h, looks))
+
     def lq_entropy_status(self) -> int:
+        """CODE_BROKEN and CODE_GAVE_UP of the decodes and encodes since the last call, added up."""
         flag = C.c_uint32(0)
         _check(load_library().lq_entropy_status(self._h, C.byref(flag)))
         return flag.value

@@ -85,8 +85,8 @@ struct lq_plan {
     uint32_t* d_code_enc = nullptr;        // [L][256]   entropy stage, allocated at its first use
     uint16_t* d_code_dec = nullptr;        // [L][kDecEntries]
     bool codes_ready = false;              // ... and all of the following allocated, the tables made
-    uint32_t* d_code_bad = nullptr;        // [1] set by a decode that met an invalid stream
-    EncodeScratch code_scratch{nullptr, 0};   // allocated with the tables
+    uint32_t* d_code_bad = nullptr;        // [1] LQ_CODE_BROKEN from a decode, LQ_CODE_GAVE_UP from an encode
+    EncodeScratch code_scratch{nullptr, 0, kMostLooks};   // allocated with the tables
     std::vector<uint8_t> code_len;         // [L][256] host copy of the word lengths
     double alt_qhat = 0.0;         // > 0: qoda_step follows Eq. (Alt) with this exponent
     double* xsum = nullptr;        // caller-owned running sum of the half iterates (qoda_set_average), or NULL
@@ -941,6 +941,14 @@ int lq_entropy_decode(lq_plan* plan, const uint32_t* stream_words, int64_t capac
     if (rc != LQ_OK) return rc;
     LQ_CUDA(launch_entropy_decode(plan->dev, stream_words, capacity_words, block_offsets, run_offsets, plan->d_code_enc, plan->d_code_dec,
                                   packed, plan->d_code_bad, (cudaStream_t)stream));
+    return LQ_OK;
+}
+
+int lq_entropy_wait(lq_plan* plan, int32_t looks)
+{
+    if (!plan) return fail(LQ_EINVAL, "NULL argument");
+    if (looks < 0) return fail(LQ_EINVAL, "looks < 0");
+    plan->code_scratch.looks = std::min(looks, kMostLooks);
     return LQ_OK;
 }
 

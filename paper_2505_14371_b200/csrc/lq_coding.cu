@@ -444,9 +444,9 @@ __device__ __noinline__ void encode_blocks(const EncodeJob J)
 }
 
 // What a tile tells the tiles behind it in the same worker's stream, one 64-bit word: its words (kTileSum) or all words up to
-// its end (kTileEnd) in the low half.  Written and read whole, and nothing else is passed on by it.
-constexpr uint64_t kTileSum = 1ull << 32, kTileEnd = 2ull << 32;
-constexpr int kMostPolls = 1 << 22;            // of a word that stays empty: some seconds
+// its end (kTileEnd) in the low half, or that it does not know where it starts (kTileLost).  Written and read whole, and nothing
+// else is passed on by it.
+constexpr uint64_t kTileSum = 1ull << 32, kTileEnd = 2ull << 32, kTileLost = 3ull << 32;
 __device__ __forceinline__ void put_state(uint64_t* a, uint64_t v) { asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(a), "l"(v) : "memory"); }
 __device__ __forceinline__ uint64_t get_state(const uint64_t* a)
 {
@@ -456,21 +456,22 @@ __device__ __forceinline__ uint64_t get_state(const uint64_t* a)
 }
 
 // The words of all tiles before tile t (one warp; state: this worker's words, one per tile): looks back 32 tiles at a time until
-// one knows everything before it.  `failed`: a tile that has not told in all the polls.
-__device__ __forceinline__ uint32_t words_before(const uint64_t* state, int t, int lane, bool& failed)
+// one knows everything before it.  `failed`: a tile before it has told nothing in `looks` looks, or gave up itself.
+__device__ __forceinline__ uint32_t words_before(const uint64_t* state, int t, int lane, int looks, bool& failed)
 {
     uint32_t before = 0;
     for (int last = t - 1; last >= 0; last -= 32) {
         const int i = last - lane;
         uint64_t v = i >= 0 ? 0ull : kTileEnd;
-        for (int poll = 0;; ++poll) {
+        for (int look = 0;; ++look) {
+            if (look >= looks) { failed = true; return 0u; }
             if ((v >> 32) == 0ull) v = get_state(state + i);
             if (__all_sync(0xffffffffu, (v >> 32) != 0ull)) break;
-            if (poll >= kMostPolls) { failed = true; return 0u; }
-            if (poll > 8) __nanosleep(100);
+            if (look > 8) __nanosleep(100);
         }
         const uint32_t ends = __ballot_sync(0xffffffffu, (v & kTileEnd) != 0ull);
         const int upto = ends ? __ffs(ends) - 1 : 31;
+        if (__any_sync(0xffffffffu, lane == upto && (v >> 32) == (kTileLost >> 32))) { failed = true; return 0u; }
         before += __reduce_add_sync(0xffffffffu, lane <= upto ? (uint32_t)v : 0u);
         if (ends) break;
     }
@@ -491,7 +492,7 @@ __global__ void __launch_bounds__(kThreads, 5) entropy_encode_kernel(PlanDev p, 
                                                                      uint32_t* __restrict__ offsets,
                                                                      uint32_t* __restrict__ out, int64_t capacity,
                                                                      uint16_t* __restrict__ run_offsets, uint64_t* states,
-                                                                     uint32_t* ticket, uint32_t* bad, uint32_t code_bytes)
+                                                                     uint32_t* ticket, int looks, uint32_t* bad, uint32_t code_bytes)
 {
     // tables of pairs of symbols, or of the single ones of wide codes, at a multiple of their size; a buffer for every warp's block
     extern __shared__ __align__(16) unsigned char enc_smem[];
@@ -567,17 +568,21 @@ __global__ void __launch_bounds__(kThreads, 5) entropy_encode_kernel(PlanDev p, 
 #pragma unroll
         for (int i = 0; i < kTileBlocks / 32; ++i) { words[lane * (kTileBlocks / 32) + i] = at; at += v[i]; }
         bool failed = false;
-        const uint32_t before = words_before(state, t, lane, failed);
+        const uint32_t before = words_before(state, t, lane, looks, failed);
         if (lane == 0) {
-            if (t > 0 && !failed) put_state(state + t, kTileEnd | (uint32_t)(before + total));
-            if (failed) atomicOr(bad, 1u);
+            if (t > 0) put_state(state + t, failed ? kTileLost : kTileEnd | (uint32_t)(before + total));
+            if (failed) atomicOr(bad, LQ_CODE_GAVE_UP);
             before_s = before; total_s = failed ? 0xffffffffu : total;
         }
     }
     __syncthreads();
-    if (total_s == 0xffffffffu) return;
     const uint32_t before = before_s;
     uint32_t* off = offsets + (int64_t)k * (p.total_blocks + 1) + L.block_off + T.block0;
+    if (total_s == 0xffffffffu) {            // gave up: offsets that no stream has, and that a decoder refuses
+        if (threadIdx.x < T.nblocks) off[threadIdx.x] = 0xffffffffu;
+        if (threadIdx.x == 0 && t == p.num_tiles - 1) off[T.nblocks] = 0xffffffffu;
+        return;
+    }
     if (threadIdx.x < T.nblocks) off[threadIdx.x] = before + words[threadIdx.x];
     if (threadIdx.x == 0 && t == p.num_tiles - 1) off[T.nblocks] = before + total_s;
     J.out = out + (int64_t)k * capacity + before;
@@ -659,7 +664,7 @@ __global__ void __launch_bounds__(128) entropy_decode_kernel(PlanDev p, const ui
     }
     if (last_pair) last_at += decode_one(last_pair, C, enc).bits;
     // no valid word, or a last coordinate that starts past the word behind the block's end
-    if (broken || first + (int64_t)(last_at >> 5) > last) atomicOr(bad, 1u);
+    if (broken || first + (int64_t)(last_at >> 5) > last) atomicOr(bad, LQ_CODE_BROKEN);
 }
 
 // Decoder on the run offsets.  A run is four lanes (128 coordinates) of a block; one CTA takes a tile (up to 128 blocks of
@@ -928,7 +933,7 @@ __global__ void __launch_bounds__(kThreads, 4) entropy_decode_runs_kernel(PlanDe
         // a broken run has read on past its own words into other threads': its words are formed again, from the block's
         if (again) broken |= walk_run_plain(r, C, len, blk, t & 7, T.size, dst);
     }
-    if (broken) atomicOr(bad, 1u);
+    if (broken) atomicOr(bad, LQ_CODE_BROKEN);
 }
 
 }  // namespace
@@ -959,7 +964,7 @@ cudaError_t launch_entropy_encode(const PlanDev& p, const uint32_t* packed, cons
     if (e != cudaSuccess) return e;
     entropy_encode_kernel<<<(unsigned)((int64_t)p.num_tiles * p.num_workers), kThreads, smem, s>>>(
         p, packed, enc_tables, offsets, out, capacity, run_offsets, scratch.states + 1, reinterpret_cast<uint32_t*>(scratch.states),
-        bad, code_bytes);
+        scratch.looks, bad, code_bytes);
     return cudaGetLastError();
 }
 

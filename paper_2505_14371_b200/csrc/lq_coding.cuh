@@ -29,9 +29,11 @@ void build_code_table_host(const uint8_t* len, const uint32_t* code, int n, uint
 
 // Scratch of the encoder, owned by the plan: a counter from which its CTAs take their tiles, then what every (worker, tile)
 // tells the tiles behind it; cleared before each encode.
+constexpr int kMostLooks = 1 << 22;      // some seconds
 struct EncodeScratch {
     uint64_t* states;        // [1 + K * num_tiles]
     size_t bytes;
+    int looks;               // at the words before a tile, until the tile gives up
 };
 cudaError_t launch_build_decode_tables(const PlanDev& p, int layer0, int layers, const uint32_t* enc_tables, uint16_t* dec_tables,
                                        cudaStream_t s);

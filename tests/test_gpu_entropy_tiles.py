@@ -90,3 +90,40 @@ def test_overlapping_encodes_stay_in_their_buffers():
     for k in range(K):
         n = int(want[1][k, blocks])
         assert torch.equal(mine[0][k, :n], want[0][k, :n])
+
+
+@pytest.mark.parametrize("sizes", [[9 * 1024 + 7] * 40, [1] * 3, [70 * 1024]])
+def test_tiles_that_give_up_say_so(sizes):
+    """No tile looks for the words before it: all but each worker's first one give up.  They leave offsets that a decode reports
+    as broken, and words that are not theirs as they were; the status names the encode, and the next encode is whole again."""
+    import paper_2505_14371_b200 as lqm
+    lqm.load_library()
+    K = 3
+    plan = lqm.Plan(sizes, 4, 2, K, 3)
+    grads = torch.randn((K, plan.padded_elems), generator=torch.Generator(device="cuda").manual_seed(1), device="cuda")
+    packed, norms = plan.empty_packed(), plan.empty_norms()
+    plan.lq_quantize_pack(grads, 1, packed, norms)
+    blocks = plan.lq_plan_blocks()
+
+    def encoded():
+        words, offs, runs = torch.full_like(packed, -1), torch.zeros((K, blocks + 1), dtype=torch.int32, device="cuda"), plan.empty_run_offsets()
+        plan.lq_entropy_encode(packed, words, offs, runs)
+        return words, offs, runs
+    whole = encoded()
+    assert plan.lq_entropy_status() == 0
+    plan.lq_entropy_wait(0)
+    words, offs, runs = encoded()
+    assert plan.lq_entropy_status() == lqm.CODE_GAVE_UP and plan.lq_entropy_status() == 0
+    first = min(8, -(-sizes[0] // 1024))                     # blocks of the first tile
+    n = whole[1][:, first]                                   # and its words
+    assert torch.equal(offs[:, :first], whole[1][:, :first]) and bool((offs[:, first:] == -1).all())
+    for k in range(K):
+        assert torch.equal(words[k, : n[k]], whole[0][k, : n[k]]) and bool((words[k, n[k]:] == -1).all())
+    for side in (runs, None):
+        plan.lq_entropy_decode(words, offs, torch.empty_like(packed), side)
+        assert plan.lq_entropy_status() == lqm.CODE_BROKEN
+    plan.lq_entropy_wait()
+    again = encoded()
+    assert plan.lq_entropy_status() == 0 and all(torch.equal(a, b) for a, b in zip(again, whole))
+    with pytest.raises(lqm.LqError):
+        plan.lq_entropy_wait(-1)
