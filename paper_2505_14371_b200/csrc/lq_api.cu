@@ -258,7 +258,6 @@ int lq_plan_create(lq_plan** out, int32_t num_layers, const int64_t* layer_sizes
     d.dec_blocks = dec_blocks;
     d.dec_shift = 0;
     while ((dec_blocks << d.dec_shift) < tile_blocks) ++d.dec_shift;
-    d.most_blocks = (int32_t)std::min<int64_t>(most_blocks, INT32_MAX);
     d.sub_tiles = tile_blocks / sub_blocks;
     d.sub_shift = 0;
     while ((1 << d.sub_shift) < d.sub_tiles) ++d.sub_shift;
@@ -268,6 +267,10 @@ int lq_plan_create(lq_plan** out, int32_t num_layers, const int64_t* layer_sizes
         d.rk0[r] = d.seed_lo + (uint32_t)(r + 2) * 0x9E3779B9u;
         d.rk1[r] = d.seed_hi + (uint32_t)(r + 2) * 0xBB67AE85u;
     }
+
+    d.small_ranks = (int16_t)small_plan_ranks((int64_t)num_layers * num_workers, num_layers, most_blocks, kSms,
+                                              small_cluster_room());
+    d.small_share = (int16_t)(d.small_ranks ? (most_blocks + d.small_ranks - 1) / d.small_ranks : 0);
 
     cudaError_t e = cudaGetDevice(&p->device);
     const size_t KL = (size_t)num_workers * (size_t)(num_layers ? num_layers : 1);

@@ -7,6 +7,7 @@
 #include <atomic>
 
 #include "lq.h"
+#include "lq_small_rule.h"
 
 namespace lq {
 
@@ -90,7 +91,8 @@ struct PlanDev {
     int32_t sub_tiles;    // sub-tiles per tile: the plan's tile size / sub_blocks, a power of two
     int32_t sub_shift;    // log2(sub_tiles)
     int32_t sub_blocks;   // blocks per sub-tile
-    int32_t most_blocks;  // blocks of the plan's largest layer
+    int16_t small_ranks;  // CTAs a (layer, worker) in the kernel of small plans, 0: the general path (small_plan_ranks) ...
+    int16_t small_share;  // ... and the most blocks that one of them has
     int32_t most_bits;    // widest code of the plan
     int32_t least_bits;   // narrowest code of the plan
     int32_t dec_blocks;   // blocks per decoder CTA; 1: its warps share them
@@ -229,7 +231,8 @@ cudaError_t launch_quantize(const PlanDev& p, const float* grads, uint32_t step,
                             const float* prev_norms, const float* levels_cur,
                             const float* levels_prev, SearchTables t, bool need_stat, cudaStream_t s);
 // layer scope, plans whose layers are all small: norms, messages and statistic in one kernel
-bool use_small(const PlanDev& p);
+inline bool use_small(const PlanDev& p) { return p.small_ranks > 0 && !p.global_norm && !p.bucket_norm; }
+ClusterRoom small_cluster_room();      // of the current device
 cudaError_t launch_layer_norms_small(const PlanDev& p, const float* grads, float* norms, cudaStream_t s);
 cudaError_t launch_quantize_small(const PlanDev& p, const float* grads, uint32_t step, uint32_t* packed, float* norms,
                                   uint32_t* hist, const uint32_t* prev_packed, const float* prev_norms,

@@ -4,20 +4,16 @@
 // general path has four (norm partials, norms, encoder, statistic).  Such plans are a chain of launches of a few us each,
 // with nothing to fill the GPU, so latency is what bounds them, and more than that of sums and look-ups the latency of fetching
 // code: warp j of a CTA takes row j of each of its blocks, and all warps run the same code.
-//
-// The rule (use_small): layers of up to 8 blocks of 1024 coordinates, a CTA each, always; larger ones while a CTA has at most 13
-// blocks and the clusters at most 444 CTAs (3 on each SM).  It asks for nothing but the plan's constants: a
-// worker range does not change which kernel encodes a layer, nor the order in which the layer's sums are formed.
-// The step in us, this kernel and the general path.  One CTA a layer: layers of one block, 80 (layer, worker) pairs 13 and 20, 2400 of them
-// 38 and 46, 9600 128 and 153; of 1 to 8 blocks, 2400 pairs 58 and 64, 4896 111 and 129.  Clusters of up to 8 blocks a CTA: 160 CTAs
-// 12 and 18, 320 15 and 20, 640 20.4 and 19.6, 1280 31 and 24.  256 CTAs of 13 blocks 19 and 22, 128 of 16 26 and 23, 288 of 24 27 and 24.
+// (Which plans: lq_small_rule.h.)
+#include <algorithm>
+#include <mutex>
+
 #include "lq_quantize_rows.cuh"
 
 namespace lq {
 
 namespace {
 
-constexpr int kMostRanks = 16, kMostShare = 13;              // CTAs of a cluster (more than 8 have to be asked for); blocks of a CTA
 // room for the words of a CTA's blocks
 __host__ __device__ constexpr int kSmallWords(int blocks, int C) { return blocks * C * 32; }
 
@@ -103,8 +99,8 @@ __device__ __forceinline__ void store_norm(const PlanDev& p, const LayerNorm& n,
 // The norms alone, in the encoder's order (lq_layer_norms gives the very norms that lq_quantize_pack sends).
 __global__ void __launch_bounds__(kQThreads) layer_norms_small_kernel(PlanDev p, const float* grads, float* norms)
 {
-    __shared__ double part[kMostRanks], scratch[kQWarps];
-    __shared__ uint32_t rows[kMostShare];                    // (not used)
+    __shared__ double part[kSmallRanks], scratch[kQWarps];
+    __shared__ uint32_t rows[kSmallShare];                    // (not used)
     float4 first;
     pdl_launch_next();
     const int ranks = gridDim.x, rank = blockIdx.x, layer = blockIdx.y, k = blockIdx.z + p.worker0;
@@ -123,8 +119,8 @@ __global__ void __launch_bounds__(kQThreads, 3) quantize_small_kernel(
     const uint32_t* prev_packed, const float* prev_norms, const float* levels_cur, const float* levels_prev, SearchTables st)
 {
     extern __shared__ unsigned char dyn_smem[];
-    __shared__ double norm_part[kMostRanks], stat_part[kMostRanks];             // per CTA of the cluster
-    __shared__ uint32_t rows[kMostShare];
+    __shared__ double norm_part[kSmallRanks], stat_part[kSmallRanks];             // per CTA of the cluster
+    __shared__ uint32_t rows[kSmallShare];
     uint32_t base;
     unsigned char* sm = table_base(dyn_smem, base);
     pdl_launch_next();
@@ -228,32 +224,62 @@ __global__ void __launch_bounds__(kQThreads, 3) quantize_small_kernel(
     }
 }
 
-// CTAs of a plan's clusters: as many as its largest layer needs for 8 blocks each, up to 8, and more, while there are blocks for
-// them and SMs (2 CTAs on each): 784 blocks of 203 530 coordinates and 4 workers on 8 CTAs each 27.7, on 16 20.5 us.
-int small_ranks(const PlanDev& p)
+}  // namespace
+
+// The most shared memory that the kernel asks for.
+constexpr unsigned kSmallTables = kSmRing + kSmSlack, kSmallMost = kSmallTables + kSmallWords(kSmallShare, LQ_MAX_BITS + 1) * 4 + LQ_HIST_STRIDE * 4;
+
+namespace {
+
+cudaError_t allow_small()
 {
-    const int64_t pairs = (int64_t)p.num_workers * p.num_layers;
-    int r = 1;
-    while (r < 8 && r * kQWarps < p.most_blocks) r *= 2;
-    while (r < kMostRanks && r < p.most_blocks && pairs * 2 * r <= 2 * kSms) r *= 2;
-    return r;
+    static std::atomic<uint64_t> memory{0}, clusters{0};
+    cudaError_t e = opt_in_shared_memory(memory, (int)kSmallMost, quantize_small_kernel<true, true>,
+                                         quantize_small_kernel<false, true>, quantize_small_kernel<false, false>);
+    if (e == cudaSuccess)
+        e = allow_clusters(clusters, layer_norms_small_kernel, quantize_small_kernel<true, true>, quantize_small_kernel<false, true>,
+                           quantize_small_kernel<false, false>);
+    return e;
 }
 
 }  // namespace
 
-bool use_small(const PlanDev& p)
+ClusterRoom small_cluster_room()
 {
-    if (p.global_norm || p.bucket_norm || p.num_layers > 65535) return false;      // (grid.y)
-    const int ranks = small_ranks(p);
-    return ranks == 1 || (p.most_blocks <= ranks * kMostShare && (int64_t)p.num_workers * p.num_layers * ranks <= 3 * kSms);
+    static std::mutex guard;
+    static ClusterRoom rooms[64];                                // asked for once per device
+    static uint64_t known = 0;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return ClusterRoom{}; }
+    const std::lock_guard<std::mutex> lock(guard);
+    if (dev < 64 && ((known >> dev) & 1u)) return rooms[dev];
+    ClusterRoom room{};
+    cudaError_t e = allow_small();
+    for (int i = 0; i < 5 && e == cudaSuccess; ++i) {
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = 1u << i; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(1u << i, 1, 1); cfg.blockDim = kQThreads; cfg.dynamicSmemBytes = kSmallMost;
+        cfg.attrs = &at; cfg.numAttrs = 1;
+        int least = INT32_MAX;
+        for (auto kernel : {quantize_small_kernel<true, true>, quantize_small_kernel<false, true>, quantize_small_kernel<false, false>}) {
+            int n = 0;
+            if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) { n = 0; cudaGetLastError(); }
+            least = std::min(least, n);
+        }
+        room.clusters[i] = least;
+    }
+    if (e != cudaSuccess) cudaGetLastError();
+    else if (dev < 64) { rooms[dev] = room; known |= 1ull << dev; }
+    return room;
 }
 
 cudaError_t launch_layer_norms_small(const PlanDev& p, const float* grads, float* norms, cudaStream_t s)
 {
-    const unsigned ranks = (unsigned)small_ranks(p);
-    static std::atomic<uint64_t> configured{0};
-    const cudaError_t e = allow_clusters(configured, layer_norms_small_kernel);
+    const cudaError_t e = allow_small();
     if (e != cudaSuccess) return e;
+    const unsigned ranks = (unsigned)p.small_ranks;
     return launch_cluster(layer_norms_small_kernel, dim3(ranks, (unsigned)p.num_layers, (unsigned)p.worker_count), kQThreads, 0, ranks,
                           s, p, grads, norms);
 }
@@ -263,18 +289,12 @@ cudaError_t launch_quantize_small(const PlanDev& p, const float* grads, uint32_t
                                   const float* levels_cur, const float* levels_prev, SearchTables t, bool need_stat, cudaStream_t s)
 {
     if (p.num_layers == 0) return cudaSuccess;
-    constexpr unsigned tables = kSmRing + kSmSlack, most = tables + kSmallWords(kMostShare, LQ_MAX_BITS + 1) * 4 + LQ_HIST_STRIDE * 4;
-    static std::atomic<uint64_t> configured{0}, clusters{0};
-    cudaError_t e = opt_in_shared_memory(configured, (int)most, quantize_small_kernel<true, true>,
-                                         quantize_small_kernel<false, true>, quantize_small_kernel<false, false>);
-    if (e == cudaSuccess)
-        e = allow_clusters(clusters, quantize_small_kernel<true, true>, quantize_small_kernel<false, true>, quantize_small_kernel<false, false>);
+    const cudaError_t e = allow_small();
     if (e != cudaSuccess) return e;
     const auto kernel = hist ? quantize_small_kernel<true, true>
                         : need_stat ? quantize_small_kernel<false, true> : quantize_small_kernel<false, false>;
-    const unsigned ranks = (unsigned)small_ranks(p);
-    const int share = (p.most_blocks + (int)ranks - 1) / (int)ranks;
-    const unsigned smem = tables + kSmallWords(share, p.most_bits + 1) * 4 + (hist ? LQ_HIST_STRIDE * 4 : 0);
+    const unsigned ranks = (unsigned)p.small_ranks;
+    const unsigned smem = kSmallTables + kSmallWords(p.small_share, p.most_bits + 1) * 4 + (hist ? LQ_HIST_STRIDE * 4 : 0);
     return launch_cluster(kernel, dim3(ranks, (unsigned)p.num_layers, (unsigned)p.worker_count), kQThreads, smem, ranks, s, p, grads, step,
                           packed, norms, hist, prev_packed, prev_norms, levels_cur, levels_prev, t);
 }

@@ -309,3 +309,31 @@ def test_objects_are_compiled_again_when_the_build_flags_change(tmp_path, monkey
     at(tmp_path / "build.py", 3000)
     b.build()
     assert sorted(os.path.basename(c) for c in ran) == sorted(names)
+
+
+@pytest.fixture(scope="module")
+def small_ranks(tmp_path_factory):
+    """small_plan_ranks(pairs, layers, blocks of the largest layer, clusters of 1, 2, 4, 8, 16 CTAs that run at once)"""
+    d = tmp_path_factory.mktemp("rule")
+    (d / "rule.cpp").write_text('#include "lq_small_rule.h"\nextern "C" int ranks(int64_t p, int64_t l, int64_t m, const int32_t* c) {\n'
+                                'lq::ClusterRoom r; for (int i = 0; i < 5; ++i) r.clusters[i] = c[i]; return lq::small_plan_ranks(p, l, m, 148, r); }\n')
+    subprocess.check_call(["g++", "-std=c++17", "-shared", "-fPIC", "-I", os.path.join(ROOT, "paper_2505_14371_b200", "csrc"),
+                           str(d / "rule.cpp"), "-o", str(d / "rule.so")])
+    f = ctypes.CDLL(str(d / "rule.so")).ranks
+    f.argtypes = [ctypes.c_int64] * 3 + [ctypes.POINTER(ctypes.c_int32)]
+    return lambda pairs, layers, most, room: f(pairs, layers, most, (ctypes.c_int32 * 5)(*room))
+
+
+WHOLE = (444, 222, 104, 48, 21)                                   # clusters that run at once on a whole B200
+
+
+@pytest.mark.parametrize("room", [WHOLE, (444, 222, 104, 48, 0), (60, 30, 12, 3, 1), (54, 24, 0, 0, 0), (0, 0, 0, 0, 0)])
+def test_small_plans_ask_for_clusters_that_the_device_has(small_ranks, room):
+    for pairs in (1, 2, 9, 18, 19, 48, 49, 104, 105, 222, 223, 5000):
+        for most in (0, 1, 2, 8, 9, 16, 17, 64, 100, 196, 208, 224, 225, 4000):
+            r = small_ranks(pairs, pairs, most, room)
+            assert r in (0, 1, 2, 4, 8, 16)
+            if most <= 8:
+                assert r >= 1                                     # a CTA a layer is always to be had
+            if r > 1 or most > 8 and r == 1:
+                assert room[r.bit_length() - 1] > 0 and most <= r * 13
