@@ -268,7 +268,7 @@ int lq_plan_create(lq_plan** out, int32_t num_layers, const int64_t* layer_sizes
         d.rk1[r] = d.seed_hi + (uint32_t)(r + 2) * 0xBB67AE85u;
     }
 
-    d.small_ranks = (int16_t)small_plan_ranks((int64_t)num_layers * num_workers, num_layers, most_blocks, kSms,
+    d.small_ranks = (int16_t)small_plan_ranks((int64_t)num_layers * num_workers, num_layers, most_blocks, blocks * num_workers, kSms,
                                               small_cluster_room());
     d.small_share = (int16_t)(d.small_ranks ? (most_blocks + d.small_ranks - 1) / d.small_ranks : 0);
 

@@ -313,15 +313,15 @@ def test_objects_are_compiled_again_when_the_build_flags_change(tmp_path, monkey
 
 @pytest.fixture(scope="module")
 def small_ranks(tmp_path_factory):
-    """small_plan_ranks(pairs, layers, blocks of the largest layer, clusters of 1, 2, 4, 8, 16 CTAs that run at once)"""
+    """small_plan_ranks(pairs, layers, blocks of the largest layer, blocks, clusters of 1, 2, 4, 8, 16 CTAs that run at once)"""
     d = tmp_path_factory.mktemp("rule")
-    (d / "rule.cpp").write_text('#include "lq_small_rule.h"\nextern "C" int ranks(int64_t p, int64_t l, int64_t m, const int32_t* c) {\n'
-                                'lq::ClusterRoom r; for (int i = 0; i < 5; ++i) r.clusters[i] = c[i]; return lq::small_plan_ranks(p, l, m, 148, r); }\n')
+    (d / "rule.cpp").write_text('#include "lq_small_rule.h"\nextern "C" int ranks(int64_t p, int64_t l, int64_t m, int64_t b, const int32_t* c) {\n'
+                                'lq::ClusterRoom r; for (int i = 0; i < 5; ++i) r.clusters[i] = c[i]; return lq::small_plan_ranks(p, l, m, b, 148, r); }\n')
     subprocess.check_call(["g++", "-std=c++17", "-shared", "-fPIC", "-I", os.path.join(ROOT, "paper_2505_14371_b200", "csrc"),
                            str(d / "rule.cpp"), "-o", str(d / "rule.so")])
     f = ctypes.CDLL(str(d / "rule.so")).ranks
-    f.argtypes = [ctypes.c_int64] * 3 + [ctypes.POINTER(ctypes.c_int32)]
-    return lambda pairs, layers, most, room: f(pairs, layers, most, (ctypes.c_int32 * 5)(*room))
+    f.argtypes = [ctypes.c_int64] * 4 + [ctypes.POINTER(ctypes.c_int32)]
+    return lambda pairs, layers, most, blocks, room: f(pairs, layers, most, blocks, (ctypes.c_int32 * 5)(*room))
 
 
 WHOLE = (444, 222, 104, 48, 21)                                   # clusters that run at once on a whole B200
@@ -331,9 +331,22 @@ WHOLE = (444, 222, 104, 48, 21)                                   # clusters tha
 def test_small_plans_ask_for_clusters_that_the_device_has(small_ranks, room):
     for pairs in (1, 2, 9, 18, 19, 48, 49, 104, 105, 222, 223, 5000):
         for most in (0, 1, 2, 8, 9, 16, 17, 64, 100, 196, 208, 224, 225, 4000):
-            r = small_ranks(pairs, pairs, most, room)
-            assert r in (0, 1, 2, 4, 8, 16)
-            if most <= 8:
-                assert r >= 1                                     # a CTA a layer is always to be had
-            if r > 1 or most > 8 and r == 1:
-                assert room[r.bit_length() - 1] > 0 and most <= r * 13
+            for blocks in (pairs * most, min(pairs * most, 1000)):
+                r = small_ranks(pairs, pairs, most, blocks, room)
+                assert r in (0, 1, 2, 4, 8, 16)
+                if most <= 8:
+                    assert r >= 1                                 # a CTA a layer is always to be had
+                if r > 1 or most > 8 and r == 1:
+                    i = r.bit_length() - 1
+                    assert room[i] >= pairs and most <= r * (12 if r == 16 and blocks > 1024 else 13)
+
+
+def test_small_plans_of_a_whole_gpu(small_ranks):
+    ranks = lambda pairs, most, blocks, layers=None: small_ranks(pairs, layers or pairs, most, blocks, WHOLE)
+    assert ranks(16, 196, 804) == 16                              # a perceptron's layers, 4 workers
+    assert ranks(64, 1, 64) == 1 and ranks(10000, 8, 80000) == 1 and ranks(65536, 1, 65536, 65536) == 0
+    assert (ranks(1, 208, 208), ranks(1, 209, 209)) == (16, 0)    # 13 blocks a CTA, ...
+    assert (ranks(16, 192, 3072), ranks(16, 193, 3088)) == (16, 0)      # ... or 12 in clusters of 16 of larger plans
+    assert (ranks(48, 104, 4992), ranks(48, 105, 5040), ranks(49, 104, 5096)) == (8, 0, 0)
+    assert (ranks(104, 32, 3328), ranks(105, 32, 3360)) == (4, 0)
+    assert (ranks(222, 16, 3552), ranks(223, 16, 3568)) == (2, 0)
