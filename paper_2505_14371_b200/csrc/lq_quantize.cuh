@@ -231,16 +231,44 @@ __device__ __forceinline__ void normalise4(const float4& v, float r, float (&u)[
         : "=f"(u[0]), "=f"(u[1]), "=f"(u[2]), "=f"(u[3]) : "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "f"(r));
 }
 
+// The step search of a row's four coordinates: addresses of their {l_tau, gap}.  (The other searches are part of quantize_coord.)
+// Its steps are loads that wait for each other, so the four take them side by side.  One after the other, 33.5 M coordinates of
+// 8 workers, random levels: 8 bits 121 us, then with the values' signs taken off at every step 159; side by side 89 (7 bits 143 -> 79,
+// with histogram 176 -> 91; where no bin holds two levels, 67 and 68).
+template <int B, int kSearch>
+__device__ __forceinline__ void step_search4(const QuantEnv& ev, const SearchPar<kSearch>& sp, const float (&u)[4], uint32_t (&t8)[4])
+{
+    if constexpr (kSearch == kSearchStep) {
+        float mag[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            // (|u| <= 1 + 2^-23 gives bits(|u|) >> 17 <= 8128; the mask keeps the pattern of a NaN inside the table too)
+            t8[e] = ev.ld + 8u * lds_u8(((__float_as_uint(u[e]) >> 17) & 0x1FFFu) | ev.lut);
+            mag[e] = fabsf(u[e]);
+        }
+#pragma unroll 1
+        for (int s = 0; s < sp.par; ++s) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) t8[e] = add8_if_le(t8[e], lds_f32(t8[e] + 8u), mag[e]);
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) t8[e] = min(t8[e], ev.ld + 8u * (uint32_t)((1 << B) - 2));
+    } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) t8[e] = 0u;
+    }
+}
+
 // One coordinate: v -> symbol, added to the lane's words `cw` at position pp; its term of the step-size
 // statistic (Eq. general_stepsize: fp32 difference of the two decoded values, squared in fp64) added to `stat`.
-// u: v scaled by the layer's 1/N; x: the coordinate's Philox word.  Bucket scope: the value tables hold the plain signed levels and the row's
+// u: v scaled by the layer's 1/N; stepped: what step_search4 found; x: the coordinate's Philox word.  Bucket scope: the value tables hold the plain signed levels and the row's
 // norms (nrow now, pn in the previous message) scale them.  `counted`: the coordinate lies inside the layer
 // (histogram mode).
 // A search by one addition for a compare, a shifted pattern and a predicated addition, and products of pairs: 67 M coordinates of 8
 // workers, 4 bits, step 1395 -> 1365 us; 17 M of 4 workers, 5 bits, 269 -> 257; Transformer-XL 1982 -> 1954.  (Differences of pairs as
 // well: no faster; two coordinates side by side through the search: 28 bytes of spills, 1982 -> 2018 us.)
 template <int B, int kSearch, bool kHist, bool kStat, bool kBucket>
-__device__ __forceinline__ void quantize_coord(const QuantEnv& ev, const SearchPar<kSearch>& sp, float v, float u, uint32_t x, int pp,
+__device__ __forceinline__ void quantize_coord(const QuantEnv& ev, const SearchPar<kSearch>& sp, float v, float u, uint32_t stepped, uint32_t x, int pp,
                                                uint32_t (&cw)[B + 1], const uint32_t (&pw)[B + 1], double& stat,
                                                float nrow, float pn, bool counted)
 {
@@ -257,10 +285,7 @@ __device__ __forceinline__ void quantize_coord(const QuantEnv& ev, const SearchP
         const uint32_t e = lds_u32(((ub >> 17) & 0x1FFCu) | ev.lut);
         t8 = (((e + ub) >> 16) & 0x7F8u) | ev.ld;
     } else {
-        // (|u| <= 1 + 2^-23 gives bits(|u|) >> 17 <= 8128; the mask keeps the pattern of a NaN inside the table too)
-        t8 = ev.ld + 8u * lds_u8(((ub >> 17) & 0x1FFFu) | ev.lut);
-        for (int s = 0; s < sp.par; ++s) t8 = add8_if_le(t8, lds_f32(t8 + 8u), fabsf(u));
-        t8 = min(t8, ev.ld + 8u * (uint32_t)(n - 2));
+        t8 = stepped;
     }
     const float2 ld = lds_f32x2(t8);
     const float den = ld.y;

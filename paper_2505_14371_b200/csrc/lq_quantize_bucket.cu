@@ -168,12 +168,14 @@ __device__ __forceinline__ double quantize_block(const PlanDev& p, const PhiloxC
             const float vv[4] = {v.x, v.y, v.z, v.w};
             float u[4];
             normalise4(v, ev.r, u);
+            uint32_t t8[4];
+            step_search4<B>(ev, sp, u, t8);
             uint32_t x[4];
             philox4x32_10_folded(ctr0 + 32 * j, pc, p, x);
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const bool counted = !kHist || blk * kBlockCoords + 128 * j + 4 * lane + e < c.size;
-                quantize_coord<B, kSearch, kHist, true, true>(ev, sp, vv[e], u[e], x[e], 4 * j + e, cw, pw, stat, nrow, pn, counted);
+                quantize_coord<B, kSearch, kHist, true, true>(ev, sp, vv[e], u[e], t8[e], x[e], 4 * j + e, cw, pw, stat, nrow, pn, counted);
             }
         } else {
             pack_zero_row<C>(cw, j, ev.ld);

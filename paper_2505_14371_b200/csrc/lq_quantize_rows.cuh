@@ -60,10 +60,12 @@ __device__ __forceinline__ double quantize_rows(const PlanDev& p, const PhiloxCo
             const float vv[4] = {v.x, v.y, v.z, v.w};
             float u[4];
             normalise4(v, ev.r, u);
+            uint32_t t8[4];
+            step_search4<B>(ev, sp, u, t8);
             pack_first_row<C>(cw, ev.ld);
 #pragma unroll
             for (int e = 0; e < 4; ++e)
-                quantize_coord<B, kSearch, kHist, kStat, false>(ev, sp, vv[e], u[e], x[e], e, cw, pw, stat, 0.f, 0.f, pos + 4 * lane + e < job.size);
+                quantize_coord<B, kSearch, kHist, kStat, false>(ev, sp, vv[e], u[e], t8[e], x[e], e, cw, pw, stat, 0.f, 0.f, pos + 4 * lane + e < job.size);
             const uint32_t at = job.words + 4u * (uint32_t)(b * (C * 32) + lane + 32 * w0);
             asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(at), "r"(cw[0] << shift) : "memory");
             if (two) asm volatile("red.shared.or.b32 [%0+128], %1;" ::"r"(at), "r"(__funnelshift_l(cw[0], cw[1], shift)) : "memory");

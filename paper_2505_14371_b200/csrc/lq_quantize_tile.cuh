@@ -98,9 +98,11 @@ __device__ __forceinline__ double quantize_tile(const PlanDev& p, const PhiloxCo
                 const float vv[4] = {v.x, v.y, v.z, v.w};
                 float u[4];
                 normalise4(v, ev.r, u);
+                uint32_t t8[4];
+                step_search4<B>(ev, sp, u, t8);
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
-                    quantize_coord<B, kSearch, kHist, kStat, false>(ev, sp, vv[e], u[e], x[e], 4 * j + e, cw, pw, stat, 0.f, 0.f, true);
+                    quantize_coord<B, kSearch, kHist, kStat, false>(ev, sp, vv[e], u[e], t8[e], x[e], 4 * j + e, cw, pw, stat, 0.f, 0.f, true);
             } else {
                 if ((mnext >> j) & 1u) cp_async16(ring + 512u * j, nsrc + 128 * j, 16);
                 cp_async_commit();
