@@ -348,11 +348,27 @@ struct EncodeJob {
     uint8_t* rows;               // the blocks' rows that hold anything, kPartialRows for a partial block (shared memory)
     int64_t room;                // words of the stream buffer from `out` on
     int nblocks, rest;           // the tile's blocks; coordinates of its last one
-    uint32_t zero_bits;          // bits of the word of level 0; its pattern
-    uint32_t zero_code;
-    uint32_t code, buf;          // shared-memory addresses: the layer's table, this warp's buffer
+    const uint32_t* enc;         // the layer's words
+    uint32_t code, single, buf;  // shared-memory addresses: the layer's table, that of its single symbols, this warp's buffer
 };
 constexpr uint32_t kPartialRows = 0xfeu;       // (a partial block is looked at as a whole)
+
+// The layer's table, by all warps of the CTA: per symbol (2 * level + sign) the level's word, the sign bit behind it unless the level is
+// 0, and their length; per pair of symbols of up to kPairBits bits the same of both.
+__device__ __forceinline__ void make_code_table(const EncodeJob& J, int C)
+{
+    const uint32_t one = C <= kPairBits ? J.single : J.code, nsym = 1u << C;
+    for (uint32_t sym = threadIdx.x; sym < nsym; sym += kThreads) {
+        const uint32_t e = J.enc[sym >> 1], l = e >> 16;
+        sts_u32(one + 4u * sym, (sym >> 1) ? ((e & 0xffffu) | ((sym & 1u) << l) | ((l + 1u) << kLenShift)) : ((e & 0xffffu) | (l << kLenShift)));
+    }
+    __syncthreads();
+    if (C <= kPairBits) {
+        for (uint32_t i = threadIdx.x; i < nsym * nsym; i += kThreads)
+            sts_u32(J.code + 4u * i, join_entries(lds_u32(one + 4u * (i & (nsym - 1u))), lds_u32(one + 4u * (i >> C))));
+        __syncthreads();
+    }
+}
 
 // A warp's blocks of a tile for one symbol width (its own function per width, so that each is compiled with
 // its own register budget).  kWrite = false: every lane's bits, the block's words and its rows.  true: the blocks are written,
@@ -364,7 +380,6 @@ __device__ __noinline__ void encode_blocks(const EncodeJob J)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int partial = J.rest < kBlockCoords ? J.nblocks - 1 : -1;
-    const bool quick_zero = J.zero_code == 0u;
     uint32_t next[C];
     auto request = [&](int b) {
         if (b >= J.nblocks) return;
@@ -372,20 +387,21 @@ __device__ __noinline__ void encode_blocks(const EncodeJob J)
 #pragma unroll
         for (int i = 0; i < C; ++i) next[i] = kWrite ? __ldcs(from + i * 32) : __ldcg(from + i * 32);
     };
+    if (!kWrite) { request(warp); make_code_table(J, C); }
+    const uint32_t zero = lds_u32(C <= kPairBits ? J.single : J.code), zero_bits = zero >> kLenShift, zero_code = zero & kCodeMask;    // the word of level 0
     if (!kWrite) {
-        request(warp);
         for (int b = warp; b < J.nblocks; b += kWarps) {
             uint32_t w[C + 1], any = 0;
 #pragma unroll
             for (int i = 0; i < C; ++i) { w[i] = next[i]; any |= w[i]; }
             w[C] = 0u;
             request(b + kWarps);
-            uint32_t rows = 0, total = 32u * J.zero_bits * 32u;
+            uint32_t rows = 0, total = 32u * zero_bits * 32u;
             if (b == partial || __any_sync(0xffffffffu, any != 0u)) {
                 uint32_t bits;
                 if (b != partial) {
                     rows = rows_of<C>(w);
-                    bits = lane_bits<C>(J.code, w, rows, J.zero_bits);
+                    bits = lane_bits<C>(J.code, w, rows, zero_bits);
                 } else {
                     rows = kPartialRows;
                     bits = lane_bits_partial<C>(J.code, w, real_positions(J.rest, lane));
@@ -397,6 +413,7 @@ __device__ __noinline__ void encode_blocks(const EncodeJob J)
         }
         return;
     }
+    const bool quick_zero = zero_code == 0u;
     // blocks without rows, where level 0's word is all zeros (untouched rows), are so many zero words
     auto loaded = [&](int b) { return b < J.nblocks && !(quick_zero && J.rows[b] == 0u); };
     if (loaded(warp)) request(warp);
@@ -409,12 +426,12 @@ __device__ __noinline__ void encode_blocks(const EncodeJob J)
         if (loaded(b + kWarps)) request(b + kWarps);
         uint32_t* out = J.out + first + lane;
         if (rows == 0u && quick_zero) {
-            if (J.runs && (lane & 3) == 0) J.runs[b * LQ_CODE_RUNS + (lane >> 2)] = (uint16_t)(32u * J.zero_bits * lane);
-            if ((int64_t)first + 32 * J.zero_bits <= J.room)       // a stream buffer that is too small is never overrun
-                for (uint32_t i = 0; i < J.zero_bits; ++i) __stcs(out + 32 * i, 0u);
+            if (J.runs && (lane & 3) == 0) J.runs[b * LQ_CODE_RUNS + (lane >> 2)] = (uint16_t)(32u * zero_bits * lane);
+            if ((int64_t)first + 32 * zero_bits <= J.room)       // a stream buffer that is too small is never overrun
+                for (uint32_t i = 0; i < zero_bits; ++i) __stcs(out + 32 * i, 0u);
             continue;
         }
-        const uint32_t bits = rows == 0u ? 32u * J.zero_bits : (uint32_t)J.lane_bits[b * 32 + lane];
+        const uint32_t bits = rows == 0u ? 32u * zero_bits : (uint32_t)J.lane_bits[b * 32 + lane];
         uint32_t incl = bits;                                // inclusive prefix sum over the lanes
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -427,7 +444,7 @@ __device__ __noinline__ void encode_blocks(const EncodeJob J)
         // eight runs of a block at once
         if (J.runs && (lane & 3) == 0) J.runs[b * LQ_CODE_RUNS + (lane >> 2)] = (uint16_t)pos;
         if (b != partial) {
-            emit_full<C>(J.code, w, lane, pos, J.buf, rows, J.zero_bits, J.zero_code);
+            emit_full<C>(J.code, w, lane, pos, J.buf, rows, zero_bits, zero_code);
         } else {
             for (uint32_t i = lane; i < nwords; i += 32) sts_u32(J.buf + 4u * i, 0u);
             __syncwarp();
@@ -510,32 +527,19 @@ __global__ void __launch_bounds__(kThreads, 5) entropy_encode_kernel(PlanDev p, 
     const Tile T = p.tiles[t];
     const int layer = T.layer, lane = threadIdx.x & 31;
     const LayerDesc L = p.layers[layer];
-    // per symbol (2 * level + sign): the level's word, the sign bit behind it unless the level is 0, and their length
-    const int C = L.bits + 1, nsym = 1 << C;
+    const int C = L.bits + 1;
     const uint32_t entries = C <= kPairBits ? 1u << (2 * C) : 1u << C;
     const uint32_t align = C == kPairBits ? 16u : 4u * entries;
     const uint32_t smem = (uint32_t)__cvta_generic_to_shared(enc_smem), code_at = (smem + align - 1u) & ~(align - 1u);
-    uint32_t* code = reinterpret_cast<uint32_t*>(enc_smem + (code_at - smem));
-    uint32_t* one = C <= kPairBits ? single : code;
-    for (int sym = threadIdx.x; sym < nsym; sym += blockDim.x) {
-        const uint32_t e = enc_tables[(int64_t)layer * kMaxLevels + (sym >> 1)], l = e >> 16;
-        one[sym] = (sym >> 1) ? ((e & 0xffffu) | ((uint32_t)(sym & 1) << l) | ((l + 1u) << kLenShift)) : ((e & 0xffffu) | (l << kLenShift));
-    }
-    __syncthreads();
-    const uint32_t zero = one[0];
-    if (C <= kPairBits) {
-        for (int i = threadIdx.x; i < 1 << (2 * C); i += blockDim.x) code[i] = join_entries(single[i & (nsym - 1)], single[i >> C]);
-        __syncthreads();
-    }
     EncodeJob J;
     J.msg = packed + (int64_t)k * p.packed_words + L.word_off + T.block0 * (int64_t)C * 32;
     J.runs = run_offsets ? run_offsets + ((int64_t)k * p.total_blocks + L.block_off + T.block0) * LQ_CODE_RUNS : nullptr;
     J.lane_bits = lane_bits; J.words = words; J.rows = rows;
     J.nblocks = T.nblocks;
     J.rest = (int)min((int64_t)kBlockCoords, L.size - (T.block0 + T.nblocks - 1) * (int64_t)kBlockCoords);
-    J.zero_bits = zero >> kLenShift; J.zero_code = zero & kCodeMask;
     J.out = nullptr; J.room = 0;
-    J.code = code_at; J.buf = smem + code_bytes + (threadIdx.x >> 5) * (kCodeBufWords * 4);
+    J.enc = enc_tables + (int64_t)layer * kMaxLevels;
+    J.code = code_at; J.single = (uint32_t)__cvta_generic_to_shared(single); J.buf = smem + code_bytes + (threadIdx.x >> 5) * (kCodeBufWords * 4);
 #define LQ_BLOCKS(WRITE)                                                                                                  \
     switch (C) {                                                                                                          \
         case 2: encode_blocks<2, WRITE>(J); break; case 3: encode_blocks<3, WRITE>(J); break;                             \
