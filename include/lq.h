@@ -276,7 +276,7 @@ int lq_symbol_counts(const lq_plan* plan, const uint32_t* packed, uint32_t* coun
  *                   (four lanes) start: side data of 16 bytes per block (1/8 bit per coordinate) that is not part of
  *                   the stream and lets the decoder work on the eight runs of a block in parallel.
  *                   The call uses scratch that the plan allocates at the first use of the stage (8 bytes per worker and
- *                   tile of 8 to 128 blocks): two encodes of one plan must not overlap on the GPU.  The tiles are
+ *                   tile of 8 to 128 blocks, and 65 per worker and block where the layers' code widths take turns): two encodes of one plan must not overlap on the GPU.  The tiles are
  *                   encoded side by side, and each waits for the words that the ones before it take.  If these do not
  *                   come (the GPU stopped for seconds, or encodes that overlap), the tile gives up: the offsets of its
  *                   blocks, and the worker's length if it is the last tile, become 0xffffffff, which a decode reports

@@ -86,7 +86,7 @@ struct lq_plan {
     uint16_t* d_code_dec = nullptr;        // [L][kDecEntries]
     bool codes_ready = false;              // ... and all of the following allocated, the tables made
     uint32_t* d_code_bad = nullptr;        // [1] LQ_CODE_BROKEN from a decode, LQ_CODE_GAVE_UP from an encode
-    EncodeScratch code_scratch{nullptr, 0, kMostLooks};   // allocated with the tables
+    EncodeScratch code_scratch{nullptr, 0, kMostLooks, false, {nullptr, nullptr}};   // allocated with the tables
     std::vector<uint8_t> code_len;         // [L][256] host copy of the word lengths
     double alt_qhat = 0.0;         // > 0: qoda_step follows Eq. (Alt) with this exponent
     double* xsum = nullptr;        // caller-owned running sum of the half iterates (qoda_set_average), or NULL
@@ -111,7 +111,7 @@ void free_plan(lq_plan* p)
     cudaFree(p->d_levels_stage); cudaFree(p->d_levels_enc[0]); cudaFree(p->d_levels_enc[1]);
     cudaFree(p->search.lut); cudaFree(p->search.ld); cudaFree(p->search.how);
     cudaFree(p->dev.norm_partial); cudaFree(p->dev.stat_partial); cudaFree(p->dev.sq_diff);
-    cudaFree(p->dev.rnorm); cudaFree(p->dev.status); cudaFree(p->dev.scalars); cudaFree(p->d_code_enc); cudaFree(p->d_code_dec); cudaFree(p->d_code_bad); cudaFree(p->code_scratch.states); cudaFree(p->d_member_off); cudaFree(p->d_member_layer); cudaFree(p->dev.alt_partial); cudaFree(p->dev.layer_total); cudaFree(p->d_row_mask[0]); cudaFree(p->d_row_mask[1]);
+    cudaFree(p->dev.rnorm); cudaFree(p->dev.status); cudaFree(p->dev.scalars); cudaFree(p->d_code_enc); cudaFree(p->d_code_dec); cudaFree(p->d_code_bad); cudaFree(p->code_scratch.states); cudaFree(p->code_scratch.sized.lane_bits); cudaFree(p->code_scratch.sized.rows); cudaFree(p->d_member_off); cudaFree(p->d_member_layer); cudaFree(p->dev.alt_partial); cudaFree(p->dev.layer_total); cudaFree(p->d_row_mask[0]); cudaFree(p->d_row_mask[1]);
     cudaFree(p->dev.energy_partial); cudaFree(p->dev.flag_partial); cudaFree(p->dev.layer_weight);
     for (auto& r : p->prof_recs) { cudaEventDestroy(r.a); cudaEventDestroy(r.b); }
     for (auto e : p->prof_pool) cudaEventDestroy(e);
@@ -835,6 +835,20 @@ int ensure_codes(lq_plan* plan)
     if (!plan->code_scratch.states) LQ_CUDA(dev_alloc_zero(&plan->code_scratch.states, states));
     plan->code_scratch.bytes = states * sizeof(uint64_t);
     try {
+        int64_t runs = 0;
+        uint32_t seen = 0;
+        for (size_t i = 0; i < plan->tiles.size(); ++i) {
+            const int b = plan->layers[(size_t)plan->tiles[i].layer].bits;
+            runs += i == 0 || plan->layers[(size_t)plan->tiles[i - 1].layer].bits != b;
+            seen |= 1u << b;
+        }
+        plan->code_scratch.by_width = entropy_by_width((int64_t)plan->dev.num_tiles * plan->dev.num_workers,
+                                                       plan->dev.total_blocks * plan->dev.num_workers, __builtin_popcount(seen), runs);
+        if (plan->code_scratch.by_width) {
+            const size_t KB = (size_t)plan->dev.num_workers * (size_t)plan->dev.total_blocks;
+            if (!plan->code_scratch.sized.lane_bits) LQ_CUDA(dev_alloc_zero(&plan->code_scratch.sized.lane_bits, KB * 32));
+            if (!plan->code_scratch.sized.rows) LQ_CUDA(dev_alloc_zero(&plan->code_scratch.sized.rows, KB));
+        }
         plan->code_len.assign(L * kMaxLevels, 0);
         std::vector<uint32_t> enc(L * kMaxLevels, 0);
         for (int m = 0; m < plan->dev.num_layers; ++m) {

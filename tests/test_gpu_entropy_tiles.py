@@ -127,3 +127,54 @@ def test_tiles_that_give_up_say_so(sizes):
     assert plan.lq_entropy_status() == 0 and all(torch.equal(a, b) for a, b in zip(again, whole))
     with pytest.raises(lqm.LqError):
         plan.lq_entropy_wait(-1)
+
+
+@pytest.mark.parametrize("by_width, layers, K, widths, runs", [
+    (True, 131, 8, [1, 2, 3, 4, 5, 6, 7, 8], 1), (False, 130, 8, [1, 2, 3, 4, 5, 6, 7, 8], 1), (True, 300, 12, [2, 3, 4, 8], 3),
+    (False, 300, 12, [2, 3, 4, 8], 20), (False, 360, 12, [7, 6], 1)])
+def test_streams_of_plans_of_several_widths(orc, by_width, layers, K, widths, runs):
+    """Plans on both sides of the rule's lines; layers of one block and a few, each with a code of its own."""
+    import paper_2505_14371_b200 as lqm
+    lqm.load_library()
+    rng = np.random.default_rng(layers)
+    sizes = [int(x) for x in rng.choice([1, 31, 200, 1023], layers)]
+    sizes[3] = 19 * 1024 + 5
+    bits = [widths[m // runs % len(widths)] for m in range(layers)]
+    plan = lqm.Plan(sizes, bits, 2, K, 11)
+    gen = torch.Generator(device="cuda").manual_seed(layers)
+    grads = torch.randn((K, plan.padded_elems), generator=gen, device="cuda") ** 3
+    grads.view(K, -1, 32)[:, ::3] = 0.0
+    grads[:, plan.elem_offsets[3] + 2048: plan.elem_offsets[3] + 6144] = 0.0
+    packed, norms = plan.empty_packed(), plan.empty_norms()
+    plan.lq_quantize_pack(grads, 1, packed, norms)
+    codes = []
+    for m, b in enumerate(bits):
+        codes.append(lqm.lq_code_build([0.3 + 0.7 * (m % 2)] + [0.5 ** min(j, 3 + m % 8) for j in range(1, 1 << b)]))
+        plan.lq_code_set(m, codes[m])
+    stream = torch.full((K, plan.lq_plan_blocks() * 416), -1, dtype=torch.int32, device="cuda")
+    offs, runs_at = torch.zeros((K, plan.lq_plan_blocks() + 1), dtype=torch.int32, device="cuda"), plan.empty_run_offsets()
+    plan.lq_entropy_wait(0)                                  # only tiles in stream order wait for others
+    plan.lq_entropy_encode(packed, stream, offs, runs_at)
+    assert plan.lq_entropy_status() == (0 if by_width else lqm.CODE_GAVE_UP)
+    plan.lq_entropy_wait()
+    stream.fill_(-1)
+    for _ in range(2):
+        plan.lq_entropy_encode(packed, stream, offs, runs_at)
+    pk, S, O = packed.cpu().numpy().view(np.uint32), stream.cpu().numpy().view(np.uint32), offs.cpu().numpy().astype(np.int64)
+    for k in range(K):
+        pos = g = 0
+        for m, d in enumerate(sizes):
+            at, l = plan.word_offsets[m], np.uint8(codes[m])
+            idx, sg = orc.unpack_layer(pk[k, at: at + orc.packed_words(d, bits[m])], d, bits[m])
+            c = orc.canonical_codes(l)
+            for lo in range(0, d, 1024):
+                words, _ = orc.entropy_encode_block(idx[lo: lo + 1024], sg[lo: lo + 1024], l, c)
+                assert O[k, g] == pos and np.array_equal(S[k, pos: pos + words.size], words), (k, m, lo)
+                pos += words.size
+                g += 1
+        assert O[k, g] == pos and np.all(S[k, pos:] == 0xffffffff)
+    back, again = torch.full_like(packed, -1), torch.full_like(stream, -1)
+    plan.lq_entropy_decode(stream, offs, back, runs_at)
+    assert plan.lq_entropy_status() == 0
+    plan.lq_entropy_encode(back, again, offs, runs_at)
+    assert torch.equal(again, stream)
