@@ -1,4 +1,4 @@
-"""The entropy encoder where its tiles meet: plans of fewer and of more tiles than a tile looks back over at a time, so that a
+"""The entropy encoder where its tiles meet: tiles of 8 to 128 blocks, of one block a warp and many; plans of fewer and of more tiles than a tile looks back over at a time, so that a
 tile's place in the stream comes from one or several looks; blocks with rows of zeros under codes whose word for level 0 is
 one zero bit, several, or not zeros at all.  Every block of every worker against the oracle's encoder, and the way back."""
 import numpy as np
@@ -14,7 +14,7 @@ def _code(lqm, kind, n):
     return [n.bit_length() - 1] * n if kind == "flat" else lqm.lq_code_build([0.9] + [0.1 / n] * (n - 1))
 
 
-@pytest.mark.parametrize("bits, kind", [(1, "fitted"), (2, "zero_long"), (3, "flat"), (4, "fitted"), (5, "zero_long"), (8, "flat")])
+@pytest.mark.parametrize("bits, kind", [(1, "fitted"), (2, "zero_long"), (3, "flat"), (4, "fitted"), (5, "zero_long"), (6, "fitted"), (7, "zero_long"), (8, "flat")])
 @pytest.mark.parametrize("layers", [1, 32, 33, 70])
 def test_streams_of_many_tiles(orc, layers, bits, kind):
     import paper_2505_14371_b200 as lqm
@@ -177,4 +177,74 @@ def test_streams_of_plans_of_several_widths(orc, by_width, layers, K, widths, ru
     plan.lq_entropy_decode(stream, offs, back, runs_at)
     assert plan.lq_entropy_status() == 0
     plan.lq_entropy_encode(back, again, offs, runs_at)
+    assert torch.equal(again, stream)
+
+
+def _sampled_blocks_match(orc, plan, packed, stream, offs, runs, codes, rng, count):
+    """`count` random blocks of every worker, and the first and last of every layer, against the oracle's encoder; all sizes of
+    blocks add up, in the order of the stream."""
+    S, O, R = stream.cpu().numpy().view(np.uint32), offs.cpu().numpy().astype(np.int64), runs.cpu().numpy().view(np.uint16)
+    blocks = [(m, i) for m, d in enumerate(plan.layer_sizes) for i in range(-(-d // 1024))]
+    ends = [g for g, (m, i) in enumerate(blocks) if i == 0 or g + 1 == len(blocks) or blocks[g + 1][0] != m]
+    assert np.all(O[:, 0] == 0) and np.all(np.diff(O, axis=1) >= 0)
+    for k in range(plan.num_workers):
+        pk = packed[k].cpu().numpy().view(np.uint32)
+        for g in {*ends, *(int(x) for x in rng.integers(0, len(blocks), count))}:
+            m, i = blocks[g]
+            b, d = plan.bits[m], min(1024, plan.layer_sizes[m] - 1024 * i)
+            at, l = plan.word_offsets[m] + i * 32 * (b + 1), np.uint8(codes[m])
+            idx, sg = orc.unpack_layer(pk[at: at + 32 * (b + 1)], d, b)
+            words, _ = orc.entropy_encode_block(idx, sg, l, orc.canonical_codes(l))
+            assert O[k, g + 1] - O[k, g] == words.size and np.array_equal(S[k, O[k, g]: O[k, g + 1]], words), (k, m, i)
+            # a lane's 32 coordinates are one after the other in the stream: where every fourth lane starts
+            size = np.where(idx > 0, l[idx].astype(np.int64) + 1, int(l[0]))
+            c = np.arange(d)
+            lane = (c // 4) % 32
+            per_lane = np.bincount(lane, weights=size, minlength=32).astype(np.int64)
+            assert np.array_equal(R[k, g], np.concatenate([[0], np.cumsum(per_lane)])[:32:4])
+        assert np.all(S[k, O[k, -1]:] == 0xffffffff)
+
+
+@pytest.mark.parametrize("sizes, bits, K, tile, kind", [
+    ([620 * 1024 + 5, 33], 4, 8, 8, "fitted"), ([1300 * 1024 + 1], 6, 8, 16, "zero_long"), ([140 * 1024 - 1] * 40, 7, 2, 16, "fitted"),
+    ([4352 * 1024 + 300, 5000], 2, 8, 32, "fitted"), ([3000 * 1024 - 100], 8, 8, 32, "fitted"), ([33000 * 1024 + 700], 3, 8, 64, "flat"),
+    ([33000 * 1024 - 100], 4, 16, 128, "fitted")])
+def test_tiles_of_many_blocks(orc, sizes, bits, K, tile, kind):
+    """Tiles of every length that plans have, more of them than CTAs run at once, with a partial one at the end: each warp takes
+    block after block, whole blocks of zeros between others of the same warp (8 blocks on) and two in a row among them."""
+    import paper_2505_14371_b200 as lqm
+    lqm.load_library()
+    plan = lqm.Plan(sizes, bits, 2, K, 5 + bits)
+    gen = torch.Generator(device="cuda").manual_seed(bits)
+    grads = torch.empty((K, plan.padded_elems), device="cuda")
+    for k in range(K):
+        grads[k].normal_(generator=gen).pow_(3)
+    grads.view(K, -1, 32)[:, ::5] = 0.0
+    whole = grads[:, : plan.padded_elems // 8192 * 8192].view(K, -1, 8, 1024)           # [.., warp, coordinate]
+    whole[:, 1::4, 2:5] = 0.0                                # a warp's every fourth block
+    whole[:, 2::4, 3:6] = 0.0                                # and the next one: two in a row
+    packed, norms = plan.empty_packed(), plan.empty_norms()
+    plan.lq_quantize_pack(grads, 1, packed, norms)
+    del grads, whole
+    lengths = _code(lqm, kind, 1 << bits)
+    for m in range(len(sizes)):
+        plan.lq_code_set(m, lengths)
+    blocks = plan.lq_plan_blocks()
+    length = 128                                             # the length of the plan's tiles
+    while length > 32 and blocks // length * K < 4096:
+        length //= 2
+    while length > 8 and blocks // length * K < 592:
+        length //= 2
+    assert length == tile
+    words = max(lengths) + 1
+    stream = torch.full((K, blocks * 32 * words), -1, dtype=torch.int32, device="cuda")
+    offs, runs = torch.zeros((K, blocks + 1), dtype=torch.int32, device="cuda"), plan.empty_run_offsets()
+    for _ in range(2):
+        plan.lq_entropy_encode(packed, stream, offs, runs)
+    assert plan.lq_entropy_status() == 0
+    _sampled_blocks_match(orc, plan, packed, stream, offs, runs, [lengths] * len(sizes), np.random.default_rng(bits), 60)
+    back, again = torch.full_like(packed, -1), torch.full_like(stream, -1)
+    plan.lq_entropy_decode(stream, offs, back, runs)
+    assert plan.lq_entropy_status() == 0
+    plan.lq_entropy_encode(back, again, offs, runs)
     assert torch.equal(again, stream)
