@@ -154,7 +154,6 @@ __global__ void __launch_bounds__(kQThreads, 4) quantize_pack_kernel(
 
     WarpCtx c;
     c.g = fresh(grads + (int64_t)kk * p.padded_elems + L.elem_off);
-    c.size = L.size;
     c.nfull = L.size / kBlockCoords;
     c.lane = lane;
     QuantEnv ev;

@@ -272,7 +272,7 @@ __device__ __forceinline__ void quantize_coord(const QuantEnv& ev, const SearchP
                                                uint32_t (&cw)[B + 1], const uint32_t (&pw)[B + 1], double& stat,
                                                float nrow, float pn, bool counted)
 {
-    constexpr int n = 1 << B, C = B + 1;
+    constexpr int C = B + 1;
     // |u| <= 1 + 2^-23 always (N >= |v| and one rounding each in 1/N and the product), and such a u
     // behaves exactly like u = 1 below, so the min(u, 1) of the definition is not needed
     const uint32_t ub = __float_as_uint(u);                  // (the searches leave the sign out)

@@ -9,7 +9,6 @@ namespace lq {
 // Everything a warp needs to walk its blocks of one (tile, worker).
 struct WarpCtx {
     const float* g;              // first coordinate of the layer in this worker's row
-    int64_t size;                // d_m
     int64_t nfull;               // blocks below this index lie wholly inside the layer
     int lane;
 };
