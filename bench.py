@@ -41,11 +41,11 @@ KERNEL_SOURCES = {"norm_partial": ["lq_norm.cu", "lq_internal.cuh"],
                   "quantize_pack": ["lq_quantize.cu", "lq_quantize_tile.cuh", "lq_quantize_rows.cuh", "lq_quantize.cuh", "lq_internal.cuh"],
                   "decode": ["lq_decode.cu", "lq_internal.cuh"]}
 NCU_SCALED = {"transformer_xl": {          # kernel: bytes per embedding / other worker-coordinate, warp instr likewise
-    "norm_partial": {"bytes": (4.0063, 4.0087), "inst": (0.15735, 0.17059), "sources": "ef7e30f7939bb94e"},
-    "quantize_pack": {"bytes": (1.2880, 5.2472), "inst": (0.21352, 1.19445), "sources": "c6377c45b8a58006"},
-    "decode": {"bytes": (2.0844, 2.5285), "inst": (0.12434, 0.21056), "sources": "c5c4255238a4cc86"}}}
+    "norm_partial": {"bytes": (4.0068, 4.0088), "inst": (0.15735, 0.17059), "sources": "f7a182d6d9a4aff3"},
+    "quantize_pack": {"bytes": (1.2854, 5.2480), "inst": (0.21387, 1.19539), "sources": "f084df386005b756"},
+    "decode": {"bytes": (2.0869, 2.5263), "inst": (0.12434, 0.21056), "sources": "438874de34dc6b49"}}}
 NCU_DIRECT = {"flat:26:4:8:2": {           # kernel: bytes and warp instructions of one launch
-    "quantize_pack": {"bytes": 2484451584.0 + 322569472.0, "inst": 630599680.0, "sources": "c6377c45b8a58006"}}}
+    "quantize_pack": {"bytes": 2484299776.0 + 323197440.0, "inst": 631123968.0, "sources": "f084df386005b756"}}}
 DENSE_POINT = "flat:26:4:8:2"             # dense companion of the headline workload: no zero rows to skip
 ISSUE_PEAK = 148 * 4 * 1.965e9            # warp instructions per second: 148 SMs x 4 schedulers x 1 per clock at 1965 MHz
 

@@ -136,7 +136,8 @@ __device__ __forceinline__ uint32_t value_addr(const uint32_t (&w)[C], int p, ui
 }
 
 // Adds a unit's workers to the sums of rows row0 .. row0 + kRows - 1, in worker order.  Two neighbours are added by one
-// instruction: 33.6 M coordinates of 16 workers at 2 bits 102.7 -> 100.5 us (80 % of the issue slots are used).
+// instruction: 33.6 M coordinates of 16 workers at 2 bits 102.7 -> 100.5 us (75 % of the issue slots are used, 5.1 warp
+// instructions per 32 symbols).
 // A clear bit of `live`: that worker's block is all zero words, which would add +0 to sums that are never -0.
 // Of 2 rows (row0 = 2 x the warp) the words are first moved so that they start with the rows' symbols: the warps run the same code,
 // which in such small grids takes longer to fetch than to run (8192 coordinates, 8 workers: the step 12.0 -> 10.0 us; 203 530 and

@@ -390,13 +390,16 @@ constexpr int kByTicket = 0, kSizes = 1, kPlaced = 2;
 
 // One warp per block, one CTA per tile (up to 128 blocks of one layer; on 32 the CTA's tables took longer than its blocks): the
 // blocks are sized, the tile tells its words to the tiles behind it and learns where it starts itself, and the blocks are written.
-// The tile's words are read a second time for that, from L2: 888 CTAs hold 80 KB each at 4 bits, 71 of its 126 MB.  Tiles are
-// taken from a counter in stream order, so that a tile only waits for tiles that run already.
-// What bounds it is instructions and, at the CTA's barriers, the warps that wait for each other (62 % of the issue slots are used).  Against a sizing pass, a scan and a writing
-// pass, each over the whole message: Transformer-XL message (755 MB in, 291 MB out, 8 workers) 598 -> 568 us, 67 M coordinates at
-// 3 bits 65.6 -> 57.3 us and at 8 bits 99.5 -> 91.5, 120 000 coordinates 18.5 -> 9.9 us (two launches instead of four).
-// 5 CTAs per SM: with 6 (40 registers) 60.5 and 98.8 us at 3 and 8 bits, the same on the large message.  Blocks dealt out as warps
-// come for them, against the waiting: 618 us, as the requests then follow a shared counter's answer.
+// The tile's words are read a second time for that, from L2: the 740 CTAs that run at a time hold 80 KB each at 4 bits, 59 of its
+// 126 MB, and 144 KB at 8, 107.  Tiles are taken from a counter in stream order, so that a tile only waits for tiles that run already.
+// What bounds it is instructions (59 % of the issue slots are used) and, at the CTA's barriers, the warps that wait for each other (the
+// largest stall, 2.9 per issue).  Against a sizing pass, a scan and a writing pass, each over the whole message: Transformer-XL message (755 MB
+// in, 291 MB out, 8 workers) 598 -> 568 us, 67 M coordinates at 3 bits 65.6 -> 57.3 us and at 8 bits 99.5 -> 91.5, 120 000 coordinates 18.5
+// -> 9.9 us (two launches instead of four).  The table of codes is made by the width's own code, behind the request of the first block:
+// 400 layers of up to 8 blocks, 64 workers 209 -> 196 us.
+// 5 CTAs per SM: with 6 (40 registers) 60.5 and 98.8 us at 3 and 8 bits, the same on the large message (by width, 512 layers of widths 1 to 8
+// in turn, 114 and 117).  Blocks dealt out as warps come for them, against the waiting: 618 us, as the requests then follow a shared
+// counter's answer.  A record per tile in stream order in place of tile and layer: 571 -> 585 us.
 template <int kMode>
 __global__ void __launch_bounds__(kThreads, 5) entropy_encode_kernel(PlanDev p, const uint32_t* __restrict__ packed,
                                                                      const uint32_t* __restrict__ enc_tables,

@@ -233,9 +233,9 @@ __device__ __forceinline__ void normalise4(const float4& v, float r, float (&u)[
 
 // The step search of a row's four coordinates: addresses of their {l_tau, gap}.  (The other searches are part of quantize_coord.)
 // Its steps are loads that wait for each other, so the four take them side by side.  One after the other, 33.5 M coordinates of
-// 8 workers, random levels: 8 bits 121 us, then with the values' signs taken off at every step 159; side by side 89 (7 bits 143 -> 79,
-// with histogram 176 -> 91; where no bin holds two levels, 67 and 68).
-template <int B, int kSearch>
+// 8 workers, random levels: 8 bits 121 us, then with the values' signs taken off at every step 159; side by side 97 (7 bits 143 -> 79,
+// with histogram 177 -> 88; where no bin holds two levels, 66 and 66).
+template <int B, bool kHist, int kSearch>
 __device__ __forceinline__ void step_search4(const QuantEnv& ev, const SearchPar<kSearch>& sp, const float (&u)[4], uint32_t (&t8)[4])
 {
     if constexpr (kSearch == kSearchStep) {
@@ -245,6 +245,7 @@ __device__ __forceinline__ void step_search4(const QuantEnv& ev, const SearchPar
             // (|u| <= 1 + 2^-23 gives bits(|u|) >> 17 <= 8128; the mask keeps the pattern of a NaN inside the table too)
             t8[e] = ev.ld + 8u * lds_u8(((__float_as_uint(u[e]) >> 17) & 0x1FFFu) | ev.lut);
             mag[e] = fabsf(u[e]);
+            if (kHist) asm("" : "+f"(mag[e]));       // (a register of its own: 4 bits, 33.5 M coordinates 72.1 -> 70.2 us)
         }
 #pragma unroll 1
         for (int s = 0; s < sp.par; ++s) {

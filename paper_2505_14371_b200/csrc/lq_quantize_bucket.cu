@@ -169,7 +169,7 @@ __device__ __forceinline__ double quantize_block(const PlanDev& p, const PhiloxC
             float u[4];
             normalise4(v, ev.r, u);
             uint32_t t8[4];
-            step_search4<B>(ev, sp, u, t8);
+            step_search4<B, kHist>(ev, sp, u, t8);
             uint32_t x[4];
             philox4x32_10_folded(ctr0 + 32 * j, pc, p, x);
 #pragma unroll

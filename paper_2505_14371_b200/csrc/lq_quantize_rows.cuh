@@ -61,7 +61,7 @@ __device__ __forceinline__ double quantize_rows(const PlanDev& p, const PhiloxCo
             float u[4];
             normalise4(v, ev.r, u);
             uint32_t t8[4];
-            step_search4<B>(ev, sp, u, t8);
+            step_search4<B, kHist>(ev, sp, u, t8);
             pack_first_row<C>(cw, ev.ld);
 #pragma unroll
             for (int e = 0; e < 4; ++e)

@@ -98,7 +98,7 @@ __device__ __forceinline__ double quantize_tile(const PlanDev& p, const PhiloxCo
                 float u[4];
                 normalise4(v, ev.r, u);
                 uint32_t t8[4];
-                step_search4<B>(ev, sp, u, t8);
+                step_search4<B, kHist>(ev, sp, u, t8);
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
                     quantize_coord<B, kSearch, kHist, kStat, false>(ev, sp, vv[e], u[e], t8[e], x[e], 4 * j + e, cw, pw, stat, 0.f, 0.f, true);
@@ -125,8 +125,19 @@ __device__ __forceinline__ double quantize_tile(const PlanDev& p, const PhiloxCo
     return stat;
 }
 
-// The whole blocks of a layer of width B.
+// The step search out of line, which leaves the other searches of the widest code more registers: 201 M coordinates, uniform levels, step
+// 736 -> 723 us (random levels, 33.5 M: encoder 89 -> 97).  Widths below gain nothing by it (7 bits, uniform 66 and 68, random 79 and 94), nor does the
+// kernel of all widths (widths 2, 3, 4 and 8, 512 layers, step 2345 -> 2365).
 template <int B, bool kHist, bool kStat>
+__device__ __noinline__ double quantize_tile_steps(const PlanDev& p, const PhiloxConsts pc, const WarpCtx c, const Tile tile, uint32_t* out,
+                                                   const uint32_t* prev, const QuantEnv ev, const uint8_t* rows_cur, const uint8_t* rows_prev,
+                                                   uint32_t ring_base)
+{
+    return quantize_tile<B, kSearchStep, kHist, kStat>(p, pc, c, tile, out, prev, ev, rows_cur, rows_prev, ring_base);
+}
+
+// The whole blocks of a layer of width B.
+template <int B, int kWidth, bool kHist, bool kStat>
 __device__ __forceinline__ double quantize_width(const PlanDev& p, const PhiloxConsts& pc, const WarpCtx& c, const Tile& tile, int search,
                                                  uint32_t* __restrict__ out, const uint32_t* __restrict__ prev, const QuantEnv& ev,
                                                  const uint8_t* rows_cur, const uint8_t* rows_prev, uint32_t ring_base)
@@ -137,7 +148,10 @@ __device__ __forceinline__ double quantize_width(const PlanDev& p, const PhiloxC
     if constexpr (B >= kWindowBits)
         if (search == kSearchWindow)
             return quantize_tile<B, kSearchWindow, kHist, kStat>(p, pc, c, tile, out, prev, ev, rows_cur, rows_prev, ring_base);
-    return quantize_tile<B, kSearchStep, kHist, kStat>(p, pc, c, tile, out, prev, ev, rows_cur, rows_prev, ring_base);
+    if constexpr (kWidth == LQ_MAX_BITS)
+        return quantize_tile_steps<B, kHist, kStat>(p, pc, c, tile, out, prev, ev, rows_cur, rows_prev, ring_base);
+    else
+        return quantize_tile<B, kSearchStep, kHist, kStat>(p, pc, c, tile, out, prev, ev, rows_cur, rows_prev, ring_base);
 }
 
 // The CTA's whole blocks for the layer's code width (kWidth, or `bits` where kWidth is 0) and search; returns the thread's
@@ -150,10 +164,10 @@ __device__ __forceinline__ double quantize_blocks(const PlanDev& p, const Philox
 {
     double stat = 0.0;
     if constexpr (kWidth != 0) {
-        stat = quantize_width<kWidth, kHist, kStat>(p, pc, c, tile, search, out, prev, ev, rows_cur, rows_prev, ring_base);
+        stat = quantize_width<kWidth, kWidth, kHist, kStat>(p, pc, c, tile, search, out, prev, ev, rows_cur, rows_prev, ring_base);
     } else {
         switch (bits) {
-#define LQ_CASE(BB) case BB: stat = quantize_width<BB, kHist, kStat>(p, pc, c, tile, search, out, prev, ev, rows_cur, rows_prev, ring_base); break;
+#define LQ_CASE(BB) case BB: stat = quantize_width<BB, 0, kHist, kStat>(p, pc, c, tile, search, out, prev, ev, rows_cur, rows_prev, ring_base); break;
             LQ_CASE(1) LQ_CASE(2) LQ_CASE(3) LQ_CASE(4) LQ_CASE(5) LQ_CASE(6) LQ_CASE(7) LQ_CASE(8)
 #undef LQ_CASE
             default: break;
