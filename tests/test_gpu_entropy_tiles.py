@@ -75,6 +75,7 @@ def test_overlapping_encodes_stay_in_their_buffers():
     want, mine, theirs = buffers(), buffers(), buffers()
     plan.lq_entropy_encode(packed, want[0][:K], want[1][:K])
     torch.cuda.synchronize()
+    plan.lq_entropy_wait(1 << 12)                            # (a tile whose word was cleared waits for nothing: not for long)
     streams = [torch.cuda.Stream(), torch.cuda.Stream()]
     for _ in range(50):
         for s, (words, offs) in zip(streams, (mine, theirs)):
@@ -83,6 +84,7 @@ def test_overlapping_encodes_stay_in_their_buffers():
     torch.cuda.synchronize()
     for words, offs in (mine, theirs):
         assert bool((words[K] == -1).all()) and bool((offs[K] == -1).all())
+    plan.lq_entropy_wait()
     plan.lq_entropy_status()
     plan.lq_entropy_encode(packed, mine[0][:K], mine[1][:K])
     assert plan.lq_entropy_status() == 0
